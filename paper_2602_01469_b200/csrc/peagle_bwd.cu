@@ -25,23 +25,30 @@ using namespace sm100;
 
 int make_bf16_map(EncodeTiledFn enc, CUtensorMap *m, const void *base, int D, int H, int T);
 int launch_bwd128_main(const CUtensorMap &tmQ, const CUtensorMap &tmdO, const CUtensorMap &tmK,
-                       const CUtensorMap &tmV, const CUtensorMap &tmDQ, const BwdParams &P, int n_sm,
-                       cudaStream_t s);
+                       const CUtensorMap &tmV, const CUtensorMap &tmDQ, const CUtensorMap &tmDK, const CUtensorMap &tmDV,
+                       const BwdParams &P, int n_sm, cudaStream_t s);
 
 // ---------------------------------------------------------------------------------------------
-// head_dim 64.  The MMA warp runs one step ahead of the compute warps
-// inside a work item:
-//   while the compute warps turn S^T(i) into P^T(i):   dK(i-1), dQ(i-1), dP^T(i)
-//   while they turn dP^T(i) into dS^T(i):              dV(i), S^T(i+1)
-// K and V of the item sit in tensor memory as bf16 (A operands of S^T and dP^T), dS^T goes both
-// over the dP^T columns (A operand of dK) and, swizzled, to shared memory (A operand of dQ).
+// head_dim 64.  The query columns of a step are two halves of 64, one per compute warpgroup, with
+// barriers of their own; the second half runs behind the first by the time of an exp phase, so that
+// the exp2 unit serves one half while the other does the rest of its step.  The products run one step
+// ahead of the compute warps:
+//   S^T(i+1) of a half behind its dV(i), once its P^T(i) is in tensor memory
+//   dP^T(i+1) of a half behind its dK(i), once its dS^T(i) is
+//   dQ(i) of both halves, once both dS^T(i) are in shared memory
+// and are issued by three warps (S^T and dV; dP^T and dK; dQ), because one warp that waits for all of
+// these in a fixed order leaves the tensor pipe idle behind every wait (one warp 3.74, three 3.05 ms
+// on the headline shape).
+// K and V of the item sit in tensor memory as bf16 (A operands of S^T and dP^T): a tensor-memory
+// operand leaves half of the shared-memory bandwidth to the other warps, a shared-memory one 5 %.
+// dS^T goes both over the dP^T columns (A operand of dK) and, swizzled, to shared memory (A operand
+// of dQ).  The scores are read as tcgen05.ld.16x256b gives them: a thread has 4 keys x 16 query columns,
+// so that it needs 16 instead of 64 of the row values -LSE and -Delta (a quarter of the loads).
 // The K tile of the next item is prefetched into a second shared-memory stage (V has one stage: it
 // is only read when it is copied to tensor memory at the start of its item); Q / dO have three
-// stages -- with two, a stage is free only when dK of step i has run, and the reload for step i+2
-// can arrive late for S^T(i+2) (3.56 -> 3.53 ms on the headline shape, same GPU, alternating runs); the items come from
-// a global cursor through a small queue.  512 threads: warps 0-7 compute, warp 8 issues
-// MMAs, warp 9 produces, warps 12-15 drain dQ (through a swizzled fp32 tile in shared memory and
-// tiled reduce-adds) and, at the end of an item, dK / dV (global reductions from registers).
+// stages; the items come from a global cursor through a small queue.  512 threads: warps 0-7
+// compute, warps 8, 10 and 11 issue MMAs, warp 9 produces, warps 12-15 drain dQ and, at the end of
+// an item, dK / dV through fp32 panels in shared memory and tiled reduce-adds.
 // The drain has warps of its own because a thread with reductions in flight stalls on its next
 // proxy fence, which the compute warps need once per step for the dS^T hand-over.
 // Registers per thread after the roles re-split the CTA's allocation (512 threads x 128): two
@@ -71,9 +78,10 @@ struct Bwd64Cfg {
     static constexpr int OFF_ROW = OFF_Q + NSQ * 2 * TILE_BYTES;  // ring of (-lse2[128], -delta[128], mq[128])
     static constexpr int ROW_BYTES = 3 * 128 * 4;
     static constexpr int OFF_BAR = OFF_ROW + NSQ * ROW_BYTES;
-    static constexpr int N_BAR = 2 * NSQ + 13 + 4;  // the last four: work-queue slots
-    static constexpr int OFF_MISC = OFF_BAR + N_BAR * 8; // tensor-memory base, abort flag, work queue
-    static constexpr int SMEM_BYTES = OFF_MISC + 32 + 1024;
+    static constexpr int N_BAR = 2 * NSQ + 17 + 4;  // the last four: work-queue slots
+    static constexpr int OFF_MISC = OFF_BAR + N_BAR * 8; // tensor-memory base, abort flag
+    static constexpr int OFF_WQ = (OFF_MISC + 8 + 15) / 16 * 16; // work queue
+    static constexpr int SMEM_BYTES = OFF_WQ + BWD_QUEUE_BYTES + 1024;
     // tensor memory: S^T | dP^T | dQ | K (bf16) | V (bf16) | dK | dV.  P^T (bf16) overwrites the
     // first half of each group's S^T columns and dS^T (bf16) the first half of its dP^T columns.
     static constexpr int TM_S = 0, TM_DP = 128, TM_DQ = 256, TM_K = 320, TM_V = 352, TM_DK = 384,
@@ -83,7 +91,8 @@ struct Bwd64Cfg {
 __global__ void __launch_bounds__(512, 1)
 bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmdO,
              const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-             const __grid_constant__ CUtensorMap tmDQ, const BwdParams P)
+             const __grid_constant__ CUtensorMap tmDQ, const __grid_constant__ CUtensorMap tmDK,
+             const __grid_constant__ CUtensorMap tmDV, const BwdParams P)
 {
     using C = Bwd64Cfg;
     constexpr int D = 64, NSQ = C::NSQ, TB = C::TILE_BYTES;
@@ -94,14 +103,15 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     const uint32_t bar0 = sb + C::OFF_BAR;
     auto BAR = [&](int i) { return bar0 + 8u * (uint32_t)i; };
     constexpr int B_QFULL = 0, B_QEMPTY = NSQ, B_KVFULL = 2 * NSQ, B_KVEMPTY = B_KVFULL + 2,
-                  B_SFULL = B_KVFULL + 4, B_DPFULL = B_KVFULL + 5, B_PFULL = B_KVFULL + 6,
-                  B_DSFULL = B_KVFULL + 7, B_DQFULL = B_KVFULL + 8, B_KVTFULL = B_KVFULL + 9,
-                  B_DQEMPTY = B_KVFULL + 10,
-                  B_ACCFREE = B_KVFULL + 12;
+                  // per half of the query columns (compute warpgroup): [0], [1]
+                  B_SFULL = B_KVFULL + 4, B_DPFULL = B_KVFULL + 6, B_PFULL = B_KVFULL + 8,
+                  B_DSFULL = B_KVFULL + 10, B_DQFULL = B_KVFULL + 12, B_KVTFULL = B_KVFULL + 13,
+                  B_DQEMPTY = B_KVFULL + 14, B_ACCFREE = B_KVFULL + 15,
+                  B_ITEMDONE = B_KVFULL + 16;
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(sp + C::OFF_MISC);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(sp + C::OFF_MISC + 4);
-    volatile int *wq = reinterpret_cast<volatile int *>(sp + C::OFF_MISC + 16);
-    constexpr int B_WQ = 2 * NSQ + 13;
+    uint8_t *wq = sp + C::OFF_WQ;
+    constexpr int B_WQ = 2 * NSQ + 17;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -109,21 +119,23 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         *abort_flag = 0;
         for (int s = 0; s < NSQ; ++s) {
             mbar_init(BAR(B_QFULL + s), 1);
-            mbar_init(BAR(B_QEMPTY + s), 1);
+            mbar_init(BAR(B_QEMPTY + s), 2); // the S^T / dV and the dP^T / dK issuer
         }
         for (int s = 0; s < 4; ++s)
             mbar_init(BAR(B_WQ + s), 1);
         for (int s = 0; s < 2; ++s) {
             mbar_init(BAR(B_KVFULL + s), 1);
             mbar_init(BAR(B_KVEMPTY + s), 1);
-            mbar_init(BAR(B_DQFULL + s), s == 0 ? 1 : 256); // [0] dQ done, [1] = B_KVTFULL
-            mbar_init(BAR(B_DQEMPTY + s), 128);              // [0] used
+            mbar_init(BAR(B_SFULL + s), 1);
+            mbar_init(BAR(B_DPFULL + s), 1);
+            mbar_init(BAR(B_PFULL + s), 4); // one arrival per warp
+            mbar_init(BAR(B_DSFULL + s), 4);
         }
-        mbar_init(BAR(B_SFULL), 1);
-        mbar_init(BAR(B_DPFULL), 1);
-        mbar_init(BAR(B_PFULL), 256);
-        mbar_init(BAR(B_DSFULL), 256);
-        mbar_init(BAR(B_ACCFREE), 128);
+        mbar_init(BAR(B_DQFULL), 1);
+        mbar_init(BAR(B_KVTFULL), 8);
+        mbar_init(BAR(B_DQEMPTY), 4);
+        mbar_init(BAR(B_ITEMDONE), 2);
+        mbar_init(BAR(B_ACCFREE), 4);
         fence_mbar_init();
     }
     if (warp == 8) {
@@ -139,104 +151,85 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         // ------------------------------------------------------------ drain (warps 12-15)
         reg_set<DRAIN_REGS, 128>();
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        const int sub = lane >> 2, cq = 2 * (lane & 3); // row inside a 16-lane load, first column
-        BwdWalk wk;
-        wk.init(P, wq, BAR(B_WQ), abort_flag, false, lane);
-        int2 ktile = make_int2(0, 0);
-        bool ok = true;
-        // adds a [32 lanes x 64 columns] block of tensor memory, scaled, to fp32 rows in global
-        // memory: row_of(lane) gives the destination row pointer or null
-        auto drain_block = [&](uint32_t tcol, float f, auto row_ptr, int barrier) {
-            uint32_t o[2][32];
-            tmem_ld_16x256b_x8(tmem + lane_base + tcol, o[0]);
-            tmem_ld_16x256b_x8(tmem + lane_base + (16u << 16) + tcol, o[1]);
-            tmem_wait_ld();
-            if (barrier >= 0) {
-                tc_fence_before();
-                mbar_arrive(BAR(barrier));
+        // A panel (this warp's 32 lanes, 32 columns) on its way out: registers -> swizzled fp32 tile
+        // in shared memory -> tiled reduce-add.  Whole 128-byte row pieces reach L2 together, which
+        // the L2 takes about 1.6 times faster than the same bytes as scattered 32-byte pieces.  The
+        // panels take two places in turn: while the reduce-add of one reads shared memory the next is
+        // written (a place is free once all but the warp's latest reduce-add have read theirs), and
+        // no warp waits for another.
+        auto send = [&](const uint32_t (&o)[32], float f, int slot, const CUtensorMap *map, int x, int y, int z) {
+            if (lane == 0)
+                bulk_wait_group_read<1>();
+            __syncwarp();
+            uint8_t *dst = sp + C::OFF_DQ + slot * TB + ((warp & 3) * 32 + lane) * 128;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                float4 v;
+                v.x = __uint_as_float(o[4 * c]) * f;
+                v.y = __uint_as_float(o[4 * c + 1]) * f;
+                v.z = __uint_as_float(o[4 * c + 2]) * f;
+                v.w = __uint_as_float(o[4 * c + 3]) * f;
+                *reinterpret_cast<float4 *>(dst + ((c ^ (lane & 7)) << 4)) = v;
             }
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-                float *ra = row_ptr((warp & 3) * 32 + hf * 16 + sub);
-                float *rb = row_ptr((warp & 3) * 32 + hf * 16 + sub + 8);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    if (ra)
-                        red_add_v2(ra + 8 * i + cq, __uint_as_float(o[hf][4 * i]) * f,
-                                   __uint_as_float(o[hf][4 * i + 1]) * f);
-                    if (rb)
-                        red_add_v2(rb + 8 * i + cq, __uint_as_float(o[hf][4 * i + 2]) * f,
-                                   __uint_as_float(o[hf][4 * i + 3]) * f);
-                }
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                tma_reduce_add_3d(map, sb + C::OFF_DQ + slot * TB + (warp & 3) * 4096, x, y, z + (warp & 3) * 32);
+                bulk_commit_group();
             }
         };
-        for (int it = 0; ok && wk.valid; ++it) {
-            if (wk.first())
-                ktile = P.ktile[wk.kt];
-            const int row0 = P.q_begin + wk.qt() * BM;
-            const int h = wk.head();
-            const bool last = wk.last();
-            ok = mbar_wait(BAR(B_DQFULL), it & 1, abort_flag);
+        bool ok = true;
+        int it = 0;
+        BwdItem item;
+        for (int w = 0; ok && bwd_take(wq, BAR(B_WQ), w, abort_flag, item); ++w) {
+        unsigned em = item.mask & 0xffu;
+        for (int i = 0, hh = 0; i < item.steps; ++i, ++it) {
+            const int row0 = (item.qt0 + __ffs(em) - 1) * BM; // row of the partition
+            const int h = item.h0 + hh;
+            if (++hh == item.nh) {
+                hh = 0;
+                em &= em - 1;
+            }
+            ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_DQFULL), it & 1, abort_flag));
+            if (!ok)
+                break;
             tc_fence_after();
-            // dQ(it): tensor memory -> registers -> swizzled fp32 tile in shared memory -> one
-            // tiled reduce-add per 32-column panel.  Whole 256-byte rows reach L2 together, which
-            // the L2 takes about 1.6 times faster than the same bytes as scattered 32-byte pieces.
-            {
-                const int rw = (warp & 3) * 32 + lane; // row of the tile = tensor-memory lane
-                uint32_t o[2][32];
-                tmem_ld32(tmem + lane_base + C::TM_DQ, o[0]);
-                tmem_ld32(tmem + lane_base + C::TM_DQ + 32, o[1]);
-                tmem_wait_ld();
-                tc_fence_before();
-                mbar_arrive(BAR(B_DQEMPTY));
-                if (threadIdx.x == 384)
-                    bulk_wait_group_read<0>(); // the previous tile has left shared memory
-                ok = bar_and(3, 128, ok);      // the four warps go on, or leave, together
-                if (!ok)
-                    break;
+            // dQ(it) (rows past the partition's end are clipped by the tensor map)
+            uint32_t o[2][32];
 #pragma unroll
-                for (int pn = 0; pn < 2; ++pn) {
-                    uint8_t *dst = sp + C::OFF_DQ + pn * TB + rw * 128;
+            for (int pn = 0; pn < 2; ++pn)
+                tmem_ld32(tmem + lane_base + C::TM_DQ + pn * 32, o[pn]);
+            tmem_wait_ld();
+            tc_fence_before();
+            warp_arrive(BAR(B_DQEMPTY));
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        float4 v;
-                        v.x = __uint_as_float(o[pn][4 * c]) * P.scale;
-                        v.y = __uint_as_float(o[pn][4 * c + 1]) * P.scale;
-                        v.z = __uint_as_float(o[pn][4 * c + 2]) * P.scale;
-                        v.w = __uint_as_float(o[pn][4 * c + 3]) * P.scale;
-                        *reinterpret_cast<float4 *>(dst + ((c ^ (rw & 7)) << 4)) = v;
-                    }
-                }
-                fence_proxy_async_smem();
-                asm volatile("bar.sync 3, 128;" ::: "memory");
-                if (threadIdx.x == 384) {
-                    // rows past the partition's end are clipped by the tensor map
-                    tma_reduce_add_3d(&tmDQ, sb + C::OFF_DQ, 0, h, row0 - P.q_begin);
-                    tma_reduce_add_3d(&tmDQ, sb + C::OFF_DQ + TB, 32, h, row0 - P.q_begin);
-                    bulk_commit_group();
-                }
-            }
-            if (last) {
-                // every MMA of the work item is complete (the barrier above covers them all)
-                const int g = wk.g;
-                drain_block(C::TM_DK, P.scale,
-                            [&](int i) -> float * {
-                                return i < ktile.y
-                                           ? P.dK_acc + ((size_t)(ktile.x + i) * P.Hkv + g) * D
-                                           : nullptr;
-                            },
-                            -1);
-                drain_block(C::TM_DV, 1.f,
-                            [&](int i) -> float * {
-                                return i < ktile.y
-                                           ? P.dV_acc + ((size_t)(ktile.x + i) * P.Hkv + g) * D
-                                           : nullptr;
-                            },
-                            B_ACCFREE);
-            }
-            wk.next();
+            for (int pn = 0; pn < 2; ++pn)
+                send(o[pn], P.scale, pn & 1, &tmDQ, 32 * pn, h, row0);
         }
-        if (threadIdx.x == 384)
+        if (!ok)
+            break;
+        // dK and dV of the work item
+        ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_ITEMDONE), w & 1, abort_flag));
+        if (!ok)
+            break;
+        tc_fence_after();
+        // Keys past a ragged tile's end have p = ds = 0, so their rows (of another range) get zeros.
+#pragma unroll
+        for (int t = 0; t < 2; ++t) { // dK, then dV
+            uint32_t o[2][32];
+            tmem_ld32(tmem + lane_base + (t ? C::TM_DV : C::TM_DK), o[0]);
+            tmem_ld32(tmem + lane_base + (t ? C::TM_DV : C::TM_DK) + 32, o[1]);
+            tmem_wait_ld();
+            if (t) {
+                tc_fence_before();
+                warp_arrive(BAR(B_ACCFREE));
+            }
+#pragma unroll
+            for (int pn = 0; pn < 2; ++pn)
+                send(o[pn], t ? 1.f : P.scale, pn, t ? &tmDV : &tmDK, 32 * pn, item.g, item.k_start);
+        }
+        }
+        if (lane == 0)
             bulk_wait_group<0>();
     } else if (warp >= 8) {
         reg_set<ISSUE_REGS, 128>();
@@ -248,157 +241,166 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                 tma_prefetch_desc(&tmK);
                 tma_prefetch_desc(&tmV);
             }
-            BwdWalk wk;
-            wk.init(P, wq, BAR(B_WQ), abort_flag, true, lane);
-            auto load_kv = [&](int w, int kt, int g) -> bool {
+            const BwdSplit split = bwd_split(P);
+            BwdItem item, nxt;
+            auto load_kv = [&](int w, const BwdItem &x) -> bool {
                 bool ok = true;
                 if (lane == 0) {
                     const int s = w & 1;
                     ok = mbar_wait(BAR(B_KVEMPTY + s), ((w >> 1) & 1) ^ 1, abort_flag) &&
                          (w == 0 || mbar_wait(BAR(B_KVTFULL), (w - 1) & 1, abort_flag));
                     if (ok) {
-                        const int start = P.ktile[kt].x;
                         mbar_arrive_expect_tx(BAR(B_KVFULL + s), 2 * TB);
-                        tma_load_3d(sb + C::OFF_KV + s * TB, &tmK, BAR(B_KVFULL + s), 0, g, start);
-                        tma_load_3d(sb + C::OFF_KV + 2 * TB, &tmV, BAR(B_KVFULL + s), 0, g, start);
+                        tma_load_3d(sb + C::OFF_KV + s * TB, &tmK, BAR(B_KVFULL + s), 0, x.g, x.k_start);
+                        tma_load_3d(sb + C::OFF_KV + 2 * TB, &tmV, BAR(B_KVFULL + s), 0, x.g, x.k_start);
                     }
                 }
                 return __all_sync(0xffffffffu, ok);
             };
-            bool ok = true;
-            if (wk.valid)
-                ok = load_kv(0, wk.kt, wk.g);
-            for (int it = 0; ok && wk.valid; ++it) {
-                const int st = it % NSQ, ph = (it / NSQ) & 1;
-                const int row0 = P.q_begin + wk.qt() * BM;
-                const int h = wk.head();
-                ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_QEMPTY + st), ph ^ 1, abort_flag));
-                if (!ok)
-                    break;
-                if (lane == 0) {
-                    mbar_arrive_expect_tx(BAR(B_QFULL + st), 2 * TB + C::ROW_BYTES);
-                    const uint32_t qa = sb + C::OFF_Q + st * 2 * TB;
-                    tma_load_3d(qa, &tmQ, BAR(B_QFULL + st), 0, h, row0);
-                    tma_load_3d(qa + TB, &tmdO, BAR(B_QFULL + st), 0, h, row0);
-                    const uint32_t ra = sb + C::OFF_ROW + st * C::ROW_BYTES;
-                    const size_t ri = (size_t)h * P.q_pad + (size_t)wk.qt() * BM;
-                    bulk_load(ra, P.nl2 + ri, 512, BAR(B_QFULL + st));
-                    bulk_load(ra + 512, P.nd + ri, 512, BAR(B_QFULL + st));
-                    bulk_load(ra + 1024, P.mqp + (size_t)wk.qt() * BM, 512, BAR(B_QFULL + st));
+            int it = 0;
+            bool more = bwd_draw(P, split, wq, BAR(B_WQ), 0, lane, item);
+            bool ok = !more || load_kv(0, item);
+            for (int w = 0; ok && more; ++w) {
+                unsigned em = item.mask & 0xffu;
+                for (int i = 0, hh = 0; i < item.steps; ++i, ++it) {
+                    const int st = it % NSQ, ph = (it / NSQ) & 1;
+                    const int qt = item.qt0 + __ffs(em) - 1, h = item.h0 + hh;
+                    if (++hh == item.nh) {
+                        hh = 0;
+                        em &= em - 1;
+                    }
+                    ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_QEMPTY + st), ph ^ 1, abort_flag));
+                    if (!ok)
+                        break;
+                    if (lane == 0) {
+                        const int row0 = P.q_begin + qt * BM;
+                        mbar_arrive_expect_tx(BAR(B_QFULL + st), 2 * TB + C::ROW_BYTES);
+                        const uint32_t qa = sb + C::OFF_Q + st * 2 * TB;
+                        tma_load_3d(qa, &tmQ, BAR(B_QFULL + st), 0, h, row0);
+                        tma_load_3d(qa + TB, &tmdO, BAR(B_QFULL + st), 0, h, row0);
+                        const uint32_t ra = sb + C::OFF_ROW + st * C::ROW_BYTES;
+                        const size_t ri = (size_t)h * P.q_pad + (size_t)qt * BM;
+                        bulk_load(ra, P.nl2 + ri, 512, BAR(B_QFULL + st));
+                        bulk_load(ra + 512, P.nd + ri, 512, BAR(B_QFULL + st));
+                        bulk_load(ra + 1024, P.mqp + (size_t)qt * BM, 512, BAR(B_QFULL + st));
+                    }
+                    // the next step's Q / dO tiles start towards L2 one step before their stage is
+                    // free; the next item is drawn, and its K / V requested, with the last step
+                    if (i + 1 < item.steps) {
+                        if (lane == 0) {
+                            const int row1 = P.q_begin + (item.qt0 + __ffs(em) - 1) * BM;
+                            tma_prefetch_3d(&tmQ, 0, item.h0 + hh, row1);
+                            tma_prefetch_3d(&tmdO, 0, item.h0 + hh, row1);
+                        }
+                    } else {
+                        more = bwd_draw(P, split, wq, BAR(B_WQ), w + 1, lane, nxt);
+                        if (more)
+                            ok = load_kv(w + 1, nxt);
+                    }
                 }
-                const bool was_last = wk.last();
-                wk.next();
-                // the next step's Q / dO tiles start towards L2 one step before their stage is free
-                if (wk.valid && lane == 0) {
-                    tma_prefetch_3d(&tmQ, 0, wk.head(), P.q_begin + wk.qt() * BM);
-                    tma_prefetch_3d(&tmdO, 0, wk.head(), P.q_begin + wk.qt() * BM);
-                }
-                if (was_last && wk.valid)
-                    ok = load_kv(wk.w, wk.kt, wk.g); // next item's K / V into the other stage
+                item = nxt;
             }
-        } else if (warp == 8) {
-            // -------------------------------------------------------- MMA issue: the whole warp
-            // walks the steps and waits, its elected lane issues (see elect_one)
+        } else {
+            // -------------------------------------------------------- MMA issue: three warps, each
+            // with its own accumulators (products into one accumulator keep one thread's order):
+            // warp 8 S^T and dV, warp 10 dP^T and dK, warp 11 dQ.  The whole warp walks the steps
+            // and waits, its elected lane issues (see elect_one).
             const uint32_t lead = elect_one();
-            constexpr uint32_t IDESC_S = idesc_bf16_f32(128, 128, 0, 0);
+            constexpr uint32_t IDESC_S = idesc_bf16_f32(128, 64, 0, 0);
             constexpr uint32_t IDESC_KV = idesc_bf16_f32(128, D, 0, 1);
             constexpr uint32_t IDESC_DQ = idesc_bf16_f32(128, D, 1, 1);
             // Lower descriptor words (16-byte units).  "k" = K-major operand, "m" = MN-major.
-            const uint32_t ds_k = desc_lo_sw128(sb + C::OFF_DS, 16);
             const uint32_t ds_m = desc_lo_sw128(sb + C::OFF_DS, TB);
-            const uint32_t kv_k = desc_lo_sw128(sb + C::OFF_KV, 16);
             const uint32_t kv_m = desc_lo_sw128(sb + C::OFF_KV, TB);
-            const uint32_t q_k = desc_lo_sw128(sb + C::OFF_Q, 16);
-            const uint32_t q_m = desc_lo_sw128(sb + C::OFF_Q, TB);
             constexpr uint32_t TBU = TB >> 4; // one tile in descriptor units
-            // S^T = K Q^T and dP^T = V dO^T: kv / q are the stage offsets in descriptor units
-            // S^T = K Q^T and dP^T = V dO^T take K / V from tensor memory (one bf16 copy per
-            // work item), so only Q / dO stream from shared memory; q = stage offset in units
-            auto issue_s = [&](uint32_t q) {
+            // warp 8: Q for S^T, dO for dV; warp 10: dO for dP^T, Q for dK
+            const uint32_t b_k = desc_lo_sw128(sb + C::OFF_Q, 16) + (warp == 8 ? 0 : TBU);
+            const uint32_t b_m = desc_lo_sw128(sb + C::OFF_Q, TB) + (warp == 8 ? TBU : 0);
+            const uint32_t t_sc = tmem + (warp == 8 ? C::TM_S : C::TM_DP), t_kv = tmem + (warp == 8 ? C::TM_K : C::TM_V),
+                           t_acc = tmem + (warp == 8 ? C::TM_DV : C::TM_DK);
+            const uint32_t bar_sc = BAR(warp == 8 ? B_SFULL : B_DPFULL), bar_in = BAR(warp == 8 ? B_PFULL : B_DSFULL);
+            // The products of one step, by half h of its query columns (64 each, one compute
+            // warpgroup's); q = offset of the step's Q / dO stage in descriptor units.
+            auto issue_score = [&](uint32_t q, int h) { // S^T = K Q^T / dP^T = V dO^T, K / V in tensor memory
 #pragma unroll
                 for (int k = 0; k < D / 16; ++k)
-                    if (lead) mma_ts_lo(tmem + C::TM_S, tmem + C::TM_K + k * 8, q_k + q + k * 2, IDESC_S, k > 0);
+                    if (lead) mma_ts_lo(t_sc + h * 64, t_kv + k * 8, b_k + q + h * 512 + k * 2, IDESC_S, k > 0);
+                if (lead) tc_commit(bar_sc + 8 * h);
             };
-            auto issue_dp = [&](uint32_t q) {
+            auto issue_acc = [&](uint32_t q, int h, bool acc) { // dV += P^T dO / dK += dS^T Q, 64 query rows
 #pragma unroll
-                for (int k = 0; k < D / 16; ++k)
-                    if (lead) mma_ts_lo(tmem + C::TM_DP, tmem + C::TM_V + k * 8, q_k + q + TBU + k * 2, IDESC_S,
-                              k > 0);
+                for (int k = 0; k < 4; ++k)
+                    if (lead) mma_ts_lo(t_acc, t_sc + h * 64 + k * 8, b_m + q + (h * 4 + k) * 128, IDESC_KV,
+                              acc || k > 0);
             };
-            // The issuing thread is a serial instruction stream, so it keeps its bookkeeping
-            // minimal: per work item only the number of steps (query tiles x heads).
-            const int G = P.Hq / P.Hkv;
             bool ok = true;
             int it = 0, w = 0;
-            for (;; ++w) {
-                // next (work item, KV head) index from the producer's queue
-                if (!mbar_wait(BAR(B_WQ + (w & 3)), (w >> 2) & 1, abort_flag))
-                    break;
-                const int idx = wq[w & 3];
-                if (idx < 0)
-                    break;
-                const int n_cur = P.bitems[idx / P.Hkv].w * G;
+            BwdItem item;
+            for (; bwd_take(wq, BAR(B_WQ), w, abort_flag, item); ++w) {
+                const int n_cur = item.steps;
                 const int ks = w & 1;
-                const uint32_t kvo = ks * TBU;
-                // K / V of this item are in tensor memory (and its K tile in shared memory)
+                if (warp == 11) {
+                    const uint32_t kvo = ks * TBU;
+                    for (int i = 0; ok && i < n_cur; ++i, ++it) {
+                        ok = mbar_wait(BAR(B_DSFULL), it & 1, abort_flag) &&
+                             mbar_wait(BAR(B_DSFULL + 1), it & 1, abort_flag) &&
+                             mbar_wait(BAR(B_DQEMPTY), (it & 1) ^ 1, abort_flag); // the accumulator has been read out
+                        if (!ok)
+                            break;
+                        tc_fence_after();
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            if (lead) mma_ss_lo(tmem + C::TM_DQ, ds_m + k * 128, kv_m + kvo + k * 128, IDESC_DQ, k > 0);
+                        if (lead) tc_commit(BAR(B_DQFULL));
+                    }
+                    if (!ok)
+                        break;
+                    if (lead) tc_commit(BAR(B_KVEMPTY + ks));
+                    continue;
+                }
+                // K / V of this item are in tensor memory
                 ok = mbar_wait(BAR(B_KVTFULL), w & 1, abort_flag) &&
                      mbar_wait(BAR(B_QFULL + it % 3), (it / 3) & 1, abort_flag);
                 if (!ok)
                     break;
                 tc_fence_after();
-                issue_s((it % 3) * 2 * TBU);
-                if (lead) tc_commit(BAR(B_SFULL));
-                issue_dp((it % 3) * 2 * TBU);
-                if (lead) tc_commit(BAR(B_DPFULL));
+                issue_score((it % 3) * 2 * TBU, 0);
+                if (warp == 10)
+                    issue_score((it % 3) * 2 * TBU, 1);
                 for (int i = 0; ok && i < n_cur; ++i, ++it) {
                     const int st = it % 3, nst = (it + 1) % 3;
                     const uint32_t qo = st * 2 * TBU, nqo = nst * 2 * TBU;
                     const bool first = i == 0, last = i == n_cur - 1;
-                    // ---- dV(it) once P^T(it) is in tensor memory, then S^T(it+1)
-                    ok = mbar_wait(BAR(B_PFULL), it & 1, abort_flag);
+                    ok = mbar_wait(bar_in, it & 1, abort_flag);
                     if (ok && first)
                         ok = mbar_wait(BAR(B_ACCFREE), (w & 1) ^ 1, abort_flag);
                     if (!ok)
                         break;
                     tc_fence_after();
-#pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        if (lead) mma_ts_lo(tmem + C::TM_DV, tmem + C::TM_S + (k / 4) * 64 + (k % 4) * 8,
-                                  q_m + qo + TBU + k * 128, IDESC_KV, !first || k > 0);
+                    issue_acc(qo, 0, !first);
+                    // The second warpgroup starts an item one exp phase behind the first, so that
+                    // the exp2 unit serves one while the other does the rest of its step.
+                    if (first && warp == 8)
+                        issue_score(qo, 1);
                     if (!last) {
                         ok = mbar_wait(BAR(B_QFULL + nst), ((it + 1) / 3) & 1, abort_flag);
                         if (!ok)
                             break;
                         tc_fence_after();
-                        issue_s(nqo);
-                        if (lead) tc_commit(BAR(B_SFULL));
+                        issue_score(nqo, 0);
                     }
-                    // ---- dK(it), dQ(it) once dS^T(it) is in tensor and shared memory, then
-                    // dP^T(it+1); the single dQ accumulator must have been read out
-                    ok = mbar_wait(BAR(B_DSFULL), it & 1, abort_flag) &&
-                         mbar_wait(BAR(B_DQEMPTY), (it & 1) ^ 1, abort_flag);
+                    ok = mbar_wait(bar_in + 8, it & 1, abort_flag);
                     if (!ok)
                         break;
                     tc_fence_after();
-#pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        if (lead) mma_ts_lo(tmem + C::TM_DK, tmem + C::TM_DP + (k / 4) * 64 + (k % 4) * 8,
-                                  q_m + qo + k * 128, IDESC_KV, !first || k > 0);
-                    if (lead) tc_commit(BAR(B_QEMPTY + st)); // dQ reads neither Q nor dO
-#pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        if (lead) mma_ss_lo(tmem + C::TM_DQ, ds_m + k * 128, kv_m + kvo + k * 128, IDESC_DQ,
-                                  k > 0);
-                    if (lead) tc_commit(BAR(B_DQFULL));
-                    if (last) {
-                        if (lead) tc_commit(BAR(B_KVEMPTY + ks));
-                    } else {
-                        issue_dp(nqo);
-                        if (lead) tc_commit(BAR(B_DPFULL));
-                    }
+                    issue_acc(qo, 1, true);
+                    if (lead) tc_commit(BAR(B_QEMPTY + st));
+                    if (!last)
+                        issue_score(nqo, 1);
                 }
                 if (!ok)
                     break;
+                if (lead) tc_commit(BAR(B_ITEMDONE));
             }
         }
     } else {
@@ -409,21 +411,28 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         const uint32_t lane_sel = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t tS = tmem + lane_sel + C::TM_S + wg * 64;
         const uint32_t tDP = tmem + lane_sel + C::TM_DP + wg * 64;
-        uint8_t *dsrow = sp + C::OFF_DS + wg * TB + r * 128;
-        BwdWalk wk;
-        wk.init(P, wq, BAR(B_WQ), abort_flag, false, lane);
+        // row of the dS^T tile that this lane addresses in stmatrix_x4 (see there): its row of the
+        // first 16, chunk added per store
+        const uint32_t dsrow = sb + C::OFF_DS + wg * TB + ((warp & 3) * 32 + (lane & 15)) * 128;
         bool ok = true;
-        int32_t mk = META_NONE_K;
-        for (int it = 0; ok && wk.valid; ++it) {
-            const int st = it % NSQ, ph = (it / NSQ) & 1;
-            if (wk.first()) {
-                const int2 ktile = P.ktile[wk.kt];
-                mk = (r < ktile.y) ? P.meta[ktile.x + r] : META_NONE_K;
+        int it = 0, st = 0; // step of this CTA, its Q / dO stage
+        BwdItem item;
+        for (int w = 0; ok && bwd_take(wq, BAR(B_WQ), w, abort_flag, item); ++w) {
+            int32_t mk[4]; // metadata of the keys of this thread's four lanes
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int kl = (warp & 3) * 32 + 8 * i + (lane >> 2);
+                mk[i] = (kl < item.k_len) ? P.meta[item.k_start + kl] : META_NONE_K;
+            }
+            {
                 // New work item: a bf16 copy of K (group 0) / V (group 1) goes to tensor memory,
                 // one row per thread.  Every S^T / dP^T product of the previous item is complete
                 // (their results were consumed in its last step), so the old copy is not in use.
-                const int ks = wk.w & 1;
-                ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_KVFULL + ks), (wk.w >> 1) & 1, abort_flag));
+                const int ks = w & 1;
+                // (The other group's last S^T / dP^T must be complete as well.)
+                ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_KVFULL + ks), (w >> 1) & 1, abort_flag) &&
+                                                 (it == 0 || mbar_wait(BAR(wg == 0 ? B_SFULL + 1 : B_DPFULL),
+                                                                       (it - 1) & 1, abort_flag)));
                 if (!ok)
                     break;
                 const uint8_t *src = sp + C::OFF_KV + (wg == 0 ? ks : 2) * TB + r * 128;
@@ -439,112 +448,113 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                 tmem_st32(tmem + lane_sel + (wg == 0 ? C::TM_K : C::TM_V), kvw);
                 tmem_wait_st();
                 tc_fence_before();
-                mbar_arrive(BAR(B_KVTFULL));
+                warp_arrive(BAR(B_KVTFULL));
             }
-            const bool full = wk.full();
+            for (unsigned em = item.mask & 0xffu; ok && em; em &= em - 1) {
+            const bool full = (item.mask >> (7 + __ffs(em))) & 1u;
+            for (int hh = 0; hh < item.nh; ++hh, ++it, st = st == NSQ - 1 ? 0 : st + 1) {
             const float *rowbuf = reinterpret_cast<const float *>(sp + C::OFF_ROW + st * C::ROW_BYTES);
-            const float4 *nl4 = reinterpret_cast<const float4 *>(rowbuf + wg * 64);
-            const float4 *nd4 = reinterpret_cast<const float4 *>(rowbuf + 128 + wg * 64);
-            const int4 *mq4 = reinterpret_cast<const int4 *>(rowbuf + 256 + wg * 64);
-            // ---- P^T
-            ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_SFULL), it & 1, abort_flag) &&
-                                             mbar_wait(BAR(B_QFULL + st), ph, abort_flag));
+            const float4 *nl4 = reinterpret_cast<const float4 *>(rowbuf + wg * 64) + (lane & 3);
+            const float4 *nd4 = reinterpret_cast<const float4 *>(rowbuf + 128 + wg * 64) + (lane & 3);
+            const int4 *mq4 = reinterpret_cast<const int4 *>(rowbuf + 256 + wg * 64) + (lane & 3);
+            // ---- P^T.  A thread holds 4 key lanes x 16 query columns (tmem_ld_16x256b_x8): for each
+            // group i of 8 columns the columns 8i + 2 (lane % 4) and the next one.
+            // The row values came with the step's Q tile, which the products read: complete.
+            ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_SFULL + wg), it & 1, abort_flag));
             if (!ok)
                 break;
             tc_fence_after();
-            uint32_t sr[2][32];
-            tmem_ld32(tS, sr[0]);
-            tmem_ld32(tS + 32, sr[1]);
-            tmem_wait_ld();
-            float p[64];
+            float4 rv[4]; // row values of the thread's columns
 #pragma unroll
-            for (int c = 0; c < 64; c += 4) {
-                const float4 l = nl4[c >> 2];
-                float a0, a1, a2, a3;
-                fma2(a0, a1, __uint_as_float(sr[c >> 5][(c + 0) & 31]),
-                     __uint_as_float(sr[c >> 5][(c + 1) & 31]), P.scale_log2, P.scale_log2, l.x, l.y);
-                fma2(a2, a3, __uint_as_float(sr[c >> 5][(c + 2) & 31]),
-                     __uint_as_float(sr[c >> 5][(c + 3) & 31]), P.scale_log2, P.scale_log2, l.z, l.w);
-                p[c + 0] = fast_exp2(a0);
-                p[c + 1] = fast_exp2(a1);
-                p[c + 2] = fast_exp2(a2);
-                p[c + 3] = fast_exp2(a3);
-            }
+            for (int m = 0; m < 4; ++m)
+                rv[m] = nl4[4 * m];
+            uint32_t sr[2][32];
+            tmem_ld_16x256b_x8(tS, sr[0]);
+            tmem_ld_16x256b_x8(tS + (16u << 16), sr[1]);
+            tmem_wait_ld();
+            float p[2][32];
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+                    for (int e = 0; e < 8; e += 2) { // group 2m (e < 4) or 2m + 1, lane t/4 or t/4 + 8
+                        const int c = 8 * m + e;
+                        float a0, a1;
+                        fma2(a0, a1, __uint_as_float(sr[hf][c]), __uint_as_float(sr[hf][c + 1]), P.scale_log2,
+                             P.scale_log2, e < 4 ? rv[m].x : rv[m].z, e < 4 ? rv[m].y : rv[m].w);
+                        p[hf][c] = fast_exp2(a0);
+                        p[hf][c + 1] = fast_exp2(a1);
+                    }
             if (!full) {
 #pragma unroll
-                for (int c = 0; c < 64; c += 4) {
-                    const int4 mq = mq4[c >> 2];
-                    if (!allowed_packed(mq.x, mk)) p[c + 0] = 0.f;
-                    if (!allowed_packed(mq.y, mk)) p[c + 1] = 0.f;
-                    if (!allowed_packed(mq.z, mk)) p[c + 2] = 0.f;
-                    if (!allowed_packed(mq.w, mk)) p[c + 3] = 0.f;
+                for (int m = 0; m < 4; ++m) {
+                    const int4 mq = mq4[4 * m];
+#pragma unroll
+                    for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            if (!allowed_packed(e < 4 ? ((e & 1) ? mq.y : mq.x) : ((e & 1) ? mq.w : mq.z),
+                                                mk[2 * hf + ((e >> 1) & 1)]))
+                                p[hf][8 * m + e] = 0.f;
                 }
             }
-            {
-                uint32_t pk[32];
 #pragma unroll
-                for (int i = 0; i < 32; ++i)
-                    pk[i] = pack_bf16x2(p[2 * i], p[2 * i + 1]);
-                tmem_st32(tS, pk); // packed P^T over the first half of this group's S^T columns
+            for (int hf = 0; hf < 2; ++hf) {
+                uint32_t pk[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    pk[i] = pack_bf16x2(p[hf][2 * i], p[hf][2 * i + 1]);
+                // packed P^T over the first half of this group's S^T columns
+                tmem_st_16x128b_x8(tS + ((16u * hf) << 16), pk);
             }
             tmem_wait_st();
             tc_fence_before();
-            mbar_arrive(BAR(B_PFULL));
+            warp_arrive(BAR(B_PFULL + wg));
             // ---- dS^T
-            ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_DPFULL), it & 1, abort_flag));
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+                rv[m] = nd4[4 * m];
+            // (and dQ of the previous step has run, so that the dS^T panel is free)
+            ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_DPFULL + wg), it & 1, abort_flag) &&
+                                             (it == 0 || mbar_wait(BAR(B_DQFULL), (it - 1) & 1, abort_flag)));
             if (!ok)
                 break;
             tc_fence_after();
-            tmem_ld32(tDP, sr[0]);
-            tmem_ld32(tDP + 32, sr[1]);
+            tmem_ld_16x256b_x8(tDP, sr[0]);
+            tmem_ld_16x256b_x8(tDP + (16u << 16), sr[1]);
             tmem_wait_ld();
             tc_fence_before();
-            uint4 dsv[8];
+            uint32_t ds[2][16];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) { // 16-byte chunk j = query columns 8j .. 8j+7
-                const float4 d0 = nd4[2 * j], d1 = nd4[2 * j + 1];
-                const int c = 8 * j;
-                float t0, t1, t2, t3, t4, t5, t6, t7;
-                add2(t0, t1, __uint_as_float(sr[c >> 5][(c + 0) & 31]), __uint_as_float(sr[c >> 5][(c + 1) & 31]), d0.x, d0.y);
-                add2(t2, t3, __uint_as_float(sr[c >> 5][(c + 2) & 31]), __uint_as_float(sr[c >> 5][(c + 3) & 31]), d0.z, d0.w);
-                add2(t4, t5, __uint_as_float(sr[c >> 5][(c + 4) & 31]), __uint_as_float(sr[c >> 5][(c + 5) & 31]), d1.x, d1.y);
-                add2(t6, t7, __uint_as_float(sr[c >> 5][(c + 6) & 31]), __uint_as_float(sr[c >> 5][(c + 7) & 31]), d1.z, d1.w);
-                mul2(t0, t1, t0, t1, p[c + 0], p[c + 1]);
-                mul2(t2, t3, t2, t3, p[c + 2], p[c + 3]);
-                mul2(t4, t5, t4, t5, p[c + 4], p[c + 5]);
-                mul2(t6, t7, t6, t7, p[c + 6], p[c + 7]);
-                dsv[j].x = pack_bf16x2(t0, t1);
-                dsv[j].y = pack_bf16x2(t2, t3);
-                dsv[j].z = pack_bf16x2(t4, t5);
-                dsv[j].w = pack_bf16x2(t6, t7);
-            }
-            // the dS^T buffer is free once dK / dQ of the previous iteration have run
-            if (it > 0) {
-                ok = __all_sync(0xffffffffu,
-                                mbar_wait(BAR(B_DQFULL), (it - 1) & 1, abort_flag));
-                if (!ok)
-                    break;
-            }
-            {
-                // the same dS^T also goes over this group's dP^T columns: operand of dK
-                uint32_t pk[32];
+            for (int m = 0; m < 4; ++m)
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    pk[4 * j] = dsv[j].x;
-                    pk[4 * j + 1] = dsv[j].y;
-                    pk[4 * j + 2] = dsv[j].z;
-                    pk[4 * j + 3] = dsv[j].w;
-                }
-                tmem_st32(tDP, pk);
-            }
+                for (int hf = 0; hf < 2; ++hf)
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                *reinterpret_cast<uint4 *>(dsrow + ((j ^ (r & 7)) << 4)) = dsv[j];
+                    for (int e = 0; e < 8; e += 2) {
+                        const int c = 8 * m + e;
+                        float t0, t1;
+                        add2(t0, t1, __uint_as_float(sr[hf][c]), __uint_as_float(sr[hf][c + 1]),
+                             e < 4 ? rv[m].x : rv[m].z, e < 4 ? rv[m].y : rv[m].w);
+                        mul2(t0, t1, t0, t1, p[hf][c], p[hf][c + 1]);
+                        ds[hf][c >> 1] = pack_bf16x2(t0, t1);
+                    }
+            // the same dS^T goes over this group's dP^T columns (operand of dK) and to shared memory
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf)
+                tmem_st_16x128b_x8(tDP + ((16u * hf) << 16), ds[hf]);
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+                for (int i = 0; i < 8; i += 2) // 16-byte chunks i, i + 1 of 16 rows
+                    stmatrix_x4(dsrow + hf * 2048 + (((i + (lane >> 4)) ^ (lane & 7)) << 4), ds[hf][2 * i],
+                                ds[hf][2 * i + 1], ds[hf][2 * i + 2], ds[hf][2 * i + 3]);
             tmem_wait_st();
             fence_proxy_async_smem();
             tc_fence_before();
-            mbar_arrive(BAR(B_DSFULL));
-            wk.next();
+            warp_arrive(BAR(B_DSFULL + wg));
+            }
+            }
         }
     }
 
@@ -612,10 +622,10 @@ __global__ void bwd_prepare(const __nv_bfloat16 *__restrict__ O, const __nv_bflo
             if (mq == META_NONE_K)
                 mq = META_NONE_Q;
         }
-        nl2[h * (size_t)q_pad + r] = l;
-        nd[h * (size_t)q_pad + r] = real ? -acc : 0.f;
+        nl2[h * (size_t)q_pad + row_slot((int)r)] = l;
+        nd[h * (size_t)q_pad + row_slot((int)r)] = real ? -acc : 0.f;
         if (h == 0)
-            mqp[r] = mq;
+            mqp[row_slot((int)r)] = mq;
     }
 }
 
@@ -666,18 +676,21 @@ static int launch_bwd_t(const Plan &p, const BwdArgs &a, EncodeTiledFn enc, int 
         return PEAGLE_ERR_CUDA;
     const int q_len = p.q_end - p.q_begin;
     const int q_pad = p.n_qt * BM;
-    // fp32 dQ staging [q_len][Hq][D] as a tensor for tiled reduce-adds: 32 columns x 128 rows
-    CUtensorMap tmDQ;
-    {
-        cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)a.Hq, (cuuint64_t)q_len};
-        cuuint64_t strides[2] = {(cuuint64_t)D * 4, (cuuint64_t)a.Hq * D * 4};
-        cuuint32_t box[3] = {32, 1, 128};
+    // fp32 sums as tensors for tiled reduce-adds, 32 columns x 32 rows: the dQ staging
+    // [q_len][Hq][D] and the caller's dK / dV [T][Hkv][D]
+    auto sum_map = [&](CUtensorMap *m, float *base, int H, int rows) {
+        cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)rows};
+        cuuint64_t strides[2] = {(cuuint64_t)D * 4, (cuuint64_t)H * D * 4};
+        cuuint32_t box[3] = {32, 1, 32};
         cuuint32_t estr[3] = {1, 1, 1};
-        if (enc(&tmDQ, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, a.dq_acc, dims, strides, box, estr,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return PEAGLE_ERR_CUDA;
-    }
+        return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, estr,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    CUtensorMap tmDQ, tmDK, tmDV;
+    if (!sum_map(&tmDQ, a.dq_acc, a.Hq, q_len) || !sum_map(&tmDK, a.dK_acc, a.Hkv, p.T) ||
+        !sum_map(&tmDV, a.dV_acc, a.Hkv, p.T))
+        return PEAGLE_ERR_CUDA;
     const size_t n_prep = (size_t)q_len * a.Hq * (D / 8);
     const size_t n_prep_pad = (size_t)q_pad * a.Hq * (D / 8);
     // Per-row values and the initial dQ staging: with SINGLE tiles, their backward does both.
@@ -724,8 +737,8 @@ static int launch_bwd_t(const Plan &p, const BwdArgs &a, EncodeTiledFn enc, int 
         if (ev0)
             cudaEventRecord(ev0, s);
         if (D == 64)
-            bwd64_kernel<<<n_sm, 512, Bwd64Cfg::SMEM_BYTES, s>>>(tmQ, tmdO, tmK, tmV, tmDQ, P);
-        else if (launch_bwd128_main(tmQ, tmdO, tmK, tmV, tmDQ, P, n_sm, s) < 0)
+            bwd64_kernel<<<n_sm, 512, Bwd64Cfg::SMEM_BYTES, s>>>(tmQ, tmdO, tmK, tmV, tmDQ, tmDK, tmDV, P);
+        else if (launch_bwd128_main(tmQ, tmdO, tmK, tmV, tmDQ, tmDK, tmDV, P, n_sm, s) < 0)
             return PEAGLE_ERR_CUDA;
         if (ev1)
             cudaEventRecord(ev1, s);

@@ -6,16 +6,17 @@
 //     warps have read dQ out.
 //   - Shared memory is full with K, V (one stage), the dS^T tile, two stages of Q, ONE stage of dO
 //     (its last reader of a step, dV, runs early in the step and its first reader of the next
-//     step, dP^T, late, so the reload fits between them) and a 32 KB fp32 tile through which dQ
-//     leaves in two halves by tiled reduce-adds (8-byte reductions from registers cost 0.6 of
-//     1.65 ms).  -LSE*log2e and -Delta of a step's rows (1 KB) come in with its Q tile; that
+//     step, dP^T, late, so the reload fits between them) and two fp32 panels of 16 KB through which
+//     dQ, dK and dV leave by tiled reduce-adds.  The fp32 reductions are what bounds the kernel: with
+//     the dQ reduce-adds left out it takes 0.57 instead of 0.71 ms (16,384 tokens, 32 heads), so the
+//     two panels alternate (one tile at a time, 64 columns of all warps together: 0.79 ms).  -LSE*log2e and -Delta of a step's rows (1 KB) come in with its Q tile; that
 //     they fit at all takes the 1 KB usually kept as slack for aligning the tiles, so the kernel
 //     requires a 1024-byte aligned base and reports an error otherwise.  Read from global memory
 //     (broadcast loads, other rows every step) they cost 16 % of the kernel.  The packed metadata
 //     of the rows, needed by the steps that are not FULL, is still read from global memory.
-// Roles (512 threads): warps 0-7 compute (a thread owns one key lane and 64 of the 128 query
-// columns), warp 8 lane 0 issues the MMAs one step ahead (dV(i), S^T(i+1) while the compute warps
-// form dS^T(i); dK(i), dQ(i), then dP^T(i+1) while they form P^T(i+1)), warp 9 produces (TMA),
+// Roles (512 threads): warps 0-7 compute (warp w key lanes 32 (w % 4) .. and half of the 128
+// query columns), warp 8 issues S^T and dV (dV(i), S^T(i+1) while the compute warps form dS^T(i)), warp 10
+// dQ, dK and dP^T (dQ(i), dK(i), then dP^T(i+1) while they form P^T(i+1)), warp 9 produces (TMA),
 // warps 12-15 drain dQ per step and dK / dV per work item.
 #include <math_constants.h>
 
@@ -52,10 +53,11 @@ struct Bwd128Cfg {
     static constexpr int OFF_DO = OFF_Q + NSQ * TILE_BYTES;      // one stage of dO
     static constexpr int OFF_DQ = OFF_DO + TILE_BYTES;           // fp32 dQ half tile on its way out: 2 panels of 32 columns
     static constexpr int OFF_BAR = OFF_DQ + TILE_BYTES;
-    static constexpr int N_BAR = 2 * NSQ + 13 + 4;               // the last four: work-queue slots
-    static constexpr int OFF_MISC = OFF_BAR + N_BAR * 8;         // tensor-memory base, abort flag, queue
+    static constexpr int N_BAR = 2 * NSQ + 14 + 4;               // the last four: work-queue slots
+    static constexpr int OFF_MISC = OFF_BAR + N_BAR * 8;         // tensor-memory base, abort flag
+    static constexpr int OFF_WQ = (OFF_MISC + 8 + 15) / 16 * 16; // work queue
     // per stage of Q: -LSE*log2e and -Delta of the step's 128 query rows (2 x 512 bytes)
-    static constexpr int OFF_ROW = (OFF_MISC + 32 + 15) / 16 * 16;
+    static constexpr int OFF_ROW = OFF_WQ + BWD_QUEUE_BYTES;
     static constexpr int ROW_BYTES = 1024;
     // No slack for alignment is left: the kernel declares its shared memory 1024-byte aligned and
     // leaves with an error if the base is not.
@@ -67,7 +69,8 @@ struct Bwd128Cfg {
 __global__ void __launch_bounds__(512, 1)
 bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmdO,
               const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-              const __grid_constant__ CUtensorMap tmDQ, const BwdParams P)
+              const __grid_constant__ CUtensorMap tmDQ, const __grid_constant__ CUtensorMap tmDK,
+             const __grid_constant__ CUtensorMap tmDV, const BwdParams P)
 {
     using C = Bwd128Cfg;
     constexpr int D = 128, NSQ = C::NSQ, TB = C::TILE_BYTES, PB = C::PANEL_BYTES;
@@ -81,14 +84,15 @@ bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
     }
     const uint32_t bar0 = sb + C::OFF_BAR;
     auto BAR = [&](int i) { return bar0 + 8u * (uint32_t)i; };
-    constexpr int B_QFULL = 0, B_QEMPTY = NSQ, B_KVFULL = 2 * NSQ, B_KVEMPTY = B_KVFULL + 1,
-                  B_SFULL = B_KVFULL + 2, B_DPFULL = B_KVFULL + 3, B_PFULL = B_KVFULL + 4,
-                  B_DSFULL = B_KVFULL + 5, B_DQFULL = B_KVFULL + 6, B_DQEMPTY = B_KVFULL + 7,
-                  B_ACCFREE = B_KVFULL + 8, B_DOFULL = B_KVFULL + 9, B_DOEMPTY = B_KVFULL + 10,
-                  B_WQ = 2 * NSQ + 13;
+    constexpr int B_QFULL = 0, B_QEMPTY = NSQ, B_KFULL = 2 * NSQ, B_KEMPTY = B_KFULL + 1,
+                  B_SFULL = B_KFULL + 2, B_DPFULL = B_KFULL + 3, B_PFULL = B_KFULL + 4,
+                  B_DSFULL = B_KFULL + 5, B_DQFULL = B_KFULL + 6, B_DQEMPTY = B_KFULL + 7,
+                  B_ACCFREE = B_KFULL + 8, B_DOFULL = B_KFULL + 9, B_DOEMPTY = B_KFULL + 10,
+                  B_ITEMDONE = B_KFULL + 11, B_VFULL = B_KFULL + 12, B_VEMPTY = B_KFULL + 13,
+                  B_WQ = B_KFULL + 14;
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(sp + C::OFF_MISC);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(sp + C::OFF_MISC + 4);
-    volatile int *wq = reinterpret_cast<volatile int *>(sp + C::OFF_MISC + 16);
+    uint8_t *wq = sp + C::OFF_WQ;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -100,8 +104,10 @@ bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         }
         for (int s = 0; s < 4; ++s)
             mbar_init(BAR(B_WQ + s), 1);
-        mbar_init(BAR(B_KVFULL), 1);
-        mbar_init(BAR(B_KVEMPTY), 1);
+        mbar_init(BAR(B_KFULL), 1);
+        mbar_init(BAR(B_KEMPTY), 1);
+        mbar_init(BAR(B_VFULL), 1);
+        mbar_init(BAR(B_VEMPTY), 1);
         mbar_init(BAR(B_SFULL), 1);
         mbar_init(BAR(B_DPFULL), 1);
         mbar_init(BAR(B_PFULL), 8);   // one arrival per compute warp
@@ -110,7 +116,8 @@ bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         mbar_init(BAR(B_DQEMPTY), 4); // one arrival per drain warp
         mbar_init(BAR(B_ACCFREE), 4);
         mbar_init(BAR(B_DOFULL), 1);
-        mbar_init(BAR(B_DOEMPTY), 1);
+        mbar_init(BAR(B_DOEMPTY), 2);  // dV and dP^T have read the tile
+        mbar_init(BAR(B_ITEMDONE), 2); // dV and dK are complete
         fence_mbar_init();
     }
     if (warp == 8) {
@@ -126,54 +133,50 @@ bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         // ------------------------------------------------------------ drain (warps 12-15)
         reg_set<DRAIN_REGS, 128>();
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        const int sub = lane >> 2, cq = 2 * (lane & 3); // row inside a 16-lane load, first column
-        BwdWalk wk;
-        wk.init(P, wq, BAR(B_WQ), abort_flag, false, lane);
-        int2 ktile = make_int2(0, 0);
-        bool ok = true;
-        // Adds a [32 lanes x 64 columns] block of tensor memory, scaled, to fp32 rows in global
-        // memory; row_ptr(lane) gives the destination row or null.  A quad of threads holds 32
-        // contiguous bytes of a row, so a reduction instruction covers whole 32-byte sectors.
-        auto drain_block = [&](uint32_t tcol, float f, auto row_ptr, int coff, int barrier) {
-            uint32_t o[2][32];
-            tmem_ld_16x256b_x8(tmem + lane_base + tcol, o[0]);
-            tmem_ld_16x256b_x8(tmem + lane_base + (16u << 16) + tcol, o[1]);
-            tmem_wait_ld();
-            if (barrier >= 0) {
-                tc_fence_before();
-                warp_arrive(BAR(barrier));
+        // A panel (this warp's 32 lanes, 32 columns) on its way out: registers -> swizzled fp32 tile
+        // in shared memory -> tiled reduce-add.  Whole 128-byte row pieces reach L2 together, which
+        // the L2 takes about 1.6 times faster than the same bytes as scattered 32-byte pieces.  The
+        // panels take two places in turn: while the reduce-add of one reads shared memory the next is
+        // written (a place is free once all but the warp's latest reduce-add have read theirs), and
+        // no warp waits for another.
+        auto send = [&](const uint32_t (&o)[32], float f, int slot, const CUtensorMap *map, int x, int y, int z) {
+            if (lane == 0)
+                bulk_wait_group_read<1>();
+            __syncwarp();
+            uint8_t *dst = sp + C::OFF_DQ + slot * PB + ((warp & 3) * 32 + lane) * 128;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                float4 v;
+                v.x = __uint_as_float(o[4 * c]) * f;
+                v.y = __uint_as_float(o[4 * c + 1]) * f;
+                v.z = __uint_as_float(o[4 * c + 2]) * f;
+                v.w = __uint_as_float(o[4 * c + 3]) * f;
+                *reinterpret_cast<float4 *>(dst + ((c ^ (lane & 7)) << 4)) = v;
             }
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-                float *ra = row_ptr((warp & 3) * 32 + hf * 16 + sub);
-                float *rb = row_ptr((warp & 3) * 32 + hf * 16 + sub + 8);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    if (ra)
-                        red_add_v2(ra + coff + 8 * i + cq, __uint_as_float(o[hf][4 * i]) * f,
-                                   __uint_as_float(o[hf][4 * i + 1]) * f);
-                    if (rb)
-                        red_add_v2(rb + coff + 8 * i + cq, __uint_as_float(o[hf][4 * i + 2]) * f,
-                                   __uint_as_float(o[hf][4 * i + 3]) * f);
-                }
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                tma_reduce_add_3d(map, sb + C::OFF_DQ + slot * PB + (warp & 3) * 4096, x, y, z + (warp & 3) * 32);
+                bulk_commit_group();
             }
         };
-        for (int it = 0; ok && wk.valid; ++it) {
-            if (wk.first())
-                ktile = P.ktile[wk.kt];
-            const int row0 = wk.qt() * BM; // row of the partition
-            const int h = wk.head();
-            const bool last = wk.last();
-            const int q_len = P.q_end - P.q_begin;
+        bool ok = true;
+        int it = 0;
+        BwdItem item;
+        for (int w = 0; ok && bwd_take(wq, BAR(B_WQ), w, abort_flag, item); ++w) {
+        unsigned em = item.mask & 0xffu;
+        for (int i = 0, hh = 0; i < item.steps; ++i, ++it) {
+            const int row0 = (item.qt0 + __ffs(em) - 1) * BM; // row of the partition
+            const int h = item.h0 + hh;
+            if (++hh == item.nh) {
+                hh = 0;
+                em &= em - 1;
+            }
             ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_DQFULL), it & 1, abort_flag));
             if (!ok)
                 break;
             tc_fence_after();
-            // dQ(it), one 64-column half at a time: tensor memory -> registers -> swizzled fp32
-            // tile in shared memory -> one tiled reduce-add per 32-column panel (rows past the
-            // partition's end are clipped by the tensor map).  The columns are released as soon
-            // as the second half is in registers.
-            (void)q_len;
+            // dQ(it) (rows past the partition's end are clipped by the tensor map)
             uint32_t o[4][32];
 #pragma unroll
             for (int pn = 0; pn < 4; ++pn)
@@ -182,55 +185,31 @@ bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
             tc_fence_before();
             warp_arrive(BAR(B_DQEMPTY));
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                if (!ok)
-                    break;
-                const int rw = (warp & 3) * 32 + lane; // row of the tile = tensor-memory lane
-                if (threadIdx.x == 384)
-                    bulk_wait_group_read<0>(); // the previous half has left shared memory
-                ok = bar_and(3, 128, ok);      // the four warps go on, or leave, together
-                if (!ok)
-                    break;
-#pragma unroll
-                for (int pn = 0; pn < 2; ++pn) {
-                    uint8_t *dst = sp + C::OFF_DQ + pn * PB + rw * 128;
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        float4 v;
-                        v.x = __uint_as_float(o[2 * half + pn][4 * c]) * P.scale;
-                        v.y = __uint_as_float(o[2 * half + pn][4 * c + 1]) * P.scale;
-                        v.z = __uint_as_float(o[2 * half + pn][4 * c + 2]) * P.scale;
-                        v.w = __uint_as_float(o[2 * half + pn][4 * c + 3]) * P.scale;
-                        *reinterpret_cast<float4 *>(dst + ((c ^ (rw & 7)) << 4)) = v;
-                    }
-                }
-                fence_proxy_async_smem();
-                asm volatile("bar.sync 3, 128;" ::: "memory");
-                if (threadIdx.x == 384) {
-                    tma_reduce_add_3d(&tmDQ, sb + C::OFF_DQ, half * 64, h, row0);
-                    tma_reduce_add_3d(&tmDQ, sb + C::OFF_DQ + PB, half * 64 + 32, h, row0);
-                    bulk_commit_group();
-                }
-            }
-            if (!ok)
-                break;
-            if (last) {
-                // every MMA of the work item is complete (the barrier above covers them all)
-                const int g = wk.g;
-                auto k_row = [&](int i) -> float * {
-                    return i < ktile.y ? P.dK_acc + ((size_t)(ktile.x + i) * P.Hkv + g) * D : nullptr;
-                };
-                auto v_row = [&](int i) -> float * {
-                    return i < ktile.y ? P.dV_acc + ((size_t)(ktile.x + i) * P.Hkv + g) * D : nullptr;
-                };
-                drain_block(C::TM_DK, P.scale, k_row, 0, -1);
-                drain_block(C::TM_DK + 64, P.scale, k_row, 64, -1);
-                drain_block(C::TM_DV, 1.f, v_row, 0, -1);
-                drain_block(C::TM_DV + 64, 1.f, v_row, 64, B_ACCFREE);
-            }
-            wk.next();
+            for (int pn = 0; pn < 4; ++pn)
+                send(o[pn], P.scale, pn & 1, &tmDQ, 32 * pn, h, row0);
         }
-        if (threadIdx.x == 384)
+        if (!ok)
+            break;
+        // dK and dV of the work item
+        ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_ITEMDONE), w & 1, abort_flag));
+        if (!ok)
+            break;
+        tc_fence_after();
+        // Keys past a ragged tile's end have p = ds = 0, so their rows (of another range) get zeros.
+#pragma unroll
+        for (int pn = 0; pn < 8; ++pn) {
+            uint32_t o[32];
+            tmem_ld32(tmem + lane_base + C::TM_DK + pn * 32, o); // dK, then dV
+            tmem_wait_ld();
+            if (pn == 7) {
+                tc_fence_before();
+                warp_arrive(BAR(B_ACCFREE));
+            }
+            const bool k = pn < 4;
+            send(o, k ? P.scale : 1.f, pn & 1, k ? &tmDK : &tmDV, 32 * (pn % 4), item.g, item.k_start);
+        }
+        }
+        if (lane == 0)
             bulk_wait_group<0>();
     } else if (warp >= 8) {
         reg_set<ISSUE_REGS, 128>();
@@ -242,62 +221,59 @@ bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                 tma_prefetch_desc(&tmK);
                 tma_prefetch_desc(&tmV);
             }
-            BwdWalk wk;
-            wk.init(P, wq, BAR(B_WQ), abort_flag, true, lane);
-            // K / V have one stage: the next item's tiles are requested once the last product of
-            // the current item has read them
-            auto load_kv = [&](int w, int kt, int g) -> bool {
-                bool ok = true;
+            const BwdSplit split = bwd_split(P);
+            BwdItem item, nxt;
+            int it = 0;
+            bool more = bwd_draw(P, split, wq, BAR(B_WQ), 0, lane, item), ok = true;
+            // waits for a place to be free, then loads a tile of two panels into it
+            auto load = [&](int empty, uint32_t parity, int full, uint32_t extra, uint32_t dst, const CUtensorMap *map,
+                            int y, int z) -> bool {
+                if (!__all_sync(0xffffffffu, mbar_wait(BAR(empty), parity, abort_flag)))
+                    return false;
                 if (lane == 0) {
-                    ok = mbar_wait(BAR(B_KVEMPTY), (w & 1) ^ 1, abort_flag);
-                    if (ok) {
-                        const int start = P.ktile[kt].x;
-                        mbar_arrive_expect_tx(BAR(B_KVFULL), 2 * TB);
-                        for (int pn = 0; pn < 2; ++pn) {
-                            tma_load_3d(sb + C::OFF_K + pn * PB, &tmK, BAR(B_KVFULL), pn * 64, g, start);
-                            tma_load_3d(sb + C::OFF_V + pn * PB, &tmV, BAR(B_KVFULL), pn * 64, g, start);
-                        }
-                    }
+                    mbar_arrive_expect_tx(BAR(full), TB + extra);
+                    for (int pn = 0; pn < 2; ++pn)
+                        tma_load_3d(dst + pn * PB, map, BAR(full), pn * 64, y, z);
                 }
-                return __all_sync(0xffffffffu, ok);
+                return true;
             };
-            bool ok = true;
-            if (wk.valid)
-                ok = load_kv(0, wk.kt, wk.g);
-            for (int it = 0; ok && wk.valid; ++it) {
-                const int st = it % NSQ, ph = (it / NSQ) & 1;
-                const int row0 = P.q_begin + wk.qt() * BM;
-                const int h = wk.head();
-                ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_QEMPTY + st), ph ^ 1, abort_flag));
-                if (!ok)
-                    break;
-                if (lane == 0) {
-                    mbar_arrive_expect_tx(BAR(B_QFULL + st), TB + C::ROW_BYTES);
-                    const uint32_t qa = sb + C::OFF_Q + st * TB;
-                    for (int pn = 0; pn < 2; ++pn)
-                        tma_load_3d(qa + pn * PB, &tmQ, BAR(B_QFULL + st), pn * 64, h, row0);
-                    const uint32_t ra = sb + C::OFF_ROW + st * C::ROW_BYTES;
-                    const size_t ri = (size_t)h * P.q_pad + (size_t)wk.qt() * BM;
-                    bulk_load(ra, P.nl2 + ri, 512, BAR(B_QFULL + st));
-                    bulk_load(ra + 512, P.nd + ri, 512, BAR(B_QFULL + st));
+            for (int w = 0; ok && more; ++w) {
+                unsigned em = item.mask & 0xffu;
+                for (int i = 0, hh = 0; i < item.steps; ++i, ++it) {
+                    const int st = it % NSQ, ph = (it / NSQ) & 1;
+                    const int qt = item.qt0 + __ffs(em) - 1, h = item.h0 + hh;
+                    const int row0 = P.q_begin + qt * BM;
+                    if (++hh == item.nh) {
+                        hh = 0;
+                        em &= em - 1;
+                    }
+                    // In the order in which the places become free: Q (two stages) after dK of the step
+                    // before the last, V and dO (one stage) after dP^T and dV, K (one stage) after dQ of
+                    // the last step.
+                    ok = load(B_QEMPTY + st, ph ^ 1, B_QFULL + st, C::ROW_BYTES, sb + C::OFF_Q + st * TB, &tmQ, h, row0);
+                    if (!ok)
+                        break;
+                    if (lane == 0) {
+                        const uint32_t ra = sb + C::OFF_ROW + st * C::ROW_BYTES;
+                        const size_t ri = (size_t)h * P.q_pad + (size_t)qt * BM;
+                        bulk_load(ra, P.nl2 + ri, 512, BAR(B_QFULL + st));
+                        bulk_load(ra + 512, P.nd + ri, 512, BAR(B_QFULL + st));
+                    }
+                    ok = (i > 0 || load(B_VEMPTY, (w & 1) ^ 1, B_VFULL, 0, sb + C::OFF_V, &tmV, item.g, item.k_start)) &&
+                         load(B_DOEMPTY, (it & 1) ^ 1, B_DOFULL, 0, sb + C::OFF_DO, &tmdO, h, row0) &&
+                         (i > 0 || load(B_KEMPTY, (w & 1) ^ 1, B_KFULL, 0, sb + C::OFF_K, &tmK, item.g, item.k_start));
+                    if (!ok)
+                        break;
+                    if (i + 1 == item.steps)
+                        more = bwd_draw(P, split, wq, BAR(B_WQ), w + 1, lane, nxt);
                 }
-                // dO has one stage: free once dV of the previous step has run
-                ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_DOEMPTY), (it & 1) ^ 1, abort_flag));
-                if (!ok)
-                    break;
-                if (lane == 0) {
-                    mbar_arrive_expect_tx(BAR(B_DOFULL), TB);
-                    for (int pn = 0; pn < 2; ++pn)
-                        tma_load_3d(sb + C::OFF_DO + pn * PB, &tmdO, BAR(B_DOFULL), pn * 64, h, row0);
-                }
-                const bool was_last = wk.last();
-                wk.next();
-                if (was_last && wk.valid)
-                    ok = load_kv(wk.w, wk.kt, wk.g);
+                item = nxt;
             }
-        } else if (warp == 8) {
-            // -------------------------------------------------------- MMA issue: the whole warp
-            // walks the steps and waits, its elected lane issues (see elect_one)
+        } else if (warp == 8 || warp == 10) {
+            // -------------------------------------------------------- MMA issue: two warps, each with
+            // its own accumulators (products into one accumulator keep one thread's order): warp 8
+            // S^T and dV, warp 10 dQ, dK and dP^T.  The whole warp walks the steps and waits, its
+            // elected lane issues (see elect_one).
             const uint32_t lead = elect_one();
             constexpr uint32_t IDESC_S = idesc_bf16_f32(128, 128, 0, 0);
             constexpr uint32_t IDESC_KV = idesc_bf16_f32(128, D, 0, 1);
@@ -316,196 +292,241 @@ bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
 #pragma unroll
                 for (int k = 0; k < D / 16; ++k)
                     if (lead) mma_ss_lo(tmem + C::TM_S, k_k + koff(k), q_k + q + koff(k), IDESC_S, k > 0);
+                if (lead) tc_commit(BAR(B_SFULL));
             };
             auto issue_dp = [&]() { // dP^T = V dO^T
 #pragma unroll
                 for (int k = 0; k < D / 16; ++k)
                     if (lead) mma_ss_lo(tmem + C::TM_DP, v_k + koff(k), do_k + koff(k), IDESC_S, k > 0);
-            };
-            const int G = P.Hq / P.Hkv;
-            bool ok = true;
-            int it = 0, w = 0;
-            for (;; ++w) {
-                if (!mbar_wait(BAR(B_WQ + (w & 3)), (w >> 2) & 1, abort_flag))
-                    break;
-                const int idx = wq[w & 3];
-                if (idx < 0)
-                    break;
-                const int n_cur = P.bitems[idx / P.Hkv].w * G;
-                ok = mbar_wait(BAR(B_KVFULL), w & 1, abort_flag) &&
-                     mbar_wait(BAR(B_QFULL + (it & 1)), (it >> 1) & 1, abort_flag) &&
-                     mbar_wait(BAR(B_DOFULL), it & 1, abort_flag);
-                // dQ of the previous item's last step must have left the dP^T columns
-                if (ok && it > 0)
-                    ok = mbar_wait(BAR(B_DQEMPTY), (it - 1) & 1, abort_flag);
-                if (!ok)
-                    break;
-                tc_fence_after();
-                issue_s((it & 1) * TBU);
-                if (lead) tc_commit(BAR(B_SFULL));
-                issue_dp();
                 if (lead) tc_commit(BAR(B_DPFULL));
-                for (int i = 0; ok && i < n_cur; ++i, ++it) {
-                    const int st = it & 1, nst = st ^ 1;
-                    static_assert(NSQ == 2, "stage = step parity");
-                    const uint32_t qo = st * TBU, nqo = nst * TBU;
-                    const bool first = i == 0, last = i == n_cur - 1;
-                    // ---- dV(it) once P^T(it) is in tensor memory, then S^T(it+1)
-                    ok = mbar_wait(BAR(B_PFULL), it & 1, abort_flag);
-                    if (ok && first)
-                        ok = mbar_wait(BAR(B_ACCFREE), (w & 1) ^ 1, abort_flag);
-                    if (!ok)
-                        break;
+                if (lead) tc_commit(BAR(B_DOEMPTY));
+            };
+            static_assert(NSQ == 2, "stage = step parity");
+            bool ok = true;
+            int it = 0;
+            BwdItem item, nxt;
+            bool have = bwd_take(wq, BAR(B_WQ), 0, abort_flag, item);
+            // The steps of consecutive items follow one another like the steps of one item: the next
+            // item's first S^T / dP^T is issued behind the last dV / dK of this one.
+            if (warp == 8) {
+                auto next_s = [&](int j, int w, bool first) { // S^T of step j, the first of item w or not
+                    if ((first && !mbar_wait(BAR(B_KFULL), w & 1, abort_flag)) ||
+                        !mbar_wait(BAR(B_QFULL + (j & 1)), (j >> 1) & 1, abort_flag))
+                        return false;
                     tc_fence_after();
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) // query rows 16k..16k+15 of P^T (bf16 over S^T)
-                        if (lead) mma_ts_lo(tmem + C::TM_DV, tmem + C::TM_S + (k / 4) * 64 + (k % 4) * 8,
-                                  do_m + k * 128, IDESC_KV, !first || k > 0);
-                    if (lead) tc_commit(BAR(B_DOEMPTY)); // dV is the step's last product with dO
-                    if (!last) {
-                        ok = mbar_wait(BAR(B_QFULL + nst), ((it + 1) >> 1) & 1, abort_flag);
+                    issue_s((j & 1) * TBU);
+                    return true;
+                };
+                if (have)
+                    ok = next_s(0, 0, true);
+                for (int w = 0; ok && have; ++w) {
+                    bool have_n = false;
+                    for (int i = 0; i < item.steps; ++i, ++it) {
+                        // ---- dV(it) once P^T(it) is in tensor memory (and dO in shared memory), then
+                        // S^T(it+1)
+                        ok = mbar_wait(BAR(B_PFULL), it & 1, abort_flag) && mbar_wait(BAR(B_DOFULL), it & 1, abort_flag);
+                        if (ok && i == 0)
+                            ok = mbar_wait(BAR(B_ACCFREE), (w & 1) ^ 1, abort_flag);
                         if (!ok)
                             break;
                         tc_fence_after();
-                        issue_s(nqo);
-                        if (lead) tc_commit(BAR(B_SFULL));
-                    }
-                    // ---- dK(it), dQ(it) once dS^T(it) is in shared memory (the compute warps then
-                    // hold dP^T(it) in registers: dQ goes over its columns)
-                    ok = mbar_wait(BAR(B_DSFULL), it & 1, abort_flag);
-                    if (!ok)
-                        break;
-                    tc_fence_after();
 #pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        if (lead) mma_ss_lo(tmem + C::TM_DK, ds_k + koff(k), q_m + qo + k * 128, IDESC_KV,
-                                  !first || k > 0);
-                    if (lead) tc_commit(BAR(B_QEMPTY + st)); // dQ reads neither Q nor dO
-#pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        if (lead) mma_ss_lo(tmem + C::TM_DQ, ds_m + k * 128, k_m + k * 128, IDESC_DQ, k > 0);
-                    if (lead) tc_commit(BAR(B_DQFULL));
-                    if (last) {
-                        if (lead) tc_commit(BAR(B_KVEMPTY));
-                    } else {
-                        // ---- dP^T(it+1) over the columns dQ(it) has just left
-                        ok = mbar_wait(BAR(B_DQEMPTY), it & 1, abort_flag) &&
-                             mbar_wait(BAR(B_DOFULL), (it + 1) & 1, abort_flag);
+                        for (int k = 0; k < 8; ++k) // query rows 16k..16k+15 of P^T (bf16 over S^T)
+                            if (lead) mma_ts_lo(tmem + C::TM_DV, tmem + C::TM_S + (k / 4) * 64 + (k % 4) * 8,
+                                      do_m + k * 128, IDESC_KV, i > 0 || k > 0);
+                        if (lead) tc_commit(BAR(B_DOEMPTY));
+                        const bool last = i + 1 == item.steps;
+                        if (last) {
+                            if (lead) tc_commit(BAR(B_ITEMDONE));
+                            have_n = bwd_take(wq, BAR(B_WQ), w + 1, abort_flag, nxt);
+                        }
+                        if (!last || have_n)
+                            ok = next_s(it + 1, w + 1, last);
                         if (!ok)
                             break;
-                        tc_fence_after();
-                        issue_dp();
-                        if (lead) tc_commit(BAR(B_DPFULL));
                     }
+                    item = nxt;
+                    have = have_n;
                 }
-                if (!ok)
-                    break;
+            } else {
+                auto next_dp = [&](int j, int w, bool first) { // dP^T of step j, over the columns dQ(j-1) has left
+                    if ((first && !mbar_wait(BAR(B_VFULL), w & 1, abort_flag)) ||
+                        (j > 0 && !mbar_wait(BAR(B_DQEMPTY), (j - 1) & 1, abort_flag)) ||
+                        !mbar_wait(BAR(B_DOFULL), j & 1, abort_flag))
+                        return false;
+                    tc_fence_after();
+                    issue_dp();
+                    return true;
+                };
+                if (have) {
+                    ok = next_dp(0, 0, true);
+                    if (item.steps == 1)
+                        if (lead) tc_commit(BAR(B_VEMPTY));
+                }
+                for (int w = 0; ok && have; ++w) {
+                    bool have_n = false;
+                    for (int i = 0; i < item.steps; ++i, ++it) {
+                        // ---- dQ(it), dK(it) once dS^T(it) is in shared memory (the compute warps then
+                        // hold dP^T(it) in registers: dQ goes over its columns).  dQ first: dP^T(it+1)
+                        // waits for the drain to read it out, dK runs meanwhile.
+                        const bool last = i + 1 == item.steps;
+                        ok = mbar_wait(BAR(B_DSFULL), it & 1, abort_flag);
+                        if (ok && i == 0)
+                            ok = mbar_wait(BAR(B_ACCFREE), (w & 1) ^ 1, abort_flag);
+                        if (!ok)
+                            break;
+                        tc_fence_after();
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            if (lead) mma_ss_lo(tmem + C::TM_DQ, ds_m + k * 128, k_m + k * 128, IDESC_DQ, k > 0);
+                        if (lead) tc_commit(BAR(B_DQFULL));
+                        if (last)
+                            if (lead) tc_commit(BAR(B_KEMPTY));
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            if (lead) mma_ss_lo(tmem + C::TM_DK, ds_k + koff(k), q_m + (it & 1) * TBU + k * 128, IDESC_KV,
+                                      i > 0 || k > 0);
+                        if (lead) tc_commit(BAR(B_QEMPTY + (it & 1)));
+                        if (last) {
+                            if (lead) tc_commit(BAR(B_ITEMDONE));
+                            have_n = bwd_take(wq, BAR(B_WQ), w + 1, abort_flag, nxt);
+                        }
+                        if (!last || have_n) {
+                            ok = next_dp(it + 1, w + 1, last);
+                            // the item's last dP^T: V may be replaced behind it
+                            if (last ? nxt.steps == 1 : i + 2 == item.steps)
+                                if (lead) tc_commit(BAR(B_VEMPTY));
+                        }
+                        if (!ok)
+                            break;
+                    }
+                    item = nxt;
+                    have = have_n;
+                }
             }
         }
     } else {
         reg_set<COMPUTE_REGS, 128>();
         // ------------------------------------------------------------ compute (warps 0-7)
         const int wg = warp >> 2;        // half of the query columns
-        const int r = threadIdx.x & 127; // key lane
         const uint32_t lane_sel = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t tS = tmem + lane_sel + C::TM_S + wg * 64;
         const uint32_t tDP = tmem + lane_sel + C::TM_DP + wg * 64;
-        uint8_t *dsrow = sp + C::OFF_DS + wg * PB + r * 128;
-        BwdWalk wk;
-        wk.init(P, wq, BAR(B_WQ), abort_flag, false, lane);
+        // row of the dS^T tile that this lane addresses in stmatrix_x4 (see there): its row of the
+        // first 16, chunk added per store
+        const uint32_t dsrow = sb + C::OFF_DS + wg * PB + ((warp & 3) * 32 + (lane & 15)) * 128;
         bool ok = true;
-        int32_t mk = META_NONE_K;
-        for (int it = 0; ok && wk.valid; ++it) {
-            if (wk.first()) {
-                const int2 ktile = P.ktile[wk.kt];
-                mk = (r < ktile.y) ? P.meta[ktile.x + r] : META_NONE_K;
+        int it = 0;
+        BwdItem item;
+        for (int w = 0; ok && bwd_take(wq, BAR(B_WQ), w, abort_flag, item); ++w) {
+            int32_t mk[4]; // metadata of the keys of this thread's four lanes
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int kl = (warp & 3) * 32 + 8 * i + (lane >> 2);
+                mk[i] = (kl < item.k_len) ? P.meta[item.k_start + kl] : META_NONE_K;
             }
-            const bool full = wk.full();
+            for (unsigned em = item.mask & 0xffu; ok && em; em &= em - 1) {
+            const int qt = item.qt0 + __ffs(em) - 1;
+            const bool full = (item.mask >> (7 + __ffs(em))) & 1u;
+            for (int hh = 0; hh < item.nh; ++hh, ++it) {
             // per-row values of this step's 64 query columns
-            const size_t rb = (size_t)wk.qt() * BM + wg * 64;
+            const size_t rb = (size_t)qt * BM + wg * 64;
             const uint8_t *rowv = sp + C::OFF_ROW + (it % NSQ) * C::ROW_BYTES + wg * 256;
-            const float4 *nl4 = reinterpret_cast<const float4 *>(rowv);
-            const float4 *nd4 = reinterpret_cast<const float4 *>(rowv + 512);
-            const int4 *mq4 = reinterpret_cast<const int4 *>(P.mqp + rb);
-            // The metadata of the next query tile is sent towards L1 now (read by the steps that are
-            // not FULL; every thread of a column group reads the same 64 values, broadcast loads)
-            {
-                int qn, hn;
-                if (lane < 2 && wk.peek(qn, hn) && qn != wk.qt())
-                    asm volatile("prefetch.global.L1 [%0];" ::"l"(P.mqp + (size_t)qn * BM + wg * 64 + lane * 32));
-            }
-            // ---- P^T (the row values arrive with the step's Q tile)
-            ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_SFULL), it & 1, abort_flag) &&
-                                             mbar_wait(BAR(B_QFULL + it % NSQ), (it / NSQ) & 1, abort_flag));
+            const float4 *nl4 = reinterpret_cast<const float4 *>(rowv) + (lane & 3);
+            const float4 *nd4 = reinterpret_cast<const float4 *>(rowv + 512) + (lane & 3);
+            const int4 *mq4 = reinterpret_cast<const int4 *>(P.mqp + rb) + (lane & 3);
+            // ---- P^T (the row values arrive with the step's Q tile).  A thread holds 4 key lanes x
+            // 16 query columns, as in bwd64_kernel.
+            // The row values came with the step's Q tile, which the products read: complete.
+            ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_SFULL), it & 1, abort_flag));
             if (!ok)
                 break;
             tc_fence_after();
-            uint32_t sr[2][32];
-            tmem_ld32(tS, sr[0]);
-            tmem_ld32(tS + 32, sr[1]);
-            tmem_wait_ld();
-            float p[64];
+            float4 rv[4]; // row values of the thread's columns
 #pragma unroll
-            for (int c = 0; c < 64; c += 4) {
-                const float4 l = nl4[c >> 2];
-                p[c + 0] = fast_exp2(fmaf(__uint_as_float(sr[c >> 5][(c + 0) & 31]), P.scale_log2, l.x));
-                p[c + 1] = fast_exp2(fmaf(__uint_as_float(sr[c >> 5][(c + 1) & 31]), P.scale_log2, l.y));
-                p[c + 2] = fast_exp2(fmaf(__uint_as_float(sr[c >> 5][(c + 2) & 31]), P.scale_log2, l.z));
-                p[c + 3] = fast_exp2(fmaf(__uint_as_float(sr[c >> 5][(c + 3) & 31]), P.scale_log2, l.w));
-            }
+            for (int m = 0; m < 4; ++m)
+                rv[m] = nl4[4 * m];
+            uint32_t sr[2][32];
+            tmem_ld_16x256b_x8(tS, sr[0]);
+            tmem_ld_16x256b_x8(tS + (16u << 16), sr[1]);
+            tmem_wait_ld();
+            float p[2][32];
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+                    for (int e = 0; e < 8; e += 2) { // group 2m (e < 4) or 2m + 1, lane t/4 or t/4 + 8
+                        const int c = 8 * m + e;
+                        float a0, a1;
+                        fma2(a0, a1, __uint_as_float(sr[hf][c]), __uint_as_float(sr[hf][c + 1]), P.scale_log2,
+                             P.scale_log2, e < 4 ? rv[m].x : rv[m].z, e < 4 ? rv[m].y : rv[m].w);
+                        p[hf][c] = fast_exp2(a0);
+                        p[hf][c + 1] = fast_exp2(a1);
+                    }
             if (!full) {
 #pragma unroll
-                for (int c = 0; c < 64; c += 4) {
-                    const int4 mq = __ldg(mq4 + (c >> 2));
-                    if (!allowed_packed(mq.x, mk)) p[c + 0] = 0.f;
-                    if (!allowed_packed(mq.y, mk)) p[c + 1] = 0.f;
-                    if (!allowed_packed(mq.z, mk)) p[c + 2] = 0.f;
-                    if (!allowed_packed(mq.w, mk)) p[c + 3] = 0.f;
+                for (int m = 0; m < 4; ++m) {
+                    const int4 mq = __ldg(mq4 + 4 * m);
+#pragma unroll
+                    for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            if (!allowed_packed(e < 4 ? ((e & 1) ? mq.y : mq.x) : ((e & 1) ? mq.w : mq.z),
+                                                mk[2 * hf + ((e >> 1) & 1)]))
+                                p[hf][8 * m + e] = 0.f;
                 }
             }
-            {
-                uint32_t pk[32];
 #pragma unroll
-                for (int i = 0; i < 32; ++i)
-                    pk[i] = pack_bf16x2(p[2 * i], p[2 * i + 1]);
-                tmem_st32(tS, pk); // packed P^T over the first half of this group's S^T columns
+            for (int hf = 0; hf < 2; ++hf) {
+                uint32_t pk[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    pk[i] = pack_bf16x2(p[hf][2 * i], p[hf][2 * i + 1]);
+                // packed P^T over the first half of this group's S^T columns
+                tmem_st_16x128b_x8(tS + ((16u * hf) << 16), pk);
             }
             tmem_wait_st();
             tc_fence_before();
             warp_arrive(BAR(B_PFULL));
             // ---- dS^T
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+                rv[m] = nd4[4 * m];
+            // (and dQ and dK of the previous step have run: their warp issues dP^T behind them, so
+            // the dS^T tile is free)
             ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_DPFULL), it & 1, abort_flag));
             if (!ok)
                 break;
             tc_fence_after();
-            tmem_ld32(tDP, sr[0]);
-            tmem_ld32(tDP + 32, sr[1]);
+            tmem_ld_16x256b_x8(tDP, sr[0]);
+            tmem_ld_16x256b_x8(tDP + (16u << 16), sr[1]);
             tmem_wait_ld();
             tc_fence_before();
-            // the dS^T tile is free once dK / dQ of the previous step have run
-            if (it > 0) {
-                ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_DQFULL), (it - 1) & 1, abort_flag));
-                if (!ok)
-                    break;
-            }
+            uint32_t ds[2][16];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) { // 16-byte chunk j = query columns 8j .. 8j+7 of this half
-                const float4 d0 = nd4[2 * j], d1 = nd4[2 * j + 1];
-                const int c = 8 * j;
-                uint4 v;
-                v.x = pack_bf16x2(p[c + 0] * (__uint_as_float(sr[c >> 5][(c + 0) & 31]) + d0.x),
-                                  p[c + 1] * (__uint_as_float(sr[c >> 5][(c + 1) & 31]) + d0.y));
-                v.y = pack_bf16x2(p[c + 2] * (__uint_as_float(sr[c >> 5][(c + 2) & 31]) + d0.z),
-                                  p[c + 3] * (__uint_as_float(sr[c >> 5][(c + 3) & 31]) + d0.w));
-                v.z = pack_bf16x2(p[c + 4] * (__uint_as_float(sr[c >> 5][(c + 4) & 31]) + d1.x),
-                                  p[c + 5] * (__uint_as_float(sr[c >> 5][(c + 5) & 31]) + d1.y));
-                v.w = pack_bf16x2(p[c + 6] * (__uint_as_float(sr[c >> 5][(c + 6) & 31]) + d1.z),
-                                  p[c + 7] * (__uint_as_float(sr[c >> 5][(c + 7) & 31]) + d1.w));
-                *reinterpret_cast<uint4 *>(dsrow + ((j ^ (r & 7)) << 4)) = v;
-            }
+            for (int m = 0; m < 4; ++m)
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+                    for (int e = 0; e < 8; e += 2) {
+                        const int c = 8 * m + e;
+                        float t0, t1;
+                        add2(t0, t1, __uint_as_float(sr[hf][c]), __uint_as_float(sr[hf][c + 1]),
+                             e < 4 ? rv[m].x : rv[m].z, e < 4 ? rv[m].y : rv[m].w);
+                        mul2(t0, t1, t0, t1, p[hf][c], p[hf][c + 1]);
+                        ds[hf][c >> 1] = pack_bf16x2(t0, t1);
+                    }
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+                for (int i = 0; i < 8; i += 2) // 16-byte chunks i, i + 1 of 16 rows
+                    stmatrix_x4(dsrow + hf * 2048 + (((i + (lane >> 4)) ^ (lane & 7)) << 4), ds[hf][2 * i],
+                                ds[hf][2 * i + 1], ds[hf][2 * i + 2], ds[hf][2 * i + 3]);
             fence_proxy_async_smem();
             warp_arrive(BAR(B_DSFULL));
-            wk.next();
+            }
+            }
         }
     }
 
@@ -528,14 +549,14 @@ bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
 }
 
 int launch_bwd128_main(const CUtensorMap &tmQ, const CUtensorMap &tmdO, const CUtensorMap &tmK,
-                       const CUtensorMap &tmV, const CUtensorMap &tmDQ, const BwdParams &P, int n_sm,
-                       cudaStream_t s)
+                       const CUtensorMap &tmV, const CUtensorMap &tmDQ, const CUtensorMap &tmDK, const CUtensorMap &tmDV,
+                       const BwdParams &P, int n_sm, cudaStream_t s)
 {
     // per device, so set before every launch (host time only)
     if (cudaFuncSetAttribute(bwd128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              Bwd128Cfg::SMEM_BYTES) != cudaSuccess)
         return PEAGLE_ERR_CUDA;
-    bwd128_kernel<<<n_sm, 512, Bwd128Cfg::SMEM_BYTES, s>>>(tmQ, tmdO, tmK, tmV, tmDQ, P);
+    bwd128_kernel<<<n_sm, 512, Bwd128Cfg::SMEM_BYTES, s>>>(tmQ, tmdO, tmK, tmV, tmDQ, tmDK, tmDV, P);
     return 1;
 }
 

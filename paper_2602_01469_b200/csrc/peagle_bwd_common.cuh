@@ -22,99 +22,98 @@ struct BwdParams {
     float scale, scale_log2;
 };
 
-// Walks the (work item, query tile, head) iterations of one CTA in execution order.  Work items
-// are handed out dynamically: the producer warp takes the next (item, KV head) index from a global
-// cursor and publishes it in a four-slot queue in shared memory; the other roles read it there.
-// A CTA that falls behind therefore takes fewer items, and the CTAs running at any time work on a
-// contiguous window of the chunk-major item list (their shared Q / dO rows and dQ staging rows
-// stay in L2), instead of drifting apart as with a static round-robin.
-struct BwdWalk {
-    const int4 *bitems;
-    int *cursor;
-    volatile int *wq;
-    volatile int *abort;
-    uint32_t wqbar;
-    int idx, total, Hkv, G, lane;
-    bool fetcher;
-    int kt, g, c, w;
-    unsigned mask, em;
-    int hh;
-    bool valid;
-    __device__ void load()
-    {
-        const int slot = w & 3;
-        if (fetcher) { // the whole producer warp, convergent
-            int v = 0;
-            if (lane == 0)
-                v = atomicAdd(cursor, 1);
-            v = __shfl_sync(0xffffffffu, v, 0);
-            idx = v < total ? v : -1;
-            if (lane == 0) {
-                wq[slot] = idx;
-                sm100::mbar_arrive(wqbar + 8u * slot);
-            }
-        } else {
-            // slot w & 3 was last used four items ago; no role is more than two items behind
-            idx = sm100::mbar_wait(wqbar + 8u * slot, (w >> 2) & 1, abort) ? wq[slot] : -1;
-        }
-        valid = idx >= 0;
-        if (!valid)
-            return;
-        const int4 item = bitems[idx / Hkv];
-        g = idx % Hkv;
-        kt = item.x;
-        c = item.y;
-        mask = (unsigned)item.z;
-        em = mask & 0xffu;
-        hh = 0;
-    }
-    __device__ void init(const BwdParams &P, volatile int *queue, uint32_t queue_bar,
-                         volatile int *abort_flag, bool is_fetcher, int lane_id)
-    {
-        bitems = P.bitems;
-        cursor = P.cursor;
-        wq = queue;
-        wqbar = queue_bar;
-        abort = abort_flag;
-        fetcher = is_fetcher;
-        lane = lane_id;
-        Hkv = P.Hkv;
-        G = P.Hq / P.Hkv;
-        total = P.counters[1] * P.Hkv;
-        w = 0;
-        load();
-    }
-    __device__ bool first() const { return hh == 0 && em == (mask & 0xffu); }
-    __device__ bool last() const { return hh == G - 1 && (em & (em - 1)) == 0; }
-    __device__ int qt() const { return c * BWD_CQ + (__ffs(em) - 1); }
-    __device__ bool full() const { return (mask >> (8 + __ffs(em) - 1)) & 1u; }
-    __device__ int head() const { return g * G + hh; }
-    // (query tile, head) of the step after this one, if it belongs to the same work item
-    __device__ bool peek(int &qt_next, int &head_next) const
-    {
-        if (hh + 1 < G) {
-            qt_next = qt();
-            head_next = g * G + hh + 1;
-            return true;
-        }
-        const unsigned rest = em & (em - 1);
-        if (rest == 0)
-            return false;
-        qt_next = c * BWD_CQ + (__ffs(rest) - 1);
-        head_next = g * G;
-        return true;
-    }
-    __device__ void next()
-    {
-        if (++hh == G) {
-            hh = 0;
-            em &= em - 1;
-            if (em == 0) {
-                ++w;
-                load();
-            }
-        }
-    }
+// Work items are handed out dynamically: the producer warp takes the next index from a global cursor
+// and publishes what the other roles need of the item in a four-slot queue in shared memory (slot
+// w & 3 for the CTA's item w; it was last used four items ago, and no role is more than two items
+// behind).  A CTA that falls behind therefore takes fewer items, and the CTAs running at any time
+// work on a contiguous window of the chunk-major item list (their shared Q / dO rows and dQ staging
+// rows stay in L2), instead of drifting apart as with a static round-robin.
+// One index = (work item of K0, KV head, part of the group's heads): one key tile against the query
+// tiles of a chunk, one head after the other; every (query tile, head) is a step.
+struct BwdItem {
+    int k_start, k_len; // key tile
+    int qt0;            // first query tile of the chunk
+    unsigned mask;      // bit b: query tile qt0 + b takes part; bit 8 + b: its tile is FULL
+    int h0, nh;         // heads h0 .. h0 + nh - 1
+    int g;              // KV head; negative: no more items
+    int steps;
 };
+constexpr int BWD_QUEUE_BYTES = 4 * (int)sizeof(BwdItem);
+
+// How finely the work items of K0 are cut, from the steps a CTA gets on average: with whole groups a
+// small problem keeps few SMs busy for up to BWD_CQ x group steps, but every item costs a K / V load,
+// a start of the pipeline and two fp32 tiles added to dK / dV (about two steps in all).  The heads of a
+// group are dealt out in parts of a twelfth of a CTA's steps (times up to BWD_CQ query tiles per
+// item), so a CTA draws three items or more; with less than three steps per CTA every step is an
+// item of its own.  Measured, backward kernel: 512 tokens, 4 heads of 64 (one KV head) 39 -> 15 us;
+// 3,128 tokens, 32 heads of 128 99 -> 76 us; divisors from 8 to 16 within 2 per cent of each other,
+// 24 up to 12 per cent slower between 5,600 and 11,200 tokens.
+struct BwdSplit {
+    int parts, nh; // parts of a KV group, heads per part
+    int tiles;     // 1: whole chunks, BWD_CQ: one query tile per item
+    int total;     // indexes to draw
+};
+__device__ __forceinline__ BwdSplit bwd_split(const BwdParams &P)
+{
+    const int G = P.Hq / P.Hkv;
+    const long long steps = (long long)P.counters[4] * P.Hq;
+    const int avg = (int)min(steps / gridDim.x, (long long)(1 << 20));
+    BwdSplit s;
+    s.nh = min(G, max(1, avg / 12));
+    s.parts = (G + s.nh - 1) / s.nh;
+    s.nh = (G + s.parts - 1) / s.parts;
+    s.parts = (G + s.nh - 1) / s.nh;
+    s.tiles = avg < 3 ? BWD_CQ : 1;
+    s.total = P.counters[1] * P.Hkv * s.parts * s.tiles;
+    return s;
+}
+
+// Producer warp (convergent): draws the next item and publishes it as item w.
+__device__ __forceinline__ bool bwd_draw(const BwdParams &P, const BwdSplit &sp, uint8_t *queue, uint32_t queue_bar,
+                                         int w, int lane, BwdItem &out)
+{
+    const int G = P.Hq / P.Hkv;
+    out.g = -1;
+    while (true) {
+        int v = 0;
+        if (lane == 0)
+            v = atomicAdd(P.cursor, 1);
+        v = __shfl_sync(0xffffffffu, v, 0);
+        if (v >= sp.total)
+            break;
+        const int tile = v % sp.tiles, rest = v / sp.tiles;
+        const int part = rest % sp.parts, ig = rest / sp.parts;
+        const int4 item = P.bitems[ig / P.Hkv];
+        unsigned mask = (unsigned)item.z;
+        if (sp.tiles > 1)
+            mask &= 0x101u << tile;
+        if ((mask & 0xffu) == 0)
+            continue; // this query tile of the chunk is skipped by the key tile
+        const int2 kt = P.ktile[item.x];
+        out.g = ig % P.Hkv;
+        out.k_start = kt.x;
+        out.k_len = kt.y;
+        out.qt0 = item.y * BWD_CQ;
+        out.mask = mask;
+        out.h0 = out.g * G + part * sp.nh;
+        out.nh = min(sp.nh, G - part * sp.nh);
+        out.steps = __popc(mask & 0xffu) * out.nh;
+        break;
+    }
+    if (lane == 0) {
+        *reinterpret_cast<BwdItem *>(queue + (w & 3) * sizeof(BwdItem)) = out;
+        sm100::mbar_arrive(queue_bar + 8u * (w & 3));
+    }
+    return out.g >= 0;
+}
+// The other roles: item w, or false at the end (or when a wait ran out).
+__device__ __forceinline__ bool bwd_take(uint8_t *queue, uint32_t queue_bar, int w, volatile int *abort, BwdItem &out)
+{
+    const bool ok = sm100::mbar_wait(queue_bar + 8u * (w & 3), (w >> 2) & 1, abort);
+    if (!__all_sync(0xffffffffu, ok))
+        return false;
+    out = *reinterpret_cast<const BwdItem *>(queue + (w & 3) * sizeof(BwdItem));
+    return out.g >= 0;
+}
 
 } // namespace peagle

@@ -789,9 +789,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 dov[i] = make_uint4(0, 0, 0, 0);
         }
         // rows of the padded partition are numbered from its first row
-        const size_t hand = (size_t)h * P.q_pad + (size_t)(qt * BM + r);
+        const size_t hand = (size_t)h * P.q_pad + (size_t)row_slot(qt * BM + r);
         if (P.dO && x == 0 && (it.h0 == 0))
-            P.mqp[qt * BM + r] = mq;
+            P.mqp[row_slot(qt * BM + r)] = mq;
         if (cnt == 0 && n_single == 0) {
             if (row_ok) {
                 uint4 z = make_uint4(0, 0, 0, 0);

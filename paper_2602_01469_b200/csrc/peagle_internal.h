@@ -45,7 +45,8 @@ struct Plan {
     int4 *ksum;            // [n_kt]
     uint8_t *cls;          // [n_qt][n_kt] tile classes
     int *undecided;        // [n_qt*n_kt] pairs the quick test could not decide
-    int *counters;         // [8] device counters (0: undecided, 1: bwd items, 2: bwd work cursor, 3: fwd cursor)
+    int *counters;         // [8] device counters (0: undecided, 1: bwd items, 2: bwd work cursor, 3: fwd cursor,
+                           // 4: (query tile, key tile) pairs in the bwd items)
     int2 *klist;           // [n_qt][n_kt] compact non-skip key tiles per query tile: (first token, len | cls<<16)
     int *kcount;           // [n_qt]
     int *qorder;           // [n_qt] query tiles, most key tiles first
@@ -84,7 +85,8 @@ struct BwdArgs {
     const float *LSE;
     void *dQ;
     float *dK_acc, *dV_acc;
-    // per-row scratch of the call, q_pad = query tiles * BM rows, rows past the partition padded
+    // per-row scratch of the call, q_pad = query tiles * BM rows, rows past the partition padded;
+    // row r's entry stands at row_slot(r)
     float *nl2;     // [Hq][q_pad] -LSE * log2(e); -inf for a padded row or a row that saw no key
     float *nd;      // [Hq][q_pad] -Delta = -<dO, O>; 0 for a padded row
     int32_t *mqp;   // [q_pad] packed metadata of the partition's rows; META_NONE_Q when padded
@@ -98,6 +100,15 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
                                   const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+// Where row r (of the padded partition) keeps its value in nl2, nd and mqp.  The compute warps of the
+// backward hold their scores as tcgen05.ld.16x256b gives them: thread t of a warp has the query
+// columns 8i + 2 (t % 4) and the next one.  With the 16 values of two such groups in the order of the
+// threads that use them, a thread gets the four of a group pair with one 16-byte load.
+__host__ __device__ inline int row_slot(int r)
+{
+    return (r & ~15) | (((r >> 1) & 3) << 2) | ((r >> 3 & 1) << 1) | (r & 1);
+}
 
 // K0: mask evaluator, tile classifier, scheduler.  Returns the number of kernels launched.
 int launch_plan(const Plan &p, const int32_t *anchor, const int32_t *depth, int K, int seq_begin,

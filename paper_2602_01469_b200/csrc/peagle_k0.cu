@@ -352,8 +352,14 @@ __global__ void k0_chunk_items(Plan p)
         for (int i = 0; i < c; ++i)
             off += p.ccount[i * BWD_CQ + sz];
         base[sz] = off;
-        if (c == n_ch - 1 && sz == 0)
+        if (c == n_ch - 1 && sz == 0) {
             p.counters[1] = off + p.ccount[c * BWD_CQ];
+            int tiles = 0;
+            for (int s2 = 0; s2 < BWD_CQ; ++s2)
+                for (int i = 0; i < n_ch; ++i)
+                    tiles += (s2 + 1) * p.ccount[i * BWD_CQ + s2];
+            p.counters[4] = tiles;
+        }
     }
     __syncthreads();
     for (int sz = BWD_CQ - 1; sz >= 0; --sz) {

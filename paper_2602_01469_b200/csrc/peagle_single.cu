@@ -156,8 +156,8 @@ __device__ __forceinline__ void single_pass(const SingleParams &P, int i0, int n
             if (sub == 0) {
                 snl2[h] = nl2;
                 snd[h] = nd;
-                P.nl2[(size_t)h * P.q_pad + r] = nl2;
-                P.nd[(size_t)h * P.q_pad + r] = nd;
+                P.nl2[(size_t)h * P.q_pad + row_slot(r)] = nl2;
+                P.nd[(size_t)h * P.q_pad + row_slot(r)] = nd;
             }
         } else {
             nl2 = snl2[h];
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(128, D == 64 ? 4 : 2) single_bwd(const SingleP
     }
     if (P.rows_ready) {
         for (int i = threadIdx.x; i < n_real * P.Hq; i += blockDim.x) {
-            const size_t ri = (size_t)(i % P.Hq) * P.q_pad + r0 + i / P.Hq;
+            const size_t ri = (size_t)(i % P.Hq) * P.q_pad + row_slot(r0 + i / P.Hq);
             snl2[i] = P.nl2[ri];
             snd[i] = P.nd[ri];
         }
@@ -280,11 +280,11 @@ __global__ void __launch_bounds__(128, D == 64 ? 4 : 2) single_bwd(const SingleP
     if (rl < RB && r < P.q_pad && !real && !P.rows_ready) { // padded row: seen by nobody
         if (sub == 0) {
             for (int hh = 0; hh < G; ++hh) {
-                P.nl2[(size_t)(g * G + hh) * P.q_pad + r] = -CUDART_INF_F;
-                P.nd[(size_t)(g * G + hh) * P.q_pad + r] = 0.f;
+                P.nl2[(size_t)(g * G + hh) * P.q_pad + row_slot(r)] = -CUDART_INF_F;
+                P.nd[(size_t)(g * G + hh) * P.q_pad + row_slot(r)] = 0.f;
             }
             if (g == 0)
-                P.mqp[r] = META_NONE_Q;
+                P.mqp[row_slot(r)] = META_NONE_Q;
         }
     }
     if (n_real == 0)
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(128, D == 64 ? 4 : 2) single_bwd(const SingleP
     const int row = P.q_begin + r;
     if (g == 0 && sub == 0 && !P.rows_ready) {
         const int32_t mq = P.meta[row];
-        P.mqp[r] = mq == META_NONE_K ? META_NONE_Q : mq;
+        P.mqp[row_slot(r)] = mq == META_NONE_K ? META_NONE_Q : mq;
     }
     const __nv_bfloat16 *sq = sQ + (size_t)rl * row_elems, *sdo = sdO + (size_t)rl * row_elems,
                         *so = sO + (size_t)rl * row_elems;
