@@ -115,22 +115,19 @@ void carve_plan(Plan &p, void *base, size_t *bytes_out)
     const size_t nq = (size_t)(p.n_qt > 0 ? p.n_qt : 1), nk = (size_t)(p.n_kt > 0 ? p.n_kt : 1);
     p.meta = c.take<int32_t>((size_t)p.T);
     p.ktile = c.take<int2>(nk);
-    p.qsum = c.take<int4>(nq);
-    p.ksum = c.take<int4>(nk);
+    p.qsum = c.take<int4>(2 * nq);
+    p.ksum = c.take<int4>(2 * nk);
+    p.ksplit = c.take<int>(nk);
     p.cls = c.take<uint8_t>(nq * nk);
     p.undecided = c.take<int>(nq * nk);
-    p.counters = c.take<int>(8);
+    p.counters = c.take<int>(PLAN_COUNTERS);
     p.klist = c.take<int2>(nq * nk);
     p.kcount = c.take<int>(nq);
     p.qorder = c.take<int>(nq);
     const size_t nch = (nq + BWD_CQ - 1) / BWD_CQ;
-    p.cmask = c.take<uint16_t>(nch * nk);
-    p.ccount = c.take<int>(nch * BWD_CQ);
-    p.bitems = c.take<int4>(nch * nk);
+    p.cdone = c.take<int>(nch);
+    p.bitems = c.take<int4>(BWD_CQ * nch * nk);
     p.scount = c.take<int>(nq);
-    p.skt = c.take<int>(nq * MAX_SINGLE);
-    p.sorder = c.take<uint8_t>(nq * MAX_SINGLE);
-    p.scol = c.take<uint8_t>(nq * MAX_SINGLE * BM);
     p.scs = c.take<uint8_t>(nq * MAX_SINGLE * BM);
     p.sbase = c.take<int>(nq * MAX_SINGLE);
     p.sperm = c.take<int>(nq);
@@ -235,7 +232,7 @@ int plan_call(peagle_ctx *ctx, const peagle_problem_t *prob, const peagle_partit
     if (c.plan.n_qt == 0)
         return PEAGLE_OK;
     ctx->launches += launch_plan(c.plan, prob->anchor, prob->depth, prob->K, c.seq_begin, c.seq_end,
-                                 c.ranges, for_bwd, prob->n_kv_heads, s);
+                                 c.ranges, for_bwd, s);
     CK(cudaGetLastError());
     return PEAGLE_OK;
 }
@@ -645,7 +642,7 @@ int peagle_attn_fwd_static(int device, const peagle_problem_t *prob,
     if (c.plan.n_qt == 0)
         return PEAGLE_OK;
     launch_plan(c.plan, prob->anchor, prob->depth, prob->K, c.seq_begin, c.seq_end, c.ranges,
-                false, prob->n_kv_heads, s);
+                false, s);
     if (cudaGetLastError() != cudaSuccess)
         return PEAGLE_ERR_CUDA;
     FwdArgs a;

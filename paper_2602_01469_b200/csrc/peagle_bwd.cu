@@ -712,10 +712,11 @@ static int launch_bwd_t(const Plan &p, const BwdArgs &a, EncodeTiledFn enc, int 
         P.ktile = p.ktile;
         P.bitems = p.bitems;
         P.counters = p.counters;
-        P.cursor = p.counters + 2;
+        P.cursor = p.counters + CNT_BWD_CURSOR;
         P.meta = p.meta;
         P.status = p.status;
         P.n_qt = p.n_qt;
+        P.n_kt = p.n_kt;
         P.q_begin = p.q_begin;
         P.q_end = p.q_end;
         P.T = p.T;

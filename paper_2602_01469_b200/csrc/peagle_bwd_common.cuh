@@ -12,7 +12,7 @@ struct BwdParams {
     int *cursor; // device counter, zero at launch: next (work item, KV head) index to hand out
     const int32_t *meta;
     int *status;
-    int n_qt, q_begin, q_end, T;
+    int n_qt, n_kt, q_begin, q_end, T;
     const float *nl2, *nd; // [Hq][q_pad] -LSE*log2(e) and -Delta, padded rows (-inf, 0)
     const int32_t *mqp;    // [q_pad] packed metadata of the partition's rows
     int q_pad;             // n_qt * BM
@@ -50,21 +50,31 @@ constexpr int BWD_QUEUE_BYTES = 4 * (int)sizeof(BwdItem);
 // 24 up to 12 per cent slower between 5,600 and 11,200 tokens.
 struct BwdSplit {
     int parts, nh; // parts of a KV group, heads per part
+    int count[BWD_CQ]; // work items of K0 with 1 .. BWD_CQ query tiles
+    int cap;           // places for the items of a size
     int tiles;     // 1: whole chunks, BWD_CQ: one query tile per item
     int total;     // indexes to draw
 };
 __device__ __forceinline__ BwdSplit bwd_split(const BwdParams &P)
 {
     const int G = P.Hq / P.Hkv;
-    const long long steps = (long long)P.counters[4] * P.Hq;
-    const int avg = (int)min(steps / gridDim.x, (long long)(1 << 20));
     BwdSplit s;
+    int items = 0;
+    long long steps = 0;
+#pragma unroll
+    for (int i = 0; i < BWD_CQ; ++i) {
+        s.count[i] = P.counters[CNT_ITEMS + i];
+        items += s.count[i];
+        steps += (long long)(i + 1) * s.count[i] * P.Hq;
+    }
+    s.cap = (P.n_qt + BWD_CQ - 1) / BWD_CQ * P.n_kt;
+    const int avg = (int)min(steps / gridDim.x, (long long)(1 << 20));
     s.nh = min(G, max(1, avg / 12));
     s.parts = (G + s.nh - 1) / s.nh;
     s.nh = (G + s.parts - 1) / s.parts;
     s.parts = (G + s.nh - 1) / s.nh;
     s.tiles = avg < 3 ? BWD_CQ : 1;
-    s.total = P.counters[1] * P.Hkv * s.parts * s.tiles;
+    s.total = items * P.Hkv * s.parts * s.tiles;
     return s;
 }
 
@@ -83,7 +93,17 @@ __device__ __forceinline__ bool bwd_draw(const BwdParams &P, const BwdSplit &sp,
             break;
         const int tile = v % sp.tiles, rest = v / sp.tiles;
         const int part = rest % sp.parts, ig = rest / sp.parts;
-        const int4 item = P.bitems[ig / P.Hkv];
+        int at = ig / P.Hkv, base = 0; // the items with most query tiles come first
+#pragma unroll
+        for (int i = BWD_CQ - 1; i >= 0; --i) {
+            if (at >= 0 && at < sp.count[i]) {
+                base = i * sp.cap + at;
+                at = -1;
+            } else if (at >= 0) {
+                at -= sp.count[i];
+            }
+        }
+        const int4 item = P.bitems[base];
         unsigned mask = (unsigned)item.z;
         if (sp.tiles > 1)
             mask &= 0x101u << tile;

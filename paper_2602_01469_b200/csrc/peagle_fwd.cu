@@ -159,7 +159,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         it.cnt = P.kcount[it.qt];
         it.klist = P.klist + (size_t)it.qt * P.n_kt;
         // the result of the SINGLE entries seeds (m, l, O) of the tile loop
-        it.n_single = min(P.scount[it.qt], MAX_SINGLE);
+        it.n_single = P.scount[it.qt];
         return it;
     };
     // Roles other than the producer: index of item w, or -1 at the end (or when a wait ran out).
@@ -945,7 +945,7 @@ static int launch_fwd_t(const Plan &p, const FwdArgs &a, EncodeTiledFn enc, int 
     P.qorder = p.qorder;
     P.meta = p.meta;
     P.status = p.status;
-    P.cursor = p.counters + 3;
+    P.cursor = p.counters + CNT_FWD_CURSOR;
     P.n_kt = p.n_kt;
     P.q_begin = p.q_begin;
     P.q_end = p.q_end;

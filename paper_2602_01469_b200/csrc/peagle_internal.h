@@ -23,7 +23,10 @@ constexpr int32_t META_NONE_K = 0x7fffffff; // packed metadata of a key outside 
 // chain tiles of the depth-major layout: one allowed pair per row).  Such tiles are taken out of
 // the tensor-core lists and handled pair by pair.  The test hook reports them as PARTIAL.
 enum TileClass : uint8_t { TILE_SKIP = 0, TILE_PARTIAL = 1, TILE_FULL = 2, TILE_SINGLE = 3 };
-constexpr int MAX_SINGLE = 16;   // SINGLE tiles kept per query tile; further ones stay PARTIAL
+constexpr int MAX_SINGLE = 16;   // SINGLE entries kept per query tile; further ones stay PARTIAL
+// device counters of a plan
+constexpr int CNT_BWD_CURSOR = 2, CNT_FWD_CURSOR = 3, CNT_DONE = 4, CNT_ITEMS = 8, PLAN_COUNTERS = 16;
+static_assert(CNT_ITEMS + BWD_CQ <= PLAN_COUNTERS, "a counter per item size");
 constexpr int NO_COL = 255;      // "this row allows no key of the tile"
 
 // Visible key ranges of one call, passed to kernels by value.
@@ -41,26 +44,24 @@ struct Plan {
     int n_qt, n_kt;        // tile counts
     int32_t *meta;         // [T] packed (anchor << 8 | depth)
     int2 *ktile;           // [n_kt] (first token, length)
-    int4 *qsum;            // [n_qt] (min anchor, max anchor, min depth, max depth)
-    int4 *ksum;            // [n_kt]
+    int4 *qsum;            // [n_qt][2] (min anchor, max anchor, min depth, max depth) of the tile's first
+                           // run of equal depth and of the rest; max anchor -1: no token
+    int4 *ksum;            // [n_kt][2]
+    int *ksplit;           // [n_kt] keys in the first run, flags for sorted runs
     uint8_t *cls;          // [n_qt][n_kt] tile classes
-    int *undecided;        // [n_qt*n_kt] pairs the quick test could not decide
-    int *counters;         // [8] device counters (0: undecided, 1: bwd items, 2: bwd work cursor, 3: fwd cursor,
-                           // 4: (query tile, key tile) pairs in the bwd items)
+    int *undecided;        // [n_qt][n_kt] key tiles that a query tile's quick test could not decide
+    int *counters;         // [PLAN_COUNTERS] device counters, zero before k0_plan: CNT_*
+    int *cdone;            // [n_ch] query tiles of a chunk that are classified
     int2 *klist;           // [n_qt][n_kt] compact non-skip key tiles per query tile: (first token, len | cls<<16)
     int *kcount;           // [n_qt]
-    int *qorder;           // [n_qt] query tiles, most key tiles first
-    uint16_t *cmask;       // [n_ch][n_kt] per chunk of BWD_CQ query tiles: bit b not skipped, bit 8+b FULL
-    int *ccount;           // [n_ch][BWD_CQ] key tiles whose word has 1, 2, .. BWD_CQ query tiles
-    int4 *bitems;          // [n_ch * n_kt] backward work items (key tile, chunk, mask word, query tiles)
+    int *qorder;           // [n_qt] query tiles, most key tiles first (no order among about equal ones)
+    int4 *bitems;          // [BWD_CQ][n_ch * n_kt] backward work items by size (1 .. BWD_CQ query tiles):
+                           // (key tile, chunk, mask word, query tiles); counters[CNT_ITEMS + size - 1] of each
     int allow_single;      // 1: the kernels of this shape take SINGLE tiles pair by pair
-    int *scount;           // [n_qt] SINGLE tiles found per query tile (may exceed MAX_SINGLE: clamp)
-    int *skt;              // [n_qt][MAX_SINGLE] key tile of a slot
-    uint8_t *sorder;       // [n_qt][MAX_SINGLE] slots by ascending key tile
-    uint8_t *scol;         // [n_qt][MAX_SINGLE][BM] per row: the one allowed key column, or NO_COL
-    int *sbase;            // [n_qt][MAX_SINGLE] first token of entry i's key tile
-    uint8_t *scs;          // [n_qt][MAX_SINGLE][BM] what the kernels read: entry i (slots by ascending
-                           // key tile) of row r is its key's column in that tile, or NO_COL
+    int *scount;           // [n_qt] SINGLE entries per query tile (at most MAX_SINGLE): windows of 128 keys,
+                           // ascending, in which every query row has at most one key
+    int *sbase;            // [n_qt][MAX_SINGLE] first token of entry i's window
+    uint8_t *scs;          // [n_qt][MAX_SINGLE][BM] key of row r in entry i's window, or NO_COL
     int *sperm;            // [n_qt] query tiles in the order the SINGLE-tile backward takes them:
                            // by the first key tile of their SINGLE entries, so that the query
                            // tiles that add to the same key rows run close together in time
@@ -112,7 +113,7 @@ __host__ __device__ inline int row_slot(int r)
 
 // K0: mask evaluator, tile classifier, scheduler.  Returns the number of kernels launched.
 int launch_plan(const Plan &p, const int32_t *anchor, const int32_t *depth, int K, int seq_begin,
-                int seq_end, const RangeList &ranges, bool for_bwd, int Hkv, cudaStream_t s);
+                int seq_end, const RangeList &ranges, bool for_bwd, cudaStream_t s);
 int launch_mask_dense(const Plan &p, const RangeList &ranges, uint8_t *out, cudaStream_t s);
 // One CTA whose bounded wait runs out after limit_ns: records PEAGLE_ERR_TIMEOUT in *status.
 int launch_wait_expiry(int *status, unsigned long long limit_ns, int *reached_end, cudaStream_t s);

@@ -2,14 +2,19 @@
 //
 // The parallel-prediction mask (paper Section 3 / 3.2) is a function of per-token metadata only,
 // so it is evaluated from a packed word per token (anchor << 8 | depth) and never stored.  For
-// one call (a query partition and the key ranges it may see) these kernels
-//   1. pack and validate the metadata and lay out the key tiles of the visible ranges,
-//   2. summarise every query tile and key tile (min/max anchor and depth),
-//   3. classify every (query tile, key tile) pair as SKIP / PARTIAL / FULL -- from the summaries
-//      where they decide, else exactly by evaluating the predicate on the tile,
-//   4. compact the non-skipped tiles into per-query-tile key lists, order query tiles
-//      longest-first, and cut the backward into (key tile, query-tile chunk) work items.
-// Everything runs on the caller's stream; nothing returns to the host.
+// one call (a query partition and the key ranges it may see) two kernels
+//   k0_tiles  pack and validate the metadata, lay out the key tiles of the visible ranges, summarise
+//             every query tile and key tile (min/max anchor and depth of its first run of equal depth
+//             and of the rest: in a depth-major layout a tile on the border of two depths holds the
+//             last anchors of one and the first of the next, and one summary would decide nothing);
+//   k0_plan   one block per query tile: classify its (query tile, key tile) pairs as SKIP / PARTIAL /
+//             FULL -- from the summaries where they decide, else exactly, by the keys each query row
+//             allows -- and compact the non-skipped ones into its key list; the last block of a chunk
+//             of query tiles cuts the backward's (key tile, chunk) work items, the last block of all
+//             orders the query tiles.
+// Everything runs on the caller's stream; nothing returns to the host.  The work is integer and small:
+// what it costs is launches and the latency of dependent steps, hence two kernels and not one per
+// step (eight kernels before: 24 us for 512 tokens, 47 us for 32,768, 95 us for the COD example).
 #include "peagle_internal.h"
 #include "sm100_ptx.cuh"
 
@@ -20,375 +25,508 @@ __device__ __forceinline__ void set_status(int *status, int err)
     atomicCAS(status, 0, err);
 }
 
-// ---- 1. pack metadata, build key tiles ---------------------------------------------------
-__global__ void k0_prepare(Plan p, const int32_t *__restrict__ anchor,
-                           const int32_t *__restrict__ depth, int K, int seq_begin, int seq_end,
-                           RangeList ranges)
+__device__ __forceinline__ int pack_meta(int a, int d, int K)
 {
-    const int t = seq_begin + blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < seq_end) {
-        const int a = anchor[t], d = depth[t];
-        if (a < 0 || a >= (1 << 23) || d < 0 || d >= K) {
-            set_status(p.status, PEAGLE_ERR_BAD_META);
-            p.meta[t] = META_NONE_K;
-        } else {
-            p.meta[t] = (a << 8) | d;
-        }
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        int kt = 0;
-        for (int i = 0; i < ranges.n; ++i)
-            for (int b = ranges.begin[i]; b < ranges.end[i]; b += BN, ++kt)
-                p.ktile[kt] = make_int2(b, min(BN, ranges.end[i] - b));
-        for (int i = 0; i < 8; ++i)
-            p.counters[i] = 0;
-    }
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < p.n_qt)
-        p.scount[i] = 0;
+    return a < 0 || a >= (1 << 23) || d < 0 || d >= K ? META_NONE_K : (a << 8) | d;
 }
 
-// ---- 2. tile summaries -----------------------------------------------------------------
-__global__ void k0_summaries(Plan p)
+constexpr int KRUN0_SORTED = 1 << 8, KRUN1_SORTED = 1 << 9; // beside the length of the first run in ksplit
+
+// ---- 1. pack metadata, lay out and summarise tiles ---------------------------------------------
+// Block b packs tokens 128 b .. of the sequence and summarises tile b (query tiles first).
+__global__ void __launch_bounds__(128) k0_tiles(Plan p, const int32_t *__restrict__ anchor,
+                                                const int32_t *__restrict__ depth, int K, int seq_begin,
+                                                int seq_end, RangeList ranges)
 {
     const int tile = blockIdx.x;
+    const int t = seq_begin + tile * 128 + threadIdx.x;
+    if (t < seq_end) {
+        const int m = pack_meta(anchor[t], depth[t], K);
+        if (m == META_NONE_K)
+            set_status(p.status, PEAGLE_ERR_BAD_META);
+        p.meta[t] = m;
+    }
+    if (tile == 0 && threadIdx.x < PLAN_COUNTERS)
+        p.counters[threadIdx.x] = 0;
+    if (threadIdx.x == 0 && tile * BWD_CQ < p.n_qt)
+        p.cdone[tile] = 0;
+    if (tile >= p.n_qt + p.n_kt)
+        return;
     int b, e;
     int4 *out;
     if (tile < p.n_qt) {
         b = p.q_begin + tile * BM;
         e = min(b + BM, p.q_end);
-        out = p.qsum + tile;
+        out = p.qsum + 2 * tile;
     } else {
-        const int2 kt = p.ktile[tile - p.n_qt];
-        b = kt.x;
-        e = kt.x + kt.y;
-        out = p.ksum + (tile - p.n_qt);
+        int kt = tile - p.n_qt, i = 0; // key tiles are numbered through the visible ranges
+        while (kt >= (ranges.end[i] - ranges.begin[i] + BN - 1) / BN)
+            kt -= (ranges.end[i] - ranges.begin[i] + BN - 1) / BN, ++i;
+        b = ranges.begin[i] + kt * BN;
+        e = min(b + BN, ranges.end[i]);
+        out = p.ksum + 2 * (tile - p.n_qt);
+        if (threadIdx.x == 0)
+            p.ktile[tile - p.n_qt] = make_int2(b, e - b);
     }
-    int a0 = INT_MAX, a1 = -1, d0 = INT_MAX, d1 = -1;
-    const int t = b + threadIdx.x;
-    if (t < e) {
-        const int m = p.meta[t];
-        if (m != META_NONE_K) {
-            a0 = a1 = m >> 8;
-            d0 = d1 = m & 0xff;
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        a0 = min(a0, __shfl_xor_sync(0xffffffffu, a0, o));
-        a1 = max(a1, __shfl_xor_sync(0xffffffffu, a1, o));
-        d0 = min(d0, __shfl_xor_sync(0xffffffffu, d0, o));
-        d1 = max(d1, __shfl_xor_sync(0xffffffffu, d1, o));
-    }
-    __shared__ int4 part[4];
-    if ((threadIdx.x & 31) == 0)
-        part[threadIdx.x >> 5] = make_int4(a0, a1, d0, d1);
+    const bool in_tile = b + (int)threadIdx.x < e;
+    const int m = in_tile ? pack_meta(anchor[b + threadIdx.x], depth[b + threadIdx.x], K) : META_NONE_K;
+    const int dn = m == META_NONE_K ? -1 : m & 0xff; // depth -1: no token, or not a valid one
+    __shared__ int split, word[128];
+    __shared__ int4 part[2][4];
+    word[threadIdx.x] = m;
+    if (threadIdx.x == 0)
+        split = e - b;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int4 r = part[0];
-        for (int w = 1; w < 4; ++w) {
-            r.x = min(r.x, part[w].x);
-            r.y = max(r.y, part[w].y);
-            r.z = min(r.z, part[w].z);
-            r.w = max(r.w, part[w].w);
-        }
-        *out = r;
+    const int first_depth = word[0] == META_NONE_K ? -1 : word[0] & 0xff;
+    if (in_tile && dn != first_depth)
+        atomicMin(&split, (int)threadIdx.x);
+    __syncthreads();
+#pragma unroll
+    for (int run = 0; run < 2; ++run) {
+        const bool in = dn >= 0 && ((int)threadIdx.x < split) == (run == 0);
+        const int a0 = __reduce_min_sync(0xffffffffu, in ? m >> 8 : INT_MAX);
+        const int a1 = __reduce_max_sync(0xffffffffu, in ? m >> 8 : -1);
+        const int d0 = __reduce_min_sync(0xffffffffu, in ? dn : INT_MAX);
+        const int d1 = __reduce_max_sync(0xffffffffu, in ? dn : -1);
+        if ((threadIdx.x & 31) == 0)
+            part[run][threadIdx.x >> 5] = make_int4(a0, a1, d0, d1);
     }
+    // runs in ascending order of their packed words can be searched instead of read through
+    const int nx = threadIdx.x + 1;
+    const bool falls = nx < e - b && word[threadIdx.x] > word[nx];
+    const int unsorted0 = __syncthreads_or(falls && nx < split);
+    const int unsorted1 = __syncthreads_or(falls && (int)threadIdx.x >= split);
+    if (threadIdx.x < 2) {
+        int4 r = part[threadIdx.x][0];
+        for (int w = 1; w < 4; ++w) {
+            const int4 o = part[threadIdx.x][w];
+            r.x = min(r.x, o.x);
+            r.y = max(r.y, o.y);
+            r.z = min(r.z, o.z);
+            r.w = max(r.w, o.w);
+        }
+        out[threadIdx.x] = r;
+    }
+    if (threadIdx.x == 0 && tile >= p.n_qt)
+        p.ksplit[tile - p.n_qt] = split | (unsorted0 ? 0 : KRUN0_SORTED) | (unsorted1 ? 0 : KRUN1_SORTED);
 }
 
-// ---- 3a. classification from summaries ---------------------------------------------------
-__global__ void k0_classify_quick(Plan p)
+// ---- 2. the plan -----------------------------------------------------------------------------
+constexpr int PLAN_THREADS = 512;
+constexpr int PLAN_GROUPS = PLAN_THREADS / BM; // pairs classified exactly at a time
+constexpr int PAIR_CACHE = 256;                // undecided pairs of a query tile kept in shared memory
+constexpr int RAW_SINGLE = 2 * MAX_SINGLE;     // one-key-per-row tiles kept before neighbours are joined
+constexpr int SORT_BUCKETS = 4096;
+
+// Class of a run of query rows and a run of keys from their summaries (min anchor, max anchor, min
+// depth, max depth; max anchor < 0: no token), or -1 where the summaries do not decide.
+__device__ __forceinline__ int classify_runs(const int4 q, const int4 k)
 {
-    const int kt = blockIdx.x * blockDim.x + threadIdx.x;
-    const int qt = blockIdx.y;
-    if (kt >= p.n_kt)
-        return;
-    const int4 q = p.qsum[qt];
-    const int4 k = p.ksum[kt];
-    const int len = p.ktile[kt].y;
-    int c = -1;
-    if (k.y < 0 || q.y < 0) {
-        c = TILE_SKIP; // a tile with no valid token
-    } else if (k.w == 0) { // every key is a depth-0 (real context) token
+    if (k.w == 0) { // every key is a depth-0 (real context) token
         if (k.y <= q.x)
-            c = (len == BN) ? TILE_FULL : TILE_PARTIAL;
-        else if (k.x > q.y)
-            c = TILE_SKIP;
+            return TILE_FULL;
+        if (k.x > q.y)
+            return TILE_SKIP;
     } else if (k.z >= 1) { // no depth-0 key: only same-anchor, not-deeper chain tokens can match
         if (k.x > q.y || k.y < q.x || k.z > q.w)
-            c = TILE_SKIP;
+            return TILE_SKIP;
     }
-    const size_t idx = (size_t)qt * p.n_kt + kt;
-    if (c >= 0) {
-        p.cls[idx] = (uint8_t)c;
-    } else {
-        p.cls[idx] = 255;
-        p.undecided[atomicAdd(&p.counters[0], 1)] = (int)idx;
+    return -1;
+}
+// Class of a tile pair, or -1: len keys, the first run has `split` of them.
+__device__ __forceinline__ int classify_quick(const int4 (&q)[2], const int4 *k2, int len, int split)
+{
+    // skip: some row does not allow some key; full: a run pair is FULL, full2: with two keys or more
+    bool skip = false, full = false, full2 = false, open = false;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const int4 k = k2[j];
+        if (k.y < 0)
+            continue;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            if (q[i].y < 0)
+                continue;
+            const int c = classify_runs(q[i], k);
+            skip |= c == TILE_SKIP;
+            full |= c == TILE_FULL;
+            full2 |= c == TILE_FULL && (j == 0 ? split : len - split) >= 2;
+            // an undecided pair may still be FULL only if all its rows belong to the chain of its keys
+            open |= c < 0;
+            skip |= c < 0 && !(k.w > 0 && q[i].x == q[i].y);
+        }
     }
+    if (!open && !full)
+        return TILE_SKIP; // also: no valid token
+    if (!open && !skip)
+        return len == BN ? TILE_FULL : TILE_PARTIAL;
+    return full2 && skip ? TILE_PARTIAL : -1;
 }
 
-// ---- 3b. exact classification of the remaining pairs ------------------------------------
-__global__ void k0_classify_exact(Plan p)
+__device__ __forceinline__ void group_sync(int group)
 {
-    __shared__ int mk[BN];
-    __shared__ int total, most, slot;
-    const int n = p.counters[0];
-    for (int w = blockIdx.x; w < n; w += gridDim.x) {
-        const int idx = p.undecided[w];
-        const int qt = idx / p.n_kt, kt = idx % p.n_kt;
-        const int2 ktile = p.ktile[kt];
-        const int r0 = p.q_begin + qt * BM, r1 = min(r0 + BM, p.q_end);
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(BM) : "memory");
+}
+
+// Compacts the elements o = 0 .. n - 1 with pred(o) in ascending order: calls emit(o, position).
+// Every thread of the block takes part.
+template <class Pred, class Emit>
+__device__ __forceinline__ int block_compact(int n, int *warp_cnt, Pred pred, Emit emit)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int base = 0;
+    for (int o0 = 0; o0 < n; o0 += PLAN_THREADS) {
+        const int o = o0 + threadIdx.x;
+        const bool mine = o < n && pred(o);
+        const unsigned bal = __ballot_sync(0xffffffffu, mine);
+        __syncthreads(); // the counts of the previous round have been read
+        if (lane == 0)
+            warp_cnt[wid] = __popc(bal);
         __syncthreads();
-        mk[threadIdx.x] = ((int)threadIdx.x < ktile.y) ? p.meta[ktile.x + threadIdx.x] : META_NONE_K;
-        if (threadIdx.x == 0) {
-            total = 0;
-            most = 0;
-            slot = -1;
+        int off = base, all = 0;
+        for (int w = 0; w < PLAN_THREADS / 32; ++w) {
+            const int c = warp_cnt[w];
+            off += w < wid ? c : 0;
+            all += c;
         }
+        if (mine)
+            emit(o, off + __popc(bal & ((1u << lane) - 1u)));
+        base += all;
+    }
+    return base;
+}
+
+// Sorts the query tiles by bucket(i), 0 .. SORT_BUCKETS - 1, ascending; the order inside a bucket is
+// arbitrary.  Every thread of the block takes part.  Up to one tile per thread the ranks are counted
+// directly (n reads of shared memory each); beyond that a counting sort over the buckets.
+template <class Bucket>
+__device__ __forceinline__ void block_sort(int n, int *hist, int *warp_sum, int *out, Bucket bucket)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __syncthreads();
+    if (n <= PLAN_THREADS) {
+        const int mine = (int)threadIdx.x < n ? bucket(threadIdx.x) * PLAN_THREADS + (int)threadIdx.x : INT_MAX;
+        hist[threadIdx.x] = mine;
         __syncthreads();
+        if ((int)threadIdx.x < n) {
+            int rank = 0;
+            for (int j = 0; j < n; j += 4) { // entries past n hold INT_MAX
+                const int4 v = *reinterpret_cast<const int4 *>(hist + j);
+                rank += (int)(v.x < mine) + (int)(v.y < mine) + (int)(v.z < mine) + (int)(v.w < mine);
+            }
+            out[rank] = threadIdx.x;
+        }
+        return;
+    }
+    constexpr int PER = SORT_BUCKETS / PLAN_THREADS;
+    for (int i = threadIdx.x; i < SORT_BUCKETS; i += PLAN_THREADS)
+        hist[i] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += PLAN_THREADS)
+        atomicAdd(&hist[bucket(i)], 1);
+    __syncthreads();
+    int sum = 0;
+    for (int j = 0; j < PER; ++j)
+        sum += hist[threadIdx.x * PER + j];
+    int scan = sum; // inclusive over the warp
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, scan, o);
+        scan += lane >= o ? v : 0;
+    }
+    if (lane == 31)
+        warp_sum[wid] = scan;
+    __syncthreads();
+    int at = scan - sum;
+    for (int w = 0; w < wid; ++w)
+        at += warp_sum[w];
+    for (int j = 0; j < PER; ++j) {
+        const int c = hist[threadIdx.x * PER + j];
+        hist[threadIdx.x * PER + j] = at;
+        at += c;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += PLAN_THREADS)
+        out[atomicAdd(&hist[bucket(i)], 1)] = i;
+}
+
+__global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, int seq_end, int for_bwd)
+{
+    __shared__ __align__(16) int hist[SORT_BUCKETS];
+    __shared__ int warp_cnt[PLAN_THREADS / 32];
+    __shared__ __align__(16) int mk[PLAN_GROUPS][BN];
+    __shared__ int2 part[PLAN_GROUPS][BM / 32];       // (allowed pairs, most keys of a row) per warp
+    __shared__ int slot_of[PLAN_GROUPS];
+    __shared__ uint8_t raw_col[RAW_SINGLE][BM];       // one-key-per-row tiles in arrival order
+    __shared__ int raw_kt[RAW_SINGLE], raw_ord[RAW_SINGLE], raw_conflict[RAW_SINGLE];
+    __shared__ int raw_min[RAW_SINGLE], raw_max[RAW_SINGLE];
+    __shared__ int4 pairs[PAIR_CACHE];                // (key tile, first token, length, first run | flags)
+    __shared__ int2 entry[RAW_SINGLE];                // sorted raw tiles of an entry: first, last
+    __shared__ int n_undecided, n_raw, n_entry, flag;
+    const int qt = blockIdx.x, tid = threadIdx.x;
+    const int lane = tid & 31;
+    uint8_t *cls = p.cls + (size_t)qt * p.n_kt;
+    int *undecided = p.undecided + (size_t)qt * p.n_kt;
+    if (tid == 0) {
+        n_undecided = 0;
+        n_raw = 0;
+    }
+    __syncthreads();
+    // ---- classes from the summaries
+    const int4 q[2] = {p.qsum[2 * qt], p.qsum[2 * qt + 1]};
+    for (int kt = tid; kt < p.n_kt; kt += PLAN_THREADS) {
+        const int2 k = p.ktile[kt];
+        const int split = p.ksplit[kt];
+        const int c = classify_quick(q, p.ksum + 2 * kt, k.y, split & 0xff);
+        cls[kt] = (uint8_t)c;
+        if (c < 0) {
+            const int at = atomicAdd(&n_undecided, 1);
+            undecided[at] = kt;
+            if (at < PAIR_CACHE)
+                pairs[at] = make_int4(kt, k.x, k.y, split);
+        }
+    }
+    __syncthreads();
+    // ---- exact classes of the rest, PLAN_GROUPS pairs at a time, a thread per query row
+    const int r0 = p.q_begin + qt * BM, r1 = min(r0 + BM, p.q_end);
+    const int group = tid / BM, row = tid % BM;
+    int mq = r0 + row < r1 ? p.meta[r0 + row] : META_NONE_Q;
+    if (mq == META_NONE_K)
+        mq = META_NONE_Q;
+    auto pair_at = [&](int w) {
+        if (w < PAIR_CACHE)
+            return pairs[w];
+        const int kt = undecided[w];
+        const int2 k = p.ktile[kt];
+        return make_int4(kt, k.x, k.y, p.ksplit[kt]);
+    };
+    // this thread's key of pair w, requested one pair ahead of its use
+    auto key_of = [&](int w) {
+        if (w >= n_undecided)
+            return META_NONE_K;
+        const int4 pr = pair_at(w);
+        return row < pr.z ? p.meta[pr.y + row] : META_NONE_K;
+    };
+    int key = key_of(group);
+    for (int w = group; w < n_undecided; w += PLAN_GROUPS) {
+        const int4 pr = pair_at(w);
+        const int kt = pr.x;
+        const int2 ktile = make_int2(pr.y, pr.z);
+        mk[group][row] = key;
+        group_sync(group);
+        key = key_of(w + PLAN_GROUPS);
+        // A row allows the keys of its own chain up to its depth, words [anchor << 8, mq], and the
+        // depth-0 keys up to its anchor, words up to mq: in a sorted run of one of the two kinds these
+        // are neighbours.
         int mine = 0, col = NO_COL;
-        if (r0 + (int)threadIdx.x < r1) {
-            const int mq = p.meta[r0 + threadIdx.x];
-            if (mq != META_NONE_K)
-                for (int c = 0; c < BN; ++c)
-                    if (allowed_packed(mq, mk[c])) {
+#pragma unroll
+        for (int run = 0; run < 2; ++run) {
+            const int lo = run == 0 ? 0 : pr.w & 0xff, hi = run == 0 ? pr.w & 0xff : ktile.y;
+            if (lo >= hi)
+                continue;
+            const int4 k = p.ksum[2 * kt + run];
+            if ((pr.w & (run == 0 ? KRUN0_SORTED : KRUN1_SORTED)) && (k.w == 0 || k.z >= 1)) {
+                auto first_above = [&](int word) { // first key of the run whose word is above `word`
+                    int a = lo, b = hi;
+                    while (a < b) {
+                        const int m = (a + b) >> 1;
+                        if (mk[group][m] <= word)
+                            a = m + 1;
+                        else
+                            b = m;
+                    }
+                    return a;
+                };
+                const int end = first_above(mq);
+                const int beg = k.w == 0 ? lo : first_above((mq & ~0xff) - 1);
+                if (end > beg) {
+                    mine += end - beg;
+                    col = end - 1;
+                }
+            } else {
+                for (int c = lo; c < hi; ++c)
+                    if (allowed_packed(mq, mk[group][c])) {
                         ++mine;
                         col = c;
                     }
+            }
         }
-        int cnt = mine, mx = mine;
-        for (int o = 16; o > 0; o >>= 1) {
-            cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-            mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        }
-        if ((threadIdx.x & 31) == 0) {
-            atomicAdd(&total, cnt);
-            atomicMax(&most, mx);
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
+        const int cnt = __reduce_add_sync(0xffffffffu, mine), most = __reduce_max_sync(0xffffffffu, mine);
+        if (lane == 0)
+            part[group][row >> 5] = make_int2(cnt, most);
+        group_sync(group);
+        if (row == 0) {
+            int total = 0, mx = 0, slot = -1;
+            for (int i = 0; i < BM / 32; ++i) {
+                total += part[group][i].x;
+                mx = max(mx, part[group][i].y);
+            }
             uint8_t c = TILE_PARTIAL;
             if (total == 0) {
                 c = TILE_SKIP;
             } else if (ktile.y == BN && total == (r1 - r0) * BN) {
                 c = TILE_FULL;
-            } else if (p.allow_single && most <= 1) {
-                const int sl = atomicAdd(&p.scount[qt], 1);
-                if (sl < MAX_SINGLE) {
+            } else if (p.allow_single && mx <= 1) {
+                slot = atomicAdd(&n_raw, 1);
+                if (slot < RAW_SINGLE) {
                     c = TILE_SINGLE;
-                    slot = sl;
-                    p.skt[qt * MAX_SINGLE + sl] = kt;
+                    raw_kt[slot] = kt;
+                    raw_min[slot] = INT_MAX;
+                    raw_max[slot] = -1;
+                } else {
+                    slot = -1;
                 }
             }
-            p.cls[idx] = c;
+            cls[kt] = c;
+            slot_of[group] = slot;
         }
-        __syncthreads();
-        if (slot >= 0)
-            p.scol[((size_t)qt * MAX_SINGLE + slot) * BM + threadIdx.x] = (uint8_t)col;
-    }
-}
-
-// ---- 4a. compact lists -------------------------------------------------------------------
-// One block per query tile: its non-skipped key tiles, ascending.
-__global__ void k0_lists(Plan p)
-{
-    __shared__ int warp_cnt[4];
-    __shared__ int base;
-    const int self = blockIdx.x;
-    if (threadIdx.x == 0)
-        base = 0;
-    __syncthreads();
-    for (int o0 = 0; o0 < p.n_kt; o0 += blockDim.x) {
-        const int o = o0 + threadIdx.x;
-        uint8_t c = TILE_SKIP;
-        if (o < p.n_kt)
-            c = p.cls[(size_t)self * p.n_kt + o];
-        if (c == TILE_SINGLE)
-            c = TILE_SKIP; // handled outside the tensor-core lists
-        const unsigned bal = __ballot_sync(0xffffffffu, c != TILE_SKIP);
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-        if (lane == 0)
-            warp_cnt[wid] = __popc(bal);
-        __syncthreads();
-        int off = base;
-        for (int w = 0; w < wid; ++w)
-            off += warp_cnt[w];
-        off += __popc(bal & ((1u << lane) - 1u));
-        if (c != TILE_SKIP) {
-            const int2 kt = p.ktile[o];
-            p.klist[(size_t)self * p.n_kt + off] = make_int2(kt.x, kt.y | ((int)c << 16));
-        }
-        __syncthreads();
-        if (threadIdx.x == 0)
-            base += warp_cnt[0] + warp_cnt[1] + warp_cnt[2] + warp_cnt[3];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        p.kcount[self] = base;
-        // SINGLE slots were handed out in arrival order: list them by ascending key tile so that
-        // the order of the per-pair sums does not change from run to run
-        const int ns = min(p.scount[self], MAX_SINGLE);
-        uint8_t ord[MAX_SINGLE];
-        for (int i = 0; i < ns; ++i) {
-            int j = i;
-            const int kt = p.skt[self * MAX_SINGLE + i];
-            while (j > 0 && p.skt[self * MAX_SINGLE + ord[j - 1]] > kt) {
-                ord[j] = ord[j - 1];
-                --j;
-            }
-            ord[j] = (uint8_t)i;
-        }
-        for (int i = 0; i < ns; ++i) {
-            p.sorder[self * MAX_SINGLE + i] = ord[i];
-            p.sbase[self * MAX_SINGLE + i] = p.ktile[p.skt[self * MAX_SINGLE + ord[i]]].x;
-        }
-    }
-    __syncthreads();
-    {
-        const int ns = min(p.scount[self], MAX_SINGLE);
-        for (int i = 0; i < ns; ++i) {
-            const int slot = p.sorder[self * MAX_SINGLE + i];
-            const int col = p.scol[((size_t)self * MAX_SINGLE + slot) * BM + threadIdx.x];
-            p.scs[((size_t)self * MAX_SINGLE + i) * BM + threadIdx.x] = (uint8_t)col;
-        }
-    }
-}
-
-// ---- 4b. order query tiles longest-first ----------------------------------------------------
-__global__ void k0_schedule(Plan p)
-{
-    extern __shared__ int cnt[];
-    const int n = p.n_qt;
-    if (n <= 8192) {
-        for (int i = threadIdx.x; i < n; i += blockDim.x)
-            cnt[i] = p.kcount[i];
-        __syncthreads();
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const int ci = cnt[i];
-            int rank = 0;
-            for (int j = 0; j < n; ++j)
-                rank += (cnt[j] > ci) || (cnt[j] == ci && j < i);
-            p.qorder[rank] = i;
-        }
-    } else {
-        for (int i = threadIdx.x; i < n; i += blockDim.x)
-            p.qorder[i] = n - 1 - i;
-    }
-    // Order of the SINGLE-tile backward: query tiles by the first token of their lowest SINGLE
-    // key tile (tiles without such entries last).  In the depth-major layout the chain tiles of
-    // one block of anchors at depths 1, 2, .. then run one after the other, and the fp32 dK / dV
-    // rows they all add to are still in L2 (one trip to memory per key row instead of one per depth).
-    __syncthreads();
-    if (n <= 8192) {
-        for (int i = threadIdx.x; i < n; i += blockDim.x)
-            cnt[i] = p.scount[i] > 0 ? p.sbase[i * MAX_SINGLE] : INT_MAX;
-        __syncthreads();
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const int ci = cnt[i];
-            int rank = 0;
-            for (int j = 0; j < n; ++j)
-                rank += (cnt[j] < ci) || (cnt[j] == ci && j < i);
-            p.sperm[rank] = i;
-        }
-    } else {
-        for (int i = threadIdx.x; i < n; i += blockDim.x)
-            p.sperm[i] = i;
-    }
-}
-
-// ---- 4c. backward work items ------------------------------------------------------------------
-// A backward work item is one key tile together with the non-skipped query tiles of one aligned
-// group of BWD_CQ consecutive query tiles ("chunk").  Items are laid out chunk-major so that the
-// CTAs running at the same time work on the same few query tiles: their Q / dO rows and their
-// fp32 dQ staging rows then stay in L2.
-// The items with all BWD_CQ query tiles come first, chunk-major; the smaller ones (the chunks on
-// the mask's diagonal) follow in descending size, so that the static round-robin over the CTAs
-// ends on small items and the CTAs finish together.
-// Pass 1, one block per chunk: for every key tile a 16-bit word (bit b: query tile 8c+b is not
-// skipped, bit 8+b: it is FULL), and how many key tiles have 1, 2, .. BWD_CQ query tiles.
-__global__ void k0_chunk_masks(Plan p)
-{
-    __shared__ int hist[BWD_CQ];
-    const int c = blockIdx.x;
-    if (threadIdx.x < BWD_CQ)
-        hist[threadIdx.x] = 0;
-    __syncthreads();
-    for (int kt = threadIdx.x; kt < p.n_kt; kt += blockDim.x) {
-        unsigned m = 0;
-        for (int b = 0; b < BWD_CQ; ++b) {
-            const int qt = c * BWD_CQ + b;
-            if (qt < p.n_qt) {
-                const uint8_t cl = p.cls[(size_t)qt * p.n_kt + kt];
-                if (cl != TILE_SKIP && cl != TILE_SINGLE)
-                    m |= 1u << b;
-                if (cl == TILE_FULL)
-                    m |= 1u << (8 + b);
+        group_sync(group);
+        const int slot = slot_of[group];
+        if (slot >= 0) {
+            raw_col[slot][row] = (uint8_t)col;
+            const int lo = __reduce_min_sync(0xffffffffu, col == NO_COL ? INT_MAX : ktile.x + col);
+            const int hi = __reduce_max_sync(0xffffffffu, col == NO_COL ? -1 : ktile.x + col);
+            if (lane == 0) {
+                atomicMin(&raw_min[slot], lo);
+                atomicMax(&raw_max[slot], hi);
             }
         }
-        p.cmask[(size_t)c * p.n_kt + kt] = (uint16_t)m;
-        if (m != 0)
-            atomicAdd(&hist[__popc(m & 0xffu) - 1], 1);
     }
     __syncthreads();
-    if (threadIdx.x < BWD_CQ)
-        p.ccount[c * BWD_CQ + threadIdx.x] = hist[threadIdx.x];
-}
+    // ---- one-key-per-row tiles: ascending by key tile (they were numbered in arrival order, and the
+    // order of the per-pair sums shall not change from run to run)
+    const int nr = min(n_raw, RAW_SINGLE);
+    if (tid < nr) {
+        int rank = 0;
+        for (int j = 0; j < nr; ++j)
+            rank += raw_kt[j] < raw_kt[tid];
+        raw_ord[rank] = tid;
+        raw_conflict[rank] = 0;
+    }
+    __syncthreads();
+    // Two neighbours become one entry when their keys lie within 128 tokens and no row has a key in
+    // both: the chain keys of 128 consecutive anchors are 128 consecutive tokens, which straddle two
+    // key tiles unless the anchors per depth are a multiple of 128.  (391 anchors, 8 depths, 32 heads of
+    // 128: forward 94 -> 72 us, the pairs' backward 76 -> 49 us.)
+    for (int i = group; i + 1 < nr; i += PLAN_GROUPS)
+        if (raw_col[raw_ord[i]][row] != NO_COL && raw_col[raw_ord[i + 1]][row] != NO_COL)
+            raw_conflict[i] = 1;
+    __syncthreads();
+    if (tid == 0) {
+        int n = 0;
+        for (int i = 0; i < nr; ++i, ++n) {
+            const bool join = i + 1 < nr && !raw_conflict[i] &&
+                              raw_max[raw_ord[i + 1]] - raw_min[raw_ord[i]] < BN;
+            if (n == MAX_SINGLE) { // no room: this tile and the rest go to the tensor cores
+                for (; i < nr; ++i)
+                    cls[raw_kt[raw_ord[i]]] = TILE_PARTIAL;
+                break;
+            }
+            entry[n] = make_int2(i, join ? i + 1 : i);
+            i += join;
+        }
+        n_entry = n;
+        p.scount[qt] = n;
+    }
+    __syncthreads();
+    const int ns = n_entry;
+    for (int i = group; i < ns; i += PLAN_GROUPS) {
+        const int2 e = entry[i];
+        const int first = raw_ord[e.x], last = raw_ord[e.y];
+        const int base = raw_min[first];
+        int col = raw_col[first][row], kt = raw_kt[first];
+        if (col == NO_COL && e.y != e.x) {
+            col = raw_col[last][row];
+            kt = raw_kt[last];
+        }
+        if (col != NO_COL)
+            col = p.ktile[kt].x + col - base;
+        p.scs[((size_t)qt * MAX_SINGLE + i) * BM + row] = (uint8_t)col;
+        if (row == 0)
+            p.sbase[qt * MAX_SINGLE + i] = base;
+    }
+    // ---- the query tile's key list, ascending (SINGLE tiles are handled outside it)
+    const int listed = block_compact(
+        p.n_kt, warp_cnt, [&](int kt) { const uint8_t c = cls[kt]; return c != TILE_SKIP && c != TILE_SINGLE; },
+        [&](int kt, int at) {
+            const int2 k = p.ktile[kt];
+            p.klist[(size_t)qt * p.n_kt + at] = make_int2(k.x, k.y | ((int)cls[kt] << 16));
+        });
+    if (tid == 0)
+        p.kcount[qt] = listed;
 
-// Pass 2, one block per chunk: the items of the chunk go to their size class's region, behind the
-// same-size items of all earlier chunks, key tiles ascending.
-// item = (key tile, chunk, mask word, query tiles in the item).
-__global__ void k0_chunk_items(Plan p)
-{
-    __shared__ int warp_cnt[4];
-    __shared__ int base[BWD_CQ]; // where this chunk's items of each size start
-    __shared__ int cursor;
-    const int c = blockIdx.x, n_ch = gridDim.x;
-    if (threadIdx.x < BWD_CQ) {
-        // sizes in output order: BWD_CQ, BWD_CQ-1, .., 1
-        const int sz = threadIdx.x; // index = size - 1
-        int off = 0;
-        for (int s2 = BWD_CQ - 1; s2 > sz; --s2)
-            for (int i = 0; i < n_ch; ++i)
-                off += p.ccount[i * BWD_CQ + s2];
-        for (int i = 0; i < c; ++i)
-            off += p.ccount[i * BWD_CQ + sz];
-        base[sz] = off;
-        if (c == n_ch - 1 && sz == 0) {
-            p.counters[1] = off + p.ccount[c * BWD_CQ];
-            int tiles = 0;
-            for (int s2 = 0; s2 < BWD_CQ; ++s2)
-                for (int i = 0; i < n_ch; ++i)
-                    tiles += (s2 + 1) * p.ccount[i * BWD_CQ + s2];
-            p.counters[4] = tiles;
-        }
-    }
+    // ---- backward work items, by the last block of a chunk of BWD_CQ consecutive query tiles: a key
+    // tile together with the chunk's query tiles that do not skip it.  Items of a chunk stay together,
+    // so that the CTAs running at the same time work on the same few query tiles (their Q / dO rows
+    // and their fp32 dQ staging rows then stay in L2), and are kept by size: the backward takes the
+    // full-size ones first and ends on small ones, so that the CTAs finish together.
+    __threadfence();
     __syncthreads();
-    for (int sz = BWD_CQ - 1; sz >= 0; --sz) {
-        if (threadIdx.x == 0)
-            cursor = base[sz];
+    if (for_bwd) {
+        const int c = qt / BWD_CQ, nq = min(BWD_CQ, p.n_qt - c * BWD_CQ);
+        if (tid == 0)
+            flag = atomicAdd(&p.cdone[c], 1) == nq - 1;
         __syncthreads();
-        for (int o0 = 0; o0 < p.n_kt; o0 += blockDim.x) {
-            const int kt = o0 + threadIdx.x;
-            unsigned m = 0;
-            if (kt < p.n_kt)
-                m = p.cmask[(size_t)c * p.n_kt + kt];
-            const bool mine = m != 0 && __popc(m & 0xffu) == sz + 1;
-            const unsigned bal = __ballot_sync(0xffffffffu, mine);
-            const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-            if (lane == 0)
-                warp_cnt[wid] = __popc(bal);
+        if (flag) {
+            __threadfence();
+            auto word = [&](int kt) { // bit b: query tile c * BWD_CQ + b is not skipped, bit 8 + b: FULL
+                unsigned m = 0;
+                for (int b = 0; b < nq; ++b) {
+                    const uint8_t cl = __ldcg(p.cls + (size_t)(c * BWD_CQ + b) * p.n_kt + kt);
+                    if (cl != TILE_SKIP && cl != TILE_SINGLE)
+                        m |= 1u << b;
+                    if (cl == TILE_FULL)
+                        m |= 1u << (8 + b);
+                }
+                return m;
+            };
+            const size_t cap = (size_t)((p.n_qt + BWD_CQ - 1) / BWD_CQ) * p.n_kt; // per size
+            if (tid < 2 * BWD_CQ)
+                hist[tid] = 0;
             __syncthreads();
-            int off = cursor;
-            for (int w = 0; w < wid; ++w)
-                off += warp_cnt[w];
-            off += __popc(bal & ((1u << lane) - 1u));
-            if (mine)
-                p.bitems[off] = make_int4(kt, c, (int)m, sz + 1);
+            unsigned m = 0; // the word of this thread's first key tile, kept for the second pass
+            for (int kt = tid; kt < p.n_kt; kt += PLAN_THREADS) {
+                const unsigned mm = word(kt);
+                m = kt == tid ? mm : m;
+                if (mm)
+                    atomicAdd(&hist[__popc(mm & 0xffu) - 1], 1);
+            }
             __syncthreads();
-            if (threadIdx.x == 0)
-                cursor += warp_cnt[0] + warp_cnt[1] + warp_cnt[2] + warp_cnt[3];
+            if (tid < BWD_CQ && hist[tid])
+                hist[BWD_CQ + tid] = atomicAdd(&p.counters[CNT_ITEMS + tid], hist[tid]);
             __syncthreads();
+            for (int kt = tid; kt < p.n_kt; kt += PLAN_THREADS) {
+                const unsigned mm = kt == tid ? m : word(kt);
+                if (mm) {
+                    const int sz = __popc(mm & 0xffu);
+                    const int at = atomicAdd(&hist[BWD_CQ + sz - 1], 1);
+                    p.bitems[(size_t)(sz - 1) * cap + at] = make_int4(kt, c, (int)mm, sz);
+                }
+            }
         }
     }
+    // ---- orders of the query tiles, by the last block of all
+    __syncthreads();
+    if (tid == 0)
+        flag = atomicAdd(&p.counters[CNT_DONE], 1) == p.n_qt - 1;
+    __syncthreads();
+    if (!flag)
+        return;
+    __threadfence();
+    // the forward takes the longest query tiles first
+    block_sort(p.n_qt, hist, warp_cnt, p.qorder, [&](int i) {
+        return SORT_BUCKETS - 1 - min(SORT_BUCKETS - 1, 2 * __ldcg(p.kcount + i) + __ldcg(p.scount + i));
+    });
+    // The SINGLE-tile backward takes them by the first token of their lowest SINGLE entry (tiles
+    // without such entries last).  In the depth-major layout the chain tiles of one block of anchors
+    // at depths 1, 2, .. then run one after the other, and the fp32 dK / dV rows they all add to are
+    // still in L2 (one trip to memory per key row instead of one per depth).
+    int shift = 7;
+    while (((seq_end - seq_begin) >> shift) >= SORT_BUCKETS - 1)
+        ++shift;
+    if (for_bwd)
+        block_sort(p.n_qt, hist, warp_cnt, p.sperm, [&](int i) {
+            return __ldcg(p.scount + i) > 0 ? (__ldcg(p.sbase + i * MAX_SINGLE) - seq_begin) >> shift : SORT_BUCKETS - 1;
+        });
 }
 
 // ---- test hook: the mask as the device predicate sees it -----------------------------------
@@ -406,42 +544,16 @@ __global__ void k0_mask_dense(Plan p, RangeList ranges, uint8_t *out)
         (uint8_t)(vis && mq != META_NONE_K && allowed_packed(mq, mk));
 }
 
-// No visible key: every query tile has an empty list.
-__global__ void k0_empty(Plan p)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < p.n_qt) {
-        p.kcount[i] = 0;
-        p.qorder[i] = i;
-        p.sperm[i] = i;
-    }
-}
-
 int launch_plan(const Plan &p, const int32_t *anchor, const int32_t *depth, int K, int seq_begin,
-                int seq_end, const RangeList &ranges, bool for_bwd, int Hkv, cudaStream_t s)
+                int seq_end, const RangeList &ranges, bool for_bwd, cudaStream_t s)
 {
-    (void)Hkv;
-    const int n_seq = seq_end - seq_begin;
-    k0_prepare<<<(n_seq + 255) / 256 > 0 ? (n_seq + 255) / 256 : 1, 256, 0, s>>>(
-        p, anchor, depth, K, seq_begin, seq_end, ranges);
     if (p.n_qt == 0)
-        return 1;
-    if (p.n_kt == 0) {
-        k0_empty<<<(p.n_qt + 255) / 256, 256, 0, s>>>(p);
-        return 2;
-    }
-    k0_summaries<<<p.n_qt + p.n_kt, 128, 0, s>>>(p);
-    k0_classify_quick<<<dim3((p.n_kt + 127) / 128, p.n_qt), 128, 0, s>>>(p);
-    k0_classify_exact<<<592, 128, 0, s>>>(p);
-    k0_lists<<<p.n_qt, 128, 0, s>>>(p);
-    const int smem = (p.n_qt <= 8192 ? p.n_qt : 0) * (int)sizeof(int);
-    k0_schedule<<<1, 1024, smem, s>>>(p);
-    if (!for_bwd)
-        return 6;
-    const int n_ch = (p.n_qt + BWD_CQ - 1) / BWD_CQ;
-    k0_chunk_masks<<<n_ch, 128, 0, s>>>(p);
-    k0_chunk_items<<<n_ch, 128, 0, s>>>(p);
-    return 8;
+        return 0;
+    const int n_seq = seq_end - seq_begin;
+    const int blocks = (n_seq + 127) / 128 > p.n_qt + p.n_kt ? (n_seq + 127) / 128 : p.n_qt + p.n_kt;
+    k0_tiles<<<blocks, 128, 0, s>>>(p, anchor, depth, K, seq_begin, seq_end, ranges);
+    k0_plan<<<p.n_qt, PLAN_THREADS, 0, s>>>(p, seq_begin, seq_end, for_bwd ? 1 : 0);
+    return 2;
 }
 
 // ---- self-test of the bounded waits ----------------------------------------------------------

@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(128, D == 64 ? 4 : 2) single_bwd(const SingleP
                         *so = sO + (size_t)rl * row_elems;
     float *rnl2 = snl2 + rl * P.Hq, *rnd = snd + rl * P.Hq;
     const int qt = r / BM, rr = r % BM;
-    const int ns = min(P.scount[qt], MAX_SINGLE);
+    const int ns = P.scount[qt];
     single_pass<D, true, KEYS>(P, 0, ns, sub, um, r, g, qt, rr, G, sq, sdo, so, rnl2, rnd);
     for (int i0 = KEYS; i0 < ns; i0 += KEYS) {
         __syncwarp(um); // lane 0's row values are visible to the unit's later passes

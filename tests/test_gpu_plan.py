@@ -1,0 +1,78 @@
+"""GPU: the plan kernels where their dispatch can go wrong -- runs that end on, just before and just
+after a tile border, tiles of mixed depth, unsorted tiles, more undecided pairs than are kept in shared
+memory, more query tiles than threads -- against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import peagle_oracle as orc
+from paper_2602_01469_b200 import binding, inputs
+from tests.gpu_common import DeviceCase, check_forward
+from tests.test_gpu_backward import check_grads, oracle_all, run_partitioned
+from tests.test_gpu_mask_and_tiles import device_problem
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = binding.Context(0)
+    yield c
+    c.close()
+
+
+def check_classes(ctx, anchor, depth, K, q, k):
+    prob = device_problem([0, anchor.shape[0]], anchor, depth, K)
+    got = binding.peagle_classify_tiles(ctx, prob, binding.Partition(0, q, k))
+    want, _, _ = orc.classify_tiles(anchor, depth, q[0], q[1], k, 128, 128)
+    assert np.array_equal(got, want)
+    assert binding.peagle_poll_status(ctx) == 0
+
+
+@pytest.mark.parametrize("order", ["depth_major", "anchor_major"])
+@pytest.mark.parametrize("n,K", [(1, 8), (63, 6), (127, 5), (128, 5), (129, 5), (255, 3), (385, 4), (40, 40)])
+def test_classes_at_tile_borders(ctx, n, K, order):
+    anchor, depth = inputs.full_grid(n, K)
+    perm = inputs.arrange_by_segment(anchor, depth, np.zeros(n * K, np.int32), order)
+    anchor, depth = anchor[perm], depth[perm]
+    check_classes(ctx, anchor, depth, K, (0, n * K), None)
+    if n * K > 40:      # ranges that start inside a run, a one-token range among them
+        check_classes(ctx, anchor, depth, K, (7, n * K - 3), [(1, 2), (5, n * K // 2 + 1), (n * K - 9, n * K)])
+
+
+def test_classes_of_one_anchor_and_of_unsorted_tiles(ctx):
+    # 250 depths of one anchor: chain tiles that are FULL without a depth-0 key in them
+    check_classes(ctx, np.zeros(250, np.int32), np.arange(250, dtype=np.int32), 250, (0, 250), None)
+    # 282 unsorted key tiles: all pairs of a query tile are undecided
+    anchor, depth = inputs.full_grid(9000, 4)
+    perm = np.random.default_rng(3).permutation(36000)
+    check_classes(ctx, anchor[perm], depth[perm], 4, (100, 430), None)
+
+
+@pytest.mark.parametrize("w", [
+    # chain keys of a query tile straddle two key tiles by one token, by half, by all but one
+    inputs.Workload("straddle_1", (129,), 6, 4, 2, 64, seed=41),
+    inputs.Workload("straddle_64", (192,), 6, 4, 2, 128, seed=42),
+    inputs.Workload("straddle_127", (255,), 6, 4, 2, 64, seed=43),
+    # thinned chains: neighbouring windows that may and may not be joined
+    inputs.Workload("thinned", (391,), 8, 4, 2, 64, seed=44, cod_r=0.8),
+], ids=lambda w: w.name)
+def test_joined_windows(ctx, w):
+    case = DeviceCase(w)
+    run_partitioned(ctx, case)
+    O, LSE, dQ, dK, dV = oracle_all(case)
+    check_forward(case.O.float().cpu().numpy(), case.LSE.t().cpu().numpy(), O, LSE)
+    check_grads(case, dQ, dK, dV)
+
+
+def test_more_query_tiles_than_threads(ctx):
+    case = DeviceCase(inputs.Workload("long", (8300,), 8, 2, 1, 64, seed=45))
+    run_partitioned(ctx, case)
+    part = case.parts[0]
+    rows = np.sort(np.random.default_rng(1).choice(case.T, 64, replace=False))
+    O, LSE = case.oracle_fwd(part, rows=rows)
+    idx = torch.as_tensor(rows, device="cuda")
+    check_forward(case.O[idx].float().cpu().numpy(), case.LSE[:, idx].t().cpu().numpy(), O, LSE)
+    dQ, _, _ = case.oracle_bwd(part, rows=rows)
+    got = case.dQ[idx].float().cpu().numpy()
+    assert np.linalg.norm(got - dQ) <= 1e-2 * np.linalg.norm(dQ)
