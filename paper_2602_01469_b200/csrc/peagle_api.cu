@@ -34,11 +34,11 @@ struct peagle_ctx {
 namespace {
 
 // SINGLE tiles are taken out of the backward's tensor-core lists when the kernel that does them
-// pair by pair fits: a block of at most 16 KV heads x 8 lanes, a query row of all heads (Q, dO, O
-// and two fp32 values per head) within its shared memory.  Otherwise such tiles stay PARTIAL.
+// pair by pair fits: a block of at most 16 KV heads x 8 lanes, a query row of all heads within its
+// shared memory.  Otherwise such tiles stay PARTIAL.
 bool single_tiles_ok(const peagle_problem_t *prob)
 {
-    return prob->n_kv_heads <= 16 && (size_t)prob->n_q_heads * (6 * prob->head_dim + 8) <= 200 * 1024;
+    return prob->n_kv_heads <= 16 && single_row_bytes(prob->n_q_heads, prob->head_dim) <= 200 * 1024;
 }
 
 int cuda_fail(peagle_ctx *ctx, cudaError_t e, const char *what)
@@ -270,6 +270,7 @@ int run_fwd(peagle_ctx *ctx, const peagle_problem_t *prob, const Call &c, const 
         a.nl2 = hand->nl2;
         a.nd = hand->nd;
         a.mqp = hand->mqp;
+        a.dq_acc = hand->dq_acc;
     }
     a.Q = Q;
     a.K = K;

@@ -24,6 +24,7 @@ namespace peagle {
 using namespace sm100;
 
 int make_bf16_map(EncodeTiledFn enc, CUtensorMap *m, const void *base, int D, int H, int T);
+int make_f32_map(EncodeTiledFn enc, CUtensorMap *m, float *base, int D, int H, int rows, int box_rows);
 int launch_bwd128_main(const CUtensorMap &tmQ, const CUtensorMap &tmdO, const CUtensorMap &tmK,
                        const CUtensorMap &tmV, const CUtensorMap &tmDQ, const CUtensorMap &tmDK, const CUtensorMap &tmDV,
                        const BwdParams &P, int n_sm, cudaStream_t s);
@@ -678,30 +679,16 @@ static int launch_bwd_t(const Plan &p, const BwdArgs &a, EncodeTiledFn enc, int 
     const int q_pad = p.n_qt * BM;
     // fp32 sums as tensors for tiled reduce-adds, 32 columns x 32 rows: the dQ staging
     // [q_len][Hq][D] and the caller's dK / dV [T][Hkv][D]
-    auto sum_map = [&](CUtensorMap *m, float *base, int H, int rows) {
-        cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)rows};
-        cuuint64_t strides[2] = {(cuuint64_t)D * 4, (cuuint64_t)H * D * 4};
-        cuuint32_t box[3] = {32, 1, 32};
-        cuuint32_t estr[3] = {1, 1, 1};
-        return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-    };
     CUtensorMap tmDQ, tmDK, tmDV;
-    if (!sum_map(&tmDQ, a.dq_acc, a.Hq, q_len) || !sum_map(&tmDK, a.dK_acc, a.Hkv, p.T) ||
-        !sum_map(&tmDV, a.dV_acc, a.Hkv, p.T))
+    if (make_f32_map(enc, &tmDQ, a.dq_acc, D, a.Hq, q_len, 32) || make_f32_map(enc, &tmDK, a.dK_acc, D, a.Hkv, p.T, 32) ||
+        make_f32_map(enc, &tmDV, a.dV_acc, D, a.Hkv, p.T, 32))
         return PEAGLE_ERR_CUDA;
     const size_t n_prep = (size_t)q_len * a.Hq * (D / 8);
     const size_t n_prep_pad = (size_t)q_pad * a.Hq * (D / 8);
-    // Per-row values and the initial dQ staging: with SINGLE tiles, their backward does both.
-    int launches = launch_bwd_single(p, a, s);
-    if (launches < 0)
-        return launches;
-    if (launches == 0 && a.rows_ready) {
-        // the forward of this partition left the per-row values; only the staging needs clearing
-        if (cudaMemsetAsync(a.dq_acc, 0, (size_t)q_len * a.Hq * D * sizeof(float), s) != cudaSuccess)
-            return PEAGLE_ERR_CUDA;
-    } else if (launches == 0) {
+    int launches = 0;
+    // Per-row values and a cleared dQ staging: the forward of the partition leaves both when it runs in
+    // the driver, where dO is known.
+    if (!a.rows_ready) {
         bwd_prepare<D><<<(unsigned)((n_prep_pad + 255) / 256), 256, 0, s>>>(
             static_cast<const __nv_bfloat16 *>(a.O), static_cast<const __nv_bfloat16 *>(a.dO), a.LSE,
             p.meta, a.nl2, a.nd, a.mqp, a.dq_acc, p.q_begin, q_len, q_pad, a.Hq, p.T);
@@ -744,6 +731,10 @@ static int launch_bwd_t(const Plan &p, const BwdArgs &a, EncodeTiledFn enc, int 
         if (ev1)
             cudaEventRecord(ev1, s);
         ++launches;
+    }
+    if (p.allow_single) {
+        const int n = launch_finish_single(p, a, s);
+        return n < 0 ? n : launches + n;
     }
     bwd_finish_dq<<<(unsigned)((n_prep + 255) / 256), 256, 0, s>>>(
         a.dq_acc, static_cast<__nv_bfloat16 *>(a.dQ) + (size_t)p.q_begin * a.Hq * D, n_prep);

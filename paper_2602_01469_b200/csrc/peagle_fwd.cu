@@ -95,7 +95,9 @@ struct FwdCfg {
     // warp); head_dim 128 has no room for the two staging tiles and stores its rows directly
     static constexpr bool O_STAGED = (D == 64);
     static constexpr int OFF_OST = OFF_V + NS * TILE_BYTES;
-    static constexpr int OFF_META = OFF_OST + (O_STAGED ? 2 * TILE_BYTES : 0);
+    // 128 x 32 fp32 zeros, the source of the stores that clear the backward's dQ staging
+    static constexpr int OFF_ZERO = OFF_OST + (O_STAGED ? 2 * TILE_BYTES : 0);
+    static constexpr int OFF_META = OFF_ZERO + PANEL_BYTES;
     static constexpr int OFF_BAR = OFF_META + NS * BN * 4;
     static constexpr int N_BAR = 1 + 4 * NS + 8 + 9;
     static constexpr int OFF_MISC = OFF_BAR + N_BAR * 8; // tmem slot, abort flag, item queue
@@ -114,7 +116,7 @@ template <int D>
 __global__ void __launch_bounds__(384, 1)
 fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
            const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
-           const FwdParams P)
+           const __grid_constant__ CUtensorMap tmZ, const FwdParams P)
 {
     using C = FwdCfg<D>;
     constexpr int NS = C::NS;
@@ -195,6 +197,11 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     if (warp == 8) {
         tmem_alloc(sb + C::OFF_MISC, 512);
         tmem_relinquish();
+    }
+    if (P.dO) {
+        for (int i = threadIdx.x; i < C::PANEL_BYTES / 16; i += 384)
+            reinterpret_cast<uint4 *>(sp + C::OFF_ZERO)[i] = make_uint4(0, 0, 0, 0);
+        fence_proxy_async_smem();
     }
     tc_fence_before();
     __syncthreads();
@@ -317,7 +324,17 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     m_cur[i] = m_nxt[i];
             }
             kpos += (uint32_t)(n_single + cnt);
+            // Hand-over to the backward: the item's rows of the fp32 dQ staging are cleared here, where
+            // the memory system is idle (the map ends at the partition's last row).
+            if (P.dO && live && lane == 0) {
+                for (int x = 0; x < ntile; ++x)
+                    for (int pn = 0; pn < D / 32; ++pn)
+                        tma_store_3d(&tmZ, sb + C::OFF_ZERO, pn * 32, it.h0 + x, it.qt * BM);
+                bulk_commit_group();
+            }
         }
+        if (lane == 0)
+            bulk_wait_group<0>();
     } else if (warp == 8 || warp == 10) {
         // ------------------------------------------------------------ MMA issue
         // Lane 0 of warp 8 issues every MMA of tile A, lane 0 of warp 10 those of tile B: the two
@@ -930,6 +947,20 @@ int make_bf16_map(EncodeTiledFn enc, CUtensorMap *m, const void *base, int D, in
     return make_map(enc, m, base, D, H, T);
 }
 
+// Tensor map of fp32 sums [rows][H][D]: 32 columns x box_rows rows, for tiled reduce-adds and stores.
+int make_f32_map(EncodeTiledFn enc, CUtensorMap *m, float *base, int D, int H, int rows, int box_rows)
+{
+    cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)rows};
+    cuuint64_t strides[2] = {(cuuint64_t)D * 4, (cuuint64_t)H * D * 4};
+    cuuint32_t box[3] = {32, 1, (cuuint32_t)box_rows};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+               ? 0
+               : -1;
+}
+
 template <int D>
 static int launch_fwd_t(const Plan &p, const FwdArgs &a, EncodeTiledFn enc, int n_sm,
                         cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1)
@@ -938,6 +969,9 @@ static int launch_fwd_t(const Plan &p, const FwdArgs &a, EncodeTiledFn enc, int 
     CUtensorMap tmQ, tmK, tmV, tmO;
     if (make_map(enc, &tmQ, a.Q, D, a.Hq, p.T) || make_map(enc, &tmK, a.K, D, a.Hkv, p.T) ||
         make_map(enc, &tmV, a.V, D, a.Hkv, p.T) || make_map(enc, &tmO, a.O, D, a.Hq, p.q_end))
+        return PEAGLE_ERR_CUDA;
+    CUtensorMap tmZ = tmO;
+    if (a.dO && make_f32_map(enc, &tmZ, a.dq_acc, D, a.Hq, p.q_end - p.q_begin, BM))
         return PEAGLE_ERR_CUDA;
     FwdParams P;
     P.klist = p.klist;
@@ -976,7 +1010,7 @@ static int launch_fwd_t(const Plan &p, const FwdArgs &a, EncodeTiledFn enc, int 
     P.n_items = p.n_qt * n_hb;
     if (ev0)
         cudaEventRecord(ev0, s);
-    fwd_kernel<D><<<std::min(P.n_items, n_sm), 384, FwdCfg<D>::SMEM_BYTES, s>>>(tmQ, tmK, tmV, tmO, P);
+    fwd_kernel<D><<<std::min(P.n_items, n_sm), 384, FwdCfg<D>::SMEM_BYTES, s>>>(tmQ, tmK, tmV, tmO, tmZ, P);
     if (ev1)
         cudaEventRecord(ev1, s);
     return 1;

@@ -75,10 +75,11 @@ struct FwdArgs {
     int Hq, Hkv, D;
     float scale;
     // optional hand-over to the backward of the same partition (all null when not wanted):
-    // dO and the backward's per-row scratch, which the forward's epilogue then fills
+    // dO, the backward's per-row scratch, which the forward's epilogue then fills, and its dQ staging
     const void *dO = nullptr;
     float *nl2 = nullptr, *nd = nullptr;
     int32_t *mqp = nullptr;
+    float *dq_acc = nullptr; // the backward's dQ staging, which the forward clears
 };
 
 struct BwdArgs {
@@ -94,7 +95,7 @@ struct BwdArgs {
     float *dq_acc;  // [q_len][Hq][D] scratch, fp32
     int Hq, Hkv, D;
     float scale;
-    bool rows_ready = false; // nl2 / nd / mqp were written by the forward of this partition
+    bool rows_ready = false; // nl2 / nd / mqp were written, dq_acc was cleared by the forward of this partition
 };
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
@@ -124,9 +125,11 @@ int launch_fwd(const Plan &p, const FwdArgs &a, EncodeTiledFn enc, int n_sm, cud
                cudaEvent_t ev0, cudaEvent_t ev1);
 int launch_bwd(const Plan &p, const BwdArgs &a, EncodeTiledFn enc, int n_sm, cudaStream_t s,
                cudaEvent_t ev0, cudaEvent_t ev1);
-// Backward of the SINGLE tiles (head_dim 64 with SINGLE tiles enabled, else returns 0): adds to
-// dK_acc / dV_acc, and prepares the tile kernel's per-row values and the initial dQ staging.
-int launch_bwd_single(const Plan &p, const BwdArgs &a, cudaStream_t s);
+// The backward's last pass where SINGLE entries are enabled: their pairs, added to dK_acc / dV_acc and to
+// the dQ staging that the tile kernel left, and dQ rounded to bf16.
+int launch_finish_single(const Plan &p, const BwdArgs &a, cudaStream_t s);
+// Shared memory that it takes per query row.
+size_t single_row_bytes(int Hq, int D);
 int launch_cast_grads(const float *dK_acc, const float *dV_acc, void *dK, void *dV, size_t n,
                       cudaStream_t s);
 int launch_cast_one(const float *src, void *dst, size_t n, cudaStream_t s);
