@@ -30,10 +30,9 @@ int launch_bwd128_main(const CUtensorMap &tmQ, const CUtensorMap &tmdO, const CU
                        const BwdParams &P, int n_sm, cudaStream_t s);
 
 // ---------------------------------------------------------------------------------------------
-// head_dim 64.  The query columns of a step are two halves of 64, one per compute warpgroup, with
-// barriers of their own; the second half runs behind the first by the time of an exp phase, so that
-// the exp2 unit serves one half while the other does the rest of its step.  The products run one step
-// ahead of the compute warps:
+// head_dim 64.  The query columns of a step are two halves of 64, eight compute warps each, with
+// barriers of their own, so that the halves drift apart and the exp2 unit serves one while the other
+// does the rest of its step.  The products run one step ahead of the compute warps:
 //   S^T(i+1) of a half behind its dV(i), once its P^T(i) is in tensor memory
 //   dP^T(i+1) of a half behind its dK(i), once its dS^T(i) is
 //   dQ(i) of both halves, once both dS^T(i) are in shared memory
@@ -43,28 +42,32 @@ int launch_bwd128_main(const CUtensorMap &tmQ, const CUtensorMap &tmdO, const CU
 // K and V of the item sit in tensor memory as bf16 (A operands of S^T and dP^T): a tensor-memory
 // operand leaves half of the shared-memory bandwidth to the other warps, a shared-memory one 5 %.
 // dS^T goes both over the dP^T columns (A operand of dK) and, swizzled, to shared memory (A operand
-// of dQ).  The scores are read as tcgen05.ld.16x256b gives them: a thread has 4 keys x 16 query columns,
-// so that it needs 16 instead of 64 of the row values -LSE and -Delta (a quarter of the loads).
+// of dQ).  Sixteen compute warps of 32 keys x 32 query columns: their time is the latency of waits,
+// tensor-memory and shared-memory accesses more than arithmetic, so four warps per scheduler hide more
+// of each other than two (with eight warps of 64 columns the kernel takes 8 % longer).  The scores are
+// read as tcgen05.ld.16x256b gives them: a thread has 4 keys x 8 query columns, so that it needs 8
+// instead of 32 of the row values -LSE and -Delta.
+// What bounds it now is shared memory: a step moves about 250 KB through it (112 KB operands, 64 KB dQ on
+// its way out, 34 KB Q / dO / row values, 32 KB dS^T), 1,950 of its 2,750 clocks; without the dQ tile's
+// writes and reads it would take 12 % less time.
 // The K tile of the next item is prefetched into a second shared-memory stage (V has one stage: it
 // is only read when it is copied to tensor memory at the start of its item); Q / dO have three
-// stages; the items come from a global cursor through a small queue.  512 threads: warps 0-7
-// compute, warps 8, 10 and 11 issue MMAs, warp 9 produces, warps 12-15 drain dQ and, at the end of
-// an item, dK / dV through fp32 panels in shared memory and tiled reduce-adds.
+// stages (with two, 10 % slower); the items come from a global cursor through a small queue.  768
+// threads: warps 0-15 compute, warps 16, 18 and 19 issue MMAs, warp 17 produces, warps 20-23 drain dQ and,
+// at the end of an item, dK / dV through fp32 panels in shared memory and tiled reduce-adds.
 // The drain has warps of its own because a thread with reductions in flight stalls on its next
 // proxy fence, which the compute warps need once per step for the dS^T hand-over.
-// Registers per thread after the roles re-split the CTA's allocation (512 threads x 128): two
-// warpgroups of compute warps, the warpgroup of the issuing / producing warps, the drain warpgroup.
-// The thread that issues the products wants its descriptors resident: with 56 (head_dim 128: 40)
-// registers for its warpgroup the compiler spilled them and re-formed them per product, and the
-// kernel was 9 (7) per cent slower than with 88.
+// Registers per thread after the roles re-split the CTA's allocation (768 threads x 80): four warpgroups
+// of compute warps, the warpgroup of the issuing / producing warps, the drain warpgroup.
 #ifndef BWD64_COMPUTE_REGS
-#define BWD64_COMPUTE_REGS 160
-#define BWD64_ISSUE_REGS 88
-#define BWD64_DRAIN_REGS 104
+#define BWD64_COMPUTE_REGS 88
+#define BWD64_ISSUE_REGS 48
+#define BWD64_DRAIN_REGS 80
 #endif
 namespace {
 constexpr int COMPUTE_REGS = BWD64_COMPUTE_REGS, ISSUE_REGS = BWD64_ISSUE_REGS, DRAIN_REGS = BWD64_DRAIN_REGS;
-static_assert(256 * COMPUTE_REGS + 128 * ISSUE_REGS + 128 * DRAIN_REGS <= 512 * 128,
+constexpr int THREADS = 768, LAUNCH_REGS = 80; // 24 warps
+static_assert(512 * COMPUTE_REGS + 128 * ISSUE_REGS + 128 * DRAIN_REGS <= THREADS * LAUNCH_REGS,
               "the re-split must fit the launch allocation, or setmaxnreg.inc waits for ever");
 } // namespace
 
@@ -89,7 +92,7 @@ struct Bwd64Cfg {
                          TM_DV = 448;
 };
 
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(THREADS, 1)
 bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmdO,
              const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
              const __grid_constant__ CUtensorMap tmDQ, const __grid_constant__ CUtensorMap tmDK,
@@ -129,17 +132,17 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             mbar_init(BAR(B_KVEMPTY + s), 1);
             mbar_init(BAR(B_SFULL + s), 1);
             mbar_init(BAR(B_DPFULL + s), 1);
-            mbar_init(BAR(B_PFULL + s), 4); // one arrival per warp
-            mbar_init(BAR(B_DSFULL + s), 4);
+            mbar_init(BAR(B_PFULL + s), 8); // one arrival per warp
+            mbar_init(BAR(B_DSFULL + s), 8);
         }
         mbar_init(BAR(B_DQFULL), 1);
-        mbar_init(BAR(B_KVTFULL), 8);
+        mbar_init(BAR(B_KVTFULL), 16);
         mbar_init(BAR(B_DQEMPTY), 4);
         mbar_init(BAR(B_ITEMDONE), 2);
         mbar_init(BAR(B_ACCFREE), 4);
         fence_mbar_init();
     }
-    if (warp == 8) {
+    if (warp == 16) {
         tmem_alloc(sb + C::OFF_MISC, 512);
         tmem_relinquish();
     }
@@ -148,9 +151,9 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    if (warp >= 12) {
-        // ------------------------------------------------------------ drain (warps 12-15)
-        reg_set<DRAIN_REGS, 128>();
+    if (warp >= 20) {
+        // ------------------------------------------------------------ drain (warps 20-23)
+        reg_set<DRAIN_REGS, LAUNCH_REGS>();
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         // A panel (this warp's 32 lanes, 32 columns) on its way out: registers -> swizzled fp32 tile
         // in shared memory -> tiled reduce-add.  Whole 128-byte row pieces reach L2 together, which
@@ -232,9 +235,9 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         }
         if (lane == 0)
             bulk_wait_group<0>();
-    } else if (warp >= 8) {
-        reg_set<ISSUE_REGS, 128>();
-        if (warp == 9) {
+    } else if (warp >= 16) {
+        reg_set<ISSUE_REGS, LAUNCH_REGS>();
+        if (warp == 17) {
             // -------------------------------------------------------- producer
             if (lane == 0) {
                 tma_prefetch_desc(&tmQ);
@@ -304,7 +307,7 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         } else {
             // -------------------------------------------------------- MMA issue: three warps, each
             // with its own accumulators (products into one accumulator keep one thread's order):
-            // warp 8 S^T and dV, warp 10 dP^T and dK, warp 11 dQ.  The whole warp walks the steps
+            // warp 16 S^T and dV, warp 18 dP^T and dK, warp 19 dQ.  The whole warp walks the steps
             // and waits, its elected lane issues (see elect_one).
             const uint32_t lead = elect_one();
             constexpr uint32_t IDESC_S = idesc_bf16_f32(128, 64, 0, 0);
@@ -314,12 +317,12 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             const uint32_t ds_m = desc_lo_sw128(sb + C::OFF_DS, TB);
             const uint32_t kv_m = desc_lo_sw128(sb + C::OFF_KV, TB);
             constexpr uint32_t TBU = TB >> 4; // one tile in descriptor units
-            // warp 8: Q for S^T, dO for dV; warp 10: dO for dP^T, Q for dK
-            const uint32_t b_k = desc_lo_sw128(sb + C::OFF_Q, 16) + (warp == 8 ? 0 : TBU);
-            const uint32_t b_m = desc_lo_sw128(sb + C::OFF_Q, TB) + (warp == 8 ? TBU : 0);
-            const uint32_t t_sc = tmem + (warp == 8 ? C::TM_S : C::TM_DP), t_kv = tmem + (warp == 8 ? C::TM_K : C::TM_V),
-                           t_acc = tmem + (warp == 8 ? C::TM_DV : C::TM_DK);
-            const uint32_t bar_sc = BAR(warp == 8 ? B_SFULL : B_DPFULL), bar_in = BAR(warp == 8 ? B_PFULL : B_DSFULL);
+            // warp 16: Q for S^T, dO for dV; warp 18: dO for dP^T, Q for dK
+            const uint32_t b_k = desc_lo_sw128(sb + C::OFF_Q, 16) + (warp == 16 ? 0 : TBU);
+            const uint32_t b_m = desc_lo_sw128(sb + C::OFF_Q, TB) + (warp == 16 ? TBU : 0);
+            const uint32_t t_sc = tmem + (warp == 16 ? C::TM_S : C::TM_DP), t_kv = tmem + (warp == 16 ? C::TM_K : C::TM_V),
+                           t_acc = tmem + (warp == 16 ? C::TM_DV : C::TM_DK);
+            const uint32_t bar_sc = BAR(warp == 16 ? B_SFULL : B_DPFULL), bar_in = BAR(warp == 16 ? B_PFULL : B_DSFULL);
             // The products of one step, by half h of its query columns (64 each, one compute
             // warpgroup's); q = offset of the step's Q / dO stage in descriptor units.
             auto issue_score = [&](uint32_t q, int h) { // S^T = K Q^T / dP^T = V dO^T, K / V in tensor memory
@@ -331,7 +334,7 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             auto issue_acc = [&](uint32_t q, int h, bool acc) { // dV += P^T dO / dK += dS^T Q, 64 query rows
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    if (lead) mma_ts_lo(t_acc, t_sc + h * 64 + k * 8, b_m + q + (h * 4 + k) * 128, IDESC_KV,
+                    if (lead) mma_ts_lo(t_acc, t_sc + h * 64 + (k >> 1) * 32 + (k & 1) * 8, b_m + q + (h * 4 + k) * 128, IDESC_KV,
                               acc || k > 0);
             };
             bool ok = true;
@@ -340,7 +343,7 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             for (; bwd_take(wq, BAR(B_WQ), w, abort_flag, item); ++w) {
                 const int n_cur = item.steps;
                 const int ks = w & 1;
-                if (warp == 11) {
+                if (warp == 19) {
                     const uint32_t kvo = ks * TBU;
                     for (int i = 0; ok && i < n_cur; ++i, ++it) {
                         ok = mbar_wait(BAR(B_DSFULL), it & 1, abort_flag) &&
@@ -366,8 +369,7 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                     break;
                 tc_fence_after();
                 issue_score((it % 3) * 2 * TBU, 0);
-                if (warp == 10)
-                    issue_score((it % 3) * 2 * TBU, 1);
+                issue_score((it % 3) * 2 * TBU, 1);
                 for (int i = 0; ok && i < n_cur; ++i, ++it) {
                     const int st = it % 3, nst = (it + 1) % 3;
                     const uint32_t qo = st * 2 * TBU, nqo = nst * 2 * TBU;
@@ -379,10 +381,6 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                         break;
                     tc_fence_after();
                     issue_acc(qo, 0, !first);
-                    // The second warpgroup starts an item one exp phase behind the first, so that
-                    // the exp2 unit serves one while the other does the rest of its step.
-                    if (first && warp == 8)
-                        issue_score(qo, 1);
                     if (!last) {
                         ok = mbar_wait(BAR(B_QFULL + nst), ((it + 1) / 3) & 1, abort_flag);
                         if (!ok)
@@ -405,13 +403,14 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             }
         }
     } else {
-        reg_set<COMPUTE_REGS, 128>();
-        // ------------------------------------------------------------ compute (warps 0-7)
-        const int wg = warp >> 2;
-        const int r = threadIdx.x & 127; // key lane for S/dP/dK/dV, query row for dQ
+        reg_set<COMPUTE_REGS, LAUNCH_REGS>();
+        // ------------------------------------------------------------ compute (warps 0-15)
+        const int wg = warp >> 3;       // half of the query columns
+        const int ch = (warp >> 2) & 1; // 32 of its 64 columns
+        const int r = (warp & 3) * 32 + lane;
         const uint32_t lane_sel = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t tS = tmem + lane_sel + C::TM_S + wg * 64;
-        const uint32_t tDP = tmem + lane_sel + C::TM_DP + wg * 64;
+        const uint32_t tS = tmem + lane_sel + C::TM_S + wg * 64 + ch * 32;
+        const uint32_t tDP = tmem + lane_sel + C::TM_DP + wg * 64 + ch * 32;
         // row of the dS^T tile that this lane addresses in stmatrix_x4 (see there): its row of the
         // first 16, chunk added per store
         const uint32_t dsrow = sb + C::OFF_DS + wg * TB + ((warp & 3) * 32 + (lane & 15)) * 128;
@@ -427,7 +426,7 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             }
             {
                 // New work item: a bf16 copy of K (group 0) / V (group 1) goes to tensor memory,
-                // one row per thread.  Every S^T / dP^T product of the previous item is complete
+                // half a row per thread.  Every S^T / dP^T product of the previous item is complete
                 // (their results were consumed in its last step), so the old copy is not in use.
                 const int ks = w & 1;
                 // (The other group's last S^T / dP^T must be complete as well.)
@@ -437,16 +436,16 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                 if (!ok)
                     break;
                 const uint8_t *src = sp + C::OFF_KV + (wg == 0 ? ks : 2) * TB + r * 128;
-                uint32_t kvw[32];
+                uint32_t kvw[16];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const uint4 v = *reinterpret_cast<const uint4 *>(src + ((c ^ (r & 7)) << 4));
+                for (int c = 0; c < 4; ++c) {
+                    const uint4 v = *reinterpret_cast<const uint4 *>(src + (((4 * ch + c) ^ (r & 7)) << 4));
                     kvw[4 * c] = v.x;
                     kvw[4 * c + 1] = v.y;
                     kvw[4 * c + 2] = v.z;
                     kvw[4 * c + 3] = v.w;
                 }
-                tmem_st32(tmem + lane_sel + (wg == 0 ? C::TM_K : C::TM_V), kvw);
+                tmem_st16(tmem + lane_sel + (wg == 0 ? C::TM_K : C::TM_V) + ch * 16, kvw);
                 tmem_wait_st();
                 tc_fence_before();
                 warp_arrive(BAR(B_KVTFULL));
@@ -455,27 +454,27 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             const bool full = (item.mask >> (7 + __ffs(em))) & 1u;
             for (int hh = 0; hh < item.nh; ++hh, ++it, st = st == NSQ - 1 ? 0 : st + 1) {
             const float *rowbuf = reinterpret_cast<const float *>(sp + C::OFF_ROW + st * C::ROW_BYTES);
-            const float4 *nl4 = reinterpret_cast<const float4 *>(rowbuf + wg * 64) + (lane & 3);
-            const float4 *nd4 = reinterpret_cast<const float4 *>(rowbuf + 128 + wg * 64) + (lane & 3);
-            const int4 *mq4 = reinterpret_cast<const int4 *>(rowbuf + 256 + wg * 64) + (lane & 3);
-            // ---- P^T.  A thread holds 4 key lanes x 16 query columns (tmem_ld_16x256b_x8): for each
+            const float4 *nl4 = reinterpret_cast<const float4 *>(rowbuf + wg * 64 + ch * 32) + (lane & 3);
+            const float4 *nd4 = reinterpret_cast<const float4 *>(rowbuf + 128 + wg * 64 + ch * 32) + (lane & 3);
+            const int4 *mq4 = reinterpret_cast<const int4 *>(rowbuf + 256 + wg * 64 + ch * 32) + (lane & 3);
+            // ---- P^T.  A thread holds 4 key lanes x 8 query columns (tmem_ld_16x256b_x4): for each
             // group i of 8 columns the columns 8i + 2 (lane % 4) and the next one.
             // The row values came with the step's Q tile, which the products read: complete.
             ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_SFULL + wg), it & 1, abort_flag));
             if (!ok)
                 break;
             tc_fence_after();
-            float4 rv[4]; // row values of the thread's columns
+            float4 rv[2]; // row values of the thread's columns
 #pragma unroll
-            for (int m = 0; m < 4; ++m)
+            for (int m = 0; m < 2; ++m)
                 rv[m] = nl4[4 * m];
-            uint32_t sr[2][32];
-            tmem_ld_16x256b_x8(tS, sr[0]);
-            tmem_ld_16x256b_x8(tS + (16u << 16), sr[1]);
+            uint32_t sr[2][16];
+            tmem_ld_16x256b_x4(tS, sr[0]);
+            tmem_ld_16x256b_x4(tS + (16u << 16), sr[1]);
             tmem_wait_ld();
-            float p[2][32];
+            float p[2][16];
 #pragma unroll
-            for (int m = 0; m < 4; ++m)
+            for (int m = 0; m < 2; ++m)
 #pragma unroll
                 for (int hf = 0; hf < 2; ++hf)
 #pragma unroll
@@ -489,7 +488,7 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                     }
             if (!full) {
 #pragma unroll
-                for (int m = 0; m < 4; ++m) {
+                for (int m = 0; m < 2; ++m) {
                     const int4 mq = mq4[4 * m];
 #pragma unroll
                     for (int hf = 0; hf < 2; ++hf)
@@ -501,34 +500,34 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                 }
             }
 #pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-                uint32_t pk[16];
+            for (int m = 0; m < 2; ++m)
+                rv[m] = nd4[4 * m]; // used by dS^T, requested ahead of the hand-over
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
+            for (int hf = 0; hf < 2; ++hf) {
+                uint32_t pk[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
                     pk[i] = pack_bf16x2(p[hf][2 * i], p[hf][2 * i + 1]);
-                // packed P^T over the first half of this group's S^T columns
-                tmem_st_16x128b_x8(tS + ((16u * hf) << 16), pk);
+                // packed P^T over the first half of this warp's S^T columns
+                tmem_st_16x128b_x4(tS + ((16u * hf) << 16), pk);
             }
             tmem_wait_st();
             tc_fence_before();
             warp_arrive(BAR(B_PFULL + wg));
             // ---- dS^T
-#pragma unroll
-            for (int m = 0; m < 4; ++m)
-                rv[m] = nd4[4 * m];
             // (and dQ of the previous step has run, so that the dS^T panel is free)
             ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_DPFULL + wg), it & 1, abort_flag) &&
                                              (it == 0 || mbar_wait(BAR(B_DQFULL), (it - 1) & 1, abort_flag)));
             if (!ok)
                 break;
             tc_fence_after();
-            tmem_ld_16x256b_x8(tDP, sr[0]);
-            tmem_ld_16x256b_x8(tDP + (16u << 16), sr[1]);
+            tmem_ld_16x256b_x4(tDP, sr[0]);
+            tmem_ld_16x256b_x4(tDP + (16u << 16), sr[1]);
             tmem_wait_ld();
             tc_fence_before();
-            uint32_t ds[2][16];
+            uint32_t ds[2][8];
 #pragma unroll
-            for (int m = 0; m < 4; ++m)
+            for (int m = 0; m < 2; ++m)
 #pragma unroll
                 for (int hf = 0; hf < 2; ++hf)
 #pragma unroll
@@ -543,12 +542,12 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             // the same dS^T goes over this group's dP^T columns (operand of dK) and to shared memory
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf)
-                tmem_st_16x128b_x8(tDP + ((16u * hf) << 16), ds[hf]);
+                tmem_st_16x128b_x4(tDP + ((16u * hf) << 16), ds[hf]);
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf)
 #pragma unroll
-                for (int i = 0; i < 8; i += 2) // 16-byte chunks i, i + 1 of 16 rows
-                    stmatrix_x4(dsrow + hf * 2048 + (((i + (lane >> 4)) ^ (lane & 7)) << 4), ds[hf][2 * i],
+                for (int i = 0; i < 4; i += 2) // 16-byte chunks 4 ch + i, + 1 of 16 rows
+                    stmatrix_x4(dsrow + hf * 2048 + (((4 * ch + i + (lane >> 4)) ^ (lane & 7)) << 4), ds[hf][2 * i],
                                 ds[hf][2 * i + 1], ds[hf][2 * i + 2], ds[hf][2 * i + 3]);
             tmem_wait_st();
             fence_proxy_async_smem();
@@ -570,7 +569,7 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         }
         __syncthreads();
     }
-    if (warp == 8) {
+    if (warp == 16) {
         __syncwarp();
         tc_fence_after();
         tmem_dealloc(tmem, 512);
@@ -725,7 +724,7 @@ static int launch_bwd_t(const Plan &p, const BwdArgs &a, EncodeTiledFn enc, int 
         if (ev0)
             cudaEventRecord(ev0, s);
         if (D == 64)
-            bwd64_kernel<<<n_sm, 512, Bwd64Cfg::SMEM_BYTES, s>>>(tmQ, tmdO, tmK, tmV, tmDQ, tmDK, tmDV, P);
+            bwd64_kernel<<<n_sm, THREADS, Bwd64Cfg::SMEM_BYTES, s>>>(tmQ, tmdO, tmK, tmV, tmDQ, tmDK, tmDV, P);
         else if (launch_bwd128_main(tmQ, tmdO, tmK, tmV, tmDQ, tmDK, tmDV, P, n_sm, s) < 0)
             return PEAGLE_ERR_CUDA;
         if (ev1)
