@@ -99,7 +99,7 @@ struct FwdCfg {
     static constexpr int OFF_ZERO = OFF_OST + (O_STAGED ? 2 * TILE_BYTES : 0);
     static constexpr int OFF_META = OFF_ZERO + PANEL_BYTES;
     static constexpr int OFF_BAR = OFF_META + NS * BN * 4;
-    static constexpr int N_BAR = 1 + 4 * NS + 8 + 9;
+    static constexpr int N_BAR = 1 + 4 * NS + 8 + 9 + 8;
     static constexpr int OFF_MISC = OFF_BAR + N_BAR * 8; // tmem slot, abort flag, item queue
     static constexpr int SMEM_BYTES = OFF_MISC + 32 + 1024; // + slack for 1024-byte alignment
     static constexpr int TM_S = 0;      // S_A at 0, S_B at 128
@@ -120,6 +120,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
 {
     using C = FwdCfg<D>;
     constexpr int NS = C::NS;
+    constexpr bool TURNS = D == 128;
+    constexpr int EB = 8, POLY = 2; // see the exponentials
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t sb = (raw + 1023u) & ~1023u;
@@ -131,7 +133,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     constexpr int B_QFULL = 0, B_KFULL = 1, B_KEMPTY = 1 + NS, B_VFULL = 1 + 2 * NS,
                   B_VEMPTY = 1 + 3 * NS, B_SFULL = 1 + 4 * NS, B_PFULL = B_SFULL + 2,
                   B_PVDONE = B_SFULL + 4, B_SREAD = B_SFULL + 6, B_WQFULL = B_SFULL + 8,
-                  B_WQFREE = B_WQFULL + 4, B_QEMPTY = B_WQFREE + 4;
+                  B_WQFREE = B_WQFULL + 4, B_QEMPTY = B_WQFREE + 4, B_TURN = B_QEMPTY + 1;
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(sp + C::OFF_MISC);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(sp + C::OFF_MISC + 4);
     volatile int *wq = reinterpret_cast<volatile int *>(sp + C::OFF_MISC + 8); // 4 slots
@@ -184,6 +186,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             mbar_init(BAR(B_PFULL + x), 4);   // one arrival per softmax warp of the tile
             mbar_init(BAR(B_PVDONE + x), 1);
             mbar_init(BAR(B_SREAD + x), 4);
+            for (int i = 0; i < 4; ++i)
+                mbar_init(BAR(B_TURN + 4 * x + i), 1);
         }
         for (int i = 0; i < 4; ++i) {
             mbar_init(BAR(B_WQFULL + i), 1);
@@ -764,27 +768,63 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     tmem_wait_st();
                 }
             }
-            const float neg_m = (m == -CUDART_INF_F) ? 0.f : -m;
-            float sum = 0.f;
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                uint32_t pk[32];
-#pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    const int c0 = 2 * i + 64 * c; // columns c0, c0+1 of this row
-                    const float p0 = fast_exp2(fmaf(__uint_as_float(xr[c0 >> 5][c0 & 31]),
-                                                    P.scale_log2, neg_m));
-                    // every fourth exponential goes to the FMA pipe: the two softmax groups
-                    // together would otherwise keep the exp2 unit busy for 2,048 clocks a step
-                    // (a larger share makes instruction issue the limit instead)
-                    const float a1 = fmaf(__uint_as_float(xr[(c0 + 1) >> 5][(c0 + 1) & 31]),
-                                          P.scale_log2, neg_m);
-                    const float p1 = (i & 1) ? exp2_fma(a1) : fast_exp2(a1);
-                    sum += p0 + p1;
-                    pk[i] = pack_bf16x2(p0, p1);
-                }
-                tmem_st32(tP + c * 32, pk);
+            // head_dim 128: the two tiles' warps of a scheduler take turns with the exponentials.  Left alone
+            // the tiles fall into step, and then both do exponentials at once and both wait at once for
+            // P V and the next S (which share tensor memory here), 2,000 of a period of 5,100 clocks.  At
+            // head_dim 64, where S is ready early, turns measured slower.
+            if (TURNS && P.two && (x == 1 || tt > 0)) {
+                ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_TURN + 4 * x + (warp & 3)), (x == 1 ? tt : tt - 1) & 1, abort_flag));
+                if (!ok)
+                    break;
             }
+            const float neg_m = (m == -CUDART_INF_F) ? 0.f : -m;
+            // Batches of EB pairs of columns, one step apart: the arguments of a batch, the exponentials of
+            // the one before, and sum and packing of the one before that are independent of one another,
+            // so that a warp does not wait for its own results.
+            const F2 scale2 = f2(P.scale_log2, P.scale_log2), nm2 = f2(neg_m, neg_m);
+            F2 sum2[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
+            F2 arg[2][EB], ex[2][EB];
+            uint32_t pk[32];
+#pragma unroll
+            for (int b = 0; b < 64 / EB + 2; ++b) {
+                if (b < 64 / EB) {
+#pragma unroll
+                    for (int k = 0; k < EB; ++k) {
+                        const int c0 = 2 * (EB * b + k); // columns c0, c0 + 1
+                        arg[b & 1][k] = fma_f2(f2(__uint_as_float(xr[c0 >> 5][c0 & 31]), __uint_as_float(xr[c0 >> 5][(c0 & 31) + 1])),
+                                               scale2, nm2);
+                    }
+                }
+                if (b >= 1 && b <= 64 / EB) {
+#pragma unroll
+                    for (int k = 0; k < EB; ++k) {
+                        const F2 x2 = arg[(b - 1) & 1][k];
+                        // a quarter of the exponentials goes to the FMA pipe (an eighth and three
+                        // eighths measured 3 and 5 per cent slower)
+                        if ((EB * (b - 1) + k) % 8 < POLY) {
+                            ex[(b - 1) & 1][k] = exp2_fma2(x2);
+                        } else {
+                            const float2 v = unf2(x2);
+                            ex[(b - 1) & 1][k] = f2(fast_exp2(v.x), fast_exp2(v.y));
+                        }
+                    }
+                }
+                if (b >= 2) {
+#pragma unroll
+                    for (int k = 0; k < EB; ++k) {
+                        const F2 e2 = ex[b & 1][k];
+                        const float2 v = unf2(e2);
+                        sum2[k & 1] = add_f2(sum2[k & 1], e2);
+                        pk[(EB * (b - 2) + k) % 32] = pack_bf16x2(v.x, v.y);
+                    }
+                    if ((EB * (b - 1)) % 32 == 0)
+                        tmem_st32(tP + (EB * (b - 1) / 32 - 1) * 32, pk);
+                }
+            }
+            const float2 sv = unf2(add_f2(sum2[0], sum2[1]));
+            const float sum = sv.x + sv.y;
+            if (TURNS && P.two && lane == 0)
+                mbar_arrive(BAR(B_TURN + 4 * (x ^ 1) + (warp & 3))); // the other tile's turn
             l += sum;
             tmem_wait_st();
             tc_fence_before();

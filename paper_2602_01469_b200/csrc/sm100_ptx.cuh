@@ -421,6 +421,13 @@ __device__ __forceinline__ F2 mul_f2(F2 a, F2 b)
     return r;
 }
 
+__device__ __forceinline__ F2 add_f2(F2 a, F2 b)
+{
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+
 // ------------------------------------------------------------------ cheap MMA issue
 // The single issuing thread should spend a couple of instructions per MMA, not a descriptor
 // build.  With the stride field fixed at 1024 bytes the upper word of a 128-byte-swizzle
@@ -601,6 +608,21 @@ __device__ __forceinline__ float exp2_fma(float x)
     p = fmaf(p, f, 0.69327623f);
     p = fmaf(p, f, 0.99992895f);
     return __int_as_float(__float_as_int(p) + (__float_as_int(xr) << 23));
+}
+
+// The same on a pair.
+__device__ __forceinline__ F2 exp2_fma2(F2 x)
+{
+    const float2 c = unf2(x);
+    x = f2(fmaxf(c.x, -126.f), fmaxf(c.y, -126.f));
+    const F2 xr = add_f2(x, f2(12582912.f, 12582912.f));
+    const F2 f = fma_f2(add_f2(xr, f2(-12582912.f, -12582912.f)), f2(-1.f, -1.f), x);
+    F2 p = fma_f2(f, f2(0.05508868f, 0.05508868f), f2(0.24260405f, 0.24260405f));
+    p = fma_f2(p, f, f2(0.69327623f, 0.69327623f));
+    p = fma_f2(p, f, f2(0.99992895f, 0.99992895f));
+    const float2 pv = unf2(p), n = unf2(xr);
+    return f2(__int_as_float(__float_as_int(pv.x) + (__float_as_int(n.x) << 23)),
+              __int_as_float(__float_as_int(pv.y) + (__float_as_int(n.y) << 23)));
 }
 
 // ------------------------------------------------------------------ CTA pairs (clusters of two)
