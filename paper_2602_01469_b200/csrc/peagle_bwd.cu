@@ -150,6 +150,8 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    pdl_trigger();
+    pdl_wait();
 
     if (warp >= 20) {
         // ------------------------------------------------------------ drain (warps 20-23)
@@ -586,6 +588,8 @@ __global__ void bwd_prepare(const __nv_bfloat16 *__restrict__ O, const __nv_bflo
                             int32_t *__restrict__ mqp, float *__restrict__ dq_acc, int q_begin,
                             int q_len, int q_pad, int Hq, int T)
 {
+    pdl_trigger();
+    pdl_wait();
     constexpr int TPR = D / 8; // threads per (row, head)
     const size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t n = (size_t)q_pad * Hq * TPR;
@@ -632,6 +636,8 @@ __global__ void bwd_prepare(const __nv_bfloat16 *__restrict__ O, const __nv_bflo
 __global__ void bwd_finish_dq(const float *__restrict__ dq_acc, __nv_bfloat16 *__restrict__ dQ,
                               size_t n8)
 {
+    pdl_trigger();
+    pdl_wait();
     const size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (gid >= n8)
         return;
@@ -649,6 +655,8 @@ __global__ void cast_grads_kernel(const float *__restrict__ a, const float *__re
                                   __nv_bfloat16 *__restrict__ oa, __nv_bfloat16 *__restrict__ ob,
                                   size_t n8)
 {
+    pdl_trigger();
+    pdl_wait();
     const size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (gid >= 2 * n8)
         return;
@@ -688,7 +696,8 @@ static int launch_bwd_t(const Plan &p, const BwdArgs &a, EncodeTiledFn enc, int 
     // Per-row values and a cleared dQ staging: the forward of the partition leaves both when it runs in
     // the driver, where dO is known.
     if (!a.rows_ready) {
-        bwd_prepare<D><<<(unsigned)((n_prep_pad + 255) / 256), 256, 0, s>>>(
+        launch_dependent(
+            bwd_prepare<D>, (unsigned)((n_prep_pad + 255) / 256), 256, 0, s,
             static_cast<const __nv_bfloat16 *>(a.O), static_cast<const __nv_bfloat16 *>(a.dO), a.LSE,
             p.meta, a.nl2, a.nd, a.mqp, a.dq_acc, p.q_begin, q_len, q_pad, a.Hq, p.T);
         launches = 1;
@@ -724,7 +733,7 @@ static int launch_bwd_t(const Plan &p, const BwdArgs &a, EncodeTiledFn enc, int 
         if (ev0)
             cudaEventRecord(ev0, s);
         if (D == 64)
-            bwd64_kernel<<<n_sm, THREADS, Bwd64Cfg::SMEM_BYTES, s>>>(tmQ, tmdO, tmK, tmV, tmDQ, tmDK, tmDV, P);
+            launch_dependent(bwd64_kernel, n_sm, THREADS, Bwd64Cfg::SMEM_BYTES, s, tmQ, tmdO, tmK, tmV, tmDQ, tmDK, tmDV, P);
         else if (launch_bwd128_main(tmQ, tmdO, tmK, tmV, tmDQ, tmDK, tmDV, P, n_sm, s) < 0)
             return PEAGLE_ERR_CUDA;
         if (ev1)
@@ -735,8 +744,8 @@ static int launch_bwd_t(const Plan &p, const BwdArgs &a, EncodeTiledFn enc, int 
         const int n = launch_finish_single(p, a, s);
         return n < 0 ? n : launches + n;
     }
-    bwd_finish_dq<<<(unsigned)((n_prep + 255) / 256), 256, 0, s>>>(
-        a.dq_acc, static_cast<__nv_bfloat16 *>(a.dQ) + (size_t)p.q_begin * a.Hq * D, n_prep);
+    launch_dependent(
+        bwd_finish_dq, (unsigned)((n_prep + 255) / 256), 256, 0, s, a.dq_acc, static_cast<__nv_bfloat16 *>(a.dQ) + (size_t)p.q_begin * a.Hq * D, n_prep);
     return launches + 1;
 }
 
@@ -757,8 +766,8 @@ int launch_cast_one(const float *src, void *dst, size_t n, cudaStream_t s)
         return 0;
     // the kernel takes two arrays of n8 pieces; here both are the one array, and the grid covers it
     // once (threads past n8 in the last block repeat the first pieces with the same values)
-    cast_grads_kernel<<<(unsigned)((n8 + 255) / 256), 256, 0, s>>>(
-        src, src, static_cast<__nv_bfloat16 *>(dst), static_cast<__nv_bfloat16 *>(dst), n8);
+    launch_dependent(
+        cast_grads_kernel, (unsigned)((n8 + 255) / 256), 256, 0, s, src, src, static_cast<__nv_bfloat16 *>(dst), static_cast<__nv_bfloat16 *>(dst), n8);
     return 1;
 }
 
@@ -766,8 +775,8 @@ int launch_cast_grads(const float *dK_acc, const float *dV_acc, void *dK, void *
                       cudaStream_t s)
 {
     const size_t n8 = n / 8;
-    cast_grads_kernel<<<(unsigned)((2 * n8 + 255) / 256), 256, 0, s>>>(
-        dK_acc, dV_acc, static_cast<__nv_bfloat16 *>(dK), static_cast<__nv_bfloat16 *>(dV), n8);
+    launch_dependent(
+        cast_grads_kernel, (unsigned)((2 * n8 + 255) / 256), 256, 0, s, dK_acc, dV_acc, static_cast<__nv_bfloat16 *>(dK), static_cast<__nv_bfloat16 *>(dV), n8);
     return 1;
 }
 

@@ -77,7 +77,9 @@ bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t sb = smem_u32(smem_raw);
     uint8_t *sp = smem_raw;
+    pdl_trigger();
     if (sb & 1023u) { // the swizzled tiles need this alignment; nothing has been set up yet
+        pdl_wait();
         if (threadIdx.x == 0)
             atomicCAS(P.status, 0, PEAGLE_ERR_ALIGN);
         return;
@@ -128,6 +130,7 @@ bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    pdl_wait();
 
     if (warp >= 12) {
         // ------------------------------------------------------------ drain (warps 12-15)
@@ -556,7 +559,7 @@ int launch_bwd128_main(const CUtensorMap &tmQ, const CUtensorMap &tmdO, const CU
     if (cudaFuncSetAttribute(bwd128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              Bwd128Cfg::SMEM_BYTES) != cudaSuccess)
         return PEAGLE_ERR_CUDA;
-    bwd128_kernel<<<n_sm, 512, Bwd128Cfg::SMEM_BYTES, s>>>(tmQ, tmdO, tmK, tmV, tmDQ, tmDK, tmDV, P);
+    launch_dependent(bwd128_kernel, n_sm, 512, Bwd128Cfg::SMEM_BYTES, s, tmQ, tmdO, tmK, tmV, tmDQ, tmDK, tmDV, P);
     return 1;
 }
 

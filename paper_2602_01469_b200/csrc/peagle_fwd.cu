@@ -211,6 +211,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    pdl_trigger();
+    pdl_wait();
 
     // Warps 8-11 hand most of their registers to the eight softmax warps.
     if (warp >= 8)
@@ -1050,7 +1052,7 @@ static int launch_fwd_t(const Plan &p, const FwdArgs &a, EncodeTiledFn enc, int 
     P.n_items = p.n_qt * n_hb;
     if (ev0)
         cudaEventRecord(ev0, s);
-    fwd_kernel<D><<<std::min(P.n_items, n_sm), 384, FwdCfg<D>::SMEM_BYTES, s>>>(tmQ, tmK, tmV, tmO, tmZ, P);
+    launch_dependent(fwd_kernel<D>, std::min(P.n_items, n_sm), 384, FwdCfg<D>::SMEM_BYTES, s, tmQ, tmK, tmV, tmO, tmZ, P);
     if (ev1)
         cudaEventRecord(ev1, s);
     return 1;

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "../../include/peagle.h"
 
 namespace peagle {
@@ -110,6 +112,27 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
 __host__ __device__ inline int row_slot(int r)
 {
     return (r & ~15) | (((r >> 1) & 3) << 2) | ((r >> 3 & 1) << 1) | (r & 1);
+}
+
+// Launches a kernel that begins with pdl_wait / pdl_trigger (sm100_ptx.cuh): its launch and set-up overlap
+// the kernel before it.  A call of a few tokens is a chain of kernels of a few microseconds each, and the
+// gaps between them were a fifth of its time (512 tokens, 4 heads: 56 -> 47 us a step).  Not for the
+// projection products and the rotary prologue, where it measured nothing.
+template <class... Params, class... Args>
+inline cudaError_t launch_dependent(void (*kernel)(Params...), unsigned grid, unsigned threads, size_t smem,
+                                    cudaStream_t s, Args &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
 // K0: mask evaluator, tile classifier, scheduler.  Returns the number of kernels launched.

@@ -38,6 +38,8 @@ __global__ void __launch_bounds__(128) k0_tiles(Plan p, const int32_t *__restric
                                                 const int32_t *__restrict__ depth, int K, int seq_begin,
                                                 int seq_end, RangeList ranges)
 {
+    sm100::pdl_trigger();
+    sm100::pdl_wait();
     const int tile = blockIdx.x;
     const int t = seq_begin + tile * 128 + threadIdx.x;
     if (t < seq_end) {
@@ -262,6 +264,8 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
     __shared__ int4 pairs[PAIR_CACHE];                // (key tile, first token, length, first run | flags)
     __shared__ int2 entry[RAW_SINGLE];                // sorted raw tiles of an entry: first, last
     __shared__ int n_undecided, n_raw, n_entry, flag;
+    sm100::pdl_trigger();
+    sm100::pdl_wait();
     const int qt = blockIdx.x, tid = threadIdx.x;
     const int lane = tid & 31;
     uint8_t *cls = p.cls + (size_t)qt * p.n_kt;
@@ -551,8 +555,8 @@ int launch_plan(const Plan &p, const int32_t *anchor, const int32_t *depth, int 
         return 0;
     const int n_seq = seq_end - seq_begin;
     const int blocks = (n_seq + 127) / 128 > p.n_qt + p.n_kt ? (n_seq + 127) / 128 : p.n_qt + p.n_kt;
-    k0_tiles<<<blocks, 128, 0, s>>>(p, anchor, depth, K, seq_begin, seq_end, ranges);
-    k0_plan<<<p.n_qt, PLAN_THREADS, 0, s>>>(p, seq_begin, seq_end, for_bwd ? 1 : 0);
+    launch_dependent(k0_tiles, blocks, 128, 0, s, p, anchor, depth, K, seq_begin, seq_end, ranges);
+    launch_dependent(k0_plan, p.n_qt, PLAN_THREADS, 0, s, p, seq_begin, seq_end, for_bwd ? 1 : 0);
     return 2;
 }
 

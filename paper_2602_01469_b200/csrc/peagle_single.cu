@@ -216,6 +216,8 @@ __global__ void __launch_bounds__(SINGLE_THREADS, 1) bwd_finish_single(const Sin
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) uint64_t bar, bar_q; // the dQ staging; Q and dO
     __shared__ int abort_flag;
+    pdl_trigger();
+    pdl_wait();
     const int RB = P.rows_per_block;
     const int row_elems = P.Hq * D;
     float *sDQ = reinterpret_cast<float *>(smem);
@@ -351,7 +353,7 @@ int launch_finish_single(const Plan &p, const BwdArgs &a, cudaStream_t s)
     void (*kern)(const SingleParams) = a.D == 64 ? bwd_finish_single<64> : bwd_finish_single<128>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return PEAGLE_ERR_CUDA;
-    kern<<<(unsigned)((P.q_pad + rb - 1) / rb), threads, smem, s>>>(P);
+    launch_dependent(kern, (unsigned)((P.q_pad + rb - 1) / rb), threads, smem, s, P);
     return 1;
 }
 
