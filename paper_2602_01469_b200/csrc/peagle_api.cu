@@ -994,7 +994,7 @@ int peagle_attn_partitioned_host(peagle_ctx *ctx, const peagle_problem_t *prob,
     if (T == 0)
         return PEAGLE_OK;
     // Three streams: rows of Q / dO go in, partitions are computed, rows of O / LSE / dQ come
-    // back, each query range cut into slices of HOST_SLICE rows so that the copies of one slice
+    // back, each query range cut into slices of rows so that the copies of one slice
     // overlap the arithmetic of another (the slices are query partitions like any other: K / V
     // and the dK / dV accumulators are shared, exactly Section 3.2's within-sequence scheme).
     {
@@ -1012,9 +1012,8 @@ int peagle_attn_partitioned_host(peagle_ctx *ctx, const peagle_problem_t *prob,
     // From here on copies into the caller's host buffers may be in flight: every error exit
     // drains the three streams first, so that nothing writes O / LSE / dQ after the return.
     auto drained = [&](int status) {
-        cudaStreamSynchronize(s_in);
-        cudaStreamSynchronize(s_c);
-        cudaStreamSynchronize(s_out);
+        for (cudaStream_t st : ctx->hs)
+            cudaStreamSynchronize(st);
         return status;
     };
 #define CKD(call)                                          \
@@ -1039,33 +1038,64 @@ int peagle_attn_partitioned_host(peagle_ctx *ctx, const peagle_problem_t *prob,
     if (rc != PEAGLE_OK)
         return rc;
     float *dK_acc = static_cast<float *>(ctx->acc_buf.ptr), *dV_acc = dK_acc + n_kv;
+    // The metadata is pageable as a rule, and such a copy holds the host until its stream is idle: it
+    // goes first, on the stream that has nothing else yet.
+    CKD(cudaMemcpyAsync(danchor, prob->anchor, nmeta, cudaMemcpyHostToDevice, s_c));
+    CKD(cudaMemcpyAsync(ddepth, prob->depth, nmeta, cudaMemcpyHostToDevice, s_c));
     CKD(cudaMemcpyAsync(dKin, K, nkv, cudaMemcpyHostToDevice, s_in));
     CKD(cudaMemcpyAsync(dVin, V, nkv, cudaMemcpyHostToDevice, s_in));
-    CKD(cudaMemcpyAsync(danchor, prob->anchor, nmeta, cudaMemcpyHostToDevice, s_in));
-    CKD(cudaMemcpyAsync(ddepth, prob->depth, nmeta, cudaMemcpyHostToDevice, s_in));
     CKD(cudaMemsetAsync(dK_acc, 0, 2 * n_kv * sizeof(float), s_c));
     peagle_problem_t dprob = *prob;
     dprob.anchor = reinterpret_cast<const int32_t *>(danchor);
     dprob.depth = reinterpret_cast<const int32_t *>(ddepth);
-    constexpr int HOST_SLICE = 16 * BM;
+    // A slice is SLICE_BYTES of Q and dO, at most 2,048 rows.  Rows come in and go out in step: slice k - 2
+    // leaves while slice k arrives, each pair after the one before it has ended in both directions, and
+    // slice k - 1 is computed meanwhile.  Left to start when they may, the two directions fall out of step
+    // and each copy takes 10-15 % longer with a pause of 40 us before the next (copies of 268 MB each way
+    // around a kernel of 100 us a slice: 7.15 ms free running, 6.11 in step; by 8 MB and by 32 MB of each
+    // slice 6.18 and 6.54).  2,048 positions, 64 / 8 heads of 64: 8.3 -> 7.5 ms a step (8 MB slices the
+    // same, 32 MB 7.9; 16 MB is worse for short examples, which have few slices).
+    constexpr int64_t SLICE_BYTES = 12 << 20;
+    const int64_t fit = SLICE_BYTES / (int64_t)(2 * row_q * BM);
+    const int slice_rows = (int)(fit < 1 ? 1 : fit > 16 ? 16 : fit) * BM;
+    struct Slice {
+        size_t off, len;
+        cudaEvent_t in, done, out;
+    };
+    std::vector<Slice> sl;
+    auto copy_out = [&](size_t k) -> int {
+        Slice &x = sl[k];
+        CKD(cudaStreamWaitEvent(s_out, x.done, 0));
+        if (k + 1 < sl.size())
+            CKD(cudaStreamWaitEvent(s_out, sl[k + 1].in, 0));
+        CKD(cudaMemcpyAsync(static_cast<uint8_t *>(O) + x.off, dOout + x.off, x.len, cudaMemcpyDeviceToHost, s_out));
+        CKD(cudaMemcpyAsync(static_cast<uint8_t *>(dQ) + x.off, ddQ + x.off, x.len, cudaMemcpyDeviceToHost, s_out));
+        CKD(cudaEventRecord(x.out, s_out));
+        return PEAGLE_OK;
+    };
     for (int i = 0; i < nparts; ++i) {
-        for (int b0 = parts[i].q.begin; b0 < parts[i].q.end; b0 += HOST_SLICE) {
-            const int b1 = b0 + HOST_SLICE < parts[i].q.end ? b0 + HOST_SLICE : parts[i].q.end;
-            const size_t off = (size_t)b0 * row_q, len = (size_t)(b1 - b0) * row_q;
-            peagle_partition_t sl = parts[i];
-            sl.q.begin = b0;
-            sl.q.end = b1;
-            CKD(cudaMemcpyAsync(dQin + off, static_cast<const uint8_t *>(Q) + off, len,
-                               cudaMemcpyHostToDevice, s_in));
-            CKD(cudaMemcpyAsync(ddO + off, static_cast<const uint8_t *>(dO) + off, len,
-                               cudaMemcpyHostToDevice, s_in));
-            cudaEvent_t e_in = event(), e_c = event();
-            if (!e_in || !e_c)
+        for (int b0 = parts[i].q.begin; b0 < parts[i].q.end; b0 += slice_rows) {
+            const int b1 = parts[i].q.end - b0 > slice_rows ? b0 + slice_rows : parts[i].q.end;
+            const size_t k = sl.size();
+            sl.push_back({(size_t)b0 * row_q, (size_t)(b1 - b0) * row_q, event(), event(), event()});
+            const Slice x = sl[k];
+            if (!x.in || !x.done || !x.out)
                 return drained(PEAGLE_ERR_CUDA);
-            CKD(cudaEventRecord(e_in, s_in));
-            CKD(cudaStreamWaitEvent(s_c, e_in, 0));
+            peagle_partition_t part = parts[i];
+            part.q.begin = b0;
+            part.q.end = b1;
+            if (k >= 2)
+                CKD(cudaStreamWaitEvent(s_in, sl[k - 2].done, 0));
+            if (k >= 3)
+                CKD(cudaStreamWaitEvent(s_in, sl[k - 3].out, 0));
+            CKD(cudaMemcpyAsync(dQin + x.off, static_cast<const uint8_t *>(Q) + x.off, x.len,
+                               cudaMemcpyHostToDevice, s_in));
+            CKD(cudaMemcpyAsync(ddO + x.off, static_cast<const uint8_t *>(dO) + x.off, x.len,
+                               cudaMemcpyHostToDevice, s_in));
+            CKD(cudaEventRecord(x.in, s_in));
             Call c;
-            rc = plan_call(ctx, &dprob, &sl, true, s_c, c);
+            rc = plan_call(ctx, &dprob, &part, true, s_c, c); // needs the metadata only
+            CKD(cudaStreamWaitEvent(s_c, x.in, 0));
             BwdArgs hand;
             if (rc == PEAGLE_OK && c.plan.n_qt > 0)
                 rc = bwd_scratch(ctx, &dprob, c, s_c, hand);
@@ -1077,14 +1107,21 @@ int peagle_attn_partitioned_host(peagle_ctx *ctx, const peagle_problem_t *prob,
                              reinterpret_cast<float *>(dLSE), ddQ, dK_acc, dV_acc, s_c, true);
             if (rc != PEAGLE_OK)
                 return drained(rc);
-            CKD(cudaEventRecord(e_c, s_c));
-            CKD(cudaStreamWaitEvent(s_out, e_c, 0));
-            CKD(cudaMemcpyAsync(static_cast<uint8_t *>(O) + off, dOout + off, len, cudaMemcpyDeviceToHost, s_out));
-            CKD(cudaMemcpyAsync(static_cast<uint8_t *>(dQ) + off, ddQ + off, len, cudaMemcpyDeviceToHost, s_out));
-            CKD(cudaMemcpy2DAsync(LSE + b0, T * 4, reinterpret_cast<float *>(dLSE) + b0, T * 4,
-                                 (size_t)(b1 - b0) * 4, (size_t)prob->n_q_heads,
-                                 cudaMemcpyDeviceToHost, s_out));
+            CKD(cudaEventRecord(x.done, s_c));
+            if (k >= 2 && (rc = copy_out(k - 2)) != PEAGLE_OK)
+                return rc;
         }
+    }
+    for (size_t k = sl.size() < 2 ? 0 : sl.size() - 2; k < sl.size(); ++k)
+        if ((rc = copy_out(k)) != PEAGLE_OK)
+            return rc;
+    for (int i = 0; i < nparts; ++i) {
+        const size_t p0 = (size_t)parts[i].q.begin, np = (size_t)(parts[i].q.end - parts[i].q.begin);
+        if (np == T)
+            CKD(cudaMemcpyAsync(LSE, dLSE, nlse, cudaMemcpyDeviceToHost, s_out));
+        else if (np > 0)
+            CKD(cudaMemcpy2DAsync(LSE + p0, T * 4, reinterpret_cast<float *>(dLSE) + p0, T * 4, np * 4,
+                                  (size_t)prob->n_q_heads, cudaMemcpyDeviceToHost, s_out));
     }
     ctx->launches += launch_cast_grads(dK_acc, dV_acc, ddK, ddV, n_kv, s_c);
     CKD(cudaGetLastError());
@@ -1095,9 +1132,8 @@ int peagle_attn_partitioned_host(peagle_ctx *ctx, const peagle_problem_t *prob,
     CKD(cudaStreamWaitEvent(s_out, e_done, 0));
     CKD(cudaMemcpyAsync(dK, ddK, nkv, cudaMemcpyDeviceToHost, s_out));
     CKD(cudaMemcpyAsync(dV, ddV, nkv, cudaMemcpyDeviceToHost, s_out));
-    CKD(cudaStreamSynchronize(s_in));
-    CKD(cudaStreamSynchronize(s_c));
-    CKD(cudaStreamSynchronize(s_out));
+    for (cudaStream_t st : ctx->hs)
+        CKD(cudaStreamSynchronize(st));
     return PEAGLE_OK;
 #undef CKD
 }
