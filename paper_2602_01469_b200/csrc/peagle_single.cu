@@ -38,8 +38,11 @@ struct SingleParams {
     float scale, scale_log2;
 };
 
-// A row of D bf16 is spread over LANES = D / 8 consecutive lanes of a warp, a unit: lane `sub` holds the
-// elements 8 sub .. 8 sub + 7 (one 16-byte load), as fp32 in neighbouring pairs.
+// A row of D elements is spread over LANES = D / 8 consecutive lanes of a warp, a unit: lane `sub` holds the
+// elements 4 sub .. 4 sub + 3 of each half of the row, as fp32 in neighbouring pairs.  (With 8 sub ..
+// 8 sub + 7, one load of bf16, the fp32 rows were read, written and added to with 32 bytes between the
+// lanes' 16: two-way bank conflicts in shared memory and half-used sectors in the adds to dK and dV.
+// 2,048 positions, 32 heads of 128: 240 -> 219 us; 4,096, 64 heads of 64: 435 -> 421 us.)
 struct Chunk {
     F2 v[4];
 };
@@ -52,9 +55,11 @@ __device__ __forceinline__ Chunk unpack_chunk(const uint4 t)
         c.v[i] = f2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xffff0000u));
     return c;
 }
+template <int D>
 __device__ __forceinline__ Chunk load_chunk(const __nv_bfloat16 *row, int sub)
 {
-    return unpack_chunk(reinterpret_cast<const uint4 *>(row)[sub]);
+    const uint2 a = reinterpret_cast<const uint2 *>(row)[sub], b = reinterpret_cast<const uint2 *>(row + D / 2)[sub];
+    return unpack_chunk(make_uint4(a.x, a.y, b.x, b.y));
 }
 __device__ __forceinline__ float dot_chunk(const Chunk &a, const Chunk &b)
 {
@@ -80,26 +85,25 @@ __device__ __forceinline__ void zero_chunk(Chunk &c)
         c.v[i] = f2(0.f, 0.f);
 }
 // adds this lane's piece of a row (dst = the row's first element) scaled by f
+template <int D>
 __device__ __forceinline__ void red_chunk(float *dst, int sub, const Chunk &x, float f)
 {
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
         const float2 a = unf2(x.v[2 * j]), b = unf2(x.v[2 * j + 1]);
-        asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + 8 * sub + 4 * j), "f"(a.x * f),
+        asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + 4 * sub + D / 2 * j), "f"(a.x * f),
                      "f"(a.y * f), "f"(b.x * f), "f"(b.y * f)
                      : "memory");
     }
 }
 
-// 8 dQ values of row r, head h from element e on, rounded to bf16.
-__device__ __forceinline__ void store_dq(const SingleParams &P, int r, int h, int D, int e, const float4 a, const float4 b)
+// This lane's dQ values of row r, head h, rounded to bf16.
+template <int D>
+__device__ __forceinline__ void store_dq(const SingleParams &P, int r, int h, int sub, const float4 a, const float4 b)
 {
-    uint4 v;
-    v.x = pack_bf16x2(a.x, a.y);
-    v.y = pack_bf16x2(a.z, a.w);
-    v.z = pack_bf16x2(b.x, b.y);
-    v.w = pack_bf16x2(b.z, b.w);
-    *reinterpret_cast<uint4 *>(P.dQ + ((size_t)(P.q_begin + r) * P.Hq + h) * D + e) = v;
+    __nv_bfloat16 *row = P.dQ + ((size_t)(P.q_begin + r) * P.Hq + h) * D;
+    reinterpret_cast<uint2 *>(row)[sub] = make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
+    reinterpret_cast<uint2 *>(row + D / 2)[sub] = make_uint2(pack_bf16x2(b.x, b.y), pack_bf16x2(b.z, b.w));
 }
 
 constexpr int KEYS = 2; // keys per pass: their dK / dV sums are kept in registers across the heads
@@ -122,8 +126,13 @@ __device__ __forceinline__ void next_keys(const SingleParams &P, unsigned &keys,
             out.tok[i] = __shfl_sync(um, at < D / 8 ? t0 : t1, ub + at % (D / 8));
         keys &= keys - 1;
         const size_t kr = ((size_t)max(out.tok[i], 0) * P.Hkv + g) * D;
-        out.k[i] = __ldg(reinterpret_cast<const uint4 *>(P.K + kr) + sub);
-        out.v[i] = __ldg(reinterpret_cast<const uint4 *>(P.V + kr) + sub);
+        auto row_of = [&](const __nv_bfloat16 *row) {
+            const uint2 a = __ldg(reinterpret_cast<const uint2 *>(row) + sub);
+            const uint2 b = __ldg(reinterpret_cast<const uint2 *>(row + D / 2) + sub);
+            return make_uint4(a.x, a.y, b.x, b.y);
+        };
+        out.k[i] = row_of(P.K + kr);
+        out.v[i] = row_of(P.V + kr);
     }
 }
 
@@ -146,8 +155,8 @@ __device__ __forceinline__ void single_pass(const SingleParams &P, const KeyRows
     const bool mine = tok[0] >= 0 && (!second || tok[1] >= 0);
     for (int hh = 0; hh < G; ++hh) {
         const int h = g * G + hh;
-        const Chunk q = load_chunk(sq + (size_t)h * D, sub);
-        const Chunk dO = load_chunk(sdo + (size_t)h * D, sub);
+        const Chunk q = load_chunk<D>(sq + (size_t)h * D, sub);
+        const Chunk dO = load_chunk<D>(sdo + (size_t)h * D, sub);
         const float nl2 = snl2[h], nd = snd[h];
         // The four sums <q, k0>, <q, k1>, <dO, v0>, <dO, v1> over the unit's lanes: halve what a lane
         // carries with every exchange (even lanes keep the scores, odd lanes dp; then one key each), so
@@ -172,8 +181,8 @@ __device__ __forceinline__ void single_pass(const SingleParams &P, const KeyRows
         axpy_chunk(dk[1], q, ds1);
         axpy_chunk(dv[0], dO, p0);
         axpy_chunk(dv[1], dO, p1);
-        float4 *acc = reinterpret_cast<float4 *>(sdq + (size_t)h * D + 8 * sub);
-        const float4 x = acc[0], y = acc[1];
+        float4 *acc = reinterpret_cast<float4 *>(sdq + (size_t)h * D) + sub;
+        const float4 x = acc[0], y = acc[D / 8];
         Chunk dq;
         dq.v[0] = f2(x.x, x.y);
         dq.v[1] = f2(x.z, x.w);
@@ -184,18 +193,18 @@ __device__ __forceinline__ void single_pass(const SingleParams &P, const KeyRows
         const float2 d0 = unf2(dq.v[0]), d1 = unf2(dq.v[1]), d2 = unf2(dq.v[2]), d3 = unf2(dq.v[3]);
         const float4 lo = make_float4(d0.x, d0.y, d1.x, d1.y), hi = make_float4(d2.x, d2.y, d3.x, d3.y);
         if (LAST) {
-            store_dq(P, r, h, D, 8 * sub, lo, hi);
+            store_dq<D>(P, r, h, sub, lo, hi);
         } else {
             acc[0] = lo;
-            acc[1] = hi;
+            acc[D / 8] = hi;
         }
     }
 #pragma unroll
     for (int i = 0; i < KEYS; ++i)
         if (tok[i] >= 0) {
             const size_t kr = ((size_t)tok[i] * P.Hkv + g) * D;
-            red_chunk(P.dK_acc + kr, sub, dk[i], P.scale);
-            red_chunk(P.dV_acc + kr, sub, dv[i], 1.f);
+            red_chunk<D>(P.dK_acc + kr, sub, dk[i], P.scale);
+            red_chunk<D>(P.dV_acc + kr, sub, dv[i], 1.f);
         }
 }
 
@@ -294,8 +303,8 @@ __global__ void __launch_bounds__(SINGLE_THREADS, 1) bwd_finish_single(const Sin
     if (!any) { // nothing to add: round what the tile kernel left
         for (int hh = 0; hh < G; ++hh) {
             const int h = g * G + hh;
-            const float4 *acc = reinterpret_cast<const float4 *>(sdq + (size_t)h * D + 8 * sub);
-            store_dq(P, r, h, D, 8 * sub, acc[0], acc[1]);
+            const float4 *acc = reinterpret_cast<const float4 *>(sdq + (size_t)h * D) + sub;
+            store_dq<D>(P, r, h, sub, acc[0], acc[D / 8]);
         }
         return;
     }
