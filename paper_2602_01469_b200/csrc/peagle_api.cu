@@ -216,7 +216,7 @@ int validate_partition(const peagle_problem_t *prob, const peagle_partition_t *p
 
 // Runs K0 for one call.  On return c.plan points into ctx->plan_buf.
 int plan_call(peagle_ctx *ctx, const peagle_problem_t *prob, const peagle_partition_t *part,
-              bool for_bwd, cudaStream_t s, Call &c)
+              bool for_bwd, cudaStream_t s, Call &c, float *zero = nullptr, size_t zero_n = 0)
 {
     int rc = validate_partition(prob, part, c);
     if (rc != PEAGLE_OK)
@@ -232,7 +232,7 @@ int plan_call(peagle_ctx *ctx, const peagle_problem_t *prob, const peagle_partit
     if (c.plan.n_qt == 0)
         return PEAGLE_OK;
     ctx->launches += launch_plan(c.plan, prob->anchor, prob->depth, prob->K, c.seq_begin, c.seq_end,
-                                 c.ranges, for_bwd, s);
+                                 c.ranges, for_bwd, s, zero, zero_n);
     CK(cudaGetLastError());
     return PEAGLE_OK;
 }
@@ -685,17 +685,29 @@ int peagle_attn_bwd(peagle_ctx *ctx, const peagle_problem_t *prob, const peagle_
     return run_bwd(ctx, prob, c, Q, K, V, O, dO, LSE, dQ, dK_acc, dV_acc, s);
 }
 
-// Runs forward + backward of the given partitions in order, adding into fp32 dK / dV accumulators.
+// Runs forward + backward of the given partitions in order, adding into fp32 dK / dV accumulators.  With
+// `clear` both are set to zero first (dV_acc follows dK_acc).
 static int run_partitions(peagle_ctx *ctx, const peagle_problem_t *prob,
                           const peagle_partition_t *parts, int32_t nparts, const void *Q,
                           const void *K, const void *V, const void *dO, void *O, float *LSE,
-                          void *dQ, float *dK_acc, float *dV_acc, cudaStream_t s)
+                          void *dQ, float *dK_acc, float *dV_acc, cudaStream_t s, bool clear)
 {
+    // Up to 32 MB the plan of the first partition that has rows clears the sums on the side (12.8 MB: 7 us
+    // of a step of 220, 0.3 MB: 2 of 48); above, a fill at memory speed takes longer than the plan, and
+    // the two together as long as one after the other (67 MB: 41 against 20 + 23 us).
+    constexpr size_t SIDE_CLEAR = 8 << 20; // floats
+    size_t zero_n = clear ? 2 * (size_t)prob->total_tokens * prob->n_kv_heads * prob->head_dim : 0;
+    if (zero_n > SIDE_CLEAR) {
+        CK(cudaMemsetAsync(dK_acc, 0, zero_n * sizeof(float), s));
+        zero_n = 0;
+    }
     for (int i = 0; i < nparts; ++i) {
         Call c;
-        int rc = plan_call(ctx, prob, &parts[i], true, s, c);
+        int rc = plan_call(ctx, prob, &parts[i], true, s, c, dK_acc, zero_n);
         if (rc != PEAGLE_OK)
             return rc;
+        if (c.plan.n_qt > 0)
+            zero_n = 0;
         // dO is known here, so the forward's epilogue leaves the backward's per-row values
         // (the separate peagle_attn_bwd forms them itself from O, dO and LSE)
         BwdArgs hand;
@@ -711,6 +723,8 @@ static int run_partitions(peagle_ctx *ctx, const peagle_problem_t *prob,
         if (rc != PEAGLE_OK)
             return rc;
     }
+    if (zero_n > 0)
+        CK(cudaMemsetAsync(dK_acc, 0, zero_n * sizeof(float), s));
     return PEAGLE_OK;
 }
 
@@ -754,8 +768,7 @@ int peagle_attn_partitioned(peagle_ctx *ctx, const peagle_problem_t *prob,
         return rc;
     float *dK_acc = static_cast<float *>(ctx->acc_buf.ptr);
     float *dV_acc = dK_acc + n_kv;
-    CK(cudaMemsetAsync(dK_acc, 0, 2 * n_kv * sizeof(float), s));
-    rc = run_partitions(ctx, prob, parts, nparts, Q, K, V, dO, O, LSE, dQ, dK_acc, dV_acc, s);
+    rc = run_partitions(ctx, prob, parts, nparts, Q, K, V, dO, O, LSE, dQ, dK_acc, dV_acc, s, true);
     if (rc != PEAGLE_OK)
         return rc;
     ctx->launches += launch_cast_grads(dK_acc, dV_acc, dK, dV, n_kv, s);
@@ -779,7 +792,7 @@ int peagle_attn_partitioned_acc(peagle_ctx *ctx, const peagle_problem_t *prob,
         return PEAGLE_ERR_ALIGN;
     CK(cudaSetDevice(ctx->device));
     return run_partitions(ctx, prob, parts, nparts, Q, K, V, dO, O, LSE, dQ, dK_acc, dV_acc,
-                          static_cast<cudaStream_t>(stream));
+                          static_cast<cudaStream_t>(stream), false);
 }
 
 int peagle_cast_grads(peagle_ctx *ctx, const float *dK_acc, const float *dV_acc, int64_t count,

@@ -135,9 +135,11 @@ inline cudaError_t launch_dependent(void (*kernel)(Params...), unsigned grid, un
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// K0: mask evaluator, tile classifier, scheduler.  Returns the number of kernels launched.
+// K0: mask evaluator, tile classifier, scheduler; it also clears `zero_n` floats (a multiple of 4) at `zero`
+// (16-byte aligned).  Returns the number of kernels launched.
 int launch_plan(const Plan &p, const int32_t *anchor, const int32_t *depth, int K, int seq_begin,
-                int seq_end, const RangeList &ranges, bool for_bwd, cudaStream_t s);
+                int seq_end, const RangeList &ranges, bool for_bwd, cudaStream_t s, float *zero = nullptr,
+                size_t zero_n = 0);
 int launch_mask_dense(const Plan &p, const RangeList &ranges, uint8_t *out, cudaStream_t s);
 // One CTA whose bounded wait runs out after limit_ns: records PEAGLE_ERR_TIMEOUT in *status.
 int launch_wait_expiry(int *status, unsigned long long limit_ns, int *reached_end, cudaStream_t s);

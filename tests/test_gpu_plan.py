@@ -76,3 +76,24 @@ def test_more_query_tiles_than_threads(ctx):
     dQ, _, _ = case.oracle_bwd(part, rows=rows)
     got = case.dQ[idx].float().cpu().numpy()
     assert np.linalg.norm(got - dQ) <= 1e-2 * np.linalg.norm(dQ)
+
+
+@pytest.mark.parametrize("w", [
+    inputs.Workload("sums_small", (200,), 3, 4, 2, 64, seed=46),        # cleared beside the plan
+    inputs.Workload("sums_above_32mb", (2050,), 8, 2, 2, 128, seed=47),  # by a fill of their own
+], ids=lambda w: w.name)
+def test_sums_of_an_earlier_call_are_cleared(ctx, w):
+    case = DeviceCase(w)
+    run_partitioned(ctx, case)
+    first = [t.float().cpu().numpy() for t in (case.dQ, case.dK, case.dV)]
+    # a partition without rows in front: the next one's plan has to clear them
+    empty = binding.Partition(0, (5, 5), case.parts[0]["k"])
+    case.bparts = [empty] + case.bparts
+    run_partitioned(ctx, case)
+    for t, want in zip((case.dQ, case.dK, case.dV), first):
+        # two fp32 sums of the same terms in another order, each rounded once to bf16
+        assert np.linalg.norm(t.float().cpu().numpy() - want) <= 2.0**-8 * np.linalg.norm(want)
+    for none in ([], [empty]):
+        case.bparts = none
+        run_partitioned(ctx, case)
+        assert not case.dK.any() and not case.dV.any()
