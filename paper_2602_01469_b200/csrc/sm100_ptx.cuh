@@ -24,7 +24,8 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
 // A kernel launched with launch_dependent (peagle_internal.h) may start while the kernel before it in the
 // stream still runs: pdl_wait returns once that kernel is complete and its writes are visible, pdl_trigger
 // lets the kernel after this one start.  Every thread of every kernel calls pdl_wait before it touches
-// global memory or leaves: a kernel that is complete then implies that all before it are.
+// global memory or leaves: a kernel that is complete then implies that all before it are.  (One exception,
+// with its reasons: bwd_prepare.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
