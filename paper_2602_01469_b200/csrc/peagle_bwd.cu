@@ -150,8 +150,8 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
 
     if (warp >= 20) {
         // ------------------------------------------------------------ drain (warps 20-23)
@@ -642,8 +642,8 @@ __global__ void bwd_prepare(const __nv_bfloat16 *__restrict__ O, const __nv_bflo
 __global__ void bwd_finish_dq(const float *__restrict__ dq_acc, __nv_bfloat16 *__restrict__ dQ,
                               size_t n8)
 {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (gid >= n8)
         return;
@@ -661,8 +661,8 @@ __global__ void cast_grads_kernel(const float *__restrict__ a, const float *__re
                                   __nv_bfloat16 *__restrict__ oa, __nv_bfloat16 *__restrict__ ob,
                                   size_t n8)
 {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (gid >= 2 * n8)
         return;

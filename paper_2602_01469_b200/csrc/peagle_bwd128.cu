@@ -77,7 +77,6 @@ bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t sb = smem_u32(smem_raw);
     uint8_t *sp = smem_raw;
-    pdl_trigger();
     if (sb & 1023u) { // the swizzled tiles need this alignment; nothing has been set up yet
         pdl_wait();
         if (threadIdx.x == 0)
@@ -131,6 +130,7 @@ bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     pdl_wait();
+    pdl_trigger();
 
     if (warp >= 12) {
         // ------------------------------------------------------------ drain (warps 12-15)

@@ -211,8 +211,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
 
     // Warps 8-11 hand most of their registers to the eight softmax warps.
     if (warp >= 8)

@@ -38,8 +38,8 @@ __global__ void __launch_bounds__(128) k0_tiles(Plan p, const int32_t *__restric
                                                 const int32_t *__restrict__ depth, int K, int seq_begin,
                                                 int seq_end, RangeList ranges)
 {
-    sm100::pdl_trigger();
     sm100::pdl_wait();
+    sm100::pdl_trigger();
     const int tile = blockIdx.x;
     const int t = seq_begin + tile * 128 + threadIdx.x;
     if (t < seq_end) {
@@ -266,9 +266,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
     __shared__ int2 entry[RAW_SINGLE];                // sorted raw tiles of an entry: first, last
     __shared__ int n_undecided, n_raw, n_entry, flag;
     sm100::pdl_wait();
-    // in this order: what starts now finds all kernels before this one complete (3,128 tokens, 32 heads of
-    // 128: 214 -> 208 us against the other order)
-    sm100::pdl_trigger();
+    sm100::pdl_trigger(); // after the wait: bwd_prepare counts on it
     const int qt = blockIdx.x, tid = threadIdx.x;
     // The blocks past the query tiles clear the fp32 sums that the backward adds to: memory is idle while
     // the others wait for one dependent step after another, and a fill of its own is a launch that

@@ -225,8 +225,8 @@ __global__ void __launch_bounds__(SINGLE_THREADS, 1) bwd_finish_single(const Sin
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) uint64_t bar, bar_q; // the dQ staging; Q and dO
     __shared__ int abort_flag;
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const int RB = P.rows_per_block;
     const int row_elems = P.Hq * D;
     float *sDQ = reinterpret_cast<float *>(smem);

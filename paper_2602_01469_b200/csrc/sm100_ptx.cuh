@@ -23,9 +23,11 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
 // ------------------------------------------------------------------ dependent launches
 // A kernel launched with launch_dependent (peagle_internal.h) may start while the kernel before it in the
 // stream still runs: pdl_wait returns once that kernel is complete and its writes are visible, pdl_trigger
-// lets the kernel after this one start.  Every thread of every kernel calls pdl_wait before it touches
-// global memory or leaves: a kernel that is complete then implies that all before it are.  (One exception,
-// with its reasons: bwd_prepare.)
+// lets the kernel after this one start.  The wait comes first: only the next kernel is then set up beside
+// this one, while with the trigger first all the kernels of a chain settle on the SMs at once and take
+// each other's places (512 tokens, 4 heads: 43 -> 40 us a step; 3,128 tokens, 32 heads of 128: 214 -> 205).
+// Every thread of every kernel calls pdl_wait before it touches global memory or leaves: a kernel that is
+// complete then implies that all before it are.  (One exception, with its reasons: bwd_prepare.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
