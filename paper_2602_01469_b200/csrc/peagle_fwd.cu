@@ -121,7 +121,6 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     using C = FwdCfg<D>;
     constexpr int NS = C::NS;
     constexpr bool TURNS = D == 128;
-    constexpr int EB = 8, POLY = 2; // see the exponentials
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t sb = (raw + 1023u) & ~1023u;
@@ -780,51 +779,49 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     break;
             }
             const float neg_m = (m == -CUDART_INF_F) ? 0.f : -m;
-            // Batches of EB pairs of columns, one step apart: the arguments of a batch, the exponentials of
-            // the one before, and sum and packing of the one before that are independent of one another,
-            // so that a warp does not wait for its own results.
+            // A quarter of the exponentials goes to the FMA pipe (an eighth and three eighths measured 3 and
+            // 5 per cent slower): every fourth column, two at a time as packed pairs.  The cubic is 7e-5
+            // off at argument 0, so which columns take it decides how exact the first rows of a sequence
+            // are, whose few keys stand in the first columns: with the fourth column of every four, rows
+            // of up to three keys are exact to fp32 rounding; with the first four of every sixteen,
+            // which keeps all pairs packed, their log-sum-exp was 7e-5 off (and the kernel at head_dim 64
+            // 2 per cent faster: 3,891 positions, 64 heads, 1,711 against 1,745 us; head_dim 128 1 per
+            // cent).  All arguments, then all exponentials, then sum and packing: what a warp does not
+            // have to wait for is then far ahead (in batches of 16 columns 1,766 to 1,811 us).
             const F2 scale2 = f2(P.scale_log2, P.scale_log2), nm2 = f2(neg_m, neg_m);
-            F2 sum2[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
-            F2 arg[2][EB], ex[2][EB];
-            uint32_t pk[32];
+            F2 e01[32], e3[16]; // of columns 4k ..: the first two; the last one of two neighbours
+            float e2[32], a3[32], sum = 0.f;
+            auto x_of = [&](int c) { return __uint_as_float(xr[c >> 5][c & 31]); };
 #pragma unroll
-            for (int b = 0; b < 64 / EB + 2; ++b) {
-                if (b < 64 / EB) {
-#pragma unroll
-                    for (int k = 0; k < EB; ++k) {
-                        const int c0 = 2 * (EB * b + k); // columns c0, c0 + 1
-                        arg[b & 1][k] = fma_f2(f2(__uint_as_float(xr[c0 >> 5][c0 & 31]), __uint_as_float(xr[c0 >> 5][(c0 & 31) + 1])),
-                                               scale2, nm2);
-                    }
-                }
-                if (b >= 1 && b <= 64 / EB) {
-#pragma unroll
-                    for (int k = 0; k < EB; ++k) {
-                        const F2 x2 = arg[(b - 1) & 1][k];
-                        // a quarter of the exponentials goes to the FMA pipe (an eighth and three
-                        // eighths measured 3 and 5 per cent slower)
-                        if ((EB * (b - 1) + k) % 8 < POLY) {
-                            ex[(b - 1) & 1][k] = exp2_fma2(x2);
-                        } else {
-                            const float2 v = unf2(x2);
-                            ex[(b - 1) & 1][k] = f2(fast_exp2(v.x), fast_exp2(v.y));
-                        }
-                    }
-                }
-                if (b >= 2) {
-#pragma unroll
-                    for (int k = 0; k < EB; ++k) {
-                        const F2 e2 = ex[b & 1][k];
-                        const float2 v = unf2(e2);
-                        sum2[k & 1] = add_f2(sum2[k & 1], e2);
-                        pk[(EB * (b - 2) + k) % 32] = pack_bf16x2(v.x, v.y);
-                    }
-                    if ((EB * (b - 1)) % 32 == 0)
-                        tmem_st32(tP + (EB * (b - 1) / 32 - 1) * 32, pk);
-                }
+            for (int k = 0; k < 32; ++k) {
+                e01[k] = fma_f2(f2(x_of(4 * k), x_of(4 * k + 1)), scale2, nm2);
+                e2[k] = fmaf(x_of(4 * k + 2), P.scale_log2, neg_m);
+                a3[k] = fmaf(x_of(4 * k + 3), P.scale_log2, neg_m);
             }
-            const float2 sv = unf2(add_f2(sum2[0], sum2[1]));
-            const float sum = sv.x + sv.y;
+#pragma unroll
+            for (int k = 0; k < 32; ++k) {
+                const float2 v = unf2(e01[k]);
+                e01[k] = f2(fast_exp2(v.x), fast_exp2(v.y));
+                e2[k] = fast_exp2(e2[k]);
+            }
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+                e3[k] = exp2_fma2(f2(a3[2 * k], a3[2 * k + 1]));
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                uint32_t pk[32];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const int k = 16 * c + i;
+                    const float2 v01 = unf2(e01[k]), v3 = unf2(e3[k >> 1]);
+                    const float last = k & 1 ? v3.y : v3.x;
+                    sum += v01.x + v01.y;
+                    sum += e2[k] + last;
+                    pk[2 * i] = pack_bf16x2(v01.x, v01.y);
+                    pk[2 * i + 1] = pack_bf16x2(e2[k], last);
+                }
+                tmem_st32(tP + c * 32, pk);
+            }
             if (TURNS && P.two && lane == 0)
                 mbar_arrive(BAR(B_TURN + 4 * (x ^ 1) + (warp & 3))); // the other tile's turn
             l += sum;

@@ -103,6 +103,21 @@ def test_forward_no_visible_keys_at_all(ctx):
     assert torch.all(case.O[:20] == 0) and torch.isneginf(case.LSE[:, :20]).all()
 
 
+@pytest.mark.parametrize("D", [64, 128])
+def test_rows_of_few_keys_to_fp32_rounding(ctx, D):
+    """The first three rows of a sequence see one to three keys, which all take the exact exponential:
+    what is left is fp32 rounding of a score below 8 in magnitude (the dot product of D terms, 2^-24
+    relative for each of its partial sums: 8 D 2^-24 <= 6e-5 at worst, about sqrt(D) 2^-24 x 8 = 5e-6 in
+    practice) and of exp2 / log2 (2^-22).  The cubic that a quarter of the columns takes is 7e-5 off."""
+    case = DeviceCase(inputs.Workload("few_keys", (70, 130), 1, 4, 2, D, seed=51))
+    run_fwd_all(ctx, case)
+    for p in case.parts:
+        rows = np.arange(p["q"][0], p["q"][0] + 3)
+        _, want = case.oracle_fwd(p, rows=rows)
+        got = case.LSE[:, torch.as_tensor(rows, device="cuda")].t().cpu().numpy()
+        assert np.abs(got - want).max() <= 1e-5
+
+
 @pytest.mark.parametrize("name", ["qwen3coder_n2048", "gptoss_n4096", "p90_n11008_s4"])
 def test_forward_full_size_sampled_rows(ctx, name):
     """Full-size launch; rows sampled from every partition (first/last tiles, ragged tail,
