@@ -35,6 +35,9 @@
  *     the device (bad metadata, a wait that ran out) are recorded in a status word that
  *     peagle_poll_status() returns.
  *   - A row whose visible allowed set is empty gets O = 0, LSE = -inf and zero gradients.
+ *   - Tiles are loaded whole.  K and V rows that a query may not see, up to 127 rows past the end
+ *     of a visible range among them (rows of the next sequence, say), enter products with weight zero:
+ *     they have to be finite.  Rows of Q, O and dO outside the partition are not used.
  *   - Token order inside a sequence is free; only speed depends on it.
  */
 #ifndef PEAGLE_H_

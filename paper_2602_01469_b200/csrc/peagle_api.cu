@@ -3,6 +3,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 #include <vector>
 
@@ -871,6 +872,22 @@ int peagle_layer_partitioned(peagle_ctx *ctx, const peagle_problem_t *prob,
     float *dX_acc = reinterpret_cast<float *>(take(b_dx)), *dW_acc = reinterpret_cast<float *>(take(b_dw));
     CK(cudaMemsetAsync(dX_acc, 0, T * dm * 4, s));
     CK(cudaMemsetAsync(dW_acc, 0, nqkv * dm * 4, s));
+    // The last key tile of a visible range is loaded whole: up to BN - 1 rows of K / V past the range's end
+    // enter its products with weight zero.  They may belong to a segment that is projected later or
+    // not at all, and hold whatever an earlier call left there; a NaN times zero would reach O, dQ
+    // and dW, so such rows are cleared.
+    for (int i = 0; i < nparts; ++i) {
+        Call c;
+        rc = validate_partition(prob, &parts[i], c);
+        if (rc != PEAGLE_OK)
+            return rc;
+        for (int r = 0; r < c.ranges.n; ++r) {
+            const size_t e = (size_t)c.ranges.end[r], over = (size_t)(e - c.ranges.begin[r]) % BN;
+            const size_t rows = over ? std::min(BN - over, T - e) : 0;
+            if (rows > 0) // K and V in one call: two lines of rows * nkv elements, Vb behind Kb
+                CK(cudaMemset2DAsync(Kb + e * nkv * 2, b_kv, 0, rows * nkv * 2, 2, s));
+        }
+    }
     const uint8_t *Xb = static_cast<const uint8_t *>(X), *Wb = static_cast<const uint8_t *>(W);
     const uint8_t *Wkv = Wb + nq * dm * 2; // rows of W that make the key and value heads
     auto gemm = [&](const void *A, long long lda, int a_t, const void *B, long long ldb, int b_t, void *C,

@@ -77,6 +77,16 @@ def test_segmented_layer_matches_oracle(ctx, w, d_model):
     check_against_oracle(w, run_layer(ctx, w, d_model))
 
 
+def test_layer_does_not_see_what_an_earlier_call_left(ctx):
+    """Scratch is carved anew per shape: the first call's fp32 sums of dX lie where the second call's K
+    and V rows will be, and every other half of an fp32 word is an arbitrary bf16, NaN among them.
+    Segments and sequences of the second call end inside a tile, so that tiles reach rows which are
+    projected later."""
+    run_layer(ctx, inputs.Workload("layer_before", (300,), 4, 2, 1, 64, seed=37), 2048)
+    w = inputs.Workload("layer_after", (110, 40), 4, 16, 8, 64, n_segments=3, seed=38)
+    check_against_oracle(w, run_layer(ctx, w, 64))
+
+
 def test_p90_shape_segmented_equals_single_pass_and_sampled_forward(ctx):
     """The P90-length configuration's segmentation (n = 11,008 in four segments; the layer is taken
     narrower -- 8 / 2 heads, d_model 512 -- so that the oracle's share stays in seconds): the
