@@ -219,7 +219,10 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         if (!ok)
             break;
         tc_fence_after();
-        // Keys past a ragged tile's end have p = ds = 0, so their rows (of another range) get zeros.
+        // Keys past a ragged tile's end are another range's, often another sequence's.  Their sums have weight
+        // zero throughout, but a zero times an Inf or NaN of a row of Q or dO is not zero, so zeros are
+        // what they get.
+        const int rows = item.k_len - (warp & 3) * 32; // of this warp's 32 keys, how many are the tile's
 #pragma unroll
         for (int t = 0; t < 2; ++t) { // dK, then dV
             uint32_t o[2][32];
@@ -230,9 +233,16 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                 tc_fence_before();
                 warp_arrive(BAR(B_ACCFREE));
             }
+            if (lane >= rows) {
 #pragma unroll
-            for (int pn = 0; pn < 2; ++pn)
-                send(o[pn], t ? 1.f : P.scale, pn, t ? &tmDV : &tmDK, 32 * pn, item.g, item.k_start);
+                for (int i = 0; i < 32; ++i)
+                    o[0][i] = o[1][i] = 0;
+            }
+            if (rows > 0) {
+#pragma unroll
+                for (int pn = 0; pn < 2; ++pn)
+                    send(o[pn], t ? 1.f : P.scale, pn, t ? &tmDV : &tmDK, 32 * pn, item.g, item.k_start);
+            }
         }
         }
         if (lane == 0)

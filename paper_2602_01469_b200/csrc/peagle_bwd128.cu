@@ -198,7 +198,13 @@ bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         if (!ok)
             break;
         tc_fence_after();
-        // Keys past a ragged tile's end have p = ds = 0, so their rows (of another range) get zeros.
+        // Keys past a ragged tile's end are another range's, often another sequence's.  Their sums have weight
+        // zero throughout, but a zero times an Inf or NaN of a row of Q or dO is not zero, so zeros are
+        // what they get.  (The item is read again: carried through its steps these words would be
+        // spilled; see the queue for why the slot still holds it.)
+        const BwdItem &done = *reinterpret_cast<const BwdItem *>(wq + (w & 3) * sizeof(BwdItem));
+        const int k_start = done.k_start, g = done.g;
+        const int rows = done.k_len - (warp & 3) * 32; // of this warp's 32 keys, how many are the tile's
 #pragma unroll
         for (int pn = 0; pn < 8; ++pn) {
             uint32_t o[32];
@@ -208,8 +214,14 @@ bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                 tc_fence_before();
                 warp_arrive(BAR(B_ACCFREE));
             }
+            if (lane >= rows) {
+#pragma unroll
+                for (int i = 0; i < 32; ++i)
+                    o[i] = 0;
+            }
             const bool k = pn < 4;
-            send(o, k ? P.scale : 1.f, pn & 1, k ? &tmDK : &tmDV, 32 * (pn % 4), item.g, item.k_start);
+            if (rows > 0)
+                send(o, k ? P.scale : 1.f, pn & 1, k ? &tmDK : &tmDV, 32 * (pn % 4), g, k_start);
         }
         }
         if (lane == 0)

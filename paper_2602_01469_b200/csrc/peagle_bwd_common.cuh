@@ -23,11 +23,21 @@ struct BwdParams {
 };
 
 // Work items are handed out dynamically: the producer warp takes the next index from a global cursor
-// and publishes what the other roles need of the item in a four-slot queue in shared memory (slot
-// w & 3 for the CTA's item w; it was last used four items ago, and no role is more than two items
-// behind).  A CTA that falls behind therefore takes fewer items, and the CTAs running at any time
-// work on a contiguous window of the chunk-major item list (their shared Q / dO rows and dQ staging
-// rows stay in L2), instead of drifting apart as with a static round-robin.
+// and publishes what the other roles need of the item in a four-slot queue in shared memory.  A CTA that
+// falls behind therefore takes fewer items, and the CTAs running at any time work on a contiguous window
+// of the chunk-major item list (their shared Q / dO rows and dQ staging rows stay in L2), instead of
+// drifting apart as with a static round-robin.
+// Slot w & 3 has the CTA's item w.  The producer writes it with the last step of item w - 1, when every
+// role has taken item w - 4, also where items are single steps:
+//   bwd64_kernel   K of item w - 1 was requested before, so the K stage of item w - 3 was free
+//                  (B_KVEMPTY): dQ of its last step was complete, which follows that step's dS^T
+//                  (compute warps, S^T and dP^T issuers) and the drain's read of dQ of the step before
+//                  (B_DQEMPTY), in item w - 4 or later.  The drain may still be sending dK / dV of item
+//                  w - 4, from its registers.
+//   bwd128_kernel  K of item w - 1 was requested before, so K of item w - 2 was free (B_KEMPTY): dQ of its
+//                  last step was complete, behind that step's dP^T, which followed the drain's read of dQ
+//                  of the step before, in item w - 3 or later.  The drain is therefore through with item
+//                  w - 4 altogether, and may read its slot again at the item's end.
 // One index = (work item of K0, KV head, part of the group's heads): one key tile against the query
 // tiles of a chunk, one head after the other; every (query tile, head) is a step.
 struct BwdItem {

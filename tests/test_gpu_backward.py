@@ -145,6 +145,22 @@ def test_bwd_rows_that_see_nothing_get_zero_gradients(ctx):
     assert torch.all(dK_acc[:140] == 0) and torch.all(dK_acc[160:] == 0)
 
 
+@pytest.mark.parametrize("D", [64, 128])
+def test_non_finite_gradient_stays_in_its_sequence(ctx, D):
+    """The last key tile of the first sequence is ragged and its lanes past the end are keys of the second
+    one: an Inf or NaN in dO of the first sequence must not reach their dK / dV rows.  Sequence lengths that
+    end inside a warp's 32 keys, on its border, and with whole warps past the end."""
+    for n in (170, 160, 130):
+        case = DeviceCase(inputs.Workload("neighbours", (n, 90), 1, 4, 2, D, seed=52))
+        case.ddO[n - 2] = float("nan")
+        case.ddO[n - 1] = float("inf")
+        run_partitioned(ctx, case)
+        sl = case.seq_slice(1)
+        _, _, dQ, dK, dV = oracle_all(case)
+        for name, got, want in zip(("dQ", "dK", "dV"), (case.dQ, case.dK, case.dV), (dQ, dK, dV)):
+            check_rows(name, got[sl].float().cpu().numpy(), want[sl])
+
+
 def full_size_checks(case, n_rows=16, n_keys=6, seed=0):
     """Checks that hold at any size, plus outputs the oracle can compute one by one."""
     w = case.w
