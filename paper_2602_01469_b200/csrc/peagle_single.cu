@@ -112,7 +112,8 @@ struct KeyRows {
     int tok[KEYS];           // -1: none
     uint4 k[KEYS], v[KEYS]; // this lane's elements of the keys' rows, packed bf16
 };
-// Takes the next KEYS keys of the row (bits of `keys`: entries, ascending) and requests their rows.
+// Takes the next KEYS keys of the row (bits of `keys`: entries, ascending; at least one) and requests their
+// rows.
 // Lane `sub` of a unit has the key of entry sub in t0 and, with 8 lanes, that of entry sub + 8 in t1.
 template <int D>
 __device__ __forceinline__ void next_keys(const SingleParams &P, unsigned &keys, int t0, int t1, int sub, unsigned um,
@@ -125,7 +126,9 @@ __device__ __forceinline__ void next_keys(const SingleParams &P, unsigned &keys,
         if (at >= 0)
             out.tok[i] = __shfl_sync(um, at < D / 8 ? t0 : t1, ub + at % (D / 8));
         keys &= keys - 1;
-        const size_t kr = ((size_t)max(out.tok[i], 0) * P.Hkv + g) * D;
+        // an absent key takes the row of the first one, which the query sees: with weight zero it is
+        // harmless unless the row has an Inf or NaN, and then the result has one anyway
+        const size_t kr = ((size_t)(out.tok[i] >= 0 ? out.tok[i] : out.tok[0]) * P.Hkv + g) * D;
         auto row_of = [&](const __nv_bfloat16 *row) {
             const uint2 a = __ldg(reinterpret_cast<const uint2 *>(row) + sub);
             const uint2 b = __ldg(reinterpret_cast<const uint2 *>(row + D / 2) + sub);

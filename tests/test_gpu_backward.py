@@ -161,6 +161,21 @@ def test_non_finite_gradient_stays_in_its_sequence(ctx, D):
             check_rows(name, got[sl].float().cpu().numpy(), want[sl])
 
 
+@pytest.mark.parametrize("D", [64, 128])
+def test_non_finite_first_token_stays_in_its_sequence(ctx, D):
+    """Chain keys are taken two at a time; a row with an odd number of them must not read another
+    sequence's K / V row in place of the second."""
+    case = DeviceCase(inputs.Workload("first_token", (40, 130), 4, 4, 2, D, seed=53))
+    case.dK_[0] = float("nan")
+    case.dV_[0] = float("inf")
+    run_partitioned(ctx, case)
+    sl = case.seq_slice(1)
+    O, LSE, dQ, dK, dV = oracle_all(case)
+    check_forward(case.O[sl].float().cpu().numpy(), case.LSE[:, sl].t().cpu().numpy(), O[sl], LSE[sl])
+    for name, got, want in zip(("dQ", "dK", "dV"), (case.dQ, case.dK, case.dV), (dQ, dK, dV)):
+        check_rows(name, got[sl].float().cpu().numpy(), want[sl])
+
+
 def full_size_checks(case, n_rows=16, n_keys=6, seed=0):
     """Checks that hold at any size, plus outputs the oracle can compute one by one."""
     w = case.w
