@@ -875,7 +875,10 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                        return fin;
                    }()) {
             tc_fence_after();
-            const float inv = l > 0.f ? 1.f / l : 0.f;
+            // A row with no key in any of its tiles has m = -inf, but not l = 0: the cubic never goes below
+            // 2^-126.  Its O is zero all the same.
+            const bool seen = m > -CUDART_INF_F && l > 0.f;
+            const float inv = seen ? 1.f / l : 0.f;
             uint4 *dst = reinterpret_cast<uint4 *>(P.O + ((size_t)row * P.Hq + h) * D);
             float delta = 0.f;
             auto dot8 = [&](const uint4 w, const uint32_t *o8) {
@@ -932,11 +935,11 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     }
                 }
             }
-            const float lse2 = l > 0.f ? m + log2f(l) : -CUDART_INF_F;
+            const float lse2 = seen ? m + log2f(l) : -CUDART_INF_F;
             if (row_ok)
                 P.LSE[(size_t)h * P.T + row] = lse2 * 0.6931471805599453f;
             if (P.dO) { // the accumulator is not normalised: Delta = inv * <dO, O_acc>
-                P.nl2[hand] = (row_ok && l > 0.f) ? -lse2 : -CUDART_INF_F;
+                P.nl2[hand] = (row_ok && seen) ? -lse2 : -CUDART_INF_F;
                 P.nd[hand] = row_ok ? -delta * inv : 0.f;
             }
         } else {

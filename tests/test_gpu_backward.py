@@ -176,6 +176,20 @@ def test_non_finite_first_token_stays_in_its_sequence(ctx, D):
         check_rows(name, got[sl].float().cpu().numpy(), want[sl])
 
 
+@pytest.mark.parametrize("D", [64, 128])
+def test_rows_of_a_tensor_core_tile_that_see_nothing(ctx, D):
+    """Rows 0-63 stand before every visible key, in a tile whose other rows see several."""
+    w = inputs.Workload("later_keys", (200,), 1, 4, 2, D, seed=55)
+    anchor, depth = inputs.full_grid(200, 1)
+    parts = [{"seq": 0, "q": (0, 200), "k": [(64, 180)]}]
+    case = DeviceCase(w, anchor=anchor, depth=depth, cu=np.array([0, 200], np.int32), parts=parts)
+    run_partitioned(ctx, case)
+    O, LSE, dQ, dK, dV = oracle_all(case)
+    check_forward(case.O.float().cpu().numpy(), case.LSE.t().cpu().numpy(), O, LSE)
+    check_grads(case, dQ, dK, dV)
+    assert not case.O[:64].any() and not case.dQ[:64].any()
+
+
 def full_size_checks(case, n_rows=16, n_keys=6, seed=0):
     """Checks that hold at any size, plus outputs the oracle can compute one by one."""
     w = case.w
