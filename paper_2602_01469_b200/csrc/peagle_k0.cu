@@ -381,9 +381,9 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
             } else if (ktile.y == BN && total == (r1 - r0) * BN) {
                 c = TILE_FULL;
             } else if (p.allow_single && mx <= 1) {
+                c = TILE_SINGLE;
                 slot = atomicAdd(&n_raw, 1);
                 if (slot < RAW_SINGLE) {
-                    c = TILE_SINGLE;
                     raw_kt[slot] = kt;
                     raw_min[slot] = INT_MAX;
                     raw_max[slot] = -1;
@@ -407,6 +407,38 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
         }
     }
     __syncthreads();
+    // More one-key-per-row tiles than there are places (from 33 depths on).  Which of them came first
+    // differs from run to run, so the lowest are taken, and looked at once more; the rest goes to the
+    // tensor cores.
+    if (n_raw > RAW_SINGLE) {
+        block_compact(
+            p.n_kt, warp_cnt, [&](int kt) { return cls[kt] == TILE_SINGLE; },
+            [&](int kt, int at) {
+                if (at < RAW_SINGLE) {
+                    raw_kt[at] = kt;
+                    raw_min[at] = INT_MAX;
+                    raw_max[at] = -1;
+                } else {
+                    cls[kt] = TILE_PARTIAL;
+                }
+            });
+        __syncthreads();
+#pragma unroll 1
+        for (int i = group; i < RAW_SINGLE; i += PLAN_GROUPS) {
+            const int2 k = p.ktile[raw_kt[i]];
+            int col = NO_COL;
+#pragma unroll 1
+            for (int c = 0; c < k.y; ++c)
+                if (allowed_packed(mq, p.meta[k.x + c]))
+                    col = c;
+            raw_col[i][row] = (uint8_t)col;
+            if (col != NO_COL) {
+                atomicMin(&raw_min[i], k.x + col);
+                atomicMax(&raw_max[i], k.x + col);
+            }
+        }
+        __syncthreads();
+    }
     // ---- one-key-per-row tiles: ascending by key tile (they were numbered in arrival order, and the
     // order of the per-pair sums shall not change from run to run)
     const int nr = min(n_raw, RAW_SINGLE);

@@ -65,6 +65,23 @@ def test_joined_windows(ctx, w):
     check_grads(case, dQ, dK, dV)
 
 
+@pytest.mark.parametrize("n,K", [(150, 48), (128, 40), (70, 120)])
+def test_more_chain_tiles_than_places_repeat_bit_for_bit(ctx, n, K):
+    """From 33 depths on a query tile has more one-key-per-row tiles than the plan keeps: the same ones are
+    chosen in every run, so that O and LSE, which are summed in a fixed order, repeat."""
+    case = DeviceCase(inputs.Workload("deep", (n,), K, 4, 2, 64, seed=54))
+    part = case.bparts[0]
+    first = None
+    for _ in range(10):
+        binding.peagle_attn_fwd(ctx, case.prob, part, case.dQ_, case.dK_, case.dV_, case.O, case.LSE)
+        assert binding.peagle_poll_status(ctx) == 0
+        if first is None:
+            first = (case.O.clone(), case.LSE.clone())
+        assert torch.equal(case.O, first[0]) and torch.equal(case.LSE, first[1])
+    O, LSE = case.oracle_fwd(case.parts[0])
+    check_forward(case.O.float().cpu().numpy(), case.LSE.t().cpu().numpy(), O, LSE)
+
+
 def test_more_query_tiles_than_threads(ctx):
     case = DeviceCase(inputs.Workload("long", (8300,), 8, 2, 1, 64, seed=45))
     run_partitioned(ctx, case)
