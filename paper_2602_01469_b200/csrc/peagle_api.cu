@@ -215,9 +215,8 @@ int validate_partition(const peagle_problem_t *prob, const peagle_partition_t *p
     return PEAGLE_OK;
 }
 
-// Runs K0 for one call.  On return c.plan points into ctx->plan_buf.
-int plan_call(peagle_ctx *ctx, const peagle_problem_t *prob, const peagle_partition_t *part,
-              bool for_bwd, cudaStream_t s, Call &c, float *zero = nullptr, size_t zero_n = 0)
+// Checks one call and lays out its plan in ctx->plan_buf.
+int plan_layout(peagle_ctx *ctx, const peagle_problem_t *prob, const peagle_partition_t *part, cudaStream_t s, Call &c)
 {
     int rc = validate_partition(prob, part, c);
     if (rc != PEAGLE_OK)
@@ -230,12 +229,27 @@ int plan_call(peagle_ctx *ctx, const peagle_problem_t *prob, const peagle_partit
     carve_plan(c.plan, ctx->plan_buf.ptr, nullptr);
     c.plan.status = ctx->status;
     c.plan.allow_single = single_tiles_ok(prob) ? 1 : 0;
+    return PEAGLE_OK;
+}
+
+// Runs K0 for a call that is laid out.
+int plan_launch(peagle_ctx *ctx, const peagle_problem_t *prob, const Call &c, bool for_bwd, cudaStream_t s,
+                const PlanSide &side)
+{
     if (c.plan.n_qt == 0)
         return PEAGLE_OK;
     ctx->launches += launch_plan(c.plan, prob->anchor, prob->depth, prob->K, c.seq_begin, c.seq_end,
-                                 c.ranges, for_bwd, s, zero, zero_n);
+                                 c.ranges, for_bwd, s, side);
     CK(cudaGetLastError());
     return PEAGLE_OK;
+}
+
+// Both.
+int plan_call(peagle_ctx *ctx, const peagle_problem_t *prob, const peagle_partition_t *part,
+              bool for_bwd, cudaStream_t s, Call &c, const PlanSide &side = PlanSide())
+{
+    const int rc = plan_layout(ctx, prob, part, s, c);
+    return rc != PEAGLE_OK ? rc : plan_launch(ctx, prob, c, for_bwd, s, side);
 }
 
 // Scratch of one backward call inside ctx->bwd_buf: per-row values and the fp32 dQ staging.
@@ -294,7 +308,7 @@ int run_fwd(peagle_ctx *ctx, const peagle_problem_t *prob, const Call &c, const 
 
 int run_bwd(peagle_ctx *ctx, const peagle_problem_t *prob, const Call &c, const void *Q,
             const void *K, const void *V, const void *O, const void *dO, const float *LSE,
-            void *dQ, float *dK_acc, float *dV_acc, cudaStream_t s, bool rows_ready = false)
+            void *dQ, float *dK_acc, float *dV_acc, cudaStream_t s)
 {
     if (c.plan.n_qt == 0)
         return PEAGLE_OK;
@@ -302,7 +316,6 @@ int run_bwd(peagle_ctx *ctx, const peagle_problem_t *prob, const Call &c, const 
     int rc = bwd_scratch(ctx, prob, c, s, a);
     if (rc != PEAGLE_OK)
         return rc;
-    a.rows_ready = rows_ready;
     a.Q = Q;
     a.K = K;
     a.V = V;
@@ -680,7 +693,24 @@ int peagle_attn_bwd(peagle_ctx *ctx, const peagle_problem_t *prob, const peagle_
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     CK(cudaSetDevice(ctx->device));
     Call c;
-    rc = plan_call(ctx, prob, part, true, s, c);
+    rc = plan_layout(ctx, prob, part, s, c);
+    if (rc != PEAGLE_OK || c.plan.n_qt == 0)
+        return rc;
+    BwdArgs rows;
+    rc = bwd_scratch(ctx, prob, c, s, rows);
+    if (rc != PEAGLE_OK)
+        return rc;
+    PlanSide side;
+    side.O = O;
+    side.dO = dO;
+    side.LSE = LSE;
+    side.nl2 = rows.nl2;
+    side.nd = rows.nd;
+    side.mqp = rows.mqp;
+    side.dq_acc = rows.dq_acc;
+    side.Hq = prob->n_q_heads;
+    side.D = prob->head_dim;
+    rc = plan_launch(ctx, prob, c, true, s, side);
     if (rc != PEAGLE_OK)
         return rc;
     return run_bwd(ctx, prob, c, Q, K, V, O, dO, LSE, dQ, dK_acc, dV_acc, s);
@@ -704,13 +734,16 @@ static int run_partitions(peagle_ctx *ctx, const peagle_problem_t *prob,
     }
     for (int i = 0; i < nparts; ++i) {
         Call c;
-        int rc = plan_call(ctx, prob, &parts[i], true, s, c, dK_acc, zero_n);
+        PlanSide side;
+        side.zero = dK_acc;
+        side.zero_n = zero_n;
+        int rc = plan_call(ctx, prob, &parts[i], true, s, c, side);
         if (rc != PEAGLE_OK)
             return rc;
         if (c.plan.n_qt > 0)
             zero_n = 0;
         // dO is known here, so the forward's epilogue leaves the backward's per-row values
-        // (the separate peagle_attn_bwd forms them itself from O, dO and LSE)
+        // (the separate peagle_attn_bwd forms them beside its plan from O, dO and LSE)
         BwdArgs hand;
         if (c.plan.n_qt > 0) {
             rc = bwd_scratch(ctx, prob, c, s, hand);
@@ -720,7 +753,7 @@ static int run_partitions(peagle_ctx *ctx, const peagle_problem_t *prob,
         rc = run_fwd(ctx, prob, c, Q, K, V, O, LSE, s, dO, &hand);
         if (rc != PEAGLE_OK)
             return rc;
-        rc = run_bwd(ctx, prob, c, Q, K, V, O, dO, LSE, dQ, dK_acc, dV_acc, s, true);
+        rc = run_bwd(ctx, prob, c, Q, K, V, O, dO, LSE, dQ, dK_acc, dV_acc, s);
         if (rc != PEAGLE_OK)
             return rc;
     }
@@ -949,7 +982,7 @@ int peagle_layer_partitioned(peagle_ctx *ctx, const peagle_problem_t *prob,
         rc = run_fwd(ctx, prob, c, Qb, Kb, Vb, O, LSE, s, dO, &hand);
         if (rc != PEAGLE_OK)
             return rc;
-        rc = run_bwd(ctx, prob, c, Qb, Kb, Vb, O, dO, LSE, dQb, dK_acc, dV_acc, s, true);
+        rc = run_bwd(ctx, prob, c, Qb, Kb, Vb, O, dO, LSE, dQb, dK_acc, dV_acc, s);
         if (rc != PEAGLE_OK)
             return rc;
         for (int r = 0; r < c.ranges.n; ++r) {
@@ -1134,7 +1167,7 @@ int peagle_attn_partitioned_host(peagle_ctx *ctx, const peagle_problem_t *prob,
                              ddO, &hand);
             if (rc == PEAGLE_OK)
                 rc = run_bwd(ctx, &dprob, c, dQin, dKin, dVin, dOout, ddO,
-                             reinterpret_cast<float *>(dLSE), ddQ, dK_acc, dV_acc, s_c, true);
+                             reinterpret_cast<float *>(dLSE), ddQ, dK_acc, dV_acc, s_c);
             if (rc != PEAGLE_OK)
                 return drained(rc);
             CKD(cudaEventRecord(x.done, s_c));

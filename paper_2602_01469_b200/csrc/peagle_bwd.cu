@@ -588,67 +588,6 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     }
 }
 
-// Per-row inputs of the backward kernels for the q_pad = n_qt * BM rows the query tiles cover:
-// -LSE * log2(e), -Delta with Delta[h][r] = <dO[q,h,:], O[q,h,:]>, and the packed metadata, with
-// neutral values for the rows past the partition's end.  Also zeroes the fp32 dQ staging.
-// Of the plan kernel before it, it needs nothing, only what that kernel waited for before it let this
-// one start: so it does not wait, and runs beside the plan (memory beside a chain of dependent steps on
-// a few SMs; two partitions of 4,000 tokens, forward and backward calls: 768 -> 739 us).  Block 0 waits
-// at its end, so that this kernel is complete only when the plan is, which is all that the next kernel
-// waits for.  Everything is read from L2.
-template <int D>
-__global__ void bwd_prepare(const __nv_bfloat16 *__restrict__ O, const __nv_bfloat16 *__restrict__ dO,
-                            const float *__restrict__ LSE, const int32_t *__restrict__ meta,
-                            float *__restrict__ nl2, float *__restrict__ nd,
-                            int32_t *__restrict__ mqp, float *__restrict__ dq_acc, int q_begin,
-                            int q_len, int q_pad, int Hq, int T)
-{
-    pdl_trigger();
-    constexpr int TPR = D / 8; // threads per (row, head)
-    const size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const size_t n = (size_t)q_pad * Hq * TPR;
-    const size_t rh = gid / TPR;
-    const size_t r = rh / Hq, h = rh % Hq;
-    const bool real = gid < n && r < (size_t)q_len;
-    float acc = 0.f;
-    if (real) {
-        const size_t src = (size_t)q_begin * Hq * D + gid * 8;
-        const uint4 a = __ldcg(reinterpret_cast<const uint4 *>(O + src));
-        const uint4 b = __ldcg(reinterpret_cast<const uint4 *>(dO + src));
-        const __nv_bfloat162 *pa = reinterpret_cast<const __nv_bfloat162 *>(&a);
-        const __nv_bfloat162 *pb = reinterpret_cast<const __nv_bfloat162 *>(&b);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float2 x = __bfloat1622float2(pa[i]), y = __bfloat1622float2(pb[i]);
-            acc += x.x * y.x + x.y * y.y;
-        }
-        float4 *z = reinterpret_cast<float4 *>(dq_acc + gid * 8);
-        z[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-        z[1] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-#pragma unroll
-    for (int o = TPR / 2; o > 0; o >>= 1)
-        acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (gid < n && (gid % TPR) == 0) {
-        float l = -CUDART_INF_F;
-        int mq = META_NONE_Q;
-        if (real) {
-            const float lse = __ldcg(LSE + h * (size_t)T + q_begin + r);
-            if (lse != -CUDART_INF_F)
-                l = -lse * 1.4426950408889634f;
-            mq = __ldcg(meta + q_begin + r);
-            if (mq == META_NONE_K)
-                mq = META_NONE_Q;
-        }
-        nl2[h * (size_t)q_pad + row_slot((int)r)] = l;
-        nd[h * (size_t)q_pad + row_slot((int)r)] = real ? -acc : 0.f;
-        if (h == 0)
-            mqp[row_slot((int)r)] = mq;
-    }
-    if (blockIdx.x == 0)
-        pdl_wait();
-}
-
 __global__ void bwd_finish_dq(const float *__restrict__ dq_acc, __nv_bfloat16 *__restrict__ dQ,
                               size_t n8)
 {
@@ -706,18 +645,8 @@ static int launch_bwd_t(const Plan &p, const BwdArgs &a, EncodeTiledFn enc, int 
     if (make_f32_map(enc, &tmDQ, a.dq_acc, D, a.Hq, q_len, 32) || make_f32_map(enc, &tmDK, a.dK_acc, D, a.Hkv, p.T, 32) ||
         make_f32_map(enc, &tmDV, a.dV_acc, D, a.Hkv, p.T, 32))
         return PEAGLE_ERR_CUDA;
-    const size_t n_prep = (size_t)q_len * a.Hq * (D / 8);
-    const size_t n_prep_pad = (size_t)q_pad * a.Hq * (D / 8);
+    const size_t n8 = (size_t)q_len * a.Hq * (D / 8);
     int launches = 0;
-    // Per-row values and a cleared dQ staging: the forward of the partition leaves both when it runs in
-    // the driver, where dO is known.
-    if (!a.rows_ready) {
-        launch_dependent(
-            bwd_prepare<D>, (unsigned)((n_prep_pad + 255) / 256), 256, 0, s,
-            static_cast<const __nv_bfloat16 *>(a.O), static_cast<const __nv_bfloat16 *>(a.dO), a.LSE,
-            p.meta, a.nl2, a.nd, a.mqp, a.dq_acc, p.q_begin, q_len, q_pad, a.Hq, p.T);
-        launches = 1;
-    }
     if (p.n_kt > 0) {
         BwdParams P;
         P.ktile = p.ktile;
@@ -761,7 +690,7 @@ static int launch_bwd_t(const Plan &p, const BwdArgs &a, EncodeTiledFn enc, int 
         return n < 0 ? n : launches + n;
     }
     launch_dependent(
-        bwd_finish_dq, (unsigned)((n_prep + 255) / 256), 256, 0, s, a.dq_acc, static_cast<__nv_bfloat16 *>(a.dQ) + (size_t)p.q_begin * a.Hq * D, n_prep);
+        bwd_finish_dq, (unsigned)((n8 + 255) / 256), 256, 0, s, a.dq_acc, static_cast<__nv_bfloat16 *>(a.dQ) + (size_t)p.q_begin * a.Hq * D, n8);
     return launches + 1;
 }
 

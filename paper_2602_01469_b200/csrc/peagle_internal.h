@@ -90,14 +90,14 @@ struct BwdArgs {
     void *dQ;
     float *dK_acc, *dV_acc;
     // per-row scratch of the call, q_pad = query tiles * BM rows, rows past the partition padded;
-    // row r's entry stands at row_slot(r)
+    // row r's entry stands at row_slot(r).  Written, and dq_acc cleared, by the forward of the partition
+    // in the driver, where dO is known, else beside the plan (PlanSide).
     float *nl2;     // [Hq][q_pad] -LSE * log2(e); -inf for a padded row or a row that saw no key
     float *nd;      // [Hq][q_pad] -Delta = -<dO, O>; 0 for a padded row
     int32_t *mqp;   // [q_pad] packed metadata of the partition's rows; META_NONE_Q when padded
     float *dq_acc;  // [q_len][Hq][D] scratch, fp32
     int Hq, Hkv, D;
     float scale;
-    bool rows_ready = false; // nl2 / nd / mqp were written, dq_acc was cleared by the forward of this partition
 };
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
@@ -135,11 +135,23 @@ inline cudaError_t launch_dependent(void (*kernel)(Params...), unsigned grid, un
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// K0: mask evaluator, tile classifier, scheduler; it also clears `zero_n` floats (a multiple of 4) at `zero`
-// (16-byte aligned).  Returns the number of kernels launched.
+// What the plan kernel does on the side, in blocks of its own: it clears `zero_n` floats (a multiple of 4) at
+// `zero` (16-byte aligned), and with O set it prepares the backward of the call's rows from O, dO and LSE (see
+// BwdArgs).
+struct PlanSide {
+    float *zero = nullptr;
+    size_t zero_n = 0;
+    const void *O = nullptr, *dO = nullptr;
+    const float *LSE = nullptr;
+    float *nl2 = nullptr, *nd = nullptr;
+    int32_t *mqp = nullptr;
+    float *dq_acc = nullptr;
+    int Hq = 0, D = 0;
+};
+
+// K0: mask evaluator, tile classifier, scheduler.  Returns the number of kernels launched.
 int launch_plan(const Plan &p, const int32_t *anchor, const int32_t *depth, int K, int seq_begin,
-                int seq_end, const RangeList &ranges, bool for_bwd, cudaStream_t s, float *zero = nullptr,
-                size_t zero_n = 0);
+                int seq_end, const RangeList &ranges, bool for_bwd, cudaStream_t s, const PlanSide &side = PlanSide());
 int launch_mask_dense(const Plan &p, const RangeList &ranges, uint8_t *out, cudaStream_t s);
 // One CTA whose bounded wait runs out after limit_ns: records PEAGLE_ERR_TIMEOUT in *status.
 int launch_wait_expiry(int *status, unsigned long long limit_ns, int *reached_end, cudaStream_t s);

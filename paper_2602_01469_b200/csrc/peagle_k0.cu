@@ -15,6 +15,9 @@
 // Everything runs on the caller's stream; nothing returns to the host.  The work is integer and small:
 // what it costs is launches and the latency of dependent steps, hence two kernels and not one per
 // step (eight kernels before: 24 us for 512 tokens, 47 us for 32,768, 95 us for the COD example).
+#include <cuda_bf16.h>
+#include <math_constants.h>
+
 #include "peagle_internal.h"
 #include "sm100_ptx.cuh"
 
@@ -251,8 +254,59 @@ __device__ __forceinline__ void block_sort(int n, int *hist, int *warp_sum, int 
         out[atomicAdd(&hist[bucket(i)], 1)] = i;
 }
 
+// The backward's inputs for the q_pad = n_qt * BM rows that the query tiles cover: -LSE * log2(e), -Delta with
+// Delta[h][r] = <dO[q,h,:], O[q,h,:]>, and the packed metadata, with neutral values for the rows past the
+// partition's end; and a cleared fp32 dQ staging.  D / 8 neighbouring lanes per (row, head), 8 elements each.
+// Bound by memory (8 bytes per element of O).  Beside the plan rather than as a kernel of its own: the
+// plan is a chain of dependent steps on a few SMs (two partitions of 4,000 tokens, 64 heads of 64, forward and
+// backward calls: 768 us with a kernel behind the plan, 725 us this way).
+__device__ __forceinline__ void prepare_rows(const Plan &p, const PlanSide &a, int block, int blocks)
+{
+    const int tpr = a.D / 8, q_len = p.q_end - p.q_begin;
+    const size_t q_pad = (size_t)p.n_qt * BM, n = q_pad * a.Hq * tpr; // a multiple of 32: warps stay whole
+    for (size_t gid = (size_t)block * PLAN_THREADS + threadIdx.x; gid < n; gid += (size_t)blocks * PLAN_THREADS) {
+        const size_t rh = gid / tpr, r = rh / a.Hq, h = rh % a.Hq;
+        const bool real = r < (size_t)q_len;
+        float acc = 0.f;
+        if (real) {
+            const size_t src = ((size_t)p.q_begin * a.Hq * tpr + gid);
+            const uint4 x4 = reinterpret_cast<const uint4 *>(a.O)[src], y4 = reinterpret_cast<const uint4 *>(a.dO)[src];
+            const __nv_bfloat162 *pa = reinterpret_cast<const __nv_bfloat162 *>(&x4);
+            const __nv_bfloat162 *pb = reinterpret_cast<const __nv_bfloat162 *>(&y4);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 x = __bfloat1622float2(pa[i]), y = __bfloat1622float2(pb[i]);
+                acc += x.x * y.x + x.y * y.y;
+            }
+            float4 *z = reinterpret_cast<float4 *>(a.dq_acc) + 2 * gid;
+            z[0] = make_float4(0.f, 0.f, 0.f, 0.f);
+            z[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        for (int o = tpr / 2; o > 0; o >>= 1)
+            acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (gid % tpr == 0) {
+            float l = -CUDART_INF_F;
+            int mq = META_NONE_Q;
+            if (real) {
+                const float lse = a.LSE[h * (size_t)p.T + p.q_begin + r];
+                if (lse != -CUDART_INF_F)
+                    l = -lse * 1.4426950408889634f;
+                mq = p.meta[p.q_begin + r];
+                if (mq == META_NONE_K)
+                    mq = META_NONE_Q;
+            }
+            a.nl2[h * q_pad + row_slot((int)r)] = l;
+            a.nd[h * q_pad + row_slot((int)r)] = real ? -acc : 0.f;
+            if (h == 0)
+                a.mqp[row_slot((int)r)] = mq;
+        }
+    }
+}
+
+// PREP: the side blocks prepare rows.  (In one kernel for both uses, plans that do not were 1 to 2 us slower.)
+template <bool PREP>
 __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, int seq_end, int for_bwd,
-                                                        float4 *zero, size_t zero_n4)
+                                                        const PlanSide side)
 {
     __shared__ __align__(16) int hist[SORT_BUCKETS];
     __shared__ int warp_cnt[PLAN_THREADS / 32];
@@ -266,16 +320,19 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
     __shared__ int2 entry[RAW_SINGLE];                // sorted raw tiles of an entry: first, last
     __shared__ int n_undecided, n_raw, n_entry, flag;
     sm100::pdl_wait();
-    sm100::pdl_trigger(); // after the wait: bwd_prepare counts on it
+    sm100::pdl_trigger();
     const int qt = blockIdx.x, tid = threadIdx.x;
-    // The blocks past the query tiles clear the fp32 sums that the backward adds to: memory is idle while
-    // the others wait for one dependent step after another, and a fill of its own is a launch that
-    // cannot overlap its neighbours (512 tokens, 4 heads: 48 -> 46 us a step; 3,128 tokens, 32 heads of
-    // 128: 220 -> 213 us).
+    // The blocks past the query tiles work on the side (PlanSide), while memory is idle and the others wait
+    // for one dependent step after another.  Clearing the fp32 sums that the backward adds to, as a fill of its
+    // own, is a launch that cannot overlap its neighbours (512 tokens, 4 heads: 48 -> 46 us a step; 3,128
+    // tokens, 32 heads of 128: 220 -> 213 us).
     if (qt >= p.n_qt) {
-        const size_t step = (size_t)(gridDim.x - p.n_qt) * PLAN_THREADS;
-        for (size_t i = (size_t)(qt - p.n_qt) * PLAN_THREADS + tid; i < zero_n4; i += step)
+        const int block = qt - p.n_qt, blocks = gridDim.x - p.n_qt;
+        float4 *zero = reinterpret_cast<float4 *>(side.zero);
+        for (size_t i = (size_t)block * PLAN_THREADS + tid; i < side.zero_n / 4; i += (size_t)blocks * PLAN_THREADS)
             zero[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if constexpr (PREP)
+            prepare_rows(p, side, block, blocks);
         return;
     }
     const int lane = tid & 31;
@@ -602,17 +659,21 @@ __global__ void k0_mask_dense(Plan p, RangeList ranges, uint8_t *out)
 }
 
 int launch_plan(const Plan &p, const int32_t *anchor, const int32_t *depth, int K, int seq_begin,
-                int seq_end, const RangeList &ranges, bool for_bwd, cudaStream_t s, float *zero, size_t zero_n)
+                int seq_end, const RangeList &ranges, bool for_bwd, cudaStream_t s, const PlanSide &side)
 {
     if (p.n_qt == 0)
         return 0;
     const int n_seq = seq_end - seq_begin;
     const int blocks = (n_seq + 127) / 128 > p.n_qt + p.n_kt ? (n_seq + 127) / 128 : p.n_qt + p.n_kt;
     launch_dependent(k0_tiles, blocks, 128, 0, s, p, anchor, depth, K, seq_begin, seq_end, ranges);
-    // 64 KB a block, and no more blocks than are resident beside the plan's own
-    const size_t clear = zero_n * 4 / 65536 + (zero_n > 0);
-    launch_dependent(k0_plan, p.n_qt + (unsigned)(clear < 256 ? clear : 256), PLAN_THREADS, 0, s, p, seq_begin,
-                     seq_end, for_bwd ? 1 : 0, reinterpret_cast<float4 *>(zero), zero_n / 4);
+    // A side block clears 64 KB or prepares 1,024 pieces of 8 elements, more where there are more than 256 or
+    // 1,184 blocks (the plan's own come first; four are resident on an SM).  Preparation of two partitions of
+    // 4,000 tokens, 64 heads of 64, with at most 296 / 444 / 592 / 1,184 blocks or any number: the case takes
+    // 747 / 730 / 734 / 729 / 729 us.
+    const size_t prep = side.O ? (size_t)p.n_qt * BM * side.Hq * (side.D / 8) : 0;
+    const size_t want = side.zero_n * 4 / 65536 + (side.zero_n > 0) + (prep + 1023) / 1024, most = side.O ? 1184 : 256;
+    launch_dependent(side.O ? k0_plan<true> : k0_plan<false>, p.n_qt + (unsigned)(want < most ? want : most),
+                     PLAN_THREADS, 0, s, p, seq_begin, seq_end, for_bwd ? 1 : 0, side);
     return 2;
 }
 

@@ -27,7 +27,7 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
 // this one, while with the trigger first all the kernels of a chain settle on the SMs at once and take
 // each other's places (512 tokens, 4 heads: 43 -> 40 us a step; 3,128 tokens, 32 heads of 128: 214 -> 205).
 // Every thread of every kernel calls pdl_wait before it touches global memory or leaves: a kernel that is
-// complete then implies that all before it are.  (One exception, with its reasons: bwd_prepare.)
+// complete then implies that all before it are.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -190,6 +190,26 @@ def test_rows_of_a_tensor_core_tile_that_see_nothing(ctx, D):
     assert not case.O[:64].any() and not case.dQ[:64].any()
 
 
+@pytest.mark.parametrize("heads", [(3, 1, 64), (8, 2, 128)], ids=str)
+def test_separate_backward_at_tile_remainders(ctx, heads):
+    """peagle_attn_bwd forms its rows' values beside the plan: partitions of one row, of a tile less one
+    row, of a tile and one row, and the rest."""
+    w = inputs.Workload("remainders", (150,), 2, *heads, seed=56)
+    case = DeviceCase(w)
+    case.parts = [{"seq": 0, "q": q, "k": [(0, 300)]} for q in ((0, 1), (1, 128), (128, 257), (257, 300))]
+    dK_acc = torch.zeros(case.T, w.n_kv_heads, w.head_dim, dtype=torch.float32, device="cuda")
+    dV_acc = torch.zeros_like(dK_acc)
+    for p in case.parts:
+        bp = binding.Partition(0, p["q"], p["k"])
+        binding.peagle_attn_fwd(ctx, case.prob, bp, case.dQ_, case.dK_, case.dV_, case.O, case.LSE)
+        binding.peagle_attn_bwd(ctx, case.prob, bp, case.dQ_, case.dK_, case.dV_, case.O, case.ddO, case.LSE,
+                                case.dQ, dK_acc, dV_acc)
+    binding.peagle_cast_grads(ctx, dK_acc, dV_acc, case.dK, case.dV)
+    assert binding.peagle_poll_status(ctx) == 0
+    O, LSE, dQ, dK, dV = oracle_all(case)
+    check_grads(case, dQ, dK, dV)
+
+
 def full_size_checks(case, n_rows=16, n_keys=6, seed=0):
     """Checks that hold at any size, plus outputs the oracle can compute one by one."""
     w = case.w
