@@ -201,7 +201,9 @@ bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
         // Keys past a ragged tile's end are another range's, often another sequence's.  Their sums have weight
         // zero throughout, but a zero times an Inf or NaN of a row of Q or dO is not zero, so zeros are
         // what they get.  (The item is read again: carried through its steps these words would be
-        // spilled; see the queue for why the slot still holds it.)
+        // spilled; see the queue for why the slot still holds it.  A warp none of whose rows are the tile's
+        // sends its zeros too: a branch around it costs 44 bytes of spills and 2 of 76 us at 391 positions,
+        // 32 heads.)
         const BwdItem &done = *reinterpret_cast<const BwdItem *>(wq + (w & 3) * sizeof(BwdItem));
         const int k_start = done.k_start, g = done.g;
         const int rows = done.k_len - (warp & 3) * 32; // of this warp's 32 keys, how many are the tile's
@@ -220,8 +222,7 @@ bwd128_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ C
                     o[i] = 0;
             }
             const bool k = pn < 4;
-            if (rows > 0)
-                send(o, k ? P.scale : 1.f, pn & 1, k ? &tmDK : &tmDV, 32 * (pn % 4), g, k_start);
+            send(o, k ? P.scale : 1.f, pn & 1, k ? &tmDK : &tmDV, 32 * (pn % 4), g, k_start);
         }
         }
         if (lane == 0)
