@@ -120,14 +120,13 @@ void carve_plan(Plan &p, void *base, size_t *bytes_out)
     p.ksum = c.take<int4>(2 * nk);
     p.ksplit = c.take<int>(nk);
     p.cls = c.take<uint8_t>(nq * nk);
-    p.undecided = c.take<int>(nq * nk);
     p.counters = c.take<int>(PLAN_COUNTERS);
     p.klist = c.take<int2>(nq * nk);
     p.kcount = c.take<int>(nq);
     p.qorder = c.take<int>(nq);
     const size_t nch = (nq + BWD_CQ - 1) / BWD_CQ;
     p.cdone = c.take<int>(nch);
-    p.bitems = c.take<int4>(BWD_CQ * nch * nk);
+    p.bitems = c.take<int2>(BWD_CQ * nch * nk);
     p.scount = c.take<int>(nq);
     p.scs = c.take<uint8_t>(nq * MAX_SINGLE * BM);
     p.sbase = c.take<int>(nq * MAX_SINGLE);

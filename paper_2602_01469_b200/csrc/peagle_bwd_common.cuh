@@ -7,7 +7,7 @@ namespace peagle {
 
 struct BwdParams {
     const int2 *ktile;
-    const int4 *bitems;
+    const int2 *bitems;
     const int *counters;
     int *cursor; // device counter, zero at launch: next (work item, KV head) index to hand out
     const int32_t *meta;
@@ -113,8 +113,8 @@ __device__ __forceinline__ bool bwd_draw(const BwdParams &P, const BwdSplit &sp,
                 at -= sp.count[i];
             }
         }
-        const int4 item = P.bitems[base];
-        unsigned mask = (unsigned)item.z;
+        const int2 item = P.bitems[base];
+        unsigned mask = item_mask(item);
         if (sp.tiles > 1)
             mask &= 0x101u << tile;
         if ((mask & 0xffu) == 0)
@@ -123,7 +123,7 @@ __device__ __forceinline__ bool bwd_draw(const BwdParams &P, const BwdSplit &sp,
         out.g = ig % P.Hkv;
         out.k_start = kt.x;
         out.k_len = kt.y;
-        out.qt0 = item.y * BWD_CQ;
+        out.qt0 = item_chunk(item) * BWD_CQ;
         out.mask = mask;
         out.h0 = out.g * G + part * sp.nh;
         out.nh = min(sp.nh, G - part * sp.nh);

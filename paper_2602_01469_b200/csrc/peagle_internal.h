@@ -16,8 +16,8 @@ constexpr int MAX_KRANGES = 32;  // visible key ranges per partition
 #ifndef PEAGLE_BWD_CQ
 #define PEAGLE_BWD_CQ 4 // measured: 2 / 4 / 8 give 3.33 / 3.27 / 3.38 ms for the head_dim 64 main kernel
 #endif
-constexpr int BWD_CQ = PEAGLE_BWD_CQ; // query tiles per backward work item (aligned chunk; at most 8)
-static_assert(BWD_CQ >= 1 && BWD_CQ <= 8, "the chunk's mask word has eight bits per field");
+constexpr int BWD_CQ = PEAGLE_BWD_CQ; // query tiles per backward work item (aligned chunk; at most 4)
+static_assert(BWD_CQ >= 1 && BWD_CQ <= 4, "pack_item has four bits per field");
 constexpr int32_t META_NONE_Q = -1;         // packed metadata of a row outside the partition (sees nothing)
 constexpr int32_t META_NONE_K = 0x7fffffff; // packed metadata of a key outside the batch (seen by nobody)
 
@@ -51,14 +51,13 @@ struct Plan {
     int4 *ksum;            // [n_kt][2]
     int *ksplit;           // [n_kt] keys in the first run, flags for sorted runs
     uint8_t *cls;          // [n_qt][n_kt] tile classes
-    int *undecided;        // [n_qt][n_kt] key tiles that a query tile's quick test could not decide
     int *counters;         // [PLAN_COUNTERS] device counters, zero before k0_plan: CNT_*
     int *cdone;            // [n_ch] query tiles of a chunk that are classified
     int2 *klist;           // [n_qt][n_kt] compact non-skip key tiles per query tile: (first token, len | cls<<16)
     int *kcount;           // [n_qt]
     int *qorder;           // [n_qt] query tiles, most key tiles first (no order among about equal ones)
-    int4 *bitems;          // [BWD_CQ][n_ch * n_kt] backward work items by size (1 .. BWD_CQ query tiles):
-                           // (key tile, chunk, mask word, query tiles); counters[CNT_ITEMS + size - 1] of each
+    int2 *bitems;          // [BWD_CQ][n_ch * n_kt] backward work items by size (1 .. BWD_CQ query tiles):
+                           // packed by pack_item; counters[CNT_ITEMS + size - 1] of each
     int allow_single;      // 1: the kernels of this shape take SINGLE tiles pair by pair
     int *scount;           // [n_qt] SINGLE entries per query tile (at most MAX_SINGLE): windows of 128 keys,
                            // ascending, in which every query row has at most one key
@@ -69,6 +68,16 @@ struct Plan {
                            // tiles that add to the same key rows run close together in time
     int *status;           // device status word
 };
+
+// A backward work item in two words: key tile; chunk of query tiles << 8 | which of them are FULL << 4 | which
+// take part.  (A plan has BWD_CQ places per key tile and chunk for them, and grows with the square of the
+// length.)  `mask`: bit b, query tile b of the chunk takes part; bit 8 + b, it is FULL.
+__device__ __forceinline__ int2 pack_item(int key_tile, int chunk, unsigned mask)
+{
+    return make_int2(key_tile, (int)((unsigned)chunk << 8 | (mask >> 8 & 15u) << 4 | (mask & 15u)));
+}
+__device__ __forceinline__ int item_chunk(int2 item) { return (int)((unsigned)item.y >> 8); }
+__device__ __forceinline__ unsigned item_mask(int2 item) { return ((unsigned)item.y & 15u) | ((unsigned)item.y >> 4 & 15u) << 8; }
 
 struct FwdArgs {
     const void *Q, *K, *V;

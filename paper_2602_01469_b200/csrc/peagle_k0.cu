@@ -337,7 +337,8 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
     }
     const int lane = tid & 31;
     uint8_t *cls = p.cls + (size_t)qt * p.n_kt;
-    int *undecided = p.undecided + (size_t)qt * p.n_kt;
+    // kept where the query tile's key list will be, which is written when they are done with
+    int *undecided = reinterpret_cast<int *>(p.klist + (size_t)qt * p.n_kt);
     if (tid == 0) {
         n_undecided = 0;
         n_raw = 0;
@@ -603,7 +604,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
                 if (mm) {
                     const int sz = __popc(mm & 0xffu);
                     const int at = atomicAdd(&hist[BWD_CQ + sz - 1], 1);
-                    p.bitems[(size_t)(sz - 1) * cap + at] = make_int4(kt, c, (int)mm, sz);
+                    p.bitems[(size_t)(sz - 1) * cap + at] = pack_item(kt, c, mm);
                 }
             }
         }

@@ -82,6 +82,29 @@ def test_more_chain_tiles_than_places_repeat_bit_for_bit(ctx, n, K):
     check_forward(case.O.float().cpu().numpy(), case.LSE.t().cpu().numpy(), O, LSE)
 
 
+def test_plan_scratch_per_tile_pair():
+    """What grows with the square of the length: class (1 byte), key list (8) and backward items (8) per pair
+    of tiles.  A context keeps an eighth more than it needs, and the allocator rounds up to 2 MB."""
+    n = 1 << 17
+    Q = torch.randn(n, 1, 64, device="cuda").bfloat16()
+    K, V, O, LSE = torch.randn_like(Q), torch.randn_like(Q), torch.empty_like(Q), torch.empty(1, n, device="cuda")
+    anchor = torch.arange(n, dtype=torch.int32, device="cuda")
+    depth = torch.zeros_like(anchor)
+    own = binding.Context(0)
+
+    def forward(m):
+        prob = binding.Problem(np.array([0, m], np.int32), anchor, depth, 1, 1, 1, 64, 0.125)
+        binding.peagle_attn_fwd(own, prob, binding.Partition(0, (0, m), None), Q, K, V, O, LSE)
+        assert binding.peagle_poll_status(own) == 0
+        return torch.cuda.mem_get_info()[0]
+
+    used = forward(128) - forward(n)
+    own.close()
+    pairs = (n // 128) ** 2
+    linear = n * 4 + n // 128 * (2 * 32 + 2 * 32 + 16 * 128 + 16 * 4 + 64)   # metadata, summaries, SINGLE entries
+    assert used <= 1.125 * (17.5 * pairs + linear) + (4 << 20)
+
+
 def test_more_query_tiles_than_threads(ctx):
     case = DeviceCase(inputs.Workload("long", (8300,), 8, 2, 1, 64, seed=45))
     run_partitioned(ctx, case)
