@@ -723,7 +723,7 @@ static int run_partitions(peagle_ctx *ctx, const peagle_problem_t *prob,
                           void *dQ, float *dK_acc, float *dV_acc, cudaStream_t s, bool clear)
 {
     // Up to 32 MB the plan of the first partition that has rows clears the sums on the side (12.8 MB: 7 us
-    // of a step of 220, 0.3 MB: 2 of 48); above, a fill at memory speed takes longer than the plan, and
+    // of a step of 220, 0.3 MB: 1 of 46); above, a fill at memory speed takes longer than the plan, and
     // the two together as long as one after the other (67 MB: 41 against 20 + 23 us).
     constexpr size_t SIDE_CLEAR = 8 << 20; // floats
     size_t zero_n = clear ? 2 * (size_t)prob->total_tokens * prob->n_kv_heads * prob->head_dim : 0;
@@ -1115,7 +1115,7 @@ int peagle_attn_partitioned_host(peagle_ctx *ctx, const peagle_problem_t *prob,
     // slice k - 1 is computed meanwhile.  Left to start when they may, the two directions fall out of step
     // and each copy takes 10-15 % longer with a pause of 40 us before the next (copies of 268 MB each way
     // around a kernel of 100 us a slice: 7.15 ms free running, 6.11 in step; by 8 MB and by 32 MB of each
-    // slice 6.18 and 6.54).  2,048 positions, 64 / 8 heads of 64: 8.3 -> 7.5 ms a step (8 MB slices the
+    // slice 6.18 and 6.54).  2,048 positions, 64 / 8 heads of 64: 7.8 -> 7.5 ms a step (8 MB slices the
     // same, 32 MB 7.9; 16 MB is worse for short examples, which have few slices).
     constexpr int64_t SLICE_BYTES = 12 << 20;
     const int64_t fit = SLICE_BYTES / (int64_t)(2 * row_q * BM);

@@ -658,8 +658,6 @@ static int launch_bwd_t(const Plan &p, const BwdArgs &a, EncodeTiledFn enc, int 
         P.n_qt = p.n_qt;
         P.n_kt = p.n_kt;
         P.q_begin = p.q_begin;
-        P.q_end = p.q_end;
-        P.T = p.T;
         P.nl2 = a.nl2;
         P.nd = a.nd;
         P.mqp = a.mqp;

@@ -12,10 +12,13 @@ struct BwdParams {
     int *cursor; // device counter, zero at launch: next (work item, KV head) index to hand out
     const int32_t *meta;
     int *status;
-    int n_qt, n_kt, q_begin, q_end, T;
+    int n_qt, n_kt, q_begin;
     const float *nl2, *nd; // [Hq][q_pad] -LSE*log2(e) and -Delta, padded rows (-inf, 0)
     const int32_t *mqp;    // [q_pad] packed metadata of the partition's rows
     int q_pad;             // n_qt * BM
+    // The sums' addresses are in the tensor maps and no kernel reads these.  They stay because of the
+    // compiler: without them it spills 20 bytes more in bwd64_kernel, in the wrong place (4,096 positions, 64
+    // heads of 64: 3.10 -> 3.31 ms).
     float *dq_acc;         // [q_len][Hq][D]
     float *dK_acc, *dV_acc;
     int Hq, Hkv;

@@ -52,9 +52,8 @@ struct FwdParams {
     float scale_log2;
     // SINGLE tiles (one allowed key per row), handled pair by pair before the tile loop
     const int *scount;
-    const uint8_t *scs;  // [n_qt][MAX_SINGLE][BM] key column of entry i for row r, or NO_COL
-    const int *sbase;    // [n_qt][MAX_SINGLE] first token of entry i's key tile
-    const __nv_bfloat16 *Q, *K, *V;
+    const uint8_t *scs;  // [n_qt][MAX_SINGLE][BM] key of row r in entry i's window, or NO_COL
+    const int *sbase;    // [n_qt][MAX_SINGLE] first token of entry i's window
     // Optional hand-over to the backward of the same partition (the driver knows dO when the
     // forward runs): per (head, row) -LSE * log2(e) and -Delta = -<dO, O>, [Hq][q_pad] each, and
     // the rows' packed metadata [q_pad], neutral values for the rows past the partition's end.
@@ -63,23 +62,6 @@ struct FwdParams {
     int32_t *mqp;
     int q_pad;
 };
-
-// <a, b> of two rows of 64 bf16 held as 32 packed pairs; products are exact in fp32.
-__device__ __forceinline__ float dot64_bf16(const uint32_t (&a)[32], const uint4 *b)
-{
-    float acc = 0.f;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const uint4 v = b[i];
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            acc = fmaf(__uint_as_float(a[4 * i + k] << 16), __uint_as_float(w[k] << 16), acc);
-            acc = fmaf(__uint_as_float(a[4 * i + k] & 0xffff0000u), __uint_as_float(w[k] & 0xffff0000u), acc);
-        }
-    }
-    return acc;
-}
 
 template <int D>
 struct FwdCfg {
@@ -1040,9 +1022,6 @@ static int launch_fwd_t(const Plan &p, const FwdArgs &a, EncodeTiledFn enc, int 
     P.nd = a.nd;
     P.mqp = a.mqp;
     P.q_pad = p.n_qt * BM;
-    P.Q = static_cast<const __nv_bfloat16 *>(a.Q);
-    P.K = static_cast<const __nv_bfloat16 *>(a.K);
-    P.V = static_cast<const __nv_bfloat16 *>(a.V);
     // the attribute belongs to the current device's copy of the function: set before every launch
     // (host time only), so that a process that drives several GPUs gets it on each of them
     if (cudaFuncSetAttribute(fwd_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,

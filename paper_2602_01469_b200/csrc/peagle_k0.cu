@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
     const int qt = blockIdx.x, tid = threadIdx.x;
     // The blocks past the query tiles work on the side (PlanSide), while memory is idle and the others wait
     // for one dependent step after another.  Clearing the fp32 sums that the backward adds to, as a fill of its
-    // own, is a launch that cannot overlap its neighbours (512 tokens, 4 heads: 48 -> 46 us a step; 3,128
+    // own, is a launch that cannot overlap its neighbours (512 tokens, 4 heads: 46.2 -> 45.1 us a step; 3,128
     // tokens, 32 heads of 128: 220 -> 213 us).
     if (qt >= p.n_qt) {
         const int block = qt - p.n_qt, blocks = gridDim.x - p.n_qt;

@@ -34,7 +34,7 @@ struct SingleParams {
     __nv_bfloat16 *dQ;
     float *dK_acc, *dV_acc;
     int *status;
-    int q_begin, q_end, q_pad, n_qt, Hq, Hkv, T, rows_per_block;
+    int q_begin, q_end, q_pad, Hq, Hkv, rows_per_block;
     float scale, scale_log2;
 };
 
@@ -342,10 +342,8 @@ int launch_finish_single(const Plan &p, const BwdArgs &a, cudaStream_t s)
     P.q_begin = p.q_begin;
     P.q_end = p.q_end;
     P.q_pad = p.n_qt * BM;
-    P.n_qt = p.n_qt;
     P.Hq = a.Hq;
     P.Hkv = a.Hkv;
-    P.T = p.T;
     P.scale = a.scale;
     P.scale_log2 = a.scale * 1.4426950408889634f;
     P.status = p.status;

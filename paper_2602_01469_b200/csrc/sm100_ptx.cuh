@@ -187,14 +187,6 @@ __device__ __forceinline__ void tma_reduce_add_2d(const CUtensorMap *m, uint32_t
         "r"(src), "r"(x), "r"(y)
         : "memory");
 }
-// Bulk reduce-add of fp32 from shared to global memory (both 16-byte aligned, size % 16 == 0).
-__device__ __forceinline__ void bulk_reduce_add_f32(void *gdst, uint32_t ssrc, uint32_t bytes)
-{
-    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(
-                     reinterpret_cast<uint64_t>(gdst)),
-                 "r"(ssrc), "r"(bytes)
-                 : "memory");
-}
 __device__ __forceinline__ void bulk_commit_group()
 {
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
@@ -296,25 +288,6 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
 }
 
 // ------------------------------------------------------------------ MMA descriptors
-// Shared-memory matrix descriptor for a bf16 tile stored as 128-byte rows with the 128-byte
-// swizzle (what a TMA load with CU_TENSOR_MAP_SWIZZLE_128B of a 64-element-wide box produces;
-// the tile base must be 1024-byte aligned).
-//   K-major operand  (rows = M or N index, the 64 elements of a row run along K):
-//       sbo = 1024 (distance between 8-row groups), lbo unused.
-//   MN-major operand (rows = K index, the 64 elements of a row run along M or N):
-//       sbo = 1024 (distance between 8-row K groups), lbo = distance between 64-wide panels.
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr, uint32_t lbo_bytes,
-                                                    uint32_t sbo_bytes)
-{
-    uint64_t d = 0;
-    d |= static_cast<uint64_t>((addr & 0x3FFFFu) >> 4);
-    d |= static_cast<uint64_t>((lbo_bytes >> 4) & 0x3FFFu) << 16;
-    d |= static_cast<uint64_t>((sbo_bytes >> 4) & 0x3FFFu) << 32;
-    d |= 1ull << 46; // descriptor version for sm_100
-    d |= 2ull << 61; // 128-byte swizzle
-    return d;
-}
-
 // Instruction descriptor for kind::f16 with bf16 inputs and fp32 accumulation.
 // a_mn / b_mn: 1 when that operand is MN-major (transposed), 0 when K-major.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, int a_mn, int b_mn)
@@ -324,29 +297,6 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, int a_mn, in
            | (1u << 10)                    // B format: BF16
            | (static_cast<uint32_t>(a_mn) << 15) | (static_cast<uint32_t>(b_mn) << 16) |
            (static_cast<uint32_t>(N >> 3) << 17) | (static_cast<uint32_t>(M >> 4) << 24);
-}
-
-// D[tmem] (+)= A[smem] * B[smem]; one thread issues.
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                       uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// D[tmem] (+)= A[tmem] * B[smem]; A is bf16 packed two per 32-bit column, lanes = M rows.
-__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
-                                       uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
 }
 
 // ------------------------------------------------------------------ register re-allocation
@@ -444,6 +394,9 @@ __device__ __forceinline__ F2 add_f2(F2 a, F2 b)
 // build.  With the stride field fixed at 1024 bytes the upper word of a 128-byte-swizzle
 // descriptor is a constant, and the lower word is (address >> 4) | (lbo >> 4) << 16, so moving an
 // operand by `bytes` inside shared memory is one 32-bit add of bytes >> 4.
+// The tile is stored as 128-byte rows with the 128-byte swizzle (a TMA load of a box 64 elements wide with
+// CU_TENSOR_MAP_SWIZZLE_128B, base 1024-byte aligned).  K-major operand (rows = M or N index): lbo unused.
+// MN-major operand (rows = K index): lbo = distance between 64-wide panels.
 constexpr uint32_t DESC_HI_SW128 = (1024u >> 4) | (1u << 14) | (2u << 29);
 __device__ __forceinline__ uint32_t desc_lo_sw128(uint32_t addr, uint32_t lbo_bytes)
 {
@@ -486,45 +439,6 @@ __device__ __forceinline__ uint32_t elect_one()
     uint32_t r;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
     return r;
-}
-
-// The same for a whole, converged warp: every lane carries the (warp-uniform) operands and only
-// the lane with `lead` != 0 issues.  Keeping the issuing warp converged lets the compiler do the
-// descriptor arithmetic once per warp in the uniform datapath, where the instruction wants its
-// operands, instead of per lane with a transfer in front of every product.
-__device__ __forceinline__ void mma_ss_lo_w(uint32_t lead, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo,
-                                            uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "setp.ne.b32 q, %6, 0;\n\t"
-        "mov.b64 da, {%1, %5};\n\t"
-        "mov.b64 db, {%2, %5};\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),
-        "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(DESC_HI_SW128), "r"(lead)
-        : "memory");
-}
-__device__ __forceinline__ void mma_ts_lo_w(uint32_t lead, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo,
-                                            uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t.reg .b64 db;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "setp.ne.b32 q, %6, 0;\n\t"
-        "mov.b64 db, {%2, %5};\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, p;\n\t}" ::"r"(d_tmem),
-        "r"(a_tmem), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(DESC_HI_SW128), "r"(lead)
-        : "memory");
-}
-__device__ __forceinline__ void tc_commit_w(uint32_t lead, uint32_t bar)
-{
-    asm volatile(
-        "{\n\t.reg .pred q;\n\t"
-        "setp.ne.b32 q, %1, 0;\n\t"
-        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar),
-        "r"(lead)
-        : "memory");
 }
 
 // 16 lanes x (8 * 8) columns of 32-bit: register 4i+j of thread t holds lane t/4 + 8*(j/2),
@@ -581,11 +495,6 @@ __device__ __forceinline__ void stmatrix_x4(uint32_t addr, uint32_t a, uint32_t 
                  "r"(c), "r"(d)
                  : "memory");
 }
-__device__ __forceinline__ void red_add_v2(float *p, float a, float b)
-{
-    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
-}
-
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
 {
     uint32_t r;
@@ -606,22 +515,10 @@ __device__ __forceinline__ float max3(float a, float b, float c)
     return r;
 }
 
-// 2^x on the FMA pipe, for taking load off the exp2 unit (16 results per clock per SM): round x
+// 2^x of a pair on the FMA pipe, for taking load off the exp2 unit (16 results per clock per SM): round x
 // to the nearest integer n with the 1.5 * 2^23 trick, a cubic for 2^(x - n) on [-0.5, 0.5]
 // (relative error < 8e-5, far below the bf16 rounding the probabilities get anyway), n added to
 // the exponent field.  x <= 126; anything below -126 is clamped (result ~1e-38 instead of 0).
-__device__ __forceinline__ float exp2_fma(float x)
-{
-    x = fmaxf(x, -126.f);
-    const float xr = x + 12582912.f;
-    const float f = x - (xr - 12582912.f);
-    float p = fmaf(f, 0.05508868f, 0.24260405f);
-    p = fmaf(p, f, 0.69327623f);
-    p = fmaf(p, f, 0.99992895f);
-    return __int_as_float(__float_as_int(p) + (__float_as_int(xr) << 23));
-}
-
-// The same on a pair.
 __device__ __forceinline__ F2 exp2_fma2(F2 x)
 {
     const float2 c = unf2(x);
