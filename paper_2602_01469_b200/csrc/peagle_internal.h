@@ -14,7 +14,7 @@ constexpr int BM = 128;          // query rows per tile
 constexpr int BN = 128;          // keys per tile
 constexpr int MAX_KRANGES = 32;  // visible key ranges per partition
 #ifndef PEAGLE_BWD_CQ
-#define PEAGLE_BWD_CQ 4 // measured: 2 / 4 / 8 give 3.33 / 3.27 / 3.38 ms for the head_dim 64 main kernel
+#define PEAGLE_BWD_CQ 4 // 2 / 3 / 4: bwd64_kernel 3.03 / 3.00 / 3.01 ms at 4,096 positions, 22.1 / 21.8 / 21.6 at 11,008
 #endif
 constexpr int BWD_CQ = PEAGLE_BWD_CQ; // query tiles per backward work item (aligned chunk; at most 4)
 static_assert(BWD_CQ >= 1 && BWD_CQ <= 4, "pack_item has four bits per field");

@@ -337,8 +337,8 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
     }
     const int lane = tid & 31;
     uint8_t *cls = p.cls + (size_t)qt * p.n_kt;
-    // kept where the query tile's key list will be, which is written when they are done with
-    int *undecided = reinterpret_cast<int *>(p.klist + (size_t)qt * p.n_kt);
+    int2 *klist = p.klist + (size_t)qt * p.n_kt;
+    int *undecided = reinterpret_cast<int *>(klist); // done with when the key list is written
     if (tid == 0) {
         n_undecided = 0;
         n_raw = 0;
@@ -554,7 +554,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
         p.n_kt, warp_cnt, [&](int kt) { const uint8_t c = cls[kt]; return c != TILE_SKIP && c != TILE_SINGLE; },
         [&](int kt, int at) {
             const int2 k = p.ktile[kt];
-            p.klist[(size_t)qt * p.n_kt + at] = make_int2(k.x, k.y | ((int)cls[kt] << 16));
+            klist[at] = make_int2(k.x, k.y | ((int)cls[kt] << 16));
         });
     if (tid == 0)
         p.kcount[qt] = listed;
