@@ -499,16 +499,30 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                         p[hf][c + 1] = fast_exp2(a1);
                     }
             if (!full) {
+                // Where each of the warp's keys is a depth-0 token that all of its rows follow, nothing is
+                // masked: so for six of the sixteen 32 x 32 blocks of a diagonal tile.
+                int4 mq[2];
 #pragma unroll
-                for (int m = 0; m < 2; ++m) {
-                    const int4 mq = mq4[4 * m];
+                for (int m = 0; m < 2; ++m)
+                    mq[m] = mq4[4 * m];
+                int first = mq[0].x;
 #pragma unroll
-                    for (int hf = 0; hf < 2; ++hf)
+                for (int m = 0; m < 2; ++m)
+                    first = min(min(first, min(mq[m].x, mq[m].y)), min(mq[m].z, mq[m].w));
+                const int last = max(max(mk[0], mk[1]), max(mk[2], mk[3]));
+                if (!__all_sync(0xffffffffu, last <= first && ((mk[0] | mk[1] | mk[2] | mk[3]) & 0xff) == 0)) {
 #pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            if (!allowed_packed(e < 4 ? ((e & 1) ? mq.y : mq.x) : ((e & 1) ? mq.w : mq.z),
-                                                mk[2 * hf + ((e >> 1) & 1)]))
-                                p[hf][8 * m + e] = 0.f;
+                    for (int k = 0; k < 4; ++k) {
+                        const uint32_t span = allowed_span(mk[k]);
+#pragma unroll
+                        for (int m = 0; m < 2; ++m)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) { // column 16m + 8 (e / 2) + 2 (lane % 4) + e % 2
+                                const int row = e < 2 ? (e == 0 ? mq[m].x : mq[m].y) : (e == 2 ? mq[m].z : mq[m].w);
+                                if ((uint32_t)(row - mk[k]) > span)
+                                    p[k >> 1][8 * m + 4 * (e >> 1) + 2 * (k & 1) + (e & 1)] = 0.f;
+                            }
+                    }
                 }
             }
 #pragma unroll

@@ -31,6 +31,15 @@ constexpr int CNT_BWD_CURSOR = 2, CNT_FWD_CURSOR = 3, CNT_DONE = 4, CNT_ITEMS = 
 static_assert(CNT_ITEMS + BWD_CQ <= PLAN_COUNTERS, "a counter per item size");
 constexpr int NO_COL = 255;      // "this row allows no key of the tile"
 
+// Second word of a key list entry: bits 0-7 length, 8-15 keys in the first run of equal depth, 16-17 class; bit
+// KLIST_RUN0 / KLIST_RUN1: the run's keys are depth-0 tokens; bit KLIST_RUNS: each run is in ascending order and
+// all depth 0 or all deeper, so that the keys of a run which a row allows are neighbours; bit KLIST_EVEN: and the
+// anchors of a run follow one another.  (The bits above the class only where it is PARTIAL.)
+constexpr int KLIST_RUN0 = 1 << 24, KLIST_RUN1 = 1 << 25, KLIST_RUNS = 1 << 26, KLIST_EVEN = 1 << 27;
+__device__ __forceinline__ int klist_len(int word) { return word & 0xff; }
+__device__ __forceinline__ int klist_split(int word) { return word >> 8 & 0xff; }
+__device__ __forceinline__ int klist_class(int word) { return word >> 16 & 3; }
+
 // Visible key ranges of one call, passed to kernels by value.
 struct RangeList {
     int n;
@@ -53,7 +62,7 @@ struct Plan {
     uint8_t *cls;          // [n_qt][n_kt] tile classes
     int *counters;         // [PLAN_COUNTERS] device counters, zero before k0_plan: CNT_*
     int *cdone;            // [n_ch] query tiles of a chunk that are classified
-    int2 *klist;           // [n_qt][n_kt] compact non-skip key tiles per query tile: (first token, len | cls<<16)
+    int2 *klist;           // [n_qt][n_kt] compact non-skip key tiles per query tile: (first token, KLIST_* word)
     int *kcount;           // [n_qt]
     int *qorder;           // [n_qt] query tiles, most key tiles first (no order among about equal ones)
     int2 *bitems;          // [BWD_CQ][n_ch * n_kt] backward work items by size (1 .. BWD_CQ query tiles):
@@ -199,6 +208,12 @@ int launch_gemm(EncodeTiledFn enc, const void *A, long long lda, int a_t, const 
 __host__ __device__ inline bool allowed_packed(int32_t mq, int32_t mk)
 {
     return (mk <= mq) && (((mk & 0xff) == 0) || ((mk ^ mq) < 256));
+}
+// The same as an interval: key mk is seen by the rows mk .. mk + allowed_span(mk), a subtraction and an
+// unsigned comparison per pair.
+__host__ __device__ inline uint32_t allowed_span(int32_t mk)
+{
+    return (mk & 0xff) == 0 ? (uint32_t)(0x7fffffff - mk) : (uint32_t)(255 - (mk & 0xff));
 }
 
 } // namespace peagle
