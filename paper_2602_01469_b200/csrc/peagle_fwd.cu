@@ -24,8 +24,7 @@
 // P from tensor memory and V from shared memory (MN-major).
 // Only tiles the classifier kept are visited; FULL tiles skip the per-element predicate; SINGLE
 // tiles (one allowed key per row) pass through the same ring first and are done pair by pair on
-// the CUDA cores, their result seeding the running (m, l, O): O in registers at head_dim 64, in
-// tensor memory at head_dim 128.
+// the CUDA cores, their result seeding the running (m, l, O).
 #include <math_constants.h>
 
 #include <algorithm>
@@ -77,13 +76,17 @@ struct FwdCfg {
     // warp); head_dim 128 has no room for the two staging tiles and stores its rows directly
     static constexpr bool O_STAGED = (D == 64);
     static constexpr int OFF_OST = OFF_V + NS * TILE_BYTES;
-    // 128 x 32 fp32 zeros, the source of the stores that clear the backward's dQ staging
+    // ZERO_ROWS x 32 fp32 zeros, the source of the stores that clear the backward's dQ staging
+    static constexpr int ZERO_ROWS = (D == 64) ? 128 : 64;
     static constexpr int OFF_ZERO = OFF_OST + (O_STAGED ? 2 * TILE_BYTES : 0);
-    static constexpr int OFF_META = OFF_ZERO + PANEL_BYTES;
+    // SINGLE entries of the item: the rows' keys [entry][row], the scores [entry][thread]
+    static constexpr int OFF_COL = OFF_ZERO + ZERO_ROWS * 128;
+    static constexpr int OFF_SCORE = OFF_COL + MAX_SINGLE * BM;
+    static constexpr int OFF_META = OFF_SCORE + MAX_SINGLE * 256 * 4;
     static constexpr int OFF_BAR = OFF_META + NS * BN * 4;
     static constexpr int N_BAR = 1 + 4 * NS + 10 + 9 + 8;
-    static constexpr int OFF_MISC = OFF_BAR + N_BAR * 8; // tmem slot, abort flag, item queue
-    static constexpr int SMEM_BYTES = OFF_MISC + 32 + 1024; // + slack for 1024-byte alignment
+    static constexpr int OFF_MISC = (OFF_BAR + N_BAR * 8 + 15) / 16 * 16; // tmem slot, abort flag; item queue
+    static constexpr int SMEM_BYTES = OFF_MISC + 16 + 4 * 16 + 1024;      // + slack for 1024-byte alignment
     static constexpr int TM_S = 0;      // S_A at 0, S_B at 128
     static constexpr int TM_O = 256;    // O_A at 256, O_B at 256 + D
     // head_dim 64 leaves 128 columns for the bf16 probabilities (64 columns per tile), so the next
@@ -163,6 +166,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     using C = FwdCfg<D>;
     constexpr int NS = C::NS;
     constexpr bool TURNS = D == 128;
+    constexpr int STAGE_ARRIVALS = 4;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t sb = (raw + 1023u) & ~1023u;
@@ -178,40 +182,25 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                   B_WQFREE = B_WQFULL + 4, B_QEMPTY = B_WQFREE + 4, B_TURN = B_QEMPTY + 1;
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(sp + C::OFF_MISC);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(sp + C::OFF_MISC + 4);
-    volatile int *wq = reinterpret_cast<volatile int *>(sp + C::OFF_MISC + 8); // 4 slots
+    int4 *wq = reinterpret_cast<int4 *>(sp + C::OFF_MISC + 16); // 4 slots
     int32_t *smeta = reinterpret_cast<int32_t *>(sp + C::OFF_META);
 
     // The warp index read through a shuffle is a value the compiler knows to be the same in every
     // lane, so what depends on it (tensor-memory addresses, barrier addresses) moves to the uniform
-    // datapath.  Measured, not reasoned: head_dim 128 0.508 -> 0.482 ms, head_dim 64 1.82 -> 1.89 ms.
-    const int warp = D == 128 ? __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0) : (int)(threadIdx.x >> 5);
+    // datapath.  Measured, not reasoned: 3,891 positions, 64 heads of 64, 1,794 -> 1,675 us without it and with.
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
     const int lane = threadIdx.x & 31;
     const int ntile = P.two ? 2 : 1;
     const int n_hb = P.two ? P.Hq / 2 : P.Hq;
     // Work item w of this CTA = (query tile, head block), handed out by a global counter in the
     // order of the schedule (query tiles with the most key tiles first).  The producer warp draws
-    // the index and passes it to the other roles through a four-slot queue in shared memory.
-    struct Item {
-        int qt, h0, g, row0, cnt, n_single;
-        const int2 *klist;
-    };
-    auto decode = [&](int idx) {
-        Item it;
-        it.qt = P.qorder[idx / n_hb];
-        const int hb = idx % n_hb;
-        it.h0 = P.two ? 2 * hb : hb;
-        it.g = it.h0 / (P.Hq / P.Hkv);
-        it.row0 = P.q_begin + it.qt * BM;
-        it.cnt = P.kcount[it.qt];
-        it.klist = P.klist + (size_t)it.qt * P.n_kt;
-        // the result of the SINGLE entries seeds (m, l, O) of the tile loop
-        it.n_single = P.scount[it.qt];
-        return it;
-    };
-    // Roles other than the producer: index of item w, or -1 at the end (or when a wait ran out).
+    // the index, looks the item up and passes it to the other roles through a four-slot queue in shared
+    // memory: query tile (negative: no more items), head block, key tiles, SINGLE entries.
+    const int heads = ntile; // of a block
+    // Roles other than the producer: item w, query tile -1 at the end (or when a wait ran out).
     auto take = [&](int w) {
         const int slot = w & 3;
-        return mbar_wait_warp(BAR(B_WQFULL + slot), (w >> 2) & 1, abort_flag) ? wq[slot] : -1;
+        return mbar_wait_warp(BAR(B_WQFULL + slot), (w >> 2) & 1, abort_flag) ? wq[slot] : make_int4(-1, 0, 0, 0);
     };
 
     if (threadIdx.x == 0) {
@@ -219,9 +208,12 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         mbar_init(BAR(B_QFULL), 1);
         for (int s = 0; s < NS; ++s) {
             mbar_init(BAR(B_KFULL + s), 1);
-            mbar_init(BAR(B_KEMPTY + s), P.two ? 2 : 1); // one commit per MMA-issuing thread
+            // a stage is free when, for each tile, a commit of the issuing warp and STAGE_ARRIVALS more
+            // have arrived: for a key tile the issuing warp's own, for a SINGLE entry one per softmax
+            // warp (and the issuing warp, which only has to see the phase pass, in place of the commit)
+            mbar_init(BAR(B_KEMPTY + s), ntile * (1 + STAGE_ARRIVALS));
             mbar_init(BAR(B_VFULL + s), 1);
-            mbar_init(BAR(B_VEMPTY + s), P.two ? 2 : 1);
+            mbar_init(BAR(B_VEMPTY + s), ntile * (1 + STAGE_ARRIVALS));
         }
         for (int x = 0; x < 2; ++x) {
             mbar_init(BAR(B_SFULL + x), 1);
@@ -237,7 +229,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             mbar_init(BAR(B_WQFREE + i), 4 * ntile); // one arrival per softmax warp
         }
         // Q may be overwritten once the MMA threads are done with it and every softmax warp has
-        // read its rows (or has no use for them)
+        // read its rows (or has no use for them).  Items without any key load no Q and have no phase here;
+        // for the others no warp arrives for an item before the issuing warps have taken it, or the
+        // arrivals of two items could mix.
         mbar_init(BAR(B_QEMPTY), 5 * ntile);
         fence_mbar_init();
     }
@@ -246,7 +240,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         tmem_relinquish();
     }
     if (P.dO) {
-        for (int i = threadIdx.x; i < C::PANEL_BYTES / 16; i += 384)
+        for (int i = threadIdx.x; i < C::ZERO_ROWS * 8; i += 384)
             reinterpret_cast<uint4 *>(sp + C::OFF_ZERO)[i] = make_uint4(0, 0, 0, 0);
         fence_proxy_async_smem();
     }
@@ -269,53 +263,78 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         }
         uint32_t kpos = 0; // position in the K / V ring, running over the items
         bool live = true;
-        for (int w = 0; live; ++w) {
-            // draw the next item once the queue slot's last reader (four items ago) is done
-            const int slot = w & 3;
-            int idx = -1;
-            if (lane == 0 && mbar_wait(BAR(B_WQFREE + slot), ((w >> 2) & 1) ^ 1, abort_flag)) {
-                idx = atomicAdd(P.cursor, 1);
-                idx = idx < P.n_items ? idx : -1;
-                wq[slot] = idx;
-                mbar_arrive(BAR(B_WQFULL + slot));
-            }
-            idx = __shfl_sync(0xffffffffu, idx, 0);
-            if (idx < 0)
-                break;
-            const Item it = decode(idx);
-            const int cnt = it.cnt, n_single = it.n_single, g = it.g;
-            const int2 *klist = it.klist;
-            if (lane == 0) {
-                live = mbar_wait(BAR(B_QEMPTY), (w & 1) ^ 1, abort_flag);
-                if (live) {
-                    mbar_arrive_expect_tx(BAR(B_QFULL), ntile * C::TILE_BYTES);
-                    for (int x = 0; x < ntile; ++x)
-                        for (int pn = 0; pn < C::PANELS; ++pn)
-                            tma_load_3d(sb + C::OFF_Q + x * C::TILE_BYTES + pn * C::PANEL_BYTES, &tmQ,
-                                        BAR(B_QFULL), pn * 64, it.h0 + x, it.row0);
+        // Draws item w once the queue slot's last reader (four items ago) is done.  A chain of an atomic and two
+        // dependent loads, 2,000 clocks, so it is started ahead of the last key tile of the item before.
+        auto draw = [&](int w) {
+            int4 e = make_int4(-1, 0, 0, 0);
+            if (mbar_wait_warp(BAR(B_WQFREE + (w & 3)), ((w >> 2) & 1) ^ 1, abort_flag) && lane == 0) {
+                const int idx = atomicAdd(P.cursor, 1);
+                if (idx < P.n_items) {
+                    e.x = P.qorder[idx / n_hb];
+                    e.y = idx % n_hb;
+                    e.z = P.kcount[e.x];
+                    e.w = P.scount[e.x];
                 }
+                wq[w & 3] = e;
+                mbar_arrive(BAR(B_WQFULL + (w & 3)));
             }
-            live = __all_sync(0xffffffffu, live);
-            // The key tiles of the SINGLE entries go through the same K / V ring first; the softmax
-            // warps read their rows from shared memory.
-            for (int i = 0; live && i < n_single; ++i) {
-                const uint32_t pos = kpos + i;
-                const int st = pos % NS, ph = (pos / NS) & 1;
-                const int start = P.sbase[it.qt * MAX_SINGLE + i];
-                live = mbar_wait_warp(BAR(B_KEMPTY + st), ph ^ 1, abort_flag) &&
-                       mbar_wait_warp(BAR(B_VEMPTY + st), ph ^ 1, abort_flag);
-                if (live && lane == 0) {
-                    mbar_arrive_expect_tx(BAR(B_KFULL + st), C::TILE_BYTES);
-                    mbar_arrive_expect_tx(BAR(B_VFULL + st), C::TILE_BYTES);
-                    for (int pn = 0; pn < C::PANELS; ++pn) {
-                        tma_load_3d(sb + C::OFF_K + st * C::TILE_BYTES + pn * C::PANEL_BYTES, &tmK,
-                                    BAR(B_KFULL + st), pn * 64, g, start);
-                        tma_load_3d(sb + C::OFF_V + st * C::TILE_BYTES + pn * C::PANEL_BYTES, &tmV,
-                                    BAR(B_VFULL + st), pn * 64, g, start);
-                    }
+            return make_int4(__shfl_sync(0xffffffffu, e.x, 0), __shfl_sync(0xffffffffu, e.y, 0),
+                             __shfl_sync(0xffffffffu, e.z, 0), __shfl_sync(0xffffffffu, e.w, 0));
+        };
+        int4 item = draw(0), next = make_int4(-1, 0, 0, 0);
+        int qn = 0; // items with keys
+        for (int w = 0; live && item.x >= 0; ++w, item = next) {
+            const int qt = item.x, h0 = item.y * heads, cnt = item.z, n_single = item.w;
+            const int g = h0 / (P.Hq / P.Hkv), row0 = P.q_begin + qt * BM;
+            const int2 *klist = P.klist + (size_t)qt * P.n_kt;
+            const int window = lane < n_single ? P.sbase[qt * MAX_SINGLE + lane] : 0; // first token of entry `lane`
+            auto load = [&](int off, const CUtensorMap *map, int full, uint32_t pos, int start) { // one K or V tile
+                const int st = pos % NS;
+                if (lane == 0) {
+                    mbar_arrive_expect_tx(BAR(full + st), C::TILE_BYTES);
+                    for (int pn = 0; pn < C::PANELS; ++pn)
+                        tma_load_3d(sb + off + st * C::TILE_BYTES + pn * C::PANEL_BYTES, map, BAR(full + st), pn * 64, g,
+                                    start);
                 }
                 __syncwarp();
+            };
+            auto stage_free = [&](int empty, uint32_t pos) {
+                return mbar_wait_warp(BAR(empty + pos % NS), ((pos / NS) & 1) ^ 1, abort_flag);
+            };
+            if (cnt + n_single > 0)
+                live = mbar_wait_warp(BAR(B_QEMPTY), (qn++ & 1) ^ 1, abort_flag);
+            if (cnt + n_single > 0 && live && lane == 0) {
+                mbar_arrive_expect_tx(BAR(B_QFULL), ntile * C::TILE_BYTES + n_single * BM);
+                for (int x = 0; x < ntile; ++x)
+                    for (int pn = 0; pn < C::PANELS; ++pn)
+                        tma_load_3d(sb + C::OFF_Q + x * C::TILE_BYTES + pn * C::PANEL_BYTES, &tmQ, BAR(B_QFULL), pn * 64,
+                                    h0 + x, row0);
+                if (n_single > 0)
+                    bulk_load(sb + C::OFF_COL, P.scs + (size_t)qt * MAX_SINGLE * BM, n_single * BM, BAR(B_QFULL));
             }
+            __syncwarp();
+            // The key tiles of the SINGLE entries go through the same K / V ring first; the softmax warps read
+            // their rows from shared memory: K of all entries, then V of all entries (so V of the first
+            // NS entries beside K, the others behind).
+            for (int i = 0; live && i < n_single; ++i) {
+                const int start = __shfl_sync(0xffffffffu, window, i);
+                live = stage_free(B_KEMPTY, kpos + i);
+                if (live)
+                    load(C::OFF_K, &tmK, B_KFULL, kpos + i, start);
+                if (live && i < NS) {
+                    live = stage_free(B_VEMPTY, kpos + i);
+                    if (live)
+                        load(C::OFF_V, &tmV, B_VFULL, kpos + i, start);
+                }
+            }
+            for (int i = NS; live && i < n_single; ++i) {
+                const int start = __shfl_sync(0xffffffffu, window, i);
+                live = stage_free(B_VEMPTY, kpos + i);
+                if (live)
+                    load(C::OFF_V, &tmV, B_VFULL, kpos + i, start);
+            }
+            if (live && cnt < 2)
+                next = draw(w + 1);
             // List entries and key metadata are fetched one key tile ahead, so that no global
             // load latency sits between a stage becoming free and its TMA loads.
             auto tile_meta = [&](int2 e, int32_t (&mv)[BN / 32]) {
@@ -334,34 +353,25 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 tile_meta(e_cur, m_cur);
             for (int j = 0; live && j < cnt; ++j) {
                 const uint32_t pos = kpos + n_single + j;
-                const int st = pos % NS, ph = (pos / NS) & 1;
+                const int st = pos % NS;
                 const int start = e_cur.x;
                 const int2 e_nn = j + 2 < cnt ? klist[j + 2] : e_nxt;
                 if (j + 1 < cnt)
                     tile_meta(e_nxt, m_nxt);
-                live = mbar_wait_warp(BAR(B_KEMPTY + st), ph ^ 1, abort_flag);
+                live = stage_free(B_KEMPTY, pos);
                 if (!live)
                     break;
-                if (lane == 0) {
-                    mbar_arrive_expect_tx(BAR(B_KFULL + st), C::TILE_BYTES);
-                    for (int pn = 0; pn < C::PANELS; ++pn)
-                        tma_load_3d(sb + C::OFF_K + st * C::TILE_BYTES + pn * C::PANEL_BYTES, &tmK,
-                                    BAR(B_KFULL + st), pn * 64, g, start);
-                }
-                __syncwarp();
-                live = mbar_wait_warp(BAR(B_VEMPTY + st), ph ^ 1, abort_flag);
+                load(C::OFF_K, &tmK, B_KFULL, pos, start);
+                live = stage_free(B_VEMPTY, pos);
                 if (!live)
                     break;
 #pragma unroll
                 for (int i = 0; i < BN / 32; ++i)
                     smeta[st * BN + lane + 32 * i] = m_cur[i];
                 __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive_expect_tx(BAR(B_VFULL + st), C::TILE_BYTES);
-                    for (int pn = 0; pn < C::PANELS; ++pn)
-                        tma_load_3d(sb + C::OFF_V + st * C::TILE_BYTES + pn * C::PANEL_BYTES, &tmV,
-                                    BAR(B_VFULL + st), pn * 64, g, start);
-                }
+                load(C::OFF_V, &tmV, B_VFULL, pos, start);
+                if (j + 2 == cnt)
+                    next = draw(w + 1);
                 e_cur = e_nxt;
                 e_nxt = e_nn;
 #pragma unroll
@@ -374,7 +384,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             if (P.dO && live && lane == 0) {
                 for (int x = 0; x < ntile; ++x)
                     for (int pn = 0; pn < D / 32; ++pn)
-                        tma_store_3d(&tmZ, sb + C::OFF_ZERO, pn * 32, it.h0 + x, it.qt * BM);
+                        for (int rr = 0; rr < BM && row0 + rr < P.q_end; rr += C::ZERO_ROWS)
+                            tma_store_3d(&tmZ, sb + C::OFF_ZERO, pn * 32, h0 + x, qt * BM + rr);
                 bulk_commit_group();
             }
         }
@@ -406,6 +417,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     if (lead) mma_ss_lo(tS, q_lo + off, kb + off, IDESC_S, k > 0);
                 }
                 if (lead) tc_commit(BAR(B_SFULL + x));
+                if (lead) mbar_arrive_n(BAR(B_KEMPTY + st), STAGE_ARRIVALS);
                 if (lead) tc_commit(BAR(B_KEMPTY + st));
             };
             auto issue_pv = [&](int st, int half, bool acc) { // 64 keys
@@ -417,28 +429,36 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 if (half == 0)
                     return;
                 if (lead) tc_commit(BAR(B_PVDONE + x));
+                if (lead) mbar_arrive_n(BAR(B_VEMPTY + st), STAGE_ARRIVALS);
                 if (lead) tc_commit(BAR(B_VEMPTY + st));
             };
             uint32_t kpos = 0; // position in the K / V ring, running over the items
             uint32_t t = 0;    // key tiles of this thread's tile so far (phases of S, P, PV)
+            int qn = 0;        // items with keys so far (phases of Q)
             bool ok = true;
             for (int w = 0; ok; ++w) {
-                const int idx = take(w);
-                if (idx < 0)
+                const int4 item = take(w);
+                if (item.x < 0)
                     break;
-                const Item it = decode(idx);
-                const int cnt = it.cnt, n_single = it.n_single;
-                ok = mbar_wait_warp(BAR(B_QFULL), w & 1, abort_flag);
-                // The SINGLE entries come first in the ring.  Their phases are waited for one by
-                // one: a parity wait is only meaningful on the phase that follows the last one
-                // seen.
-                for (int i = 0; ok && i < n_single; ++i) {
-                    const uint32_t pos = kpos + i;
-                    ok = mbar_wait_warp(BAR(B_KFULL + pos % NS), (pos / NS) & 1, abort_flag) &&
-                         mbar_wait_warp(BAR(B_VFULL + pos % NS), (pos / NS) & 1, abort_flag);
-                }
+                const int cnt = item.z, n_single = item.w;
+                if (cnt + n_single == 0)
+                    continue;
+                ok = mbar_wait_warp(BAR(B_QFULL), qn++ & 1, abort_flag);
                 if (ok && cnt == 0)
                     if (lead) mbar_arrive(BAR(B_QEMPTY)); // no product reads this Q
+                // The SINGLE entries come first in the ring: K of all, then V of all.  This warp waits for their
+                // phases one by one, and a stage is not refilled before it has: a parity wait is only
+                // meaningful on the phase that follows the last one seen.
+                for (int i = 0; ok && i < n_single; ++i) {
+                    const uint32_t pos = kpos + i;
+                    ok = mbar_wait_warp(BAR(B_KFULL + pos % NS), (pos / NS) & 1, abort_flag);
+                    if (ok && lead) mbar_arrive(BAR(B_KEMPTY + pos % NS));
+                }
+                for (int i = 0; ok && i < n_single; ++i) {
+                    const uint32_t pos = kpos + i;
+                    ok = mbar_wait_warp(BAR(B_VFULL + pos % NS), (pos / NS) & 1, abort_flag);
+                    if (ok && lead) mbar_arrive(BAR(B_VEMPTY + pos % NS));
+                }
                 if (ok && cnt > 0) {
                     const uint32_t p0 = kpos + n_single;
                     // S of the previous item's last key tile must be in the softmax registers
@@ -509,21 +529,27 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         const uint32_t tP = tmem + lane_sel + C::TM_P + x * C::P_STRIDE;
         uint32_t kpos = 0; // position in the K / V ring, running over the items
         uint32_t t = 0;    // key tiles of this tile so far (phases of S, P, PV)
+        int qn = 0;        // items with keys so far (phases of Q)
         bool ok = true;
-        for (int w = 0; ok; ++w) {
-        const int idx = __shfl_sync(0xffffffffu, take(w), 0);
-        __syncwarp();
-        if (lane == 0 && idx >= 0)
-            mbar_arrive(BAR(B_WQFREE + (w & 3))); // this warp has read the queue slot
-        if (idx < 0)
-            break;
-        const Item it = decode(idx);
-        const int qt = it.qt, cnt = it.cnt, n_single = it.n_single;
-        const int2 *klist = it.klist;
-        const int h = it.h0 + x;
-        const int row = it.row0 + r;
+        // Item w, and its row's metadata, are fetched ahead of the epilogue of item w - 1 (two dependent reads of
+        // global memory and the draw itself, 1,500 to 3,500 clocks per item before the queue carried the item).
+        auto fetch = [&](int w, int32_t &meta) {
+            const int4 e = take(w);
+            __syncwarp();
+            if (lane == 0 && e.x >= 0)
+                mbar_arrive(BAR(B_WQFREE + (w & 3))); // this warp has read the queue slot
+            const int row = P.q_begin + e.x * BM + r;
+            meta = e.x >= 0 && row < P.q_end ? P.meta[row] : META_NONE_Q;
+            return e;
+        };
+        int32_t mq;
+        int4 item = fetch(0, mq);
+        for (int w = 0; ok && item.x >= 0; ++w) {
+        const int qt = item.x, h0 = item.y * heads, cnt = item.z, n_single = item.w;
+        const int2 *klist = P.klist + (size_t)qt * P.n_kt;
+        const int h = h0 + x;
+        const int row0 = P.q_begin + qt * BM, row = row0 + r;
         const bool row_ok = row < P.q_end;
-        int32_t mq = row_ok ? P.meta[row] : META_NONE_Q;
         if (mq == META_NONE_K)
             mq = META_NONE_Q;
         float m = -CUDART_INF_F, l = 0.f;
@@ -533,212 +559,101 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             if (D == 128)
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(pre + 64));
         }
-        if (n_single == 0 && lane == 0)
-            mbar_arrive(BAR(B_QEMPTY)); // no row of Q is read by this warp
-        if constexpr (D == 64) {
-            if (n_single > 0) {
-                // One allowed key per row and tile: the score and the weighted value on the CUDA
-                // cores, rows read from the staged K / V tiles, as an online softmax; the result
-                // becomes the starting (m, l, O) of the tile loop.
-                ok = mbar_wait_warp(BAR(B_QFULL), w & 1, abort_flag);
-                float qf[64]; // the row of Q, unpacked once
-                {
-                    const uint8_t *qrow = sp + C::OFF_Q + x * C::TILE_BYTES + r * 128;
+        if (n_single > 0) {
+            // One allowed key per row and entry, on the CUDA cores from the staged K / V rows: the scores of
+            // all entries, then the softmax over them and the weighted values, which become the starting
+            // (m, l, O) of the tile loop.  A row of Q and a row of O are then not held at the same time, and
+            // each of the two passes needs K or V only.  Bound by unpacking bf16 (a row's element is two
+            // instructions, one of them packed).  (One pass with an online softmax, O in tensor memory at
+            // head_dim 128, and a barrier of the tile's warps after every entry: 1,900 clocks per entry at
+            // head_dim 64, 3,300 at 128.)
+            ok = mbar_wait_warp(BAR(B_QFULL), qn & 1, abort_flag);
+            const uint8_t *cols = sp + C::OFF_COL + r;
+            float *score = reinterpret_cast<float *>(sp + C::OFF_SCORE) + threadIdx.x;
+            auto row_piece = [&](uint32_t off, int rr, int c) { // elements 8c .. 8c + 7 of row rr of a staged tile
+                return *reinterpret_cast<const uint4 *>(sp + off + (c >> 3) * C::PANEL_BYTES + rr * 128 +
+                                                        (((c & 7) ^ (rr & 7)) << 4));
+            };
+            auto pair = [](uint32_t w2) { return f2(__uint_as_float(w2 << 16), __uint_as_float(w2 & 0xffff0000u)); };
+            if (ok) {
+                F2 q[D / 2];
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const uint4 v = *reinterpret_cast<const uint4 *>(qrow + ((c ^ (r & 7)) << 4));
-                        const uint32_t qw[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            qf[8 * c + 2 * k] = __uint_as_float(qw[k] << 16);
-                            qf[8 * c + 2 * k + 1] = __uint_as_float(qw[k] & 0xffff0000u);
-                        }
-                    }
+                for (int c = 0; c < D / 8; ++c) {
+                    const uint4 v = row_piece(C::OFF_Q + x * C::TILE_BYTES, r, c);
+                    q[4 * c] = pair(v.x);
+                    q[4 * c + 1] = pair(v.y);
+                    q[4 * c + 2] = pair(v.z);
+                    q[4 * c + 3] = pair(v.w);
                 }
-                __syncwarp();
-                if (lane == 0)
-                    mbar_arrive(BAR(B_QEMPTY)); // this warp's rows of Q are in registers
-                float o[64];
-#pragma unroll
-                for (int i = 0; i < 64; ++i)
-                    o[i] = 0.f;
-                int col_nxt = P.scs[((size_t)qt * MAX_SINGLE) * BM + r];
+#pragma unroll 1
                 for (int i = 0; ok && i < n_single; ++i) {
                     const uint32_t pos = kpos + i;
-                    const int st = pos % NS, ph = (pos / NS) & 1;
-                    const int col = col_nxt;
-                    if (i + 1 < n_single) // requested one entry ahead of its use
-                        col_nxt = P.scs[((size_t)qt * MAX_SINGLE + i + 1) * BM + r];
-                    ok = mbar_wait_warp(BAR(B_KFULL + st), ph, abort_flag) &&
-                         mbar_wait_warp(BAR(B_VFULL + st), ph, abort_flag);
-                    if (ok && col != NO_COL && row_ok) {
-                        const uint8_t *krow = sp + C::OFF_K + st * C::TILE_BYTES + col * 128;
-                        const uint8_t *vrow = sp + C::OFF_V + st * C::TILE_BYTES + col * 128;
-                        float acc4[4] = {0.f, 0.f, 0.f, 0.f}; // four chains of dependent adds
+                    const int st = pos % NS;
+                    const int col = cols[i * BM];
+                    ok = mbar_wait_warp(BAR(B_KFULL + st), (pos / NS) & 1, abort_flag);
+                    if (!ok)
+                        break;
+                    float s2 = -CUDART_INF_F;
+                    if (col != NO_COL && row_ok) {
+                        F2 acc[4]; // four chains of dependent adds
 #pragma unroll
-                        for (int c = 0; c < 8; ++c) {
-                            const uint4 v = *reinterpret_cast<const uint4 *>(krow + ((c ^ (col & 7)) << 4));
+                        for (int c = 0; c < D / 8; ++c) {
+                            const uint4 v = row_piece(C::OFF_K + st * C::TILE_BYTES, col, c);
                             const uint32_t kw[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                acc4[k] = fmaf(qf[8 * c + 2 * k], __uint_as_float(kw[k] << 16), acc4[k]);
-                                acc4[k] = fmaf(qf[8 * c + 2 * k + 1], __uint_as_float(kw[k] & 0xffff0000u),
-                                               acc4[k]);
-                            }
+                            for (int k = 0; k < 4; ++k)
+                                acc[k] = c == 0 ? mul_f2(q[k], pair(kw[k])) : fma_f2(q[4 * c + k], pair(kw[k]), acc[k]);
                         }
-                        const float s2 = ((acc4[0] + acc4[1]) + (acc4[2] + acc4[3])) * P.scale_log2;
-                        // As in the tile loop, the running sums move to a new maximum only when it
-                        // grew by more than 2^8 (always for the first key, where m is -inf and
-                        // the sums are still zero).
-                        if (s2 > m + 8.f) {
-                            const float alpha = fast_exp2(m - s2); // 0 for the first key
-                            l *= alpha;
-#pragma unroll
-                            for (int e = 0; e < 64; ++e)
-                                o[e] *= alpha;
-                            m = s2;
-                        }
-                        const float pr = fast_exp2(s2 - m);
-                        l += pr;
-#pragma unroll
-                        for (int c = 0; c < 8; ++c) {
-                            const uint4 v = *reinterpret_cast<const uint4 *>(vrow + ((c ^ (col & 7)) << 4));
-                            const uint32_t vw[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                o[8 * c + 2 * k] = fmaf(pr, __uint_as_float(vw[k] << 16), o[8 * c + 2 * k]);
-                                o[8 * c + 2 * k + 1] =
-                                    fmaf(pr, __uint_as_float(vw[k] & 0xffff0000u), o[8 * c + 2 * k + 1]);
-                            }
-                        }
+                        const float2 a = unf2(add_f2(add_f2(acc[0], acc[1]), add_f2(acc[2], acc[3])));
+                        s2 = (a.x + a.y) * P.scale_log2;
                     }
-                    // every thread of this tile's four warps is done with the stage (and the four
-                    // warps leave together if a wait ran out)
-                    ok = bar_and(1 + x, 128, ok);
-                    if (!ok)
-                        break;
-                    if (r == 0) {
-                        mbar_arrive(BAR(B_KEMPTY + st));
-                        mbar_arrive(BAR(B_VEMPTY + st));
-                    }
-                }
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    uint32_t ov[32];
-#pragma unroll
-                    for (int i = 0; i < 32; ++i)
-                        ov[i] = __float_as_uint(o[32 * c + i]);
-                    tmem_st32(tO + c * 32, ov);
-                }
-                tmem_wait_st(); // ordered before the first P V product by the P hand-over below
-            }
-        } else {
-            if (n_single > 0) {
-                // head_dim 128: the same pair-by-pair online softmax, but a row of O (128 fp32) does
-                // not fit beside the row of Q in registers, so O is kept in tensor memory and
-                // updated 32 columns at a time (load, scale and add, store).  Tensor-memory
-                // accesses are warp-wide, so rows without a key in an entry take part with
-                // weight 0.
-                ok = mbar_wait_warp(BAR(B_QFULL), w & 1, abort_flag);
-                uint32_t qp[64]; // the row of Q as packed bf16 pairs, panel-major
-#pragma unroll
-                for (int pn = 0; pn < 2; ++pn) {
-                    const uint8_t *qrow = sp + C::OFF_Q + x * C::TILE_BYTES + pn * C::PANEL_BYTES + r * 128;
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const uint4 v = *reinterpret_cast<const uint4 *>(qrow + ((c ^ (r & 7)) << 4));
-                        qp[32 * pn + 4 * c + 0] = v.x;
-                        qp[32 * pn + 4 * c + 1] = v.y;
-                        qp[32 * pn + 4 * c + 2] = v.z;
-                        qp[32 * pn + 4 * c + 3] = v.w;
-                    }
-                }
-                __syncwarp();
-                if (lane == 0)
-                    mbar_arrive(BAR(B_QEMPTY)); // this warp's rows of Q are in registers
-                int col_nxt = P.scs[((size_t)qt * MAX_SINGLE) * BM + r];
-                for (int i = 0; ok && i < n_single; ++i) {
-                    const uint32_t pos = kpos + i;
-                    const int st = pos % NS, ph = (pos / NS) & 1;
-                    const int col = col_nxt;
-                    if (i + 1 < n_single) // requested one entry ahead of its use
-                        col_nxt = P.scs[((size_t)qt * MAX_SINGLE + i + 1) * BM + r];
-                    ok = mbar_wait_warp(BAR(B_KFULL + st), ph, abort_flag) && mbar_wait_warp(BAR(B_VFULL + st), ph, abort_flag);
-                    if (ok) {
-                        const bool have = col != NO_COL && row_ok;
-                        const int kc = have ? col : 0;
-                        const uint8_t *krow = sp + C::OFF_K + st * C::TILE_BYTES + kc * 128;
-                        const uint8_t *vrow = sp + C::OFF_V + st * C::TILE_BYTES + kc * 128;
-                        float acc4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                        for (int pn = 0; pn < 2; ++pn) {
-#pragma unroll
-                            for (int c = 0; c < 8; ++c) {
-                                const uint4 v = *reinterpret_cast<const uint4 *>(
-                                    krow + pn * C::PANEL_BYTES + ((c ^ (kc & 7)) << 4));
-                                const uint32_t kw[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                                for (int k = 0; k < 4; ++k) {
-                                    const uint32_t qw = qp[32 * pn + 4 * c + k];
-                                    acc4[k] = fmaf(__uint_as_float(qw << 16), __uint_as_float(kw[k] << 16), acc4[k]);
-                                    acc4[k] = fmaf(__uint_as_float(qw & 0xffff0000u),
-                                                   __uint_as_float(kw[k] & 0xffff0000u), acc4[k]);
-                                }
-                            }
-                        }
-                        const float s2 = ((acc4[0] + acc4[1]) + (acc4[2] + acc4[3])) * P.scale_log2;
-                        float alpha = 1.f, pr = 0.f;
-                        if (have) {
-                            if (s2 > m + 8.f) { // as in the tile loop; always for the row's first key
-                                alpha = fast_exp2(m - s2); // 0 for the first key
-                                l *= alpha;
-                                m = s2;
-                            }
-                            pr = fast_exp2(s2 - m);
-                            l += pr;
-                        }
-#pragma unroll
-                        for (int q4 = 0; q4 < 4; ++q4) { // columns 32 q4 .. 32 q4 + 31 of O
-                            uint32_t ov[32];
-                            if (i > 0) {
-                                tmem_ld32(tO + q4 * 32, ov);
-                                tmem_wait_ld();
-                            } else {
-#pragma unroll
-                                for (int e = 0; e < 32; ++e)
-                                    ov[e] = 0u;
-                            }
-                            const uint8_t *vp = vrow + (q4 >> 1) * C::PANEL_BYTES;
-#pragma unroll
-                            for (int cc = 0; cc < 4; ++cc) {
-                                const int c = (q4 & 1) * 4 + cc;
-                                const uint4 v = *reinterpret_cast<const uint4 *>(vp + ((c ^ (kc & 7)) << 4));
-                                const uint32_t vw[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                                for (int k = 0; k < 4; ++k) {
-                                    const int e = 8 * cc + 2 * k;
-                                    ov[e] = __float_as_uint(fmaf(pr, __uint_as_float(vw[k] << 16),
-                                                                 alpha * __uint_as_float(ov[e])));
-                                    ov[e + 1] = __float_as_uint(fmaf(pr, __uint_as_float(vw[k] & 0xffff0000u),
-                                                                     alpha * __uint_as_float(ov[e + 1])));
-                                }
-                            }
-                            tmem_st32(tO + q4 * 32, ov);
-                        }
-                        tmem_wait_st(); // before the next entry loads these columns, and ordered before
-                                        // the first P V product by the P hand-over below
-                    }
-                    // every thread of this tile's four warps is done with the stage (and the four
-                    // warps leave together if a wait ran out)
-                    ok = bar_and(1 + x, 128, ok);
-                    if (!ok)
-                        break;
-                    if (r == 0) {
-                        mbar_arrive(BAR(B_KEMPTY + st));
-                        mbar_arrive(BAR(B_VEMPTY + st));
-                    }
+                    score[i * 256] = s2;
+                    m = fmaxf(m, s2);
+                    warp_arrive(BAR(B_KEMPTY + st)); // this warp is done with the rows
                 }
             }
+            const float neg_m = m == -CUDART_INF_F ? 0.f : -m;
+            F2 o[D / 2];
+#pragma unroll
+            for (int i = 0; i < D / 2; ++i)
+                o[i] = f2(0.f, 0.f);
+#pragma unroll 1
+            for (int i = 0; ok && i < n_single; ++i) {
+                const uint32_t pos = kpos + i;
+                const int st = pos % NS;
+                const int col = cols[i * BM];
+                const float pr = fast_exp2(score[i * 256] + neg_m);
+                ok = mbar_wait_warp(BAR(B_VFULL + st), (pos / NS) & 1, abort_flag);
+                if (!ok)
+                    break;
+                if (col != NO_COL && row_ok) {
+                    l += pr;
+                    const F2 pp = f2(pr, pr);
+#pragma unroll
+                    for (int c = 0; c < D / 8; ++c) {
+                        const uint4 v = row_piece(C::OFF_V + st * C::TILE_BYTES, col, c);
+                        o[4 * c] = fma_f2(pp, pair(v.x), o[4 * c]);
+                        o[4 * c + 1] = fma_f2(pp, pair(v.y), o[4 * c + 1]);
+                        o[4 * c + 2] = fma_f2(pp, pair(v.z), o[4 * c + 2]);
+                        o[4 * c + 3] = fma_f2(pp, pair(v.w), o[4 * c + 3]);
+                    }
+                }
+                warp_arrive(BAR(B_VEMPTY + st));
+            }
+#pragma unroll
+            for (int c = 0; c < D / 32; ++c) {
+                uint32_t ov[32];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const float2 v = unf2(o[16 * c + i]);
+                    ov[2 * i] = __float_as_uint(v.x);
+                    ov[2 * i + 1] = __float_as_uint(v.y);
+                }
+                tmem_st32(tO + c * 32, ov);
+            }
+            tmem_wait_st(); // ordered before the first P V product by the P hand-over below
+            // Q and the entries' columns are done with (the issuing warps need Q for longer anyway)
+            warp_arrive(BAR(B_QEMPTY));
         }
         int word_nxt = cnt > 0 ? klist[0].y : 0;
         for (int j = 0; ok && j < cnt; ++j) {
@@ -860,6 +775,11 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             tc_fence_before();
             warp_arrive(BAR(B_PFULL + (C::P_HALVES ? 2 : 0) + x));
         }
+        if (ok && cnt > 0 && n_single == 0 && lane == 0)
+            mbar_arrive(BAR(B_QEMPTY)); // this warp reads no row of Q; not ahead of the issuing warp, see Q's phases
+        __syncwarp();
+        int32_t mq_next = META_NONE_Q;
+        const int4 item_next = fetch(w + 1, mq_next);
         // ---- epilogue: normalise, store O and LSE
         // Delta of the row needs the row of dO: requested here, ahead of the wait for the last
         // P V product (the row was sent towards L2 when the item began)
@@ -877,7 +797,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         }
         // rows of the padded partition are numbered from its first row
         const size_t hand = (size_t)h * P.q_pad + (size_t)row_slot(qt * BM + r);
-        if (P.dO && x == 0 && (it.h0 == 0))
+        if (P.dO && x == 0 && h0 == 0)
             P.mqp[row_slot(qt * BM + r)] = mq;
         if (cnt == 0 && n_single == 0) {
             if (row_ok) {
@@ -942,7 +862,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 fence_proxy_async_smem();
                 asm volatile("bar.sync %0, 128;" ::"r"(1 + x) : "memory");
                 if (r == 0) {
-                    tma_store_3d(&tmO, sb + C::OFF_OST + x * C::TILE_BYTES, 0, h, it.row0);
+                    tma_store_3d(&tmO, sb + C::OFF_OST + x * C::TILE_BYTES, 0, h, row0);
                     bulk_commit_group();
                 }
             } else
@@ -976,6 +896,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         }
         kpos += (uint32_t)(n_single + cnt);
         t += (uint32_t)cnt;
+        qn += cnt + n_single > 0;
+        item = item_next;
+        mq = mq_next;
         } // items
     }
 
@@ -1042,7 +965,7 @@ static int launch_fwd_t(const Plan &p, const FwdArgs &a, EncodeTiledFn enc, int 
         make_map(enc, &tmV, a.V, D, a.Hkv, p.T) || make_map(enc, &tmO, a.O, D, a.Hq, p.q_end))
         return PEAGLE_ERR_CUDA;
     CUtensorMap tmZ = tmO;
-    if (a.dO && make_f32_map(enc, &tmZ, a.dq_acc, D, a.Hq, p.q_end - p.q_begin, BM))
+    if (a.dO && make_f32_map(enc, &tmZ, a.dq_acc, D, a.Hq, p.q_end - p.q_begin, FwdCfg<D>::ZERO_ROWS))
         return PEAGLE_ERR_CUDA;
     FwdParams P;
     P.klist = p.klist;

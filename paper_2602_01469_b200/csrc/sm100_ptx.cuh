@@ -44,6 +44,10 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n) // n arrivals
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n) : "memory");
+}
 // One arrival for a whole (converged) warp: every lane has finished and fenced its own work, the
 // warp meets, lane 0 arrives.  A barrier counted per thread costs one serialised shared-memory
 // atomic per thread and phase -- hundreds of clocks on a hand-over that happens every step.
