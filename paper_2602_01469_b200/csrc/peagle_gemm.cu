@@ -13,9 +13,12 @@
 // and B by TMA into a ring of stages (128-byte swizzle), warp 1 lane 0 issues tcgen05.mma (four
 // k = 16 products per slab) into one of two accumulators in tensor memory and releases the stages
 // by commits, warps 2-5 read an accumulator when its last commit arrives, hand it back as soon as
-// it is in registers, and either store bf16 rows or add into an fp32 C (tiles of one launch are
-// disjoint and launches on a stream are ordered, so the addition is a plain load-add-store).
+// it is in registers, and either store bf16 rows or add into an fp32 C (in gemm_kernel the tiles of one launch
+// are disjoint and launches on a stream are ordered, so the addition is a plain load-add-store; the pairs of
+// gemm2_kernel add by reductions).
 #include <cstdint>
+
+#include <algorithm>
 
 #include "peagle_internal.h"
 #include "sm100_ptx.cuh"
@@ -266,6 +269,46 @@ struct Gemm2Cfg {
     static_assert(N_BAR * 8 + 32 <= 1024 && SMEM <= 227 * 1024, "shared memory of one CTA");
 };
 
+// A pair's work: whole tiles in waves of n_pairs, then, where C is added to, its share of the last, partly
+// filled wave, whose k slabs are dealt out evenly: the pairs that share a tile add their parts to C one after
+// the other.  Whole waves stay whole because the pairs then walk k together and find each other's slabs in L2.  A
+// share is at least MIN_SHARE slabs, since every part of a tile costs an epilogue of about ten.  The order of the
+// parts is not fixed, so the last bit of such a tile may differ from run to run.  (dW of 5,120 x 2,880 over 32,768
+// rows: 240 tiles on 74 pairs, 3.24 instead of 4 waves; projection, rotary kernels and their backward for these
+// sizes 2,561 -> 2,463 us.)
+struct PairWalk {
+    static constexpr int MIN_SHARE = 8;
+    int t, i0, i1; // the segment: tile, k slabs i0 .. i1 - 1
+    int w = 0, waves, rest, u, u1;
+    int pair, n_pairs, n_k;
+    __device__ PairWalk(int pair_, int n_pairs_, int n_tiles, int n_k_, bool deal)
+        : pair(pair_), n_pairs(n_pairs_), n_k(n_k_)
+    {
+        waves = deal ? n_tiles / n_pairs : (n_tiles - pair + n_pairs - 1) / n_pairs;
+        rest = waves * n_pairs; // first tile of the part that is dealt out
+        const long long units = deal ? (long long)(n_tiles - rest) * n_k : 0;
+        const int shares = (int)min((long long)n_pairs, max(1ll, units / MIN_SHARE));
+        u = pair < shares ? (int)(units * pair / shares) : 0;
+        u1 = pair < shares ? (int)(units * (pair + 1) / shares) : 0;
+    }
+    __device__ bool next()
+    {
+        if (w < waves) {
+            t = pair + w++ * n_pairs;
+            i0 = 0;
+            i1 = n_k;
+            return true;
+        }
+        if (u >= u1)
+            return false;
+        t = rest + u / n_k;
+        i0 = u % n_k;
+        i1 = min(n_k, i0 + (u1 - u));
+        u += i1 - i0;
+        return true;
+    }
+};
+
 __global__ void __launch_bounds__(192, 1)
 gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
              const __grid_constant__ CUtensorMap tmC, const GemmParams P)
@@ -288,7 +331,7 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     const int n_k = (P.K + GK - 1) / GK;
     const int tiles_n = (P.N + NT - 1) / NT;
     const int n_tiles = tiles_n * ((P.M + 2 * GT - 1) / (2 * GT));
-    const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+    PairWalk work((int)blockIdx.x >> 1, (int)gridDim.x >> 1, n_tiles, n_k, P.c_f32_add != 0);
 
     if (threadIdx.x == 0) {
         *abort_flag = 0;
@@ -320,10 +363,10 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
             tma_prefetch_desc(&tmB);
             bool live = true;
             int it = 0;
-            for (int t = pair; live && t < n_tiles; t += n_pairs) {
-                const int m0 = (t / tiles_n) * 2 * GT + (int)rank * GT;
-                const int nb = (t % tiles_n) * NT + (int)rank * (NT / 2); // this CTA's half of B
-                for (int i = 0; i < n_k; ++i, ++it) {
+            while (live && work.next()) {
+                const int m0 = (work.t / tiles_n) * 2 * GT + (int)rank * GT;
+                const int nb = (work.t % tiles_n) * NT + (int)rank * (NT / 2); // this CTA's half of B
+                for (int i = work.i0; i < work.i1; ++i, ++it) {
                     const int s = it % ST;
                     if (!mbar_wait_cluster(EMPTY(s), ((it / ST) & 1) ^ 1, abort_flag)) {
                         live = false;
@@ -358,13 +401,13 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
             const uint32_t a_step = P.a_t ? 128u : 2u, b_step = P.b_t ? 128u : 2u;
             bool ok = true;
             int it = 0, j = 0;
-            for (int t = pair; ok && t < n_tiles; t += n_pairs, ++j) {
+            for (; ok && work.next(); ++j) {
                 const int buf = j & 1;
                 ok = mbar_wait_cluster(ACCEMPTY(buf), ((j >> 1) & 1) ^ 1, abort_flag);
                 if (!ok)
                     break;
                 tc_fence_after();
-                for (int i = 0; ok && i < n_k; ++i, ++it) {
+                for (int i = work.i0; ok && i < work.i1; ++i, ++it) {
                     const int s = it % ST;
                     ok = mbar_wait_cluster(FULL(s), (it / ST) & 1, abort_flag);
                     if (!ok)
@@ -376,7 +419,7 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
 #pragma unroll
                     for (int k = 0; k < GK / 16; ++k)
                         if (lead) mma_ss_lo_pair(tmem + buf * NT, a_lo + k * a_step, b_lo + k * b_step, idesc,
-                                       (i > 0 || k > 0) ? 1u : 0u);
+                                       (i > work.i0 || k > 0) ? 1u : 0u);
                     if (lead) tc_commit_pair(EMPTY(s));
                 }
                 if (ok)
@@ -387,8 +430,8 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         // ------------------------------------------------------------ epilogue (warps 2-5, each CTA)
         const int q = warp & 3;
         int j = 0, piece = 0;
-        for (int t = pair; t < n_tiles; t += n_pairs, ++j) {
-            const int buf = j & 1;
+        for (; work.next(); ++j) {
+            const int buf = j & 1, t = work.t;
             const int m = (t / tiles_n) * 2 * GT + (int)rank * GT + q * 32 + lane;
             const int n0 = (t % tiles_n) * NT;
             // the four warps go on, or leave, together (they meet at named barriers below)
@@ -548,7 +591,9 @@ int launch_gemm(EncodeTiledFn enc, const void *A, long long lda, int a_t, const 
         if (cudaOccupancyMaxActiveClusters(&fit, gemm2_kernel, &cfg) != cudaSuccess || fit < 1)
             return PEAGLE_ERR_CUDA;
         const long long tiles2 = (long long)((N + 255) / 256) * ((M + 255) / 256);
-        const long long n_pairs = tiles2 < fit ? tiles2 : fit;
+        // an added-to C takes as many pairs as its slabs fill (see PairWalk)
+        const long long parts = c_f32_add ? std::max(tiles2, tiles2 * ((K + GK - 1) / GK) / PairWalk::MIN_SHARE) : tiles2;
+        const long long n_pairs = parts < fit ? parts : fit;
         cfg.gridDim = dim3((unsigned)(2 * n_pairs));
         // fp32 C as a tensor for the tiled reduce-adds: 32 columns (128 bytes) x 128 rows
         CUtensorMap tmC = tmA;
