@@ -196,7 +196,7 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                 hh = 0;
                 em &= em - 1;
             }
-            ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_DQFULL), it & 1, abort_flag));
+            ok = mbar_wait_warp(BAR(B_DQFULL), it & 1, abort_flag);
             if (!ok)
                 break;
             tc_fence_after();
@@ -215,7 +215,7 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         if (!ok)
             break;
         // dK and dV of the work item
-        ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_ITEMDONE), w & 1, abort_flag));
+        ok = mbar_wait_warp(BAR(B_ITEMDONE), w & 1, abort_flag);
         if (!ok)
             break;
         tc_fence_after();
@@ -285,7 +285,7 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                         hh = 0;
                         em &= em - 1;
                     }
-                    ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_QEMPTY + st), ph ^ 1, abort_flag));
+                    ok = mbar_wait_warp(BAR(B_QEMPTY + st), ph ^ 1, abort_flag);
                     if (!ok)
                         break;
                     if (lane == 0) {
@@ -358,9 +358,9 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                 if (warp == 19) {
                     const uint32_t kvo = ks * TBU;
                     for (int i = 0; ok && i < n_cur; ++i, ++it) {
-                        ok = mbar_wait(BAR(B_DSFULL), it & 1, abort_flag) &&
-                             mbar_wait(BAR(B_DSFULL + 1), it & 1, abort_flag) &&
-                             mbar_wait(BAR(B_DQEMPTY), (it & 1) ^ 1, abort_flag); // the accumulator has been read out
+                        ok = mbar_wait_warp(BAR(B_DSFULL), it & 1, abort_flag) &&
+                             mbar_wait_warp(BAR(B_DSFULL + 1), it & 1, abort_flag) &&
+                             mbar_wait_warp(BAR(B_DQEMPTY), (it & 1) ^ 1, abort_flag); // the accumulator has been read out
                         if (!ok)
                             break;
                         tc_fence_after();
@@ -375,8 +375,8 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                     continue;
                 }
                 // K / V of this item are in tensor memory
-                ok = mbar_wait(BAR(B_KVTFULL), w & 1, abort_flag) &&
-                     mbar_wait(BAR(B_QFULL + it % 3), (it / 3) & 1, abort_flag);
+                ok = mbar_wait_warp(BAR(B_KVTFULL), w & 1, abort_flag) &&
+                     mbar_wait_warp(BAR(B_QFULL + it % 3), (it / 3) & 1, abort_flag);
                 if (!ok)
                     break;
                 tc_fence_after();
@@ -386,21 +386,21 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                     const int st = it % 3, nst = (it + 1) % 3;
                     const uint32_t qo = st * 2 * TBU, nqo = nst * 2 * TBU;
                     const bool first = i == 0, last = i == n_cur - 1;
-                    ok = mbar_wait(bar_in, it & 1, abort_flag);
+                    ok = mbar_wait_warp(bar_in, it & 1, abort_flag);
                     if (ok && first)
-                        ok = mbar_wait(BAR(B_ACCFREE), (w & 1) ^ 1, abort_flag);
+                        ok = mbar_wait_warp(BAR(B_ACCFREE), (w & 1) ^ 1, abort_flag);
                     if (!ok)
                         break;
                     tc_fence_after();
                     issue_acc(qo, 0, !first);
                     if (!last) {
-                        ok = mbar_wait(BAR(B_QFULL + nst), ((it + 1) / 3) & 1, abort_flag);
+                        ok = mbar_wait_warp(BAR(B_QFULL + nst), ((it + 1) / 3) & 1, abort_flag);
                         if (!ok)
                             break;
                         tc_fence_after();
                         issue_score(nqo, 0);
                     }
-                    ok = mbar_wait(bar_in + 8, it & 1, abort_flag);
+                    ok = mbar_wait_warp(bar_in + 8, it & 1, abort_flag);
                     if (!ok)
                         break;
                     tc_fence_after();
@@ -442,9 +442,7 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                 // (their results were consumed in its last step), so the old copy is not in use.
                 const int ks = w & 1;
                 // (The other group's last S^T / dP^T must be complete as well.)
-                ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_KVFULL + ks), (w >> 1) & 1, abort_flag) &&
-                                                 (it == 0 || mbar_wait(BAR(wg == 0 ? B_SFULL + 1 : B_DPFULL),
-                                                                       (it - 1) & 1, abort_flag)));
+                ok = (mbar_wait_warp(BAR(B_KVFULL + ks), (w >> 1) & 1, abort_flag) && (it == 0 || mbar_wait_warp(BAR(wg == 0 ? B_SFULL + 1 : B_DPFULL), (it - 1) & 1, abort_flag)));
                 if (!ok)
                     break;
                 const uint8_t *src = sp + C::OFF_KV + (wg == 0 ? ks : 2) * TB + r * 128;
@@ -472,7 +470,7 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             // ---- P^T.  A thread holds 4 key lanes x 8 query columns (tmem_ld_16x256b_x4): for each
             // group i of 8 columns the columns 8i + 2 (lane % 4) and the next one.
             // The row values came with the step's Q tile, which the products read: complete.
-            ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_SFULL + wg), it & 1, abort_flag));
+            ok = mbar_wait_warp(BAR(B_SFULL + wg), it & 1, abort_flag);
             if (!ok)
                 break;
             tc_fence_after();
@@ -542,8 +540,7 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             warp_arrive(BAR(B_PFULL + wg));
             // ---- dS^T
             // (and dQ of the previous step has run, so that the dS^T panel is free)
-            ok = __all_sync(0xffffffffu, mbar_wait(BAR(B_DPFULL + wg), it & 1, abort_flag) &&
-                                             (it == 0 || mbar_wait(BAR(B_DQFULL), (it - 1) & 1, abort_flag)));
+            ok = (mbar_wait_warp(BAR(B_DPFULL + wg), it & 1, abort_flag) && (it == 0 || mbar_wait_warp(BAR(B_DQFULL), (it - 1) & 1, abort_flag)));
             if (!ok)
                 break;
             tc_fence_after();
