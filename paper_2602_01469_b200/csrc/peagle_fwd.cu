@@ -167,7 +167,6 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
 {
     using C = FwdCfg<D>;
     constexpr int NS = C::NS;
-    constexpr bool TURNS = D == 128;
     constexpr int STAGE_ARRIVALS = 4;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -532,6 +531,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         uint32_t kpos = 0; // position in the K / V ring, running over the items
         uint32_t t = 0;    // key tiles of this tile so far (phases of S, P, PV)
         int qn = 0;        // items with keys so far (phases of Q)
+        uint32_t n_turn = 0; // items with key tiles so far
         bool ok = true;
         // Item w, and its row's metadata, are fetched ahead of the epilogue of item w - 1 (two dependent reads of
         // global memory and the draw itself, 1,500 to 3,500 clocks per item before the queue carried the item).
@@ -731,12 +731,15 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     tmem_wait_st();
                 }
             }
-            // head_dim 128: the two tiles' warps of a scheduler take turns with the exponentials.  Left alone
-            // the tiles fall into step, and then both do exponentials at once and both wait at once for
-            // P V and the next S (which share tensor memory here), 2,000 of a period of 5,100 clocks.  At
-            // head_dim 64, where S is ready early, turns measured slower.
-            if (TURNS && P.two && (x == 1 || tt > 0)) {
-                ok = mbar_wait_warp(BAR(B_TURN + 4 * x + (warp & 3)), (x == 1 ? tt : tt - 1) & 1, abort_flag);
+            // Left alone the two tiles' warps of a scheduler fall into step: both do exponentials at once and both wait
+            // at once, with the exp2 unit idle for half of the time.  It is enough that tile B's first
+            // exponentials of an item start behind tile A's: the distance lasts, and a hand-over per tile costs more
+            // than it gives (3,891 positions, 64 heads of 64: 1,660 us in step, 1,547 apart, 1,737 with a turn per
+            // tile; 2,048 positions, 32 heads of 128: 346 with turns, 336 so).  Tile A waits for tile B's first
+            // turn of the item before, which is long past, so that no warp is ever two phases ahead of another's
+            // wait.
+            if (P.two && j == 0 && (x == 1 || n_turn > 0)) {
+                ok = mbar_wait_warp(BAR(B_TURN + 4 * x + (warp & 3)), (x == 1 ? n_turn : n_turn - 1) & 1, abort_flag);
                 if (!ok)
                     break;
             }
@@ -769,7 +772,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     warp_arrive(BAR(B_PFULL + x));
                 }
             }
-            if (TURNS && P.two && lane == 0)
+            if (P.two && lane == 0 && j == 0)
                 mbar_arrive(BAR(B_TURN + 4 * (x ^ 1) + (warp & 3))); // the other tile's turn
             const float2 s0 = unf2(sum2[0]), s1 = unf2(sum2[1]);
             l += (s0.x + s0.y) + (s1.x + s1.y);
@@ -943,6 +946,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         kpos += (uint32_t)(n_single + cnt);
         t += (uint32_t)cnt;
         qn += cnt + n_single > 0;
+        n_turn += cnt > 0;
         item = item_next;
         mq = mq_next;
         } // items
