@@ -58,7 +58,7 @@ struct Plan {
     int4 *qsum;            // [n_qt][2] (min anchor, max anchor, min depth, max depth) of the tile's first
                            // run of equal depth and of the rest; max anchor -1: no token
     int4 *ksum;            // [n_kt][2]
-    int *ksplit;           // [n_kt] keys in the first run, flags for sorted runs
+    int *ksplit;           // [n_kt] keys in the first run, flags of the runs
     uint8_t *cls;          // [n_qt][n_kt] tile classes
     int *counters;         // [PLAN_COUNTERS] device counters, zero before k0_plan: CNT_*
     int *cdone;            // [n_ch] query tiles of a chunk that are classified

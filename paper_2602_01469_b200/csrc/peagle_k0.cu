@@ -33,8 +33,10 @@ __device__ __forceinline__ int pack_meta(int a, int d, int K)
     return a < 0 || a >= (1 << 23) || d < 0 || d >= K ? META_NONE_K : (a << 8) | d;
 }
 
-// Beside the length of the first run in ksplit: each run is in ascending order; its anchors follow one another.
+// Beside the length of the first run in ksplit, for each run: it is in ascending order; its anchors follow one
+// another; its keys are all depth-0 tokens; all deeper ones.
 constexpr int KRUN0_SORTED = 1 << 8, KRUN1_SORTED = 1 << 9, KRUN0_EVEN = 1 << 10, KRUN1_EVEN = 1 << 11;
+constexpr int KRUN0_REAL = 1 << 12, KRUN1_REAL = 1 << 13, KRUN0_CHAIN = 1 << 14, KRUN1_CHAIN = 1 << 15;
 
 // ---- 1. pack metadata, lay out and summarise tiles ---------------------------------------------
 // Block b packs tokens 128 b .. of the sequence and summarises tile b (query tiles first).
@@ -115,10 +117,12 @@ __global__ void __launch_bounds__(128) k0_tiles(Plan p, const int32_t *__restric
             r.w = max(r.w, o.w);
         }
         out[threadIdx.x] = r;
+        int kinds = (r.w == 0 ? KRUN0_REAL : 0) | (r.z >= 1 ? KRUN0_CHAIN : 0);
+        kinds |= __shfl_down_sync(3u, kinds, 1) << 1; // the second run's bits follow the first's
+        if (threadIdx.x == 0 && tile >= p.n_qt)
+            p.ksplit[tile - p.n_qt] =
+                split | kinds | ((KRUN0_SORTED | KRUN1_SORTED | KRUN0_EVEN | KRUN1_EVEN) & ~not_so);
     }
-    if (threadIdx.x == 0 && tile >= p.n_qt)
-        p.ksplit[tile - p.n_qt] =
-            split | ((KRUN0_SORTED | KRUN1_SORTED | KRUN0_EVEN | KRUN1_EVEN) & ~not_so);
 }
 
 // ---- 2. the plan -----------------------------------------------------------------------------
@@ -319,7 +323,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
     __shared__ int2 part[PLAN_GROUPS][BM / 32];       // (allowed pairs, most keys of a row) per warp
     __shared__ int slot_of[PLAN_GROUPS];
     __shared__ uint8_t raw_col[RAW_SINGLE][BM];       // one-key-per-row tiles in arrival order
-    __shared__ int raw_kt[RAW_SINGLE], raw_ord[RAW_SINGLE], raw_conflict[RAW_SINGLE];
+    __shared__ int raw_kt[RAW_SINGLE], raw_start[RAW_SINGLE], raw_ord[RAW_SINGLE], raw_conflict[RAW_SINGLE];
     __shared__ int raw_min[RAW_SINGLE], raw_max[RAW_SINGLE];
     __shared__ int4 pairs[PAIR_CACHE];                // (key tile, first token, length, first run | flags)
     __shared__ int2 entry[RAW_SINGLE];                // sorted raw tiles of an entry: first, last
@@ -394,16 +398,20 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
         key = key_of(w + PLAN_GROUPS);
         // A row allows the keys of its own chain up to its depth, words [anchor << 8, mq], and the
         // depth-0 keys up to its anchor, words up to mq: in a sorted run of one of the two kinds these
-        // are neighbours.
+        // are neighbours, and where the run's anchors follow one another their place is a subtraction.  (With
+        // searches throughout, and the kinds of the runs read from memory pair by pair, this was half of a plan of
+        // 18 us for 391 positions.)
         int mine = 0, col = NO_COL;
 #pragma unroll
         for (int run = 0; run < 2; ++run) {
             const int lo = run == 0 ? 0 : pr.w & 0xff, hi = run == 0 ? pr.w & 0xff : ktile.y;
             if (lo >= hi)
                 continue;
-            const int4 k = p.ksum[2 * kt + run];
-            if ((pr.w & (run == 0 ? KRUN0_SORTED : KRUN1_SORTED)) && (k.w == 0 || k.z >= 1)) {
+            const int flags = pr.w >> run; // the first run's bits are this run's
+            if ((flags & KRUN0_SORTED) && (flags & (KRUN0_REAL | KRUN0_CHAIN))) {
                 auto first_above = [&](int word) { // first key of the run whose word is above `word`
+                    if (flags & KRUN0_EVEN)
+                        return lo + min(max(((word - mk[group][lo]) >> 8) + 1, 0), hi - lo);
                     int a = lo, b = hi;
                     while (a < b) {
                         const int m = (a + b) >> 1;
@@ -415,7 +423,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
                     return a;
                 };
                 const int end = first_above(mq);
-                const int beg = k.w == 0 ? lo : first_above((mq & ~0xff) - 1);
+                const int beg = flags & KRUN0_REAL ? lo : first_above((mq & ~0xff) - 1);
                 if (end > beg) {
                     mine += end - beg;
                     col = end - 1;
@@ -448,6 +456,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
                 slot = atomicAdd(&n_raw, 1);
                 if (slot < RAW_SINGLE) {
                     raw_kt[slot] = kt;
+                    raw_start[slot] = ktile.x;
                     raw_min[slot] = INT_MAX;
                     raw_max[slot] = -1;
                 } else {
@@ -479,6 +488,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
             [&](int kt, int at) {
                 if (at < RAW_SINGLE) {
                     raw_kt[at] = kt;
+                    raw_start[at] = p.ktile[kt].x;
                     raw_min[at] = INT_MAX;
                     raw_max[at] = -1;
                 } else {
@@ -543,13 +553,13 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
         const int2 e = entry[i];
         const int first = raw_ord[e.x], last = raw_ord[e.y];
         const int base = raw_min[first];
-        int col = raw_col[first][row], kt = raw_kt[first];
+        int col = raw_col[first][row], start = raw_start[first];
         if (col == NO_COL && e.y != e.x) {
             col = raw_col[last][row];
-            kt = raw_kt[last];
+            start = raw_start[last];
         }
         if (col != NO_COL)
-            col = p.ktile[kt].x + col - base;
+            col = start + col - base;
         p.scs[((size_t)qt * MAX_SINGLE + i) * BM + row] = (uint8_t)col;
         if (row == 0)
             p.sbase[qt * MAX_SINGLE + i] = base;
@@ -562,11 +572,10 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
             int word = k.y | ((int)cls[kt] << 16);
             if (cls[kt] == TILE_PARTIAL) {
                 const int split = p.ksplit[kt];
-                const int4 a = p.ksum[2 * kt], b = p.ksum[2 * kt + 1];
-                const bool runs = (split & KRUN0_SORTED) && (split & KRUN1_SORTED) && (a.w == 0 || a.z >= 1) &&
-                                  (b.w == 0 || b.z >= 1);
-                word |= (split & 0xff) << 8 | (a.w == 0 ? KLIST_RUN0 : 0) | (b.w == 0 ? KLIST_RUN1 : 0) |
-                        (runs ? KLIST_RUNS : 0) | ((split & KRUN0_EVEN) && (split & KRUN1_EVEN) ? KLIST_EVEN : 0);
+                const bool runs = (split & KRUN0_SORTED) && (split & KRUN1_SORTED) &&
+                                  (split & (KRUN0_REAL | KRUN0_CHAIN)) && (split & (KRUN1_REAL | KRUN1_CHAIN));
+                word |= (split & 0xff) << 8 | (split & KRUN0_REAL ? KLIST_RUN0 : 0) |
+                        (split & KRUN1_REAL ? KLIST_RUN1 : 0) | (runs ? KLIST_RUNS : 0) | ((split & KRUN0_EVEN) && (split & KRUN1_EVEN) ? KLIST_EVEN : 0);
             }
             klist[at] = make_int2(k.x, word);
         });
