@@ -103,6 +103,28 @@ def test_forward_no_visible_keys_at_all(ctx):
     assert torch.all(case.O[:20] == 0) and torch.isneginf(case.LSE[:, :20]).all()
 
 
+@pytest.mark.parametrize("heads", [(4, 1), (3, 1)], ids=["pairs", "odd_group"])
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("gaps", [False, True], ids=["even", "gaps"])
+def test_forward_items_of_every_kind(ctx, heads, D, gaps):
+    """Query tiles that see nothing, several in a row; one-key-per-row entries without any key tile; one and
+    several key tiles with and without entries; masks of runs whose anchors follow one another or have
+    gaps, in tiles that straddle two depths."""
+    n, K = 600, 3
+    anchor, depth = inputs.full_grid(n, K)
+    if gaps:
+        keep = anchor % 7 != 3
+        anchor, depth = anchor[keep], depth[keep]
+    T = anchor.shape[0]
+    n = T // K
+    w = inputs.Workload("kinds", (n,), K, *heads, D, seed=18)
+    for k in ([(2 * n, T)], [(0, 100)], [(0, 130), (2 * n, T)], [(n - 70, T)], [(0, T)]):
+        parts = [{"seq": 0, "q": (0, T), "k": k}]
+        case = DeviceCase(w, anchor=anchor, depth=depth, cu=np.array([0, T], np.int32), parts=parts)
+        run_fwd_all(ctx, case)
+        compare_rows(case, parts[0], np.arange(T))
+
+
 @pytest.mark.parametrize("D", [64, 128])
 def test_rows_of_few_keys_to_fp32_rounding(ctx, D):
     """The first three rows of a sequence see one to three keys, which all take the exact exponential:
