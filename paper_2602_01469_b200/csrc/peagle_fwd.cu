@@ -65,6 +65,11 @@ struct FwdParams {
 template <int D>
 struct FwdCfg {
     static constexpr int NS = (D == 64) ? 3 : 2;
+    // SINGLE entries per pass: at head_dim 64 as many as the ring holds, so that the next ones' K arrives under
+    // these ones' V and their V under that K (4,096 positions, 64 heads: 1,650 against 1,617 us); at 128, where
+    // the ring holds two and O would go through tensor memory between them, all (2,048 positions, 32
+    // heads: 365 against 378).
+    static constexpr int CHUNK = (D == 64) ? NS : MAX_SINGLE;
     static constexpr int PANELS = D / 64;
     static constexpr int PANEL_BYTES = 128 * 128; // 128 rows of 128 bytes
     static constexpr int TILE_BYTES = PANELS * PANEL_BYTES;
@@ -110,53 +115,30 @@ __device__ __forceinline__ uint32_t bits_below(int n)
     asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(max(n, 0))); // clamps: 32 and more give 0
     return r - 1u;
 }
-// The keys of a PARTIAL tile that row mq allows, a bit per key.  In runs in ascending order of one kind each
-// they are neighbours: depth-0 keys up to mq, or the keys of the row's own chain up to mq.  Where the anchors of
-// a run follow one another their place is a subtraction, else a search of eight dependent reads; the rest
-// (shuffled tokens) goes through the predicate for every key.  The warp then passes over the 32 columns that all
-// its rows see.  (The predicate for every element took 2,200 clocks of a PARTIAL tile, as much as all else in it:
-// forward of 500 positions, 64 heads of 64, 114.4 -> 106.7 us; 3,891 positions 1,714 -> 1,648; 391 positions, 32
-// heads of 128, 76.1 -> 74.0.)
+// The keys that row mq allows of a PARTIAL tile with KLIST_EVEN, a bit per key.  In a run of one kind whose anchors
+// follow one another they are neighbours, depth-0 keys up to mq or the keys of the row's own chain up to mq, and
+// their places are subtractions.  A warp then passes over the 32 columns that all its rows see.  (The predicate
+// for every element takes 2,200 clocks of a tile, as much as all else in it: forward of 500 positions, 64 heads
+// of 64, 114.4 -> 106.7 us; 3,891 positions 1,714 -> 1,648.  For the other tiles, of COD sets or anchor-major
+// orders, it stays: searches of eight dependent reads in sorted runs, or bits from the predicate, were slower.)
 __device__ __forceinline__ void row_mask(const int32_t *mk, int word, int32_t mq, uint32_t (&see)[4])
 {
-    if (word & KLIST_RUNS) {
-        const int split = klist_split(word), len = klist_len(word);
-        auto first_above = [&](int lo, int end, int w) { // first key of lo .. end - 1 (1 to 128) above w
-            if (word & KLIST_EVEN)
-                return lo + min(max(((w - mk[lo]) >> 8) + 1, 0), end - lo);
-            int at = lo;
-#pragma unroll
-            for (int s = 128; s > 0; s >>= 1) {
-                const bool below = mk[min(at + s, end) - 1] <= w;
-                at += at + s <= end && below ? s : 0;
-            }
-            return at;
-        };
-        const int own = (mq & ~0xff) - 1; // below the row's chain
-        const int e0 = first_above(0, split, mq), b0 = word & KLIST_RUN0 ? 0 : first_above(0, split, own);
-        int e1 = split, b1 = split;
-        if (split < len) {
-            e1 = first_above(split, len, mq);
-            if (!(word & KLIST_RUN1))
-                b1 = first_above(split, len, own);
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-            see[c] = (bits_below(e0 - 32 * c) & ~bits_below(b0 - 32 * c)) |
-                     (bits_below(e1 - 32 * c) & ~bits_below(b1 - 32 * c));
-    } else {
-#pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
-            uint32_t m = 0;
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-                m |= (uint32_t)allowed_packed(mq, mk[32 * c + i]) << i;
-            see[3] = c == 3 ? m : see[3];
-            see[2] = c == 2 ? m : see[2];
-            see[1] = c == 1 ? m : see[1];
-            see[0] = c == 0 ? m : see[0];
-        }
+    const int split = klist_split(word), len = klist_len(word);
+    auto first_above = [&](int lo, int end, int w) { // first key of lo .. end - 1 above w
+        return lo + min(max(((w - mk[lo]) >> 8) + 1, 0), end - lo);
+    };
+    const int own = (mq & ~0xff) - 1; // below the row's chain
+    const int e0 = first_above(0, split, mq), b0 = word & KLIST_RUN0 ? 0 : first_above(0, split, own);
+    int e1 = split, b1 = split;
+    if (split < len) {
+        e1 = first_above(split, len, mq);
+        if (!(word & KLIST_RUN1))
+            b1 = first_above(split, len, own);
     }
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        see[c] = (bits_below(e0 - 32 * c) & ~bits_below(b0 - 32 * c)) |
+                 (bits_below(e1 - 32 * c) & ~bits_below(b1 - 32 * c));
 }
 
 template <int D>
@@ -314,28 +296,29 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     bulk_load(sb + C::OFF_COL, P.scs + (size_t)qt * MAX_SINGLE * BM, n_single * BM, BAR(B_QFULL));
             }
             __syncwarp();
-            // The key tiles of the SINGLE entries go through the same K / V ring first; the softmax warps read
-            // their rows from shared memory: K of all entries, then V of all entries (so V of the first
-            // NS entries beside K, the others behind).
-            for (int i = 0; live && i < n_single; ++i) {
-                const int start = __shfl_sync(0xffffffffu, window, i);
-                live = stage_free(B_KEMPTY, kpos + i);
-                if (live)
-                    load(C::OFF_K, &tmK, B_KFULL, kpos + i, start);
-                if (live && i < NS) {
+            // The key tiles of the SINGLE entries go through the same K / V ring first, CHUNK at a time, K of all of them and
+            // then V (where a chunk is longer than the ring, the first V beside K); the softmax warps read their
+            // rows from shared memory.
+            for (int c0 = 0; live && c0 < n_single; c0 += C::CHUNK) {
+                const int c1 = min(c0 + C::CHUNK, n_single), beside = C::CHUNK > NS ? min(c1, NS) : c0;
+                for (int i = c0; live && i < c1; ++i) {
+                    const int start = __shfl_sync(0xffffffffu, window, i);
+                    live = stage_free(B_KEMPTY, kpos + i);
+                    if (live)
+                        load(C::OFF_K, &tmK, B_KFULL, kpos + i, start);
+                    if (live && i < beside) {
+                        live = stage_free(B_VEMPTY, kpos + i);
+                        if (live)
+                            load(C::OFF_V, &tmV, B_VFULL, kpos + i, start);
+                    }
+                }
+                for (int i = beside; live && i < c1; ++i) {
+                    const int start = __shfl_sync(0xffffffffu, window, i);
                     live = stage_free(B_VEMPTY, kpos + i);
                     if (live)
                         load(C::OFF_V, &tmV, B_VFULL, kpos + i, start);
                 }
             }
-            for (int i = NS; live && i < n_single; ++i) {
-                const int start = __shfl_sync(0xffffffffu, window, i);
-                live = stage_free(B_VEMPTY, kpos + i);
-                if (live)
-                    load(C::OFF_V, &tmV, B_VFULL, kpos + i, start);
-            }
-            if (live && cnt < 2)
-                next = draw(w + 1);
             // List entries and key metadata are fetched one key tile ahead, so that no global
             // load latency sits between a stage becoming free and its TMA loads.
             auto tile_meta = [&](int2 e, int32_t (&mv)[BN / 32]) {
@@ -371,7 +354,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     smeta[st * BN + lane + 32 * i] = m_cur[i];
                 __syncwarp();
                 load(C::OFF_V, &tmV, B_VFULL, pos, start);
-                if (j + 2 == cnt)
+                if (j + 2 == cnt && cnt > NS)
                     next = draw(w + 1);
                 e_cur = e_nxt;
                 e_nxt = e_nn;
@@ -379,6 +362,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 for (int i = 0; i < BN / 32; ++i)
                     m_cur[i] = m_nxt[i];
             }
+            if (live && cnt <= NS) // short items: no load waits for it
+                next = draw(w + 1);
             kpos += (uint32_t)(n_single + cnt);
             // Hand-over to the backward: the item's rows of the fp32 dQ staging are cleared here, where
             // the memory system is idle (the map ends at the partition's last row).
@@ -447,18 +432,21 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 ok = mbar_wait_warp(BAR(B_QFULL), qn++ & 1, abort_flag);
                 if (ok && cnt == 0)
                     if (lead) mbar_arrive(BAR(B_QEMPTY)); // no product reads this Q
-                // The SINGLE entries come first in the ring: K of all, then V of all.  This warp waits for their
-                // phases one by one, and a stage is not refilled before it has: a parity wait is only
+                // The SINGLE entries come first in the ring, CHUNK at a time, K and then V.  This warp waits for their phases
+                // one by one in that order, and a stage is not refilled before it has: a parity wait is only
                 // meaningful on the phase that follows the last one seen.
-                for (int i = 0; ok && i < n_single; ++i) {
-                    const uint32_t pos = kpos + i;
-                    ok = mbar_wait_warp(BAR(B_KFULL + pos % NS), (pos / NS) & 1, abort_flag);
-                    if (ok && lead) mbar_arrive(BAR(B_KEMPTY + pos % NS));
-                }
-                for (int i = 0; ok && i < n_single; ++i) {
-                    const uint32_t pos = kpos + i;
-                    ok = mbar_wait_warp(BAR(B_VFULL + pos % NS), (pos / NS) & 1, abort_flag);
-                    if (ok && lead) mbar_arrive(BAR(B_VEMPTY + pos % NS));
+                for (int c0 = 0; ok && c0 < n_single; c0 += C::CHUNK) {
+                    const int c1 = min(c0 + C::CHUNK, n_single);
+                    for (int i = c0; ok && i < c1; ++i) {
+                        const uint32_t pos = kpos + i;
+                        ok = mbar_wait_warp(BAR(B_KFULL + pos % NS), (pos / NS) & 1, abort_flag);
+                        if (ok && lead) mbar_arrive(BAR(B_KEMPTY + pos % NS));
+                    }
+                    for (int i = c0; ok && i < c1; ++i) {
+                        const uint32_t pos = kpos + i;
+                        ok = mbar_wait_warp(BAR(B_VFULL + pos % NS), (pos / NS) & 1, abort_flag);
+                        if (ok && lead) mbar_arrive(BAR(B_VEMPTY + pos % NS));
+                    }
                 }
                 if (ok && cnt > 0) {
                     const uint32_t p0 = kpos + n_single;
@@ -562,8 +550,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(pre + 64));
         }
         if (n_single > 0) {
-            // One allowed key per row and entry, on the CUDA cores from the staged K / V rows: the scores of
-            // all entries, then the softmax over them and the weighted values, which become the starting
+            // One allowed key per row and entry, on the CUDA cores from the staged K / V rows, CHUNK entries at a time:
+            // their scores, then the softmax over them and the weighted values, whose sums become the starting
             // (m, l, O) of the tile loop.  A row of Q and a row of O are then not held at the same time, and
             // each of the two passes needs K or V only.  Bound by unpacking bf16 (a row's element is two
             // instructions, one of them packed).  (One pass with an online softmax, O in tensor memory at
@@ -577,7 +565,12 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                                                         (((c & 7) ^ (rr & 7)) << 4));
             };
             auto pair = [](uint32_t w2) { return f2(__uint_as_float(w2 << 16), __uint_as_float(w2 & 0xffff0000u)); };
-            if (ok) {
+#pragma unroll 1
+            for (int c0 = 0; ok && c0 < n_single; c0 += C::CHUNK) {
+            const int c1 = min(c0 + C::CHUNK, n_single);
+            const bool again = C::CHUNK < MAX_SINGLE && c0 > 0;
+            float cm = -CUDART_INF_F; // largest of these scores
+            {
                 F2 q[D / 2];
 #pragma unroll
                 for (int c = 0; c < D / 8; ++c) {
@@ -588,7 +581,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                     q[4 * c + 3] = pair(v.w);
                 }
 #pragma unroll 1
-                for (int i = 0; ok && i < n_single; ++i) {
+                for (int i = c0; ok && i < c1; ++i) {
                     const uint32_t pos = kpos + i;
                     const int st = pos % NS;
                     const int col = cols[i * BM];
@@ -609,22 +602,34 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                         const float2 a = unf2(add_f2(add_f2(acc[0], acc[1]), add_f2(acc[2], acc[3])));
                         s2 = (a.x + a.y) * P.scale_log2;
                     }
-                    score[i * 32] = s2;
-                    m = fmaxf(m, s2);
+                    score[(i - c0) * 32] = s2;
+                    cm = fmaxf(cm, s2);
                     warp_arrive(BAR(B_KEMPTY + st)); // this warp is done with the rows
                 }
             }
-            const float neg_m = m == -CUDART_INF_F ? 0.f : -m;
+            const float m_new = fmaxf(m, cm), neg_m = m_new == -CUDART_INF_F ? 0.f : -m_new;
+            const float alpha = fast_exp2(m + neg_m); // of the sums so far; 0 while there are none
+            m = m_new;
+            l *= alpha;
             F2 o[D / 2];
 #pragma unroll
-            for (int i = 0; i < D / 2; ++i)
-                o[i] = f2(0.f, 0.f);
+            for (int c = 0; c < D / 32; ++c) {
+                uint32_t ov[32];
+                if (again) {
+                    tmem_ld32(tO + c * 32, ov);
+                    tmem_wait_ld();
+                }
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    o[16 * c + i] = again ? mul_f2(f2(__uint_as_float(ov[2 * i]), __uint_as_float(ov[2 * i + 1])), f2(alpha, alpha))
+                                           : f2(0.f, 0.f);
+            }
 #pragma unroll 1
-            for (int i = 0; ok && i < n_single; ++i) {
+            for (int i = c0; ok && i < c1; ++i) {
                 const uint32_t pos = kpos + i;
                 const int st = pos % NS;
                 const int col = cols[i * BM];
-                const float pr = fast_exp2(score[i * 32] + neg_m);
+                const float pr = fast_exp2(score[(i - c0) * 32] + neg_m);
                 ok = mbar_wait_warp(BAR(B_VFULL + st), (pos / NS) & 1, abort_flag);
                 if (!ok)
                     break;
@@ -654,6 +659,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 tmem_st32(tO + c * 32, ov);
             }
             tmem_wait_st(); // ordered before the first P V product by the P hand-over below
+            }
             // Q and the entries' columns are done with (the issuing warps need Q for longer anyway)
             warp_arrive(BAR(B_QEMPTY));
         }
@@ -680,15 +686,29 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 ok = mbar_wait_warp(BAR(B_VFULL + st), ph, abort_flag);
                 if (!ok)
                     break;
-                uint32_t see[4];
-                row_mask(smeta + st * BN, word, mq, see);
+                if (word & KLIST_EVEN) {
+                    uint32_t see[4];
+                    row_mask(smeta + st * BN, word, mq, see);
 #pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    if (!__all_sync(0xffffffffu, see[c] == ~0u)) {
+                    for (int c = 0; c < 4; ++c)
+                        if (!__all_sync(0xffffffffu, see[c] == ~0u)) {
 #pragma unroll
-                        for (int i = 0; i < 32; ++i)
-                            if (!(see[c] >> i & 1u)) xr[c][i] = 0xff800000u;
-                    }
+                            for (int i = 0; i < 32; ++i)
+                                if (!(see[c] >> i & 1u)) xr[c][i] = 0xff800000u;
+                        }
+                } else {
+                    const int4 *mk4 = reinterpret_cast<const int4 *>(smeta + st * BN);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int i = 0; i < 32; i += 4) {
+                            const int4 mk = mk4[(c * 32 + i) >> 2];
+                            if (!allowed_packed(mq, mk.x)) xr[c][i + 0] = 0xff800000u;
+                            if (!allowed_packed(mq, mk.y)) xr[c][i + 1] = 0xff800000u;
+                            if (!allowed_packed(mq, mk.z)) xr[c][i + 2] = 0xff800000u;
+                            if (!allowed_packed(mq, mk.w)) xr[c][i + 3] = 0xff800000u;
+                        }
+                }
             }
             float mx4[4]; // four independent chains of three-input maxima
 #pragma unroll

@@ -32,10 +32,9 @@ static_assert(CNT_ITEMS + BWD_CQ <= PLAN_COUNTERS, "a counter per item size");
 constexpr int NO_COL = 255;      // "this row allows no key of the tile"
 
 // Second word of a key list entry: bits 0-7 length, 8-15 keys in the first run of equal depth, 16-17 class; bit
-// KLIST_RUN0 / KLIST_RUN1: the run's keys are depth-0 tokens; bit KLIST_RUNS: each run is in ascending order and
-// all depth 0 or all deeper, so that the keys of a run which a row allows are neighbours; bit KLIST_EVEN: and the
-// anchors of a run follow one another.  (The bits above the class only where it is PARTIAL.)
-constexpr int KLIST_RUN0 = 1 << 24, KLIST_RUN1 = 1 << 25, KLIST_RUNS = 1 << 26, KLIST_EVEN = 1 << 27;
+// KLIST_RUN0 / KLIST_RUN1: the run's keys are depth-0 tokens; bit KLIST_EVEN: in each run the keys are all depth 0 or
+// all deeper and their anchors follow one another.  (The bits above the class only where it is PARTIAL.)
+constexpr int KLIST_RUN0 = 1 << 24, KLIST_RUN1 = 1 << 25, KLIST_EVEN = 1 << 26;
 __device__ __forceinline__ int klist_len(int word) { return word & 0xff; }
 __device__ __forceinline__ int klist_split(int word) { return word >> 8 & 0xff; }
 __device__ __forceinline__ int klist_class(int word) { return word >> 16 & 3; }

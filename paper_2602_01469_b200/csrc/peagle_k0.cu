@@ -572,10 +572,10 @@ __global__ void __launch_bounds__(PLAN_THREADS) k0_plan(Plan p, int seq_begin, i
             int word = k.y | ((int)cls[kt] << 16);
             if (cls[kt] == TILE_PARTIAL) {
                 const int split = p.ksplit[kt];
-                const bool runs = (split & KRUN0_SORTED) && (split & KRUN1_SORTED) &&
+                const bool even = (split & KRUN0_EVEN) && (split & KRUN1_EVEN) &&
                                   (split & (KRUN0_REAL | KRUN0_CHAIN)) && (split & (KRUN1_REAL | KRUN1_CHAIN));
                 word |= (split & 0xff) << 8 | (split & KRUN0_REAL ? KLIST_RUN0 : 0) |
-                        (split & KRUN1_REAL ? KLIST_RUN1 : 0) | (runs ? KLIST_RUNS : 0) | ((split & KRUN0_EVEN) && (split & KRUN1_EVEN) ? KLIST_EVEN : 0);
+                        (split & KRUN1_REAL ? KLIST_RUN1 : 0) | (even ? KLIST_EVEN : 0);
             }
             klist[at] = make_int2(k.x, word);
         });
