@@ -566,7 +566,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             };
             auto pair = [](uint32_t w2) { return f2(__uint_as_float(w2 << 16), __uint_as_float(w2 & 0xffff0000u)); };
 #pragma unroll 1
-            for (int c0 = 0; ok && c0 < n_single; c0 += C::CHUNK) {
+            for (int c0 = 0; ok && c0 < (C::CHUNK < MAX_SINGLE ? n_single : 1); c0 += C::CHUNK) {
             const int c1 = min(c0 + C::CHUNK, n_single);
             const bool again = C::CHUNK < MAX_SINGLE && c0 > 0;
             float cm = -CUDART_INF_F; // largest of these scores
