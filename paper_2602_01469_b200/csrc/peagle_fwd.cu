@@ -180,10 +180,16 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     // the index, looks the item up and passes it to the other roles through a four-slot queue in shared
     // memory: query tile (negative: no more items), head block, key tiles, SINGLE entries.
     const int heads = ntile; // of a block
-    // Roles other than the producer: item w, query tile -1 at the end (or when a wait ran out).
+    // Every warp of the other roles: item w, query tile -1 at the end (or when a wait ran out).  Each of them hands the
+    // slot back, the issuing warps too: items without keys take no phase of Q, so nothing else keeps the
+    // producer from drawing past a warp that has yet to read the slot.
     auto take = [&](int w) {
         const int slot = w & 3;
-        return mbar_wait_warp(BAR(B_WQFULL + slot), (w >> 2) & 1, abort_flag) ? wq[slot] : make_int4(-1, 0, 0, 0);
+        if (!mbar_wait_warp(BAR(B_WQFULL + slot), (w >> 2) & 1, abort_flag))
+            return make_int4(-1, 0, 0, 0);
+        const int4 e = wq[slot];
+        warp_arrive(BAR(B_WQFREE + slot));
+        return e;
     };
 
     if (threadIdx.x == 0) {
@@ -209,7 +215,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         }
         for (int i = 0; i < 4; ++i) {
             mbar_init(BAR(B_WQFULL + i), 1);
-            mbar_init(BAR(B_WQFREE + i), 4 * ntile); // one arrival per softmax warp
+            mbar_init(BAR(B_WQFREE + i), 5 * ntile); // one arrival per softmax and issuing warp
         }
         // Q may be overwritten once the MMA threads are done with it and every softmax warp has
         // read its rows (or has no use for them).  Items without any key load no Q and have no phase here;
@@ -246,7 +252,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         }
         uint32_t kpos = 0; // position in the K / V ring, running over the items
         bool live = true;
-        // Draws item w once the queue slot's last reader (four items ago) is done.  A chain of an atomic and two
+        // Draws item w once the queue slot's last readers (four items ago) are done.  A chain of an atomic and two
         // dependent loads, 2,000 clocks, so it is started ahead of the last key tile of the item before.
         auto draw = [&](int w) {
             int4 e = make_int4(-1, 0, 0, 0);
@@ -525,9 +531,6 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         // global memory and the draw itself, 1,500 to 3,500 clocks per item before the queue carried the item).
         auto fetch = [&](int w, int32_t &meta) {
             const int4 e = take(w);
-            __syncwarp();
-            if (lane == 0 && e.x >= 0)
-                mbar_arrive(BAR(B_WQFREE + (w & 3))); // this warp has read the queue slot
             const int row = P.q_begin + e.x * BM + r;
             meta = e.x >= 0 && row < P.q_end ? P.meta[row] : META_NONE_Q;
             return e;

@@ -125,6 +125,32 @@ def test_forward_items_of_every_kind(ctx, heads, D, gaps):
         compare_rows(case, parts[0], np.arange(T))
 
 
+@pytest.mark.parametrize("keys", ["chains", "late", "late_and_chains"])
+@pytest.mark.parametrize("D,heads", [(64, (64, 8)), (64, (24, 8)), (128, (32, 4)), (128, (24, 8))],
+                         ids=["d64_pairs", "d64_odd_group", "d128_pairs", "d128_odd_group"])
+def test_forward_many_items_without_keys(ctx, D, heads, keys):
+    """Query tiles that see nothing come last, and here they are five or more to every SM, behind items with
+    one-key-per-row entries only, key tiles only, or both: each CTA goes round its four-slot item queue on items
+    that pass no barrier of Q."""
+    n, K = 2880, 4
+    anchor, depth = inputs.full_grid(n, K)
+    T, late = n * K, 3 * n // 4
+    k = {"chains": [(3 * n, T)], "late": [(late, n)], "late_and_chains": [(late, n), (3 * n, T)]}[keys]
+    sees = ((depth == 3) & ("chains" in keys)) | ((anchor >= late) & ("late" in keys))
+    none = ~sees.reshape(T // 128, 128).any(axis=1)
+    blocks = heads[0] // 2 if (heads[0] // heads[1]) % 2 == 0 else heads[0]
+    assert none.sum() * blocks >= 5 * torch.cuda.get_device_properties(0).multi_processor_count
+    parts = [{"seq": 0, "q": (0, T), "k": k}]
+    w = inputs.Workload("empty_items", (n,), K, *heads, D, seed=19)
+    case = DeviceCase(w, anchor=anchor, depth=depth, cu=np.array([0, T], np.int32), parts=parts)
+    run_fwd_all(ctx, case)
+    blind = torch.as_tensor(~sees, device="cuda")
+    assert torch.all(case.O[blind] == 0) and torch.isneginf(case.LSE[:, blind]).all()
+    assert torch.isfinite(case.LSE[:, ~blind]).all() and torch.isfinite(case.O.float()).all()
+    edges = np.concatenate([[t, t + 127] for t in range(0, T, 1280)])
+    compare_rows(case, parts[0], np.unique(np.concatenate([edges, [late - 1, late, n - 1, 3 * n, T - 1]])))
+
+
 @pytest.mark.parametrize("D", [64, 128])
 def test_rows_of_few_keys_to_fp32_rounding(ctx, D):
     """The first three rows of a sequence see one to three keys, which all take the exact exponential:
