@@ -180,13 +180,14 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     // the index, looks the item up and passes it to the other roles through a four-slot queue in shared
     // memory: query tile (negative: no more items), head block, key tiles, SINGLE entries.
     const int heads = ntile; // of a block
-    // Every warp of the other roles: item w, query tile -1 at the end (or when a wait ran out).  Each of them hands the
+    // Every warp of the other roles: item w, query tile -1 at the end, GONE when a wait ran out.  Each of them hands the
     // slot back, the issuing warps too: items without keys take no phase of Q, so nothing else keeps the
     // producer from drawing past a warp that has yet to read the slot.
+    constexpr int GONE = -2;
     auto take = [&](int w) {
         const int slot = w & 3;
         if (!mbar_wait_warp(BAR(B_WQFULL + slot), (w >> 2) & 1, abort_flag))
-            return make_int4(-1, 0, 0, 0);
+            return make_int4(GONE, 0, 0, 0);
         const int4 e = wq[slot];
         warp_arrive(BAR(B_WQFREE + slot));
         return e;
@@ -526,7 +527,6 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         uint32_t t = 0;    // key tiles of this tile so far (phases of S, P, PV)
         int qn = 0;        // items with keys so far (phases of Q)
         uint32_t n_turn = 0; // items with key tiles so far
-        bool ok = true;
         // Item w, and its row's metadata, are fetched ahead of the epilogue of item w - 1 (two dependent reads of
         // global memory and the draw itself, 1,500 to 3,500 clocks per item before the queue carried the item).
         auto fetch = [&](int w, int32_t &meta) {
@@ -535,8 +535,16 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             meta = e.x >= 0 && row < P.q_end ? P.meta[row] : META_NONE_Q;
             return e;
         };
+        // At head_dim 64 a tile's four warps meet at named barriers, which know no limit.  So once per item they agree,
+        // at such a barrier, whether all of them go on to the next: one whose wait ran out would leave the others
+        // there for good.
+        auto together = [&](bool on) {
+            __syncwarp();
+            return C::O_STAGED ? bar_and(1 + x, 128, on) : on;
+        };
         int32_t mq;
         int4 item = fetch(0, mq);
+        bool ok = together(item.x != GONE);
         for (int w = 0; ok && item.x >= 0; ++w) {
         const int qt = item.x, h0 = item.y * heads, cnt = item.z, n_single = item.w;
         const int2 *klist = P.klist + (size_t)qt * P.n_kt;
@@ -851,17 +859,14 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
                 P.nl2[hand] = -CUDART_INF_F;
                 P.nd[hand] = 0.f;
             }
+            ok = together(item_next.x != GONE);
         } else if ([&] {
-                       bool fin = ok && (cnt == 0 || mbar_wait_warp(BAR(B_PVDONE + x), (t + cnt - 1) & 1, abort_flag));
-                       if constexpr (C::O_STAGED) {
-                           // the four warps of the tile go on together (they meet at a barrier
-                           // below); before that, the staging tile of the previous item must
-                           // have left shared memory
-                           if (r == 0)
-                               bulk_wait_group_read<0>();
-                           fin = bar_and(1 + x, 128, fin);
-                       }
-                       return fin;
+                       const bool fin = ok && item_next.x != GONE &&
+                                        (cnt == 0 || mbar_wait_warp(BAR(B_PVDONE + x), (t + cnt - 1) & 1, abort_flag));
+                       // the staging tile of the previous item must have left shared memory
+                       if (C::O_STAGED && r == 0)
+                           bulk_wait_group_read<0>();
+                       return together(fin);
                    }()) {
             tc_fence_after();
             // A row with no key in any of its tiles has m = -inf, but not l = 0: the cubic never goes below
