@@ -265,7 +265,9 @@ int peagle_rope_qkv_bwd(peagle_ctx *ctx, const void *dQ, const void *dK, const v
  * A(m, k) is A[m * lda + k], or A[k * lda + m] when a_transposed; B(n, k) is B[n * ldb + k], or
  * B[k * ldb + n] when b_transposed.  With c_fp32_accumulate == 0, C is bf16 [M][ldc] and is
  * written; otherwise C is fp32 [M][ldc] and the product is ADDED to it (launches on one stream are
- * ordered; two calls that add into the same C from different streams race).  All dev, 16-byte
+ * ordered; two calls that add into the same C from different streams race).  Such sums do not repeat
+ * to the last bit: several blocks may share an element and add their parts of its sum in any order
+ * (a C with few tiles or a partly filled last wave of them, and K long enough).  All dev, 16-byte
  * aligned; lda, ldb, ldc (elements) and N multiples of 8; K >= 1.  Elements outside M x N are not
  * touched.  So a linear layer Y = X W^T with W [d_out][d_in] is (A = X, B = W); its input gradient
  * dX = dY W is (A = dY, B = W transposed, K = d_out); its weight gradient dW += dY^T X is

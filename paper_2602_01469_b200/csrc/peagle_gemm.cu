@@ -50,6 +50,7 @@ struct GemmParams {
     int M, N, K;
     int a_t, b_t;  // 1: operand stored transposed (MN-major)
     int c_f32_add; // 0: C bf16, stored; 1: C fp32, added to
+    int shares;    // gemm2_kernel: how many shares the last wave is dealt out in; 0: whole tiles
     void *C;
     long long ldc;
     int *status;
@@ -269,27 +270,24 @@ struct Gemm2Cfg {
     static_assert(N_BAR * 8 + 32 <= 1024 && SMEM <= 227 * 1024, "shared memory of one CTA");
 };
 
-// A pair's work: whole tiles in waves of n_pairs, then, where C is added to, its share of the last, partly
-// filled wave, whose k slabs are dealt out evenly: the pairs that share a tile add their parts to C one after
-// the other.  Whole waves stay whole because the pairs then walk k together and find each other's slabs in L2.  A
-// share is at least MIN_SHARE slabs, since every part of a tile costs an epilogue of about ten.  The order of the
-// parts is not fixed, so the last bit of such a tile may differ from run to run.  (dW of 5,120 x 2,880 over 32,768
-// rows: 240 tiles on 74 pairs, 3.24 instead of 4 waves; projection, rotary kernels and their backward for these
-// sizes 2,561 -> 2,463 us.)
+// A pair's work: whole tiles in waves of n_pairs, then, where that pays (deal_last_wave), its share of the last,
+// partly filled wave, whose k slabs are dealt out.  Pairs that share a tile add their parts to C in no fixed
+// order, so the last bits of such a tile may differ from run to run.  Whole waves stay whole because the pairs
+// then walk k together and find each other's slabs in L2.
 struct PairWalk {
-    static constexpr int MIN_SHARE = 8;
     int t, i0, i1; // the segment: tile, k slabs i0 .. i1 - 1
-    int w = 0, waves, rest, u, u1;
+    int w = 0, waves, rest, u = 0, u1 = 0;
     int pair, n_pairs, n_k;
-    __device__ PairWalk(int pair_, int n_pairs_, int n_tiles, int n_k_, bool deal)
+    __device__ PairWalk(int pair_, int n_pairs_, int n_tiles, int n_k_, int shares)
         : pair(pair_), n_pairs(n_pairs_), n_k(n_k_)
     {
-        waves = deal ? n_tiles / n_pairs : (n_tiles - pair + n_pairs - 1) / n_pairs;
+        waves = shares ? n_tiles / n_pairs : (n_tiles - pair + n_pairs - 1) / n_pairs;
         rest = waves * n_pairs; // first tile of the part that is dealt out
-        const long long units = deal ? (long long)(n_tiles - rest) * n_k : 0;
-        const int shares = (int)min((long long)n_pairs, max(1ll, units / MIN_SHARE));
-        u = pair < shares ? (int)(units * pair / shares) : 0;
-        u1 = pair < shares ? (int)(units * (pair + 1) / shares) : 0;
+        if (pair < shares) {
+            const long long units = (long long)(n_tiles - rest) * n_k;
+            u = (int)(units * pair / shares);
+            u1 = (int)(units * (pair + 1) / shares);
+        }
     }
     __device__ bool next()
     {
@@ -308,6 +306,30 @@ struct PairWalk {
         return true;
     }
 };
+
+// Into how many shares the tiles of the last wave are dealt out, 0 for whole tiles.  Figures: us of one product
+// into an fp32 C, both operands transposed, 74 pairs.
+//  - Every tile in equal parts, one part to a pair: as many as there are pairs for, of at least MIN_SHARE slabs.  An
+//    epilogue per pair as with whole tiles, and the parts keep step.  (5,120 x 2,880, 18 tiles left: inner
+//    dimension 1,024 34.9 -> 32.9, 32,768 1,014 -> 816; parts of 4 slabs, 512 x 1,024 x 576: 18.6 -> 22.6.)
+//  - All slabs evenly, over the tiles' borders: a pair then has up to two epilogues, EPILOGUE slabs together with the
+//    loss of step.  Taken where it saves more than that and two ninths of the time.  (2,560 x 1,024, 40 tiles: inner
+//    1,536 17.5 -> 18.5, 4,096 30.8 -> 24.7; 8,704 x 1,024, 62 tiles left: inner 32,768 513 -> 559.)  Where the inner
+//    dimension is LONG the pairs drift too far apart for L2 unless a third is saved.  (8,192 x 1,024, 54 tiles left:
+//    inner 20,480 320 -> 288, 65,536 960 -> 1,040; 48 tiles and fewer: 1.01 to 1.3 times faster.)
+int deal_last_wave(long long tiles, long long fit, long long n_k)
+{
+    constexpr long long EPILOGUE = 18, MIN_SHARE = 8, LONG = 400; // in slabs
+    const long long left = tiles % fit;
+    if (left == 0)
+        return 0;
+    const long long parts = std::min(fit / left, n_k / MIN_SHARE);
+    const long long in_parts = parts < 2 ? n_k : (n_k + parts - 1) / parts;
+    const long long share = std::max((left * n_k + fit - 1) / fit, MIN_SHARE);
+    if (share + EPILOGUE < in_parts && 9 * share <= 7 * in_parts && (n_k <= LONG || 3 * share <= 2 * in_parts))
+        return (int)((left * n_k + share - 1) / share);
+    return parts < 2 ? 0 : (int)(left * parts);
+}
 
 __global__ void __launch_bounds__(192, 1)
 gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -331,7 +353,7 @@ gemm2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     const int n_k = (P.K + GK - 1) / GK;
     const int tiles_n = (P.N + NT - 1) / NT;
     const int n_tiles = tiles_n * ((P.M + 2 * GT - 1) / (2 * GT));
-    PairWalk work((int)blockIdx.x >> 1, (int)gridDim.x >> 1, n_tiles, n_k, P.c_f32_add != 0);
+    PairWalk work((int)blockIdx.x >> 1, (int)gridDim.x >> 1, n_tiles, n_k, P.shares);
 
     if (threadIdx.x == 0) {
         *abort_flag = 0;
@@ -567,6 +589,7 @@ int launch_gemm(EncodeTiledFn enc, const void *A, long long lda, int a_t, const 
     P.C = C;
     P.ldc = ldc;
     P.status = status;
+    P.shares = 0;
     int dev = 0, n_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -591,9 +614,9 @@ int launch_gemm(EncodeTiledFn enc, const void *A, long long lda, int a_t, const 
         if (cudaOccupancyMaxActiveClusters(&fit, gemm2_kernel, &cfg) != cudaSuccess || fit < 1)
             return PEAGLE_ERR_CUDA;
         const long long tiles2 = (long long)((N + 255) / 256) * ((M + 255) / 256);
-        // an added-to C takes as many pairs as its slabs fill (see PairWalk)
-        const long long parts = c_f32_add ? std::max(tiles2, tiles2 * ((K + GK - 1) / GK) / PairWalk::MIN_SHARE) : tiles2;
-        const long long n_pairs = parts < fit ? parts : fit;
+        if (c_f32_add)
+            P.shares = deal_last_wave(tiles2, fit, (K + GK - 1) / GK);
+        const long long n_pairs = std::min<long long>(std::max<long long>(tiles2, P.shares), fit);
         cfg.gridDim = dim3((unsigned)(2 * n_pairs));
         // fp32 C as a tensor for the tiled reduce-adds: 32 columns (128 bytes) x 128 rows
         CUtensorMap tmC = tmA;

@@ -25,7 +25,9 @@ def rand_bf16(shape, seed):
 @pytest.mark.parametrize("M,N,K", [(128, 128, 64), (200, 264, 200), (1, 8, 8), (513, 1024, 2880), (300, 72, 1000),
                                    (300, 1160, 520),   # wide tiles with a ragged last column of tiles
                                    (200, 1024, 136),   # one pair of CTAs whose second CTA holds 72 rows
-                                   (4808, 1024, 1000)])  # a whole wave of pairs, and two tiles dealt out in parts
+                                   (4808, 1024, 1000),  # a whole wave of pairs, and two tiles dealt out in parts
+                                   (4808, 1024, 200),   # the same with too few slabs to deal out
+                                   (2500, 1024, 2700)])  # 40 tiles dealt out in shares that cross their borders
 @pytest.mark.parametrize("a_t,b_t", [(0, 0), (0, 1), (1, 1), (1, 0)])
 def test_products_match_fp64(ctx, M, N, K, a_t, b_t):
     def pad8(x):
