@@ -442,7 +442,8 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                 // (their results were consumed in its last step), so the old copy is not in use.
                 const int ks = w & 1;
                 // (The other group's last S^T / dP^T must be complete as well.)
-                ok = (mbar_wait_warp(BAR(B_KVFULL + ks), (w >> 1) & 1, abort_flag) && (it == 0 || mbar_wait_warp(BAR(wg == 0 ? B_SFULL + 1 : B_DPFULL), (it - 1) & 1, abort_flag)));
+                ok = mbar_wait_warp(BAR(B_KVFULL + ks), (w >> 1) & 1, abort_flag) &&
+                     (it == 0 || mbar_wait_warp(BAR(wg == 0 ? B_SFULL + 1 : B_DPFULL), (it - 1) & 1, abort_flag));
                 if (!ok)
                     break;
                 const uint8_t *src = sp + C::OFF_KV + (wg == 0 ? ks : 2) * TB + r * 128;
@@ -540,7 +541,8 @@ bwd64_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             warp_arrive(BAR(B_PFULL + wg));
             // ---- dS^T
             // (and dQ of the previous step has run, so that the dS^T panel is free)
-            ok = (mbar_wait_warp(BAR(B_DPFULL + wg), it & 1, abort_flag) && (it == 0 || mbar_wait_warp(BAR(B_DQFULL), (it - 1) & 1, abort_flag)));
+            ok = mbar_wait_warp(BAR(B_DPFULL + wg), it & 1, abort_flag) &&
+                 (it == 0 || mbar_wait_warp(BAR(B_DQFULL), (it - 1) & 1, abort_flag));
             if (!ok)
                 break;
             tc_fence_after();

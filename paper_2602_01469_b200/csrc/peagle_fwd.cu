@@ -10,10 +10,10 @@
 //   warps 0-3  softmax of tile A (one query row per thread; online softmax in the log2 domain,
 //              log-sum-exp bookkeeping, final normalisation and store)
 //   warps 4-7  softmax of tile B
-//              (head_dim 64: the normalised O tile goes to shared memory and leaves by one tiled
-//              store per tile instead of 32 scattered 16-byte pieces per store instruction)
-//   warp  8    allocates tensor memory; lane 0 issues the MMAs of tile A
-//   warp  10   lane 0 issues the MMAs of tile B
+//              (rows of O leave through shared memory: at head_dim 64 by one tiled store per tile, at 128
+//              32 rows by 32 columns at a time; not as 32 scattered 16-byte pieces per store instruction)
+//   warp  8    allocates tensor memory; its elected lane issues the MMAs of tile A
+//   warp  10   its elected lane issues the MMAs of tile B
 //   warp  9    producer: draws the items; TMA loads of Q per item and of the K / V tiles
 //              through a ring, plus the packed metadata of each key tile for the implicit mask
 // Tensor memory (512 columns x 128 lanes, fp32): S_A | S_B (128 columns each), O_A | O_B
@@ -23,8 +23,8 @@
 // S = Q K^T takes both operands from shared memory (K-major, 128-byte swizzle); O += P V takes
 // P from tensor memory and V from shared memory (MN-major).
 // Only tiles the classifier kept are visited; FULL tiles skip the per-element predicate; SINGLE
-// tiles (one allowed key per row) pass through the same ring first and are done pair by pair on
-// the CUDA cores, their result seeding the running (m, l, O).
+// entries (windows with one allowed key per row) pass through the same ring first and are done on the CUDA
+// cores in two passes, scores and weighted values, their result seeding the running (m, l, O).
 #include <math_constants.h>
 
 #include <algorithm>
@@ -66,10 +66,11 @@ template <int D>
 struct FwdCfg {
     static constexpr int NS = (D == 64) ? 3 : 2;
     // SINGLE entries per pass: at head_dim 64 as many as the ring holds, so that the next ones' K arrives under
-    // these ones' V and their V under that K (4,096 positions, 64 heads: 1,650 against 1,617 us); at 128, where
+    // these ones' V and their V under that K (4,096 positions, 64 heads: 1,617 us, all at once 1,650); at 128, where
     // the ring holds two and O would go through tensor memory between them, all (2,048 positions, 32
-    // heads: 365 against 378).
+    // heads: 365 us, as many as the ring holds 378).
     static constexpr int CHUNK = (D == 64) ? NS : MAX_SINGLE;
+    static constexpr bool ONE_CHUNK = CHUNK >= MAX_SINGLE;
     static constexpr int PANELS = D / 64;
     static constexpr int PANEL_BYTES = 128 * 128; // 128 rows of 128 bytes
     static constexpr int TILE_BYTES = PANELS * PANEL_BYTES;
@@ -78,7 +79,8 @@ struct FwdCfg {
     static constexpr int OFF_V = OFF_K + NS * TILE_BYTES;
     // head_dim 64: the finished O tiles leave through shared memory and a tiled store (a thread
     // that writes its own row puts 32 separate 16-byte pieces into every store instruction of its
-    // warp); head_dim 128 has no room for the two staging tiles and stores its rows directly
+    // warp); head_dim 128 has no room for the two staging tiles: its rows pass through 2 KB per warp
+    // and leave by plain stores of four neighbouring lanes to a row
     static constexpr bool O_STAGED = (D == 64);
     static constexpr int OFF_OST = OFF_V + NS * TILE_BYTES;
     // ZERO_ROWS x 32 fp32 zeros, the source of the stores that clear the backward's dQ staging
@@ -386,7 +388,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             bulk_wait_group<0>();
     } else if (warp == 8 || warp == 10) {
         // ------------------------------------------------------------ MMA issue
-        // Lane 0 of warp 8 issues every MMA of tile A, lane 0 of warp 10 those of tile B: the two
+        // One lane of warp 8 issues every MMA of tile A, one of warp 10 those of tile B: the two
         // tiles are independent instruction streams (they only share the K / V stages, which are
         // released once both threads have committed), and two threads issue twice as fast as one.
         const int x = (warp - 8) >> 1;
@@ -577,99 +579,99 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             };
             auto pair = [](uint32_t w2) { return f2(__uint_as_float(w2 << 16), __uint_as_float(w2 & 0xffff0000u)); };
 #pragma unroll 1
-            for (int c0 = 0; ok && c0 < (C::CHUNK < MAX_SINGLE ? n_single : 1); c0 += C::CHUNK) {
-            const int c1 = min(c0 + C::CHUNK, n_single);
-            const bool again = C::CHUNK < MAX_SINGLE && c0 > 0;
-            float cm = -CUDART_INF_F; // largest of these scores
-            {
-                F2 q[D / 2];
+            for (int c0 = 0; ok && c0 < (C::ONE_CHUNK ? 1 : n_single); c0 += C::CHUNK) {
+                const int c1 = min(c0 + C::CHUNK, n_single);
+                const bool again = !C::ONE_CHUNK && c0 > 0;
+                float cm = -CUDART_INF_F; // largest of these scores
+                {
+                    F2 q[D / 2];
 #pragma unroll
-                for (int c = 0; c < D / 8; ++c) {
-                    const uint4 v = row_piece(C::OFF_Q + x * C::TILE_BYTES, r, c);
-                    q[4 * c] = pair(v.x);
-                    q[4 * c + 1] = pair(v.y);
-                    q[4 * c + 2] = pair(v.z);
-                    q[4 * c + 3] = pair(v.w);
+                    for (int c = 0; c < D / 8; ++c) {
+                        const uint4 v = row_piece(C::OFF_Q + x * C::TILE_BYTES, r, c);
+                        q[4 * c] = pair(v.x);
+                        q[4 * c + 1] = pair(v.y);
+                        q[4 * c + 2] = pair(v.z);
+                        q[4 * c + 3] = pair(v.w);
+                    }
+#pragma unroll 1
+                    for (int i = c0; ok && i < c1; ++i) {
+                        const uint32_t pos = kpos + i;
+                        const int st = pos % NS;
+                        const int col = cols[i * BM];
+                        ok = mbar_wait_warp(BAR(B_KFULL + st), (pos / NS) & 1, abort_flag);
+                        if (!ok)
+                            break;
+                        float s2 = -CUDART_INF_F;
+                        if (col != NO_COL && row_ok) {
+                            F2 acc[4]; // four chains of dependent adds
+#pragma unroll
+                            for (int c = 0; c < D / 8; ++c) {
+                                const uint4 v = row_piece(C::OFF_K + st * C::TILE_BYTES, col, c);
+                                const uint32_t kw[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                                for (int k = 0; k < 4; ++k)
+                                    acc[k] = c == 0 ? mul_f2(q[k], pair(kw[k])) : fma_f2(q[4 * c + k], pair(kw[k]), acc[k]);
+                            }
+                            const float2 a = unf2(add_f2(add_f2(acc[0], acc[1]), add_f2(acc[2], acc[3])));
+                            s2 = (a.x + a.y) * P.scale_log2;
+                        }
+                        score[(i - c0) * 32] = s2;
+                        cm = fmaxf(cm, s2);
+                        warp_arrive(BAR(B_KEMPTY + st)); // this warp is done with the rows
+                    }
+                }
+                const float m_new = fmaxf(m, cm), neg_m = m_new == -CUDART_INF_F ? 0.f : -m_new;
+                const float alpha = fast_exp2(m + neg_m); // of the sums so far; 0 while there are none
+                m = m_new;
+                l *= alpha;
+                F2 o[D / 2];
+#pragma unroll
+                for (int c = 0; c < D / 32; ++c) {
+                    uint32_t ov[32];
+                    if (again) {
+                        tmem_ld32(tO + c * 32, ov);
+                        tmem_wait_ld();
+                    }
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        o[16 * c + i] = again ? mul_f2(f2(__uint_as_float(ov[2 * i]), __uint_as_float(ov[2 * i + 1])), f2(alpha, alpha))
+                                               : f2(0.f, 0.f);
                 }
 #pragma unroll 1
                 for (int i = c0; ok && i < c1; ++i) {
                     const uint32_t pos = kpos + i;
                     const int st = pos % NS;
                     const int col = cols[i * BM];
-                    ok = mbar_wait_warp(BAR(B_KFULL + st), (pos / NS) & 1, abort_flag);
+                    const float pr = fast_exp2(score[(i - c0) * 32] + neg_m);
+                    ok = mbar_wait_warp(BAR(B_VFULL + st), (pos / NS) & 1, abort_flag);
                     if (!ok)
                         break;
-                    float s2 = -CUDART_INF_F;
                     if (col != NO_COL && row_ok) {
-                        F2 acc[4]; // four chains of dependent adds
+                        l += pr;
+                        const F2 pp = f2(pr, pr);
 #pragma unroll
                         for (int c = 0; c < D / 8; ++c) {
-                            const uint4 v = row_piece(C::OFF_K + st * C::TILE_BYTES, col, c);
-                            const uint32_t kw[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                            for (int k = 0; k < 4; ++k)
-                                acc[k] = c == 0 ? mul_f2(q[k], pair(kw[k])) : fma_f2(q[4 * c + k], pair(kw[k]), acc[k]);
+                            const uint4 v = row_piece(C::OFF_V + st * C::TILE_BYTES, col, c);
+                            o[4 * c] = fma_f2(pp, pair(v.x), o[4 * c]);
+                            o[4 * c + 1] = fma_f2(pp, pair(v.y), o[4 * c + 1]);
+                            o[4 * c + 2] = fma_f2(pp, pair(v.z), o[4 * c + 2]);
+                            o[4 * c + 3] = fma_f2(pp, pair(v.w), o[4 * c + 3]);
                         }
-                        const float2 a = unf2(add_f2(add_f2(acc[0], acc[1]), add_f2(acc[2], acc[3])));
-                        s2 = (a.x + a.y) * P.scale_log2;
                     }
-                    score[(i - c0) * 32] = s2;
-                    cm = fmaxf(cm, s2);
-                    warp_arrive(BAR(B_KEMPTY + st)); // this warp is done with the rows
-                }
-            }
-            const float m_new = fmaxf(m, cm), neg_m = m_new == -CUDART_INF_F ? 0.f : -m_new;
-            const float alpha = fast_exp2(m + neg_m); // of the sums so far; 0 while there are none
-            m = m_new;
-            l *= alpha;
-            F2 o[D / 2];
-#pragma unroll
-            for (int c = 0; c < D / 32; ++c) {
-                uint32_t ov[32];
-                if (again) {
-                    tmem_ld32(tO + c * 32, ov);
-                    tmem_wait_ld();
+                    warp_arrive(BAR(B_VEMPTY + st));
                 }
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    o[16 * c + i] = again ? mul_f2(f2(__uint_as_float(ov[2 * i]), __uint_as_float(ov[2 * i + 1])), f2(alpha, alpha))
-                                           : f2(0.f, 0.f);
-            }
-#pragma unroll 1
-            for (int i = c0; ok && i < c1; ++i) {
-                const uint32_t pos = kpos + i;
-                const int st = pos % NS;
-                const int col = cols[i * BM];
-                const float pr = fast_exp2(score[(i - c0) * 32] + neg_m);
-                ok = mbar_wait_warp(BAR(B_VFULL + st), (pos / NS) & 1, abort_flag);
-                if (!ok)
-                    break;
-                if (col != NO_COL && row_ok) {
-                    l += pr;
-                    const F2 pp = f2(pr, pr);
+                for (int c = 0; c < D / 32; ++c) {
+                    uint32_t ov[32];
 #pragma unroll
-                    for (int c = 0; c < D / 8; ++c) {
-                        const uint4 v = row_piece(C::OFF_V + st * C::TILE_BYTES, col, c);
-                        o[4 * c] = fma_f2(pp, pair(v.x), o[4 * c]);
-                        o[4 * c + 1] = fma_f2(pp, pair(v.y), o[4 * c + 1]);
-                        o[4 * c + 2] = fma_f2(pp, pair(v.z), o[4 * c + 2]);
-                        o[4 * c + 3] = fma_f2(pp, pair(v.w), o[4 * c + 3]);
+                    for (int i = 0; i < 16; ++i) {
+                        const float2 v = unf2(o[16 * c + i]);
+                        ov[2 * i] = __float_as_uint(v.x);
+                        ov[2 * i + 1] = __float_as_uint(v.y);
                     }
+                    tmem_st32(tO + c * 32, ov);
                 }
-                warp_arrive(BAR(B_VEMPTY + st));
-            }
-#pragma unroll
-            for (int c = 0; c < D / 32; ++c) {
-                uint32_t ov[32];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const float2 v = unf2(o[16 * c + i]);
-                    ov[2 * i] = __float_as_uint(v.x);
-                    ov[2 * i + 1] = __float_as_uint(v.y);
-                }
-                tmem_st32(tO + c * 32, ov);
-            }
-            tmem_wait_st(); // ordered before the first P V product by the P hand-over below
+                tmem_wait_st(); // ordered before the first P V product by the P hand-over below
             }
             // Q and the entries' columns are done with (the issuing warps need Q for longer anyway)
             warp_arrive(BAR(B_QEMPTY));
@@ -765,10 +767,10 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             // Left alone the two tiles' warps of a scheduler fall into step: both do exponentials at once and both wait
             // at once, with the exp2 unit idle for half of the time.  It is enough that tile B's first
             // exponentials of an item start behind tile A's: the distance lasts, and a hand-over per tile costs more
-            // than it gives (3,891 positions, 64 heads of 64: 1,660 us in step, 1,547 apart, 1,737 with a turn per
-            // tile; 2,048 positions, 32 heads of 128: 346 with turns, 336 so).  Tile A waits for tile B's first
-            // turn of the item before, which is long past, so that no warp is ever two phases ahead of another's
-            // wait.
+            // than it gives (one set of inputs again and again, 3,891 positions, 64 heads of 64: 1,660 us in step,
+            // 1,547 apart, 1,737 with a turn per tile; 2,048 positions, 32 heads of 128: 346 with turns, 336 so).
+            // Tile A waits for tile B's first turn of the item before, which is long past, so that no warp is ever
+            // two phases ahead of another's wait.
             if (P.two && j == 0 && (x == 1 || n_turn > 0)) {
                 ok = mbar_wait_warp(BAR(B_TURN + 4 * x + (warp & 3)), (x == 1 ? n_turn : n_turn - 1) & 1, abort_flag);
                 if (!ok)
@@ -779,8 +781,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             // that arguments, exponentials and sums all stay packed pairs (every fourth column: 190 more
             // instructions per tile, 3,891 positions, 64 heads of 64: 1,815 against 1,633 us; three
             // eighths 1,790).  The cubic is 7e-5 off at argument 0, so which columns take it decides how
-            // exact the first rows of a sequence are, whose few keys stand in the first columns: rows of
-            // up to six keys are exact to fp32 rounding.
+            // exact the first rows of a sequence are, whose few keys stand in the first columns: depth-0 rows of
+            // up to six keys that begin a tile are exact to fp32 rounding.
             const F2 scale2 = f2(P.scale_log2, P.scale_log2), nm2 = f2(neg_m, neg_m);
             F2 sum2[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
 #pragma unroll

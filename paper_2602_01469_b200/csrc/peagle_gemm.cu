@@ -10,7 +10,7 @@
 //   input grad   dX = dY W       A = dY [rows][d_out] K-major,  B = W [d_out][d_in] MN-major (k = d_out)
 //   weight grad  dW = dY^T X     A = dY [rows][d_out] MN-major, B = X [rows][d_in]  MN-major (k = rows)
 // Persistent CTAs take 128 x 128 or 128 x 256 tiles of C in turn: warp 0 loads 64-wide k slabs of A
-// and B by TMA into a ring of stages (128-byte swizzle), warp 1 lane 0 issues tcgen05.mma (four
+// and B by TMA into a ring of stages (128-byte swizzle), one lane of warp 1 issues tcgen05.mma (four
 // k = 16 products per slab) into one of two accumulators in tensor memory and releases the stages
 // by commits, warps 2-5 read an accumulator when its last commit arrives, hand it back as soon as
 // it is in registers, and either store bf16 rows or add into an fp32 C (in gemm_kernel the tiles of one launch

@@ -107,9 +107,9 @@ def test_forward_no_visible_keys_at_all(ctx):
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("gaps", [False, True], ids=["even", "gaps"])
 def test_forward_items_of_every_kind(ctx, heads, D, gaps):
-    """Query tiles that see nothing, several in a row; one-key-per-row entries without any key tile; one and
-    several key tiles with and without entries; masks of runs whose anchors follow one another or have
-    gaps, in tiles that straddle two depths."""
+    """Query tiles that see nothing; one-key-per-row entries without any key tile; one and several key tiles
+    with and without entries; masks of runs whose anchors follow one another or have gaps, in tiles that
+    straddle two depths.  (There are fewer items than SMs: a CTA takes one.)"""
     n, K = 600, 3
     anchor, depth = inputs.full_grid(n, K)
     if gaps:
@@ -151,16 +151,17 @@ def test_forward_many_items_without_keys(ctx, D, heads, keys):
     compare_rows(case, parts[0], np.unique(np.concatenate([edges, [late - 1, late, n - 1, 3 * n, T - 1]])))
 
 
+@pytest.mark.parametrize("K", [1, 4])
 @pytest.mark.parametrize("D", [64, 128])
-def test_rows_of_few_keys_to_fp32_rounding(ctx, D):
-    """The first three rows of a sequence see one to three keys, which all take the exact exponential:
+def test_rows_of_few_keys_to_fp32_rounding(ctx, D, K):
+    """The first six rows of a sequence see one to six keys, which all take the exact exponential:
     what is left is fp32 rounding of a score below 8 in magnitude (the dot product of D terms, 2^-24
     relative for each of its partial sums: 8 D 2^-24 <= 6e-5 at worst, about sqrt(D) 2^-24 x 8 = 5e-6 in
     practice) and of exp2 / log2 (2^-22).  The cubic that a quarter of the columns takes is 7e-5 off."""
-    case = DeviceCase(inputs.Workload("few_keys", (70, 130), 1, 4, 2, D, seed=51))
+    case = DeviceCase(inputs.Workload("few_keys", (70, 130), K, 4, 2, D, seed=51))
     run_fwd_all(ctx, case)
     for p in case.parts:
-        rows = np.arange(p["q"][0], p["q"][0] + 3)
+        rows = np.arange(p["q"][0], p["q"][0] + 6)
         _, want = case.oracle_fwd(p, rows=rows)
         got = case.LSE[:, torch.as_tensor(rows, device="cuda")].t().cpu().numpy()
         assert np.abs(got - want).max() <= 1e-5
