@@ -315,11 +315,12 @@ struct PairWalk {
 //  - All slabs evenly, over the tiles' borders: a pair then has up to two epilogues, EPILOGUE slabs together with the
 //    loss of step.  Taken where it saves more than that and two ninths of the time.  (2,560 x 1,024, 40 tiles: inner
 //    1,536 17.5 -> 18.5, 4,096 30.8 -> 24.7; 8,704 x 1,024, 62 tiles left: inner 32,768 513 -> 559.)  Where the inner
-//    dimension is LONG the pairs drift too far apart for L2 unless a third is saved.  (8,192 x 1,024, 54 tiles left:
-//    inner 20,480 320 -> 288, 65,536 960 -> 1,040; 48 tiles and fewer: 1.01 to 1.3 times faster.)
+//    dimension is LONG the pairs drift too far apart for L2 unless a third is saved, and at the power cap whole tiles
+//    lose less than the clock alone says.  (52 to 54 tiles left: 8,192 x 1,024, inner 65,536 960 -> 1,040; 5,120 x 2,536
+//    among the other products of a projection for seconds, inner 24,696 1,942 -> 1,968 in all, 12,000 955 -> 956.)
 int deal_last_wave(long long tiles, long long fit, long long n_k)
 {
-    constexpr long long EPILOGUE = 18, MIN_SHARE = 8, LONG = 400; // in slabs
+    constexpr long long EPILOGUE = 18, MIN_SHARE = 8, LONG = 200; // in slabs
     const long long left = tiles % fit;
     if (left == 0)
         return 0;
